@@ -203,11 +203,6 @@ __global__ void sqrt_kernel(double* x, int n) {
   if (i < n) x[i] = sqrt(x[i]);
 }
 
-__global__ void count_active_kernel(const int32_t* done, int R, int32_t* active) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < R && !done[i]) atomicAdd(active, 1);
-}
-
 }  // namespace
 
 void s_project(const double2* X, const int64_t* ptr, const int32_t* edge, const double* w, const double* nrm, int ns,
@@ -260,11 +255,6 @@ void tikhonov(const int32_t* tet_nb, const double* w, const double* eps, int64_t
 void sqrt_inplace(double* x, int n, cudaStream_t s) {
   note_launch(1);
   sqrt_kernel<<<(n + 127) / 128, 128, 0, s>>>(x, n); }
-void count_active(const int32_t* done, int R, int32_t* active, cudaStream_t s) {
-  note_launch(1);
-  count_active_kernel<<<(R + 127) / 128, 128, 0, s>>>(done, R, active);
-}
-
 }  // namespace mwk
 
 namespace mwk {

@@ -58,7 +58,9 @@ inline Shape shape_for(int R) {
 // warps split into S = 16 / nvec row slots per vector.  A warp walks its rows in passes of kUnroll
 // rows with all loads of a pass issued together (V_i from HBM, w shared by the block's warps
 // through L1); each pass is summed in the vector precision and added to an FP64 accumulator.
-// No block-level synchronisation.  Part index p = block * S + slot.
+// The S row slots of a vector are then added in slot order through shared memory, so a block
+// leaves one part (p = block), and the grid holds no block without rows: a short block (13k rows,
+// 8 columns) used to leave 9,728 parts, whose sums took 80 us against 17 us for the dots.
 constexpr int kDotThreads = 512;
 constexpr int kDotWarps = kDotThreads / 32;
 constexpr int kDotVecPerWarp = 4;   // nvec <= 64 = 16 warps x 4
@@ -147,17 +149,32 @@ __global__ void __launch_bounds__(kDotThreads) cgs_dots_kernel(const T* __restri
       acc[a][q] = make_double2(x, y);
     }
   }
-  if (lrow == 0 && active_c) {
-    const int64_t p = (int64_t)blockIdx.x * S + slot;
+  if (S == 1) {
+    if (lrow == 0 && active_c) {
 #pragma unroll
-    for (int a = 0; a < kDotVecPerWarp; ++a) {
-      if (a < nmine) {
-        const int i = i_first + a * i_step;
+      for (int a = 0; a < kDotVecPerWarp; ++a) {
+        if (a < nmine) {
+          const int i = i_first + a * i_step;
 #pragma unroll
-        for (int q = 0; q < CPL; ++q)
-          if (c0 + q < R) part[(p * nvec + i) * R + c0 + q] = acc[a][q];
+          for (int q = 0; q < CPL; ++q)
+            if (c0 + q < R) part[((int64_t)blockIdx.x * nvec + i) * R + c0 + q] = acc[a][q];
+        }
       }
     }
+    return;
+  }
+  // S > 1: nvec * S <= 16 warps, one vector each (warp = slot * nvec + i)
+  __shared__ double2 red[kDotWarps][32 * CPL];
+  if (lrow == 0 && active_c)
+#pragma unroll
+    for (int q = 0; q < CPL; ++q)
+      if (c0 + q < R) red[warp][c0 + q] = acc[0][q];
+  __syncthreads();
+  for (int t = threadIdx.x; t < nvec * R; t += kDotThreads) {
+    const int i = t / R, c = t - i * R;
+    double2 v = red[i][c];
+    for (int q = 1; q < S; ++q) v = cadd(v, red[q * nvec + i][c]);
+    part[(int64_t)blockIdx.x * nvec * R + t] = v;
   }
 }
 
@@ -375,27 +392,48 @@ __global__ void __launch_bounds__(kBdThreads, 2)
   }
 }
 
-// h[i][c] = sum_p part[p][i][c]: one warp per entry, lanes take parts lane, lane + 32, ...,
-// then a fixed shuffle tree (deterministic).
+// h[i][c] = sum_p part[p][i][c].  A block serves 8 neighbouring entries: 32 lanes per entry take
+// parts lane, lane + 32, ... (eight loads in flight, 128 contiguous bytes per part), then a fixed
+// tree through shared memory.  The loads' latency bounds it: a warp per entry, one strided load at
+// a time, took 7 us (304 parts) to 80 us (9,728 parts).
 // With vscale (the basis kept unscaled, V_i = vscale[i][c] * Vu_i), h[i][c] is scaled by it.
-__global__ void reduce_h_kernel(const double2* __restrict__ part, int nparts, int nvec, int R, double2* __restrict__ h,
-                                const double* __restrict__ vscale) {
-  const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (t >= nvec * R) return;
+constexpr int kRhEntries = 8;
+__global__ void __launch_bounds__(256) reduce_h_kernel(const double2* __restrict__ part, int nparts, int nvec, int R,
+                                                       double2* __restrict__ h, const double* __restrict__ vscale) {
+  __shared__ double2 red[32][kRhEntries];
+  const int e = threadIdx.x % kRhEntries, lane = threadIdx.x / kRhEntries;
+  const int n = nvec * R;
+  const int t = blockIdx.x * kRhEntries + e;
   double x = 0.0, y = 0.0;
-  for (int p = lane; p < nparts; p += 32) {
-    const double2 v = part[(int64_t)p * nvec * R + t];
-    x += v.x;
-    y += v.y;
+  if (t < n) {
+    const double2* pt = part + t;
+    int p = lane;
+    for (; p + 7 * 32 < nparts; p += 8 * 32) {
+      double2 v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = pt[(int64_t)(p + u * 32) * n];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        x += v[u].x;
+        y += v[u].y;
+      }
+    }
+#pragma unroll 8
+    for (; p < nparts; p += 32) {
+      const double2 v = pt[(int64_t)p * n];
+      x += v.x;
+      y += v.y;
+    }
   }
-  for (int off = 16; off > 0; off >>= 1) {
-    x += __shfl_xor_sync(0xffffffffu, x, off);
-    y += __shfl_xor_sync(0xffffffffu, y, off);
+  red[lane][e] = make_double2(x, y);
+  __syncthreads();
+  for (int st = 16; st > 0; st >>= 1) {
+    if (lane < st) red[lane][e] = cadd(red[lane][e], red[lane + st][e]);
+    __syncthreads();
   }
-  if (lane == 0) {
+  if (lane == 0 && t < n) {
     const double sc = vscale ? vscale[t] : 1.0;
-    h[t] = make_double2(x * sc, y * sc);
+    h[t] = make_double2(red[0][e].x * sc, red[0][e].y * sc);
   }
 }
 
@@ -668,12 +706,28 @@ __global__ void __launch_bounds__(kThreads) colnorm2_kernel(const T* __restrict_
     }
 }
 
-__global__ void reduce_cols_kernel(const double* __restrict__ part, int nparts, int R, double* __restrict__ out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= R) return;
+// Sum of part[p][c] over the parts of one column by a block of kColThreads threads (thread t takes
+// parts t, t + kColThreads, ..., then a fixed tree); valid in every thread.  One thread per column
+// walked up to 608 parts one load at a time: 64 us.
+constexpr int kColThreads = 128;
+__device__ __forceinline__ double sum_column_parts(const double* __restrict__ part, int nparts, int R, int c) {
+  __shared__ double red[kColThreads];
   double s = 0.0;
-  for (int p = 0; p < nparts; ++p) s += part[(int64_t)p * R + c];
-  out[c] = s;
+#pragma unroll 8
+  for (int p = threadIdx.x; p < nparts; p += kColThreads) s += part[(int64_t)p * R + c];
+  red[threadIdx.x] = s;
+  __syncthreads();
+  for (int st = kColThreads / 2; st > 0; st >>= 1) {
+    if ((int)threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
+    __syncthreads();
+  }
+  return red[0];
+}
+
+__global__ void __launch_bounds__(kColThreads) reduce_cols_kernel(const double* __restrict__ part, int nparts, int R,
+                                                                  double* __restrict__ out) {
+  const double s = sum_column_parts(part, nparts, R, blockIdx.x);
+  if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
@@ -705,6 +759,7 @@ __global__ void __launch_bounds__(32 * kGivensWarps) givens_kernel(
   double2* rc = rc_all[wib];
   double2* rs = rs_all[wib];
   double nn = 0.0;
+#pragma unroll 8
   for (int p = lane; p < nparts; p += 32) nn += npart[(int64_t)p * R + c];
   for (int off = 16; off > 0; off >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, off);
   const double hn = sqrt(nn);
@@ -770,25 +825,23 @@ __global__ void scale_cols_kernel(T* __restrict__ v, const double* __restrict__ 
   }
 }
 
-// Start of a cycle: ||r|| from partials, per-column target and state; columns already within
-// tol of ||b|| are marked done.
-__global__ void start_state_kernel(const double* __restrict__ npart, int nparts, int R, const double* __restrict__ bnorm,
-                                   double tol, double inner_tol, int fp64_mode, double* __restrict__ rnorm,
-                                   double2* __restrict__ g, double* __restrict__ target, int32_t* __restrict__ done,
-                                   int32_t* __restrict__ kcol, int m) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= R) return;
-  double nn = 0.0;
-  for (int p = 0; p < nparts; ++p) nn += npart[(int64_t)p * R + c];
-  const double rn = sqrt(nn);
+// Start of a cycle, one block per column: ||r|| from partials, per-column target and state; columns
+// already within tol of ||b|| are marked done, the others counted in *active (zeroed before).
+__global__ void __launch_bounds__(kColThreads) start_state_kernel(
+    const double* __restrict__ npart, int nparts, int R, const double* __restrict__ bnorm, double tol,
+    double inner_tol, int fp64_mode, double* __restrict__ rnorm, double2* __restrict__ g, double* __restrict__ target,
+    int32_t* __restrict__ done, int32_t* __restrict__ kcol, int m, int32_t* __restrict__ active) {
+  const int c = blockIdx.x;
+  const double rn = sqrt(sum_column_parts(npart, nparts, R, c));
+  double2* gc = g + (int64_t)c * (m + 1);
+  for (int i = threadIdx.x; i <= m; i += kColThreads) gc[i] = make_double2(i == 0 ? rn : 0.0, 0.0);
+  if (threadIdx.x != 0) return;
   rnorm[c] = rn;
   const double goal = tol * bnorm[c];
   const bool conv = !(rn > goal);
   done[c] = conv ? 1 : 0;
   kcol[c] = 0;
-  double2* gc = g + (int64_t)c * (m + 1);
-  for (int i = 0; i <= m; ++i) gc[i] = make_double2(0.0, 0.0);
-  gc[0] = make_double2(rn, 0.0);
+  if (!conv) atomicAdd(active, 1);
   // FP64 mode: aim a little below tol so the recomputed true residual passes;
   // mixed mode: reduce the residual by inner_tol (never below half the final goal).
   target[c] = fp64_mode ? 0.5 * goal : fmax(inner_tol * rn, 0.5 * goal);
@@ -828,27 +881,40 @@ __global__ void normalize_start32_kernel(const float2* __restrict__ r, const dou
   }
 }
 
-// Back substitution R y = g per column (R upper triangular after the rotations).
-__global__ void hessenberg_solve_kernel(const double2* __restrict__ H, const double2* __restrict__ g,
-                                        const int32_t* __restrict__ kcol, int m, int R, double2* __restrict__ y) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= R) return;
+// Back substitution R y = g (R upper triangular after the rotations), one warp per column: the
+// triangle is brought to shared memory (packed by columns, 33 KB at 63 steps) with all lanes, then
+// column by column y_i = s_i / R_ii and the lanes subtract R_li y_i from s_l, l < i.  A thread per
+// column waited for one H entry at a time: 9 us at 3 steps, 27 us at 12.
+__global__ void __launch_bounds__(32) hessenberg_solve_kernel(const double2* __restrict__ H,
+                                                              const double2* __restrict__ g,
+                                                              const int32_t* __restrict__ kcol, int m, int R,
+                                                              double2* __restrict__ y) {
+  extern __shared__ double2 tri[];                  // [k (k + 1) / 2] triangle, then [k] right-hand side
+  const int c = blockIdx.x, lane = threadIdx.x;
   const int k = kcol[c];
   double2* yc = y + (int64_t)c * m;
   const double2* gc = g + (int64_t)c * (m + 1);
-  for (int i = k; i < m; ++i) yc[i] = make_double2(0.0, 0.0);
+  double2* sv = tri + (m * (m + 1)) / 2;
+  for (int i = k + lane; i < m; i += 32) yc[i] = make_double2(0.0, 0.0);
+  for (int i = lane; i < k; i += 32) sv[i] = gc[i];
+#pragma unroll 4
+  for (int l = 0; l < k; ++l) {
+    const double2* Hl = H + ((int64_t)c * m + l) * (m + 1);
+    for (int i = lane; i <= l; i += 32) tri[(l * (l + 1)) / 2 + i] = Hl[i];
+  }
+  __syncwarp();
   for (int i = k - 1; i >= 0; --i) {
-    double2 s = gc[i];
-    for (int l = i + 1; l < k; ++l) {
-      const double2 hv = H[((int64_t)c * m + l) * (m + 1) + i];
-      const double2 p = cmul(hv, yc[l]);
-      s.x -= p.x;
-      s.y -= p.y;
-    }
-    const double2 d = H[((int64_t)c * m + i) * (m + 1) + i];
+    const double2* Ri = tri + (i * (i + 1)) / 2;
+    const double2 d = Ri[i], s = sv[i];
     const double dd = cabs2(d);
-    yc[i] = dd > 0.0 ? make_double2((s.x * d.x + s.y * d.y) / dd, (s.y * d.x - s.x * d.y) / dd)
-                     : make_double2(0.0, 0.0);
+    const double2 yi = dd > 0.0 ? make_double2((s.x * d.x + s.y * d.y) / dd, (s.y * d.x - s.x * d.y) / dd)
+                                : make_double2(0.0, 0.0);
+    if (lane == 0) yc[i] = yi;
+    for (int l = lane; l < i; l += 32) {
+      const double2 p = cmul(Ri[l], yi);
+      sv[l] = make_double2(sv[l].x - p.x, sv[l].y - p.y);
+    }
+    __syncwarp();
   }
 }
 
@@ -1111,18 +1177,22 @@ int dots_launch(const T* V, int64_t vstride, int nvec, const T* w, int64_t E, in
   }
   Shape sh = shape_for(R);
   const int S = nvec >= kDotWarps ? 1 : kDotWarps / nvec;
+  // rows of one block pass, as in the kernel (kUnroll rows per thread)
+  const int unroll = std::max<int>(1, 16 / sh.cpl / (int)(sizeof(T) / 8));
+  const int64_t chunk = (int64_t)unroll * (32 >> sh.tpr_log2) * S;
+  const int nb = (int)std::min<int64_t>(kBlocks, (E + chunk - 1) / chunk);
   switch (sh.cpl) {
     case 1:
-      cgs_dots_kernel<T, 1><<<kBlocks, kDotThreads, 0, s>>>(V, vstride, nvec, w, E, R, sh.tpr_log2, S, part);
+      cgs_dots_kernel<T, 1><<<nb, kDotThreads, 0, s>>>(V, vstride, nvec, w, E, R, sh.tpr_log2, S, part);
       break;
     case 2:
-      cgs_dots_kernel<T, 2><<<kBlocks, kDotThreads, 0, s>>>(V, vstride, nvec, w, E, R, sh.tpr_log2, S, part);
+      cgs_dots_kernel<T, 2><<<nb, kDotThreads, 0, s>>>(V, vstride, nvec, w, E, R, sh.tpr_log2, S, part);
       break;
     default:
-      cgs_dots_kernel<T, 4><<<kBlocks, kDotThreads, 0, s>>>(V, vstride, nvec, w, E, R, sh.tpr_log2, S, part);
+      cgs_dots_kernel<T, 4><<<nb, kDotThreads, 0, s>>>(V, vstride, nvec, w, E, R, sh.tpr_log2, S, part);
       break;
   }
-  return kBlocks * S;
+  return nb;
 }
 
 template <typename T>
@@ -1156,21 +1226,23 @@ int update_launch(const T* V, int64_t vstride, int nvec, const double2* h, T* w,
     cudaFuncSetAttribute(cgs_update_kernel<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
     attr = true;
   }
+  const int rows_per_block = kThreads >> sh.tpr_log2;
+  const int nb = (int)std::min<int64_t>(kBlocks, (E + rows_per_block - 1) / rows_per_block);
   switch (sh.cpl) {
     case 1:
       cgs_update_kernel<T, 1>
-          <<<kBlocks, kThreads, smem, s>>>(V, vstride, nvec, h, w, E, R, sh.tpr_log2, npart, vscale);
+          <<<nb, kThreads, smem, s>>>(V, vstride, nvec, h, w, E, R, sh.tpr_log2, npart, vscale);
       break;
     case 2:
       cgs_update_kernel<T, 2>
-          <<<kBlocks, kThreads, smem, s>>>(V, vstride, nvec, h, w, E, R, sh.tpr_log2, npart, vscale);
+          <<<nb, kThreads, smem, s>>>(V, vstride, nvec, h, w, E, R, sh.tpr_log2, npart, vscale);
       break;
     default:
       cgs_update_kernel<T, 4>
-          <<<kBlocks, kThreads, smem, s>>>(V, vstride, nvec, h, w, E, R, sh.tpr_log2, npart, vscale);
+          <<<nb, kThreads, smem, s>>>(V, vstride, nvec, h, w, E, R, sh.tpr_log2, npart, vscale);
       break;
   }
-  return kBlocks;
+  return nb;
 }
 
 __global__ void fill_f64_kernel(double* __restrict__ x, int n, double v) {
@@ -1234,7 +1306,7 @@ int cgs_dots_f32(const float2* V, int64_t vstride, int nvec, const float2* w, in
 void reduce_h(const double2* part, int nparts, int nvec, int R, double2* h, cudaStream_t s, const double* vscale) {
   note_launch(1);
   const int n = nvec * R;
-  reduce_h_kernel<<<(n * 32 + 255) / 256, 256, 0, s>>>(part, nparts, nvec, R, h, vscale);
+  reduce_h_kernel<<<(n + kRhEntries - 1) / kRhEntries, 256, 0, s>>>(part, nparts, nvec, R, h, vscale);
 }
 int cgs_update_f64(const double2* V, int64_t vstride, int nvec, const double2* h, double2* w, int64_t E, int R,
                    double* npart, cudaStream_t s, int32_t* err, int stages, const double* vscale) {
@@ -1247,22 +1319,24 @@ int cgs_update_f32(const float2* V, int64_t vstride, int nvec, const double2* h,
 int colnorm2_f64(const double2* x, int64_t E, int R, double* npart, cudaStream_t s) {
   note_launch(1);
   Shape sh = shape_for(R);
+  const int rows_per_block = kThreads >> sh.tpr_log2;
+  const int nb = (int)std::min<int64_t>(kBlocks, (E + rows_per_block - 1) / rows_per_block);
   switch (sh.cpl) {
     case 1:
-      colnorm2_kernel<double2, 1><<<kBlocks, kThreads, 0, s>>>(x, E, R, sh.tpr_log2, npart);
+      colnorm2_kernel<double2, 1><<<nb, kThreads, 0, s>>>(x, E, R, sh.tpr_log2, npart);
       break;
     case 2:
-      colnorm2_kernel<double2, 2><<<kBlocks, kThreads, 0, s>>>(x, E, R, sh.tpr_log2, npart);
+      colnorm2_kernel<double2, 2><<<nb, kThreads, 0, s>>>(x, E, R, sh.tpr_log2, npart);
       break;
     default:
-      colnorm2_kernel<double2, 4><<<kBlocks, kThreads, 0, s>>>(x, E, R, sh.tpr_log2, npart);
+      colnorm2_kernel<double2, 4><<<nb, kThreads, 0, s>>>(x, E, R, sh.tpr_log2, npart);
       break;
   }
-  return kBlocks;
+  return nb;
 }
 void reduce_cols(const double* part, int nparts, int R, double* out, cudaStream_t s) {
   note_launch(1);
-  reduce_cols_kernel<<<(R + 127) / 128, 128, 0, s>>>(part, nparts, R, out);
+  reduce_cols_kernel<<<R, kColThreads, 0, s>>>(part, nparts, R, out);
 }
 void givens_step(const double2* h, const double* npart, int nparts, int j, int m, int R, double2* H, double2* cs,
                  double2* gvec, double* target, int32_t* done, int32_t* kcol, double* scale, int32_t* active_count,
@@ -1281,10 +1355,10 @@ void scale_cols_f32(float2* v, const double* scale, int64_t E, int R, cudaStream
 }
 void start_state(const double* npart, int nparts, int R, const double* bnorm, double tol, double inner_tol,
                  int fp64_mode, double* rnorm, double2* gvec, double* target, int32_t* done, int32_t* kcol, int m,
-                 cudaStream_t s) {
+                 int32_t* active, cudaStream_t s) {
   note_launch(1);
-  start_state_kernel<<<(R + 127) / 128, 128, 0, s>>>(npart, nparts, R, bnorm, tol, inner_tol, fp64_mode, rnorm, gvec,
-                                                      target, done, kcol, m);
+  start_state_kernel<<<R, kColThreads, 0, s>>>(npart, nparts, R, bnorm, tol, inner_tol, fp64_mode, rnorm, gvec, target,
+                                               done, kcol, m, active);
 }
 void normalize_start_f64(const double2* r, const double* rnorm, const int32_t* done, int64_t E, int R, double2* v0,
                          cudaStream_t s) {
@@ -1304,7 +1378,8 @@ void normalize_start32(const float2* r, const double* rnorm, const int32_t* done
 void solve_hessenberg(const double2* H, const double2* gvec, const int32_t* kcol, int m, int R, double2* y,
                       cudaStream_t s) {
   note_launch(1);
-  hessenberg_solve_kernel<<<(R + 127) / 128, 128, 0, s>>>(H, gvec, kcol, m, R, y);
+  const size_t smem = sizeof(double2) * (m * (m + 1) / 2 + m);   // 33 KB at the largest m = 63
+  hessenberg_solve_kernel<<<R, 32, smem, s>>>(H, gvec, kcol, m, R, y);
 }
 void update_x_f64(const double2* Z, int64_t zstride, const double2* y, const int32_t* kcol, int m, double2* x,
                   int64_t E, int R, cudaStream_t s, int32_t* err) {

@@ -31,7 +31,7 @@ void mwk::note_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed
 namespace mwk {
 void start_state(const double* npart, int nparts, int R, const double* bnorm, double tol, double inner_tol,
                  int fp64_mode, double* rnorm, double2* gvec, double* target, int32_t* done, int32_t* kcol, int m,
-                 cudaStream_t s);
+                 int32_t* active, cudaStream_t s);
 void normalize_start_f64(const double2* r, const double* rnorm, const int32_t* done, int64_t E, int R, double2* v0,
                          cudaStream_t s);
 void normalize_start_f32(const double2* r, const double* rnorm, const int32_t* done, int64_t E, int R, float2* v0,
@@ -44,7 +44,6 @@ constexpr int kMaxRestart = 63;
 
 // Launch-shape value (mw_launch_shapes.spmm_threads) that selects the halo-tiled SpMM.
 constexpr int kSpmmHaloShape = 1;
-constexpr int kDotParts = mwk::kCgsDotsMaxParts;
 
 // Distance between consecutive Krylov vectors, in complex elements: E * R rounded up to 32, so
 // every vector starts on a 256-byte boundary (bulk copies need 16).
@@ -452,9 +451,7 @@ void ensure_work(Ctx* c, int R, int m, int prec) {
     w.r32 = dalloc<float2>(c, n);
   }
   w.bblk = dalloc<double2>(c, n);
-  w.part = dalloc<double2>(c, (size_t)kDotParts * 8 * R > (size_t)kRedBlocks * (kMaxRestart + 1) * R
-                                  ? (size_t)kDotParts * 8 * R
-                                  : (size_t)kRedBlocks * (kMaxRestart + 1) * R);
+  w.part = dalloc<double2>(c, (size_t)std::max(mwk::kCgsDotsMaxParts, kRedBlocks) * (kMaxRestart + 1) * R);
   w.h = dalloc<double2>(c, (size_t)(kMaxRestart + 1) * R);
   w.H = dalloc<double2>(c, (size_t)R * m * (m + 1));
   w.cs = dalloc<double2>(c, (size_t)R * 2 * m);
@@ -1538,8 +1535,7 @@ BlockStats solve_block(Ctx* c, int f, int R, const double2* B, double2* X, const
     }
     CK(cudaMemsetAsync(w.active, 0, sizeof(int32_t), s));
     mwk::start_state(w.npart, nb, R, w.bnorm, o.tol, o.inner_tol, wp == 0, w.rnorm, w.g, w.target, w.done, w.kcol,
-                     m, s);
-    mwk::count_active(w.done, R, w.active, s);
+                     m, w.active, s);
     check_launch("cycle start");
     st.outer++;
     st.have_relres = true;

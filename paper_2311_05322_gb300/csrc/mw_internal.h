@@ -219,7 +219,7 @@ int cgs_dots_f32(const float2* V, int64_t vstride, int nvec, const float2* w, in
                  double2* part, int32_t* err, cudaStream_t s, int stages = 0);
 constexpr int kCgsDotsMinStages = 2, kCgsDotsMaxStages = 6;
 // Largest part count cgs_dots can return.
-constexpr int kCgsDotsMaxParts = 152 * 4 * 8;
+constexpr int kCgsDotsMaxParts = 152 * 4;
 // Sets conditional-node handles (cudaGraphConditionalHandle values) of one captured Arnoldi
 // step to (*active != 0); at most kMaxStepHandles handles.
 constexpr int kMaxStepHandles = 8;
