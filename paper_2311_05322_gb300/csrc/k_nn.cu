@@ -129,148 +129,245 @@ __global__ void relu_back_kernel(const float* __restrict__ z, const float* __res
     dz[i] = z[i] > 0.f ? dh[i] : 0.f;
 }
 
-// convT forward, gather form: one thread per output position (b, o), all Co channels at once;
-// per axis the inputs i with o = 2i - 1 + k are i = (o + 1 - k) / 2 for the two k of matching
-// parity.  The layer's weights sit in shared memory; every input value is read once per output
-// position.  Per output the sum runs over ci, then kz, ky, kx ascending.
-template <int CO>
-__global__ void __launch_bounds__(256) convT_fwd_kernel(const float* __restrict__ x, const float* __restrict__ w,
-                                                        const float* __restrict__ b, float* __restrict__ a,
-                                                        float* __restrict__ g, int B, int Ci, int D) {
-  extern __shared__ float sw[];                     // [Ci][CO][64]
-  for (int q = threadIdx.x; q < Ci * CO * 64; q += blockDim.x) sw[q] = w[q];
+// The transposed convolutions: D = 4, 8, 16 input positions per axis, Do = 2 D.  All three are
+// bound by operand delivery to the FP32 pipes (about 19 MFLOP per sample and direction, activations
+// and weights in L1 / L2 / shared memory): the earlier forms issued one to two loads per FMA (a tap's
+// weight and value each) and ran at 3.6 TFLOP/s.  Here a thread owns a pair of neighbouring
+// positions and several channels, reads its neighbourhood once per channel with wide loads and a
+// quadruple of taps per shared-memory load, so one load feeds four to eight FMAs.  Every sum runs in
+// the order stated at its kernel; taps outside the volume are skipped, not multiplied by zero.
+//
+// Forward.  Output o = 2 j + p of cell j takes input j + d with tap k = p + 1 - 2 d (d = -1, 0, 1):
+// a thread computes the 2 x 8 outputs of cells (jz, jy, jx), (jz, jy, jx + 1) for COG channels from
+// 3 x 3 x 4 inputs.  Walking d = +1, 0, -1 along z, then y, then x takes the taps of every output in
+// ascending order: per output the sum runs over ci, then kz, ky, kx ascending.
+constexpr int kConvThreads = 128;
+constexpr int kConvCog = 2;   // output channels per thread (forward): measured equal to 4, more blocks
+template <int D, int CI, int CO, bool RELU>
+__global__ void __launch_bounds__(kConvThreads) convT_fwd_kernel(const float* __restrict__ x,
+                                                                 const float* __restrict__ w,
+                                                                 const float* __restrict__ bias,
+                                                                 float* __restrict__ y, int B) {
+  constexpr int COG = kConvCog, DD = 2 * D;
+  __shared__ float4 sw[CI * COG * 16];              // [ci][co][kz][ky] of kx quadruples
+  const int co0 = blockIdx.y * COG;
+  for (int q = threadIdx.x; q < CI * COG * 16; q += kConvThreads)
+    sw[q] = reinterpret_cast<const float4*>(w)[(q / (COG * 16) * CO + co0) * 16 + q % (COG * 16)];
   __syncthreads();
-  const int Do = 2 * D;
-  const int64_t V = (int64_t)Do * Do * Do;
-  const int64_t total = (int64_t)B * V;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t o = t % V;
-    const int bb = (int)(t / V);
-    const int ox = (int)(o % Do), oy = (int)((o / Do) % Do), oz = (int)(o / ((int64_t)Do * Do));
-    float s[CO];
+  const int64_t t = (int64_t)blockIdx.x * kConvThreads + threadIdx.x;
+  if (t >= (int64_t)B * D * D * (D / 2)) return;
+  const int jx = 2 * (int)(t % (D / 2)), jy = (int)(t / (D / 2) % D), jz = (int)(t / (D / 2 * D) % D);
+  const int64_t bb = t / (D / 2 * D * D);
+  const bool lo[3] = {jx > 0, jy > 0, jz > 0}, hi[3] = {jx + 2 < D, jy + 1 < D, jz + 1 < D};
+  float acc[COG][2][2][2][2];                       // [co][pz][py][cell][px]
 #pragma unroll
-    for (int co = 0; co < CO; ++co) s[co] = b[co];
-    for (int ci = 0; ci < Ci; ++ci) {
-      const float* xc = x + ((int64_t)bb * Ci + ci) * D * D * D;
-      const float* wc = sw + ci * CO * 64;
-      for (int kz = (oz + 1) & 1; kz < 4; kz += 2) {
-        const int iz = (oz + 1 - kz) >> 1;
-        if (iz < 0 || iz >= D) continue;
-        for (int ky = (oy + 1) & 1; ky < 4; ky += 2) {
-          const int iy = (oy + 1 - ky) >> 1;
-          if (iy < 0 || iy >= D) continue;
-          for (int kx = (ox + 1) & 1; kx < 4; kx += 2) {
-            const int ix = (ox + 1 - kx) >> 1;
-            if (ix < 0 || ix >= D) continue;
-            const float xv = xc[(iz * D + iy) * D + ix];
-            const int kk = (kz * 4 + ky) * 4 + kx;
+  for (int co = 0; co < COG; ++co)
 #pragma unroll
-            for (int co = 0; co < CO; ++co) s[co] = fmaf(xv, wc[co * 64 + kk], s[co]);
+    for (int q = 0; q < 16; ++q) acc[co][q >> 3][(q >> 2) & 1][(q >> 1) & 1][q & 1] = bias[co0 + co];
+  for (int ci = 0; ci < CI; ++ci) {
+    const float* xc = x + ((bb * CI + ci) * D + jz) * D * D + jy * D + jx;
+    float xv[3][3][4];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+        const bool ok = (a == 1 || (a == 0 ? lo[2] : hi[2])) && (e == 1 || (e == 0 ? lo[1] : hi[1]));
+        const float* r = xc + (a - 1) * D * D + (e - 1) * D;
+        const float2 m = ok ? *reinterpret_cast<const float2*>(r) : make_float2(0.f, 0.f);
+        xv[a][e][0] = ok && lo[0] ? r[-1] : 0.f;
+        xv[a][e][1] = m.x;
+        xv[a][e][2] = m.y;
+        xv[a][e][3] = ok && hi[0] ? r[2] : 0.f;
+      }
+#pragma unroll
+    for (int a = 2; a >= 0; --a) {
+      if (!(a == 1 || (a == 0 ? lo[2] : hi[2]))) continue;
+#pragma unroll
+      for (int e = 2; e >= 0; --e) {
+        if (!(e == 1 || (e == 0 ? lo[1] : hi[1]))) continue;
+#pragma unroll
+        for (int pz = 0; pz < 2; ++pz) {
+          const int kz = pz + 3 - 2 * a;
+          if (kz < 0 || kz > 3) continue;
+#pragma unroll
+          for (int py = 0; py < 2; ++py) {
+            const int ky = py + 3 - 2 * e;
+            if (ky < 0 || ky > 3) continue;
+#pragma unroll
+            for (int co = 0; co < COG; ++co) {
+              const float4 w4 = sw[(ci * COG + co) * 16 + kz * 4 + ky];
+              float(&s)[2][2] = acc[co][pz][py];
+              // even outputs take kx = 1 (d = 0), 3 (d = -1); odd ones kx = 0 (d = 1), 2 (d = 0)
+              s[0][1] = fmaf(xv[a][e][2], w4.x, s[0][1]);
+              if (hi[0]) s[1][1] = fmaf(xv[a][e][3], w4.x, s[1][1]);
+              s[0][0] = fmaf(xv[a][e][1], w4.y, s[0][0]);
+              s[1][0] = fmaf(xv[a][e][2], w4.y, s[1][0]);
+              s[0][1] = fmaf(xv[a][e][1], w4.z, s[0][1]);
+              s[1][1] = fmaf(xv[a][e][2], w4.z, s[1][1]);
+              if (lo[0]) s[0][0] = fmaf(xv[a][e][0], w4.w, s[0][0]);
+              s[1][0] = fmaf(xv[a][e][1], w4.w, s[1][0]);
+            }
           }
         }
       }
     }
-#pragma unroll
-    for (int co = 0; co < CO; ++co) {
-      const int64_t idx = ((int64_t)bb * CO + co) * V + o;
-      a[idx] = s[co];
-      if (g) g[idx] = s[co] > 0.f ? s[co] : 0.f;
-    }
   }
+#pragma unroll
+  for (int co = 0; co < COG; ++co)
+#pragma unroll
+    for (int pz = 0; pz < 2; ++pz)
+#pragma unroll
+      for (int py = 0; py < 2; ++py) {
+        float4 v = make_float4(acc[co][pz][py][0][0], acc[co][pz][py][0][1], acc[co][pz][py][1][0],
+                               acc[co][pz][py][1][1]);
+        if (RELU) {
+          v.x = v.x > 0.f ? v.x : 0.f;
+          v.y = v.y > 0.f ? v.y : 0.f;
+          v.z = v.z > 0.f ? v.z : 0.f;
+          v.w = v.w > 0.f ? v.w : 0.f;
+        }
+        float* o = y + (((bb * CO + co0 + co) * DD + 2 * jz + pz) * DD + 2 * jy + py) * DD + 2 * jx;
+        *reinterpret_cast<float4*>(o) = v;
+      }
 }
 
-// convT backward-data: dx[b][ci][i] = sum_co sum_k w[ci][co][k] dy[b][co][2i - 1 + k]; one thread
-// per input position (b, i) and group of CIG channels (the group is blockIdx.y, so layers with
-// few positions still fill the GPU), the group's weights in shared memory.  Per output the sum
-// runs over co, then kz, ky, kx ascending.
-template <int CIG>
-__global__ void __launch_bounds__(256) convT_bwd_data_kernel(const float* __restrict__ dy,
-                                                             const float* __restrict__ w, float* __restrict__ dx,
-                                                             int B, int Co, int D, int Ci) {
-  extern __shared__ float sw[];                     // [CIG][Co][64] of channels ci0 ..
+// Backward-data: dx[b][ci][i] = sum_co sum_k w[ci][co][k] dy[b][co][2i - 1 + k], then 0 where the
+// layer's input act[b][ci][i] is not positive (the ReLU before it).  A thread owns positions
+// (iz, iy, ix), (iz, iy, ix + 1) and CIG channels (the group is blockIdx.y): per (co, kz, ky) six
+// dy values serve 8 CIG FMAs.  Per output the sum runs over co, then kz, ky, kx ascending.
+template <int D, int CI, int CO, int CIG>
+__global__ void __launch_bounds__(kConvThreads) convT_bwd_data_kernel(const float* __restrict__ dy,
+                                                                      const float* __restrict__ w,
+                                                                      const float* __restrict__ act,
+                                                                      float* __restrict__ dx, int B) {
+  constexpr int DD = 2 * D;
+  __shared__ float4 sw[CO * CIG * 16];              // [co][ci][kz][ky] of kx quadruples
   const int ci0 = blockIdx.y * CIG;
-  for (int q = threadIdx.x; q < CIG * Co * 64; q += blockDim.x) sw[q] = w[(size_t)ci0 * Co * 64 + q];
+  for (int q = threadIdx.x; q < CO * CIG * 16; q += kConvThreads) {
+    const int k = q % 16, c = q / 16 % CIG, co = q / (16 * CIG);
+    sw[q] = reinterpret_cast<const float4*>(w)[((ci0 + c) * CO + co) * 16 + k];
+  }
   __syncthreads();
-  const int Do = 2 * D;
-  const int64_t V = (int64_t)D * D * D;
-  const int64_t total = (int64_t)B * V;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = t % V;
-    const int bb = (int)(t / V);
-    const int ix = (int)(i % D), iy = (int)((i / D) % D), iz = (int)(i / ((int64_t)D * D));
-    float s[CIG];
+  const int64_t t = (int64_t)blockIdx.x * kConvThreads + threadIdx.x;
+  if (t >= (int64_t)B * D * D * (D / 2)) return;
+  const int ix = 2 * (int)(t % (D / 2)), iy = (int)(t / (D / 2) % D), iz = (int)(t / (D / 2 * D) % D);
+  const int64_t bb = t / (D / 2 * D * D);
+  const bool xlo = ix > 0, xhi = ix + 2 < D;
+  float acc[CIG][2];
 #pragma unroll
-    for (int ci = 0; ci < CIG; ++ci) s[ci] = 0.f;
-    for (int co = 0; co < Co; ++co) {
-      const float* yc = dy + ((int64_t)bb * Co + co) * Do * Do * Do;
-      for (int kz = 0; kz < 4; ++kz) {
-        const int oz = 2 * iz - 1 + kz;
-        if (oz < 0 || oz >= Do) continue;
-        for (int ky = 0; ky < 4; ++ky) {
-          const int oy = 2 * iy - 1 + ky;
-          if (oy < 0 || oy >= Do) continue;
-          for (int kx = 0; kx < 4; ++kx) {
-            const int ox = 2 * ix - 1 + kx;
-            if (ox < 0 || ox >= Do) continue;
-            const float yv = yc[(oz * Do + oy) * Do + ox];
-            const int kk = (kz * 4 + ky) * 4 + kx;
+  for (int c = 0; c < CIG; ++c) acc[c][0] = acc[c][1] = 0.f;
+  for (int co = 0; co < CO; ++co) {
+    const float* yc = dy + (bb * CO + co) * DD * DD * DD;
 #pragma unroll
-            for (int ci = 0; ci < CIG; ++ci) s[ci] = fmaf(yv, sw[(ci * Co + co) * 64 + kk], s[ci]);
-          }
+    for (int kz = 0; kz < 4; ++kz) {
+      const int oz = 2 * iz - 1 + kz;
+      if (oz < 0 || oz >= DD) continue;
+      float yv[4][6];
+#pragma unroll
+      for (int ky = 0; ky < 4; ++ky) {
+        const int oy = 2 * iy - 1 + ky;
+        const bool ok = oy >= 0 && oy < DD;
+        const float* r = yc + (oz * DD + oy) * DD + 2 * ix;
+        const float4 m = ok ? *reinterpret_cast<const float4*>(r) : make_float4(0.f, 0.f, 0.f, 0.f);
+        yv[ky][0] = ok && xlo ? r[-1] : 0.f;
+        yv[ky][1] = m.x;
+        yv[ky][2] = m.y;
+        yv[ky][3] = m.z;
+        yv[ky][4] = m.w;
+        yv[ky][5] = ok && xhi ? r[4] : 0.f;
+      }
+#pragma unroll
+      for (int ky = 0; ky < 4; ++ky) {
+        const int oy = 2 * iy - 1 + ky;
+        if (oy < 0 || oy >= DD) continue;
+#pragma unroll
+        for (int c = 0; c < CIG; ++c) {
+          const float4 w4 = sw[(co * CIG + c) * 16 + kz * 4 + ky];
+          if (xlo) acc[c][0] = fmaf(yv[ky][0], w4.x, acc[c][0]);
+          acc[c][1] = fmaf(yv[ky][2], w4.x, acc[c][1]);
+          acc[c][0] = fmaf(yv[ky][1], w4.y, acc[c][0]);
+          acc[c][1] = fmaf(yv[ky][3], w4.y, acc[c][1]);
+          acc[c][0] = fmaf(yv[ky][2], w4.z, acc[c][0]);
+          acc[c][1] = fmaf(yv[ky][4], w4.z, acc[c][1]);
+          acc[c][0] = fmaf(yv[ky][3], w4.w, acc[c][0]);
+          if (xhi) acc[c][1] = fmaf(yv[ky][5], w4.w, acc[c][1]);
         }
       }
     }
+  }
 #pragma unroll
-    for (int ci = 0; ci < CIG; ++ci) dx[((int64_t)bb * Ci + ci0 + ci) * V + i] = s[ci];
+  for (int c = 0; c < CIG; ++c) {
+    const int64_t o = (((bb * CI + ci0 + c) * D + iz) * D + iy) * D + ix;
+    const float2 m = *reinterpret_cast<const float2*>(act + o);
+    *reinterpret_cast<float2*>(dx + o) = make_float2(m.x > 0.f ? acc[c][0] : 0.f, m.y > 0.f ? acc[c][1] : 0.f);
   }
 }
 
-// convT backward-weights, dW[ci][co][k] = sum_b sum_i x[b][ci][i] dy[b][co][2i - 1 + k], in two
-// fixed-order passes.  Pass 1: block (ci, co, kz, chunk) walks its chunk of the B D^3 input
-// positions for the 16 taps of one kz plane; thread t takes positions t, t + 256, ... and keeps
-// the 16 tap sums in registers; the block then sums the 256 threads' values tap by tap (thread
-// order, through shared memory) into part[chunk][ci][co][k].
-// Pass 2 sums the chunks in order.
+// Backward-weights, dW[ci][co][k] = sum_b sum_i x[b][ci][i] dy[b][co][2i - 1 + k], in two
+// fixed-order passes.  Pass 1: block (4 channels ci, co, kz; chunk) walks its chunk of the B D^3
+// input positions for the 16 taps of one kz plane; thread t takes positions t, t + 256, ... and keeps
+// the 4 x 16 tap sums in registers, so a position's 16 dy values (three loads per ky) serve 64 FMAs;
+// the block then sums the 256 threads' values tap by tap (thread order, through shared memory) into
+// part[chunk][ci][co][k].  Pass 2 sums the chunks in order.
 constexpr int kBwdWThreads = 256;
+constexpr int kBwdWCi = 4;
+constexpr size_t kBwdWSmem = sizeof(float) * kBwdWThreads * (kBwdWCi * 16 + 1);
+template <int D, int CI, int CO>
 __global__ void __launch_bounds__(kBwdWThreads) convT_bwd_w_kernel(const float* __restrict__ x,
                                                                    const float* __restrict__ dy,
-                                                                   float* __restrict__ part, int B, int Ci, int Co,
-                                                                   int D, int64_t chunk) {
-  __shared__ float red[kBwdWThreads][17];
-  const int pair = blockIdx.x >> 2, kz = blockIdx.x & 3;
-  const int ci = pair / Co, co = pair % Co;
-  const int Do = 2 * D;
-  const int64_t V = (int64_t)D * D * D, total = (int64_t)B * V;
+                                                                   float* __restrict__ part, int B, int64_t chunk) {
+  extern __shared__ float red[];                    // [256][65]
+  constexpr int DD = 2 * D, V = D * D * D;
+  const int kz = blockIdx.x & 3, co = (blockIdx.x >> 2) % CO, ci0 = (blockIdx.x >> 2) / CO * kBwdWCi;
+  const int64_t total = (int64_t)B * V;
   const int64_t p0 = (int64_t)blockIdx.y * chunk, p1 = min(total, p0 + chunk);
-  float acc[16];
+  float acc[kBwdWCi][16];
 #pragma unroll
-  for (int k = 0; k < 16; ++k) acc[k] = 0.f;
+  for (int k = 0; k < kBwdWCi * 16; ++k) acc[k >> 4][k & 15] = 0.f;
   for (int64_t t = p0 + threadIdx.x; t < p1; t += kBwdWThreads) {
-    const int64_t i = t % V;
-    const int bb = (int)(t / V);
-    const int ix = (int)(i % D), iy = (int)((i / D) % D), iz = (int)(i / ((int64_t)D * D));
+    const int i = (int)(t % V);
+    const int64_t bb = t / V;
+    const int ix = i % D, iy = i / D % D, iz = i / (D * D);
     const int oz = 2 * iz - 1 + kz;
-    if (oz < 0 || oz >= Do) continue;
-    const float xv = x[((int64_t)bb * Ci + ci) * V + i];
-    const float* yc = dy + ((int64_t)bb * Co + co) * Do * Do * Do + (int64_t)oz * Do * Do;
+    if (oz < 0 || oz >= DD) continue;
+    float xv[kBwdWCi];
+#pragma unroll
+    for (int c = 0; c < kBwdWCi; ++c) xv[c] = x[(bb * CI + ci0 + c) * V + i];
+    const float* yc = dy + (((bb * CO + co) * DD + oz) * DD + 2 * iy) * DD + 2 * ix;
+    const bool xlo = ix > 0, xhi = ix + 1 < D;
+    float yv[4][4];
 #pragma unroll
     for (int ky = 0; ky < 4; ++ky) {
-      const int oy = 2 * iy - 1 + ky;
+      const bool ok = (ky != 0 || iy > 0) && (ky != 3 || iy + 1 < D);
+      const float* r = yc + (ky - 1) * DD;
+      const float2 m = ok ? *reinterpret_cast<const float2*>(r) : make_float2(0.f, 0.f);
+      yv[ky][0] = ok && xlo ? r[-1] : 0.f;
+      yv[ky][1] = m.x;
+      yv[ky][2] = m.y;
+      yv[ky][3] = ok && xhi ? r[2] : 0.f;
+    }
 #pragma unroll
-      for (int kx = 0; kx < 4; ++kx) {
-        const int ox = 2 * ix - 1 + kx;
-        if (oy >= 0 && oy < Do && ox >= 0 && ox < Do)
-          acc[ky * 4 + kx] = fmaf(xv, yc[(int64_t)oy * Do + ox], acc[ky * 4 + kx]);
+    for (int ky = 0; ky < 4; ++ky) {
+      if (!((ky != 0 || iy > 0) && (ky != 3 || iy + 1 < D))) continue;
+#pragma unroll
+      for (int c = 0; c < kBwdWCi; ++c) {
+        if (xlo) acc[c][ky * 4] = fmaf(xv[c], yv[ky][0], acc[c][ky * 4]);
+        acc[c][ky * 4 + 1] = fmaf(xv[c], yv[ky][1], acc[c][ky * 4 + 1]);
+        acc[c][ky * 4 + 2] = fmaf(xv[c], yv[ky][2], acc[c][ky * 4 + 2]);
+        if (xhi) acc[c][ky * 4 + 3] = fmaf(xv[c], yv[ky][3], acc[c][ky * 4 + 3]);
       }
     }
   }
+  constexpr int NA = kBwdWCi * 16;
 #pragma unroll
-  for (int k = 0; k < 16; ++k) red[threadIdx.x][k] = acc[k];
+  for (int k = 0; k < NA; ++k) red[threadIdx.x * (NA + 1) + k] = acc[k >> 4][k & 15];
   __syncthreads();
-  if (threadIdx.x < 16) {
+  if (threadIdx.x < NA) {
     float sum = 0.f;
-    for (int q = 0; q < kBwdWThreads; ++q) sum += red[q][threadIdx.x];
-    part[(((int64_t)blockIdx.y * Ci + ci) * Co + co) * 64 + kz * 16 + threadIdx.x] = sum;
+#pragma unroll 16
+    for (int q = 0; q < kBwdWThreads; ++q) sum += red[q * (NA + 1) + threadIdx.x];
+    const int c = threadIdx.x >> 4;
+    part[(((int64_t)blockIdx.y * CI + ci0 + c) * CO + co) * 64 + kz * 16 + (threadIdx.x & 15)] = sum;
   }
 }
 
@@ -289,6 +386,7 @@ __global__ void chansum_kernel(const float* __restrict__ dy, int B, int Co, int6
   __shared__ float red[256];
   const int co = blockIdx.x, b = blockIdx.y;
   float s = 0.f;
+#pragma unroll 8
   for (int64_t v = threadIdx.x; v < V; v += 256) s += dy[((int64_t)b * Co + co) * V + v];
   red[threadIdx.x] = s;
   __syncthreads();
@@ -466,71 +564,58 @@ void nn_relu_back(const float* z, const float* dh, float* dz, int64_t n, cudaStr
   note_launch(1);
   relu_back_kernel<<<gsb(n), 256, 0, s>>>(z, dh, dz, n);
 }
-// The transposed convolutions keep a layer's weights (up to 16 x 16 x 64 floats, 64 KB) in
-// dynamic shared memory.
-static void allow_conv_smem() {
-  static bool done = false;
-  if (done) return;
-  const int sm = 16 * 16 * 64 * (int)sizeof(float);
-  cudaFuncSetAttribute(convT_fwd_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  cudaFuncSetAttribute(convT_fwd_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  cudaFuncSetAttribute(convT_fwd_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  cudaFuncSetAttribute(convT_bwd_data_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  cudaFuncSetAttribute(convT_bwd_data_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  cudaFuncSetAttribute(convT_bwd_data_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  done = true;
+template <int D, int CI, int CO, bool RELU>
+static void conv_fwd(const float* x, const float* w, const float* b, float* y, int B, cudaStream_t s) {
+  const int64_t n = (int64_t)B * D * D * (D / 2);
+  convT_fwd_kernel<D, CI, CO, RELU>
+      <<<dim3((unsigned)((n + kConvThreads - 1) / kConvThreads), CO / kConvCog), kConvThreads, 0, s>>>(x, w, b, y, B);
 }
 
-void nn_convT_fwd(const float* x, const float* w, const float* b, float* a, float* g, int B, int Ci, int Co, int D,
-                  cudaStream_t s) {
-  allow_conv_smem();
+void nn_convT_fwd(int layer, const float* x, const float* w, const float* b, float* y, int B, cudaStream_t s) {
   note_launch(1);
-  const int64_t n = (int64_t)B * 8 * D * D * D;
-  const size_t sm = sizeof(float) * Ci * Co * 64;
-  switch (Co) {
-    case 2:
-      convT_fwd_kernel<2><<<gsb(n), 256, sm, s>>>(x, w, b, a, g, B, Ci, D);
-      break;
-    case 8:
-      convT_fwd_kernel<8><<<gsb(n), 256, sm, s>>>(x, w, b, a, g, B, Ci, D);
-      break;
-    default:
-      convT_fwd_kernel<16><<<gsb(n), 256, sm, s>>>(x, w, b, a, g, B, Ci, D);
-      break;
-  }
+  if (layer == 0)
+    conv_fwd<4, 16, 16, true>(x, w, b, y, B, s);
+  else if (layer == 1)
+    conv_fwd<8, 16, 8, true>(x, w, b, y, B, s);
+  else
+    conv_fwd<16, 8, 2, false>(x, w, b, y, B, s);
 }
-void nn_convT_bwd(const float* x, const float* w, const float* dy, float* dx, float* dw, float* db, int B, int Ci,
-                  int Co, int D, float* part, float* wpart, cudaStream_t s) {
-  allow_conv_smem();
-  note_launch(dx ? 5 : 4);
-  if (dx) {
-    // channel groups so that every layer launches about two waves of blocks
-    const int64_t n = (int64_t)B * D * D * D;
-    const int nb = gsb(n);
-    const int cig = nb * (Ci / 8) >= 2 * 152 ? 8 : (nb * (Ci / 4) >= 2 * 152 ? 4 : 1);
-    const dim3 grid((unsigned)nb, (unsigned)(Ci / cig));
-    const size_t sm = sizeof(float) * cig * Co * 64;
-    if (cig == 8)
-      convT_bwd_data_kernel<8><<<grid, 256, sm, s>>>(dy, w, dx, B, Co, D, Ci);
-    else if (cig == 4)
-      convT_bwd_data_kernel<4><<<grid, 256, sm, s>>>(dy, w, dx, B, Co, D, Ci);
-    else
-      convT_bwd_data_kernel<1><<<grid, 256, sm, s>>>(dy, w, dx, B, Co, D, Ci);
-  }
-  {
-    // enough (ci, co, chunk) blocks for every SM twice, chunks of whole thread rounds, at most
-    // kConvChunks chunks (the workspace holds kConvChunks x Ci x Co x 64 partial sums)
-    const int64_t total = (int64_t)B * D * D * D;
-    int nchunk = (int)std::min<int64_t>(kConvChunks, std::max<int64_t>(1, (2 * 152 + Ci * Co - 1) / (Ci * Co)));
-    int64_t chunk = (total + nchunk - 1) / nchunk;
-    chunk = (chunk + kBwdWThreads - 1) / kBwdWThreads * kBwdWThreads;
-    nchunk = (int)((total + chunk - 1) / chunk);
-    convT_bwd_w_kernel<<<dim3(Ci * Co * 4, nchunk), kBwdWThreads, 0, s>>>(x, dy, wpart, B, Ci, Co, D, chunk);
-    const int64_t n = (int64_t)Ci * Co * 64;
-    convT_bwd_w_final_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(wpart, nchunk, n, dw);
-  }
-  chansum_kernel<<<dim3(Co, B), 256, 0, s>>>(dy, B, Co, (int64_t)8 * D * D * D, part);
-  chansum_final_kernel<<<1, 32, 0, s>>>(part, B, Co, db);
+
+// CIG channels of dx per thread: fewer positions (small D) take fewer channels each, so that all
+// three layers launch 16k threads or more at batch 64.
+template <int D, int CI, int CO, int CIG>
+static void conv_bwd(const float* x, const float* w, const float* dy, float* dx, float* dw, float* db, int B,
+                     float* part, float* wpart, cudaStream_t s) {
+  const int64_t n = (int64_t)B * D * D * (D / 2);
+  convT_bwd_data_kernel<D, CI, CO, CIG>
+      <<<dim3((unsigned)((n + kConvThreads - 1) / kConvThreads), CI / CIG), kConvThreads, 0, s>>>(dy, w, x, dx, B);
+  // chunks of whole thread rounds, at most kConvChunks (the workspace holds kConvChunks x CI x CO x 64
+  // partial sums), as many as make CI x CO x chunks two per SM
+  const int64_t total = (int64_t)B * D * D * D;
+  int nchunk = (int)std::min<int64_t>(kConvChunks, std::max<int64_t>(1, (2 * 152 + CI * CO - 1) / (CI * CO)));
+  int64_t chunk = (total + nchunk - 1) / nchunk;
+  chunk = (chunk + kBwdWThreads - 1) / kBwdWThreads * kBwdWThreads;
+  nchunk = (int)((total + chunk - 1) / chunk);
+  static const cudaError_t attr = cudaFuncSetAttribute(
+      convT_bwd_w_kernel<D, CI, CO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBwdWSmem);
+  (void)attr;   // a failure shows at the launch
+  convT_bwd_w_kernel<D, CI, CO>
+      <<<dim3(CI / kBwdWCi * CO * 4, nchunk), kBwdWThreads, kBwdWSmem, s>>>(x, dy, wpart, B, chunk);
+  const int64_t nw = (int64_t)CI * CO * 64;
+  convT_bwd_w_final_kernel<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(wpart, nchunk, nw, dw);
+  chansum_kernel<<<dim3(CO, B), 256, 0, s>>>(dy, B, CO, (int64_t)8 * D * D * D, part);
+  chansum_final_kernel<<<1, 32, 0, s>>>(part, B, CO, db);
+}
+
+void nn_convT_bwd(int layer, const float* x, const float* w, const float* dy, float* dx, float* dw, float* db, int B,
+                  float* part, float* wpart, cudaStream_t s) {
+  note_launch(5);
+  if (layer == 0)
+    conv_bwd<4, 16, 16, 2>(x, w, dy, dx, dw, db, B, part, wpart, s);
+  else if (layer == 1)
+    conv_bwd<8, 16, 8, 4>(x, w, dy, dx, dw, db, B, part, wpart, s);
+  else
+    conv_bwd<16, 8, 2, 8>(x, w, dy, dx, dw, db, B, part, wpart, s);
 }
 void nn_mse(const float* y, const float* t, int64_t n, float* dy, double* part, double* loss, cudaStream_t s) {
   note_launch(2);

@@ -14,13 +14,15 @@ void nn_gemm_f32(const float* A, int64_t sam, int64_t sak, const float* Bf, int6
                  size_t ws_floats = 0);
 void nn_colsum(const float* dz, int B, int N, float* db, cudaStream_t s);
 void nn_relu_back(const float* z, const float* dh, float* dz, int64_t n, cudaStream_t s);
-void nn_convT_fwd(const float* x, const float* w, const float* b, float* a, float* g, int B, int Ci, int Co, int D,
-                  cudaStream_t s);
-// part: B * Co floats of per-(channel, sample) partial sums for the bias gradient; wpart:
-// kConvChunks * Ci * Co * 64 floats of partial weight-gradient sums.
+// The decoder's transposed convolutions, layer 0: 16 -> 16 at 4^3, 1: 16 -> 8 at 8^3, 2: 8 -> 2 at
+// 16^3 (input positions).  Forward: y, after the ReLU for layers 0 and 1.
+void nn_convT_fwd(int layer, const float* x, const float* w, const float* b, float* y, int B, cudaStream_t s);
+// Backward from dy: weight and bias gradients, and dx masked by the ReLU that made x (0 where x is
+// not positive).  part: B * 16 floats of per-(channel, sample) partial sums for the bias
+// gradient; wpart: kConvChunks * 16 * 16 * 64 floats of partial weight-gradient sums.
 constexpr int kConvChunks = 64;
-void nn_convT_bwd(const float* x, const float* w, const float* dy, float* dx, float* dw, float* db, int B, int Ci,
-                  int Co, int D, float* part, float* wpart, cudaStream_t s);
+void nn_convT_bwd(int layer, const float* x, const float* w, const float* dy, float* dx, float* dw, float* db, int B,
+                  float* part, float* wpart, cudaStream_t s);
 void nn_mse(const float* y, const float* t, int64_t n, float* dy, double* part, double* loss, cudaStream_t s);
 void nn_adam(float* th, const float* g, float* m, float* v, int64_t n, float lr, float b1, float b2, float eps, int step,
              cudaStream_t s);

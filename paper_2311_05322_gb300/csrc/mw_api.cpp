@@ -174,13 +174,12 @@ struct NnState {
   int step = 0;
   float *theta = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr;
   void *W1b = nullptr, *W2b = nullptr;
-  float *x = nullptr, *z1 = nullptr, *h1 = nullptr, *z2 = nullptr, *h2 = nullptr, *a1 = nullptr, *g1 = nullptr,
-        *a2 = nullptr, *g2 = nullptr, *y = nullptr, *t = nullptr;
+  float *x = nullptr, *z1 = nullptr, *h1 = nullptr, *z2 = nullptr, *h2 = nullptr, *g1 = nullptr,
+        *g2 = nullptr, *y = nullptr, *t = nullptr;
   float* gws = nullptr;       // split-K partial sums of the dense layers [32][bcap][1024]
   float* cpart = nullptr;     // per-(channel, sample) partial bias sums [bcap][16]
   float* wpart = nullptr;     // partial weight-gradient sums of the decoder [kConvChunks][16][16][64]
-  float *dy = nullptr, *dg2 = nullptr, *da2 = nullptr, *dg1 = nullptr, *da1 = nullptr, *dh2 = nullptr,
-        *dz2 = nullptr, *dh1 = nullptr, *dz1 = nullptr;
+  float *dy = nullptr, *da2 = nullptr, *da1 = nullptr, *dz2 = nullptr, *dh1 = nullptr, *dz1 = nullptr;
   double *part = nullptr, *loss = nullptr;
   float *data_x = nullptr, *data_t = nullptr;
   int64_t data_n = 0;
@@ -3557,9 +3556,9 @@ int64_t mw_nn_param_count(int32_t n_in) {
 static void nn_free(Ctx* c) {
   NnState& n = c->nn;
   for (void* p : {(void*)n.theta, (void*)n.grad, (void*)n.m, (void*)n.v, n.W1b, n.W2b, (void*)n.x, (void*)n.z1,
-                  (void*)n.h1, (void*)n.z2, (void*)n.h2, (void*)n.a1, (void*)n.g1, (void*)n.a2, (void*)n.g2,
-                  (void*)n.y, (void*)n.t, (void*)n.dy, (void*)n.dg2, (void*)n.da2, (void*)n.dg1, (void*)n.da1,
-                  (void*)n.dh2, (void*)n.dz2, (void*)n.dh1, (void*)n.dz1, (void*)n.part, (void*)n.loss,
+                  (void*)n.h1, (void*)n.z2, (void*)n.h2, (void*)n.g1, (void*)n.g2,
+                  (void*)n.y, (void*)n.t, (void*)n.dy, (void*)n.da2, (void*)n.da1,
+                  (void*)n.dz2, (void*)n.dh1, (void*)n.dz1, (void*)n.part, (void*)n.loss,
                   (void*)n.gws, (void*)n.cpart, (void*)n.wpart,
                   (void*)n.data_x, (void*)n.data_t, (void*)n.idx})
     dfree(c, p);
@@ -3569,9 +3568,9 @@ static void nn_free(Ctx* c) {
 static void nn_batch_buffers(Ctx* c, int B) {
   NnState& n = c->nn;
   if (B <= n.bcap) return;
-  for (void* p : {(void*)n.x, (void*)n.z1, (void*)n.h1, (void*)n.z2, (void*)n.h2, (void*)n.a1, (void*)n.g1, (void*)n.a2,
-                  (void*)n.g2, (void*)n.y, (void*)n.t, (void*)n.dy, (void*)n.dg2, (void*)n.da2, (void*)n.dg1,
-                  (void*)n.da1, (void*)n.dh2, (void*)n.dz2, (void*)n.dh1, (void*)n.dz1, (void*)n.idx, (void*)n.gws,
+  for (void* p : {(void*)n.x, (void*)n.z1, (void*)n.h1, (void*)n.z2, (void*)n.h2, (void*)n.g1,
+                  (void*)n.g2, (void*)n.y, (void*)n.t, (void*)n.dy, (void*)n.da2,
+                  (void*)n.da1, (void*)n.dz2, (void*)n.dh1, (void*)n.dz1, (void*)n.idx, (void*)n.gws,
                   (void*)n.cpart, (void*)n.wpart})
     dfree(c, p);
   n.wpart = dalloc<float>(c, (size_t)mwk::kConvChunks * 16 * 16 * 64);
@@ -3582,18 +3581,13 @@ static void nn_batch_buffers(Ctx* c, int B) {
   n.h1 = dalloc<float>(c, (size_t)B * kHid);
   n.z2 = dalloc<float>(c, (size_t)B * kHid);
   n.h2 = dalloc<float>(c, (size_t)B * kHid);
-  n.a1 = dalloc<float>(c, (size_t)B * 16 * 512);
   n.g1 = dalloc<float>(c, (size_t)B * 16 * 512);
-  n.a2 = dalloc<float>(c, (size_t)B * 8 * 4096);
   n.g2 = dalloc<float>(c, (size_t)B * 8 * 4096);
   n.y = dalloc<float>(c, (size_t)B * kOut);
   n.t = dalloc<float>(c, (size_t)B * kOut);
   n.dy = dalloc<float>(c, (size_t)B * kOut);
-  n.dg2 = dalloc<float>(c, (size_t)B * 8 * 4096);
   n.da2 = dalloc<float>(c, (size_t)B * 8 * 4096);
-  n.dg1 = dalloc<float>(c, (size_t)B * 16 * 512);
   n.da1 = dalloc<float>(c, (size_t)B * 16 * 512);
-  n.dh2 = dalloc<float>(c, (size_t)B * kHid);
   n.dz2 = dalloc<float>(c, (size_t)B * kHid);
   n.dh1 = dalloc<float>(c, (size_t)B * kHid);
   n.dz1 = dalloc<float>(c, (size_t)B * kHid);
@@ -3624,9 +3618,9 @@ static void nn_forward(Ctx* c, int B) {
   // each input voxel meets 4^3 taps per (ci, co) pair: 16x16 at 4^3, 16x8 at 8^3, 8x2 at 16^3
   ProfScope ps(c, MW_K_NN_CONV, 4.0 * Bd * (H + 2 * 2 * 16 * 512 + 2 * 8 * 4096 + kOut),
                2.0 * 64 * Bd * (16 * 16 * 64 + 16 * 8 * 512 + 8 * 2 * 4096));
-  mwk::nn_convT_fwd(n.h2, th + n.oC1, th + n.oc1, n.a1, n.g1, B, 16, 16, 4, s);
-  mwk::nn_convT_fwd(n.g1, th + n.oC2, th + n.oc2, n.a2, n.g2, B, 16, 8, 8, s);
-  mwk::nn_convT_fwd(n.g2, th + n.oC3, th + n.oc3, n.y, nullptr, B, 8, 2, 16, s);
+  mwk::nn_convT_fwd(0, n.h2, th + n.oC1, th + n.oc1, n.g1, B, s);
+  mwk::nn_convT_fwd(1, n.g1, th + n.oC2, th + n.oc2, n.g2, B, s);
+  mwk::nn_convT_fwd(2, n.g2, th + n.oC3, th + n.oc3, n.y, B, s);
 }
 
 // loss against n.t and gradient into n.grad
@@ -3645,16 +3639,13 @@ static void nn_backward(Ctx* c, int B) {
     // flops; the first layer's input gradient is the reshaped dh2), ReLU masks between them
     ProfScope ps(c, MW_K_NN_CONV, 4.0 * Bd * (kOut + 3 * 2 * 8 * 4096 + 3 * 2 * 16 * 512 + 2 * H),
                  4.0 * 64 * Bd * (16 * 16 * 64 + 16 * 8 * 512 + 8 * 2 * 4096));
-    mwk::nn_convT_bwd(n.g2, th + n.oC3, n.dy, n.dg2, g + n.oC3, g + n.oc3, B, 8, 2, 16, n.cpart, n.wpart, s);
-    mwk::nn_relu_back(n.a2, n.dg2, n.da2, (int64_t)B * 8 * 4096, s);
-    mwk::nn_convT_bwd(n.g1, th + n.oC2, n.da2, n.dg1, g + n.oC2, g + n.oc2, B, 16, 8, 8, n.cpart, n.wpart, s);
-    mwk::nn_relu_back(n.a1, n.dg1, n.da1, (int64_t)B * 16 * 512, s);
-    mwk::nn_convT_bwd(n.h2, th + n.oC1, n.da1, n.dh2, g + n.oC1, g + n.oc1, B, 16, 16, 4, n.cpart, n.wpart, s);
+    mwk::nn_convT_bwd(2, n.g2, th + n.oC3, n.dy, n.da2, g + n.oC3, g + n.oc3, B, n.cpart, n.wpart, s);
+    mwk::nn_convT_bwd(1, n.g1, th + n.oC2, n.da2, n.da1, g + n.oC2, g + n.oc2, B, n.cpart, n.wpart, s);
+    mwk::nn_convT_bwd(0, n.h2, th + n.oC1, n.da1, n.dz2, g + n.oC1, g + n.oc1, B, n.cpart, n.wpart, s);
   }
   // dW2 = dz2^T h1, dh1 = dz2 W2 (BF16 W2), dW1 = dz1^T x; bias sums and ReLU masks between
   ProfScope ps(c, MW_K_NN_GEMM, 4.0 * H * (H + ni) + 2.0 * H * H + 4.0 * Bd * (ni + 6 * H) + 8.0 * H,
                2.0 * Bd * H * (2 * H + ni));
-  mwk::nn_relu_back(n.z2, n.dh2, n.dz2, (int64_t)B * kHid, s);
   const size_t wsf = (size_t)32 * n.bcap * kHid;
   mwk::nn_gemm_f32(n.dz2, 1, kHid, n.h1, kHid, 1, nullptr, g + n.oW2, nullptr, kHid, kHid, B, s, n.gws, wsf);
   mwk::nn_colsum(n.dz2, B, kHid, g + n.ob2, s);
