@@ -4,16 +4,18 @@
 #include <stdint.h>
 
 namespace mwk {
-// C = A B (+ bias), optional H = relu(C).  ws (ws_floats floats, may be null): partial sums of a
+// Dense layers with BF16 weights W [N][K], FP32 elsewhere.  ws (ws_floats floats): partial sums of a
 // split K, used when the tile grid alone would leave SMs idle; the split sums in a fixed order.
-void nn_gemm_bf16(const float* A, int64_t sam, int64_t sak, const void* Bw, int64_t sbk, int64_t sbn,
-                  const float* bias, float* C, float* H, int M, int N, int K, cudaStream_t s, float* ws = nullptr,
-                  size_t ws_floats = 0);
-void nn_gemm_f32(const float* A, int64_t sam, int64_t sak, const float* Bf, int64_t sbk, int64_t sbn,
-                 const float* bias, float* C, float* H, int M, int N, int K, cudaStream_t s, float* ws = nullptr,
-                 size_t ws_floats = 0);
+// h [B][N] = relu(x [B][K] W^T + bias)
+void nn_dense_fwd(const float* x, const void* W, const float* bias, float* h, int B, int N, int K, float* ws,
+                  size_t ws_floats, cudaStream_t s);
+// dx [B][K] = dz [B][N] W where h [B][K] > 0, else 0 (h: the ReLU output that entered the layer)
+void nn_dense_bwd_data(const float* dz, const void* W, const float* h, float* dx, int B, int N, int K, float* ws,
+                       size_t ws_floats, cudaStream_t s);
+// dW [N][K] = dz^T x
+void nn_dense_bwd_w(const float* dz, const float* x, float* dW, int B, int N, int K, float* ws, size_t ws_floats,
+                    cudaStream_t s);
 void nn_colsum(const float* dz, int B, int N, float* db, cudaStream_t s);
-void nn_relu_back(const float* z, const float* dh, float* dz, int64_t n, cudaStream_t s);
 // The decoder's transposed convolutions, layer 0: 16 -> 16 at 4^3, 1: 16 -> 8 at 8^3, 2: 8 -> 2 at
 // 16^3 (input positions).  Forward: y, after the ReLU for layers 0 and 1.
 void nn_convT_fwd(int layer, const float* x, const float* w, const float* b, float* y, int B, cudaStream_t s);

@@ -174,12 +174,12 @@ struct NnState {
   int step = 0;
   float *theta = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr;
   void *W1b = nullptr, *W2b = nullptr;
-  float *x = nullptr, *z1 = nullptr, *h1 = nullptr, *z2 = nullptr, *h2 = nullptr, *g1 = nullptr,
+  float *x = nullptr, *h1 = nullptr, *h2 = nullptr, *g1 = nullptr,
         *g2 = nullptr, *y = nullptr, *t = nullptr;
   float* gws = nullptr;       // split-K partial sums of the dense layers [32][bcap][1024]
   float* cpart = nullptr;     // per-(channel, sample) partial bias sums [bcap][16]
   float* wpart = nullptr;     // partial weight-gradient sums of the decoder [kConvChunks][16][16][64]
-  float *dy = nullptr, *da2 = nullptr, *da1 = nullptr, *dz2 = nullptr, *dh1 = nullptr, *dz1 = nullptr;
+  float *dy = nullptr, *da2 = nullptr, *da1 = nullptr, *dz2 = nullptr, *dz1 = nullptr;
   double *part = nullptr, *loss = nullptr;
   float *data_x = nullptr, *data_t = nullptr;
   int64_t data_n = 0;
@@ -3555,10 +3555,10 @@ int64_t mw_nn_param_count(int32_t n_in) {
 
 static void nn_free(Ctx* c) {
   NnState& n = c->nn;
-  for (void* p : {(void*)n.theta, (void*)n.grad, (void*)n.m, (void*)n.v, n.W1b, n.W2b, (void*)n.x, (void*)n.z1,
-                  (void*)n.h1, (void*)n.z2, (void*)n.h2, (void*)n.g1, (void*)n.g2,
+  for (void* p : {(void*)n.theta, (void*)n.grad, (void*)n.m, (void*)n.v, n.W1b, n.W2b, (void*)n.x,
+                  (void*)n.h1, (void*)n.h2, (void*)n.g1, (void*)n.g2,
                   (void*)n.y, (void*)n.t, (void*)n.dy, (void*)n.da2, (void*)n.da1,
-                  (void*)n.dz2, (void*)n.dh1, (void*)n.dz1, (void*)n.part, (void*)n.loss,
+                  (void*)n.dz2, (void*)n.dz1, (void*)n.part, (void*)n.loss,
                   (void*)n.gws, (void*)n.cpart, (void*)n.wpart,
                   (void*)n.data_x, (void*)n.data_t, (void*)n.idx})
     dfree(c, p);
@@ -3568,18 +3568,16 @@ static void nn_free(Ctx* c) {
 static void nn_batch_buffers(Ctx* c, int B) {
   NnState& n = c->nn;
   if (B <= n.bcap) return;
-  for (void* p : {(void*)n.x, (void*)n.z1, (void*)n.h1, (void*)n.z2, (void*)n.h2, (void*)n.g1,
+  for (void* p : {(void*)n.x, (void*)n.h1, (void*)n.h2, (void*)n.g1,
                   (void*)n.g2, (void*)n.y, (void*)n.t, (void*)n.dy, (void*)n.da2,
-                  (void*)n.da1, (void*)n.dz2, (void*)n.dh1, (void*)n.dz1, (void*)n.idx, (void*)n.gws,
+                  (void*)n.da1, (void*)n.dz2, (void*)n.dz1, (void*)n.idx, (void*)n.gws,
                   (void*)n.cpart, (void*)n.wpart})
     dfree(c, p);
   n.wpart = dalloc<float>(c, (size_t)mwk::kConvChunks * 16 * 16 * 64);
   n.gws = dalloc<float>(c, (size_t)32 * B * kHid);
   n.cpart = dalloc<float>(c, (size_t)16 * B);
   n.x = dalloc<float>(c, (size_t)B * n.n_in);
-  n.z1 = dalloc<float>(c, (size_t)B * kHid);
   n.h1 = dalloc<float>(c, (size_t)B * kHid);
-  n.z2 = dalloc<float>(c, (size_t)B * kHid);
   n.h2 = dalloc<float>(c, (size_t)B * kHid);
   n.g1 = dalloc<float>(c, (size_t)B * 16 * 512);
   n.g2 = dalloc<float>(c, (size_t)B * 8 * 4096);
@@ -3589,7 +3587,6 @@ static void nn_batch_buffers(Ctx* c, int B) {
   n.da2 = dalloc<float>(c, (size_t)B * 8 * 4096);
   n.da1 = dalloc<float>(c, (size_t)B * 16 * 512);
   n.dz2 = dalloc<float>(c, (size_t)B * kHid);
-  n.dh1 = dalloc<float>(c, (size_t)B * kHid);
   n.dz1 = dalloc<float>(c, (size_t)B * kHid);
   n.idx = dalloc<int32_t>(c, (size_t)B);
   n.bcap = B;
@@ -3608,12 +3605,12 @@ static void nn_forward(Ctx* c, int B) {
   cudaStream_t s = c->stream;
   const double Bd = B, ni = n.n_in, H = kHid;
   {
-    // BF16 weights, FP32 inputs and biases read once; pre- and post-activation written
-    ProfScope ps(c, MW_K_NN_GEMM, 2.0 * H * (ni + H) + 4.0 * Bd * (ni + H) + 8.0 * H + 16.0 * Bd * H,
+    // BF16 weights, FP32 inputs and biases read once; activations written
+    ProfScope ps(c, MW_K_NN_GEMM, 2.0 * H * (ni + H) + 4.0 * Bd * (ni + H) + 8.0 * H + 8.0 * Bd * H,
                  2.0 * Bd * H * (ni + H));
     const size_t wsf = (size_t)32 * n.bcap * kHid;
-    mwk::nn_gemm_bf16(n.x, n.n_in, 1, n.W1b, 1, n.n_in, th + n.ob1, n.z1, n.h1, B, kHid, n.n_in, s, n.gws, wsf);
-    mwk::nn_gemm_bf16(n.h1, kHid, 1, n.W2b, 1, kHid, th + n.ob2, n.z2, n.h2, B, kHid, kHid, s, n.gws, wsf);
+    mwk::nn_dense_fwd(n.x, n.W1b, th + n.ob1, n.h1, B, kHid, n.n_in, n.gws, wsf, s);
+    mwk::nn_dense_fwd(n.h1, n.W2b, th + n.ob2, n.h2, B, kHid, kHid, n.gws, wsf, s);
   }
   // each input voxel meets 4^3 taps per (ci, co) pair: 16x16 at 4^3, 16x8 at 8^3, 8x2 at 16^3
   ProfScope ps(c, MW_K_NN_CONV, 4.0 * Bd * (H + 2 * 2 * 16 * 512 + 2 * 8 * 4096 + kOut),
@@ -3647,11 +3644,10 @@ static void nn_backward(Ctx* c, int B) {
   ProfScope ps(c, MW_K_NN_GEMM, 4.0 * H * (H + ni) + 2.0 * H * H + 4.0 * Bd * (ni + 6 * H) + 8.0 * H,
                2.0 * Bd * H * (2 * H + ni));
   const size_t wsf = (size_t)32 * n.bcap * kHid;
-  mwk::nn_gemm_f32(n.dz2, 1, kHid, n.h1, kHid, 1, nullptr, g + n.oW2, nullptr, kHid, kHid, B, s, n.gws, wsf);
+  mwk::nn_dense_bwd_w(n.dz2, n.h1, g + n.oW2, B, kHid, kHid, n.gws, wsf, s);
   mwk::nn_colsum(n.dz2, B, kHid, g + n.ob2, s);
-  mwk::nn_gemm_bf16(n.dz2, kHid, 1, n.W2b, kHid, 1, nullptr, n.dh1, nullptr, B, kHid, kHid, s, n.gws, wsf);
-  mwk::nn_relu_back(n.z1, n.dh1, n.dz1, (int64_t)B * kHid, s);
-  mwk::nn_gemm_f32(n.dz1, 1, kHid, n.x, n.n_in, 1, nullptr, g + n.oW1, nullptr, kHid, n.n_in, B, s, n.gws, wsf);
+  mwk::nn_dense_bwd_data(n.dz2, n.W2b, n.h1, n.dz1, B, kHid, kHid, n.gws, wsf, s);
+  mwk::nn_dense_bwd_w(n.dz1, n.x, g + n.oW1, B, kHid, n.n_in, n.gws, wsf, s);
   mwk::nn_colsum(n.dz1, B, kHid, g + n.ob1, s);
 }
 
