@@ -191,16 +191,6 @@ __global__ void gemm_reduce_kernel(const float* __restrict__ P, int nz, GemmArgs
   }
 }
 
-// Column sums of dZ [B][N] -> db [N] (fixed order).
-__global__ void colsum_kernel(const float* __restrict__ dz, int B, int N, float* __restrict__ db) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  float s = 0.f;
-#pragma unroll 16
-  for (int b = 0; b < B; ++b) s += dz[(int64_t)b * N + n];
-  db[n] = s;
-}
-
 // The transposed convolutions: D = 4, 8, 16 input positions per axis, Do = 2 D.  All three are
 // bound by operand delivery to the FP32 pipes (about 19 MFLOP per sample and direction, activations
 // and weights in L1 / L2 / shared memory): the earlier forms issued one to two loads per FMA (a tap's
@@ -236,9 +226,8 @@ __global__ void __launch_bounds__(kConvThreads) convT_fwd_kernel(const float* __
   for (int co = 0; co < COG; ++co)
 #pragma unroll
     for (int q = 0; q < 16; ++q) acc[co][q >> 3][(q >> 2) & 1][(q >> 1) & 1][q & 1] = bias[co0 + co];
-  for (int ci = 0; ci < CI; ++ci) {
-    const float* xc = x + ((bb * CI + ci) * D + jz) * D * D + jy * D + jx;
-    float xv[3][3][4];
+  const float* xc = x + (bb * CI * D + jz) * D * D + jy * D + jx;
+  auto load = [&](float (&v)[3][3][4]) {
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
@@ -246,11 +235,26 @@ __global__ void __launch_bounds__(kConvThreads) convT_fwd_kernel(const float* __
         const bool ok = (a == 1 || (a == 0 ? lo[2] : hi[2])) && (e == 1 || (e == 0 ? lo[1] : hi[1]));
         const float* r = xc + (a - 1) * D * D + (e - 1) * D;
         const float2 m = ok ? *reinterpret_cast<const float2*>(r) : make_float2(0.f, 0.f);
-        xv[a][e][0] = ok && lo[0] ? r[-1] : 0.f;
-        xv[a][e][1] = m.x;
-        xv[a][e][2] = m.y;
-        xv[a][e][3] = ok && hi[0] ? r[2] : 0.f;
+        v[a][e][0] = ok && lo[0] ? r[-1] : 0.f;
+        v[a][e][1] = m.x;
+        v[a][e][2] = m.y;
+        v[a][e][3] = ok && hi[0] ? r[2] : 0.f;
       }
+  };
+  float nx[3][3][4];
+  if (D < 16) load(nx);
+  for (int ci = 0; ci < CI; ++ci) {
+    float xv[3][3][4];
+    if (D < 16) {
+      // few warps per SM: the next channel's loads are in flight during this one's products
+#pragma unroll
+      for (int q = 0; q < 36; ++q) xv[q / 12][q / 4 % 3][q & 3] = nx[q / 12][q / 4 % 3][q & 3];
+      xc += D * D * D;
+      if (ci + 1 < CI) load(nx);
+    } else {
+      load(xv);
+      xc += D * D * D;
+    }
 #pragma unroll
     for (int a = 2; a >= 0; --a) {
       if (!(a == 1 || (a == 0 ? lo[2] : hi[2]))) continue;
@@ -328,42 +332,51 @@ __global__ void __launch_bounds__(kConvThreads) convT_bwd_data_kernel(const floa
   float acc[CIG][2];
 #pragma unroll
   for (int c = 0; c < CIG; ++c) acc[c][0] = acc[c][1] = 0.f;
-  for (int co = 0; co < CO; ++co) {
-    const float* yc = dy + (bb * CO + co) * DD * DD * DD;
+  const float* yb = dy + bb * CO * DD * DD * DD + 2 * ix;
+  // the 4 x 6 values of channel and plane it = 4 co + kz
+  auto load = [&](int it, float (&v)[4][6]) {
+    const int oz = 2 * iz - 1 + (it & 3);
+    const bool okz = oz >= 0 && oz < DD;
+    const float* yz = yb + ((it >> 2) * DD + oz) * DD * DD;
 #pragma unroll
-    for (int kz = 0; kz < 4; ++kz) {
-      const int oz = 2 * iz - 1 + kz;
-      if (oz < 0 || oz >= DD) continue;
-      float yv[4][6];
+    for (int ky = 0; ky < 4; ++ky) {
+      const int oy = 2 * iy - 1 + ky;
+      const bool ok = okz && oy >= 0 && oy < DD;
+      const float* r = yz + oy * DD;
+      const float4 m = ok ? *reinterpret_cast<const float4*>(r) : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[ky][0] = ok && xlo ? r[-1] : 0.f;
+      v[ky][1] = m.x;
+      v[ky][2] = m.y;
+      v[ky][3] = m.z;
+      v[ky][4] = m.w;
+      v[ky][5] = ok && xhi ? r[4] : 0.f;
+    }
+  };
+  float ny[4][6];
+  load(0, ny);
+  for (int it = 0; it < 4 * CO; ++it) {
+    float yv[4][6];
 #pragma unroll
-      for (int ky = 0; ky < 4; ++ky) {
-        const int oy = 2 * iy - 1 + ky;
-        const bool ok = oy >= 0 && oy < DD;
-        const float* r = yc + (oz * DD + oy) * DD + 2 * ix;
-        const float4 m = ok ? *reinterpret_cast<const float4*>(r) : make_float4(0.f, 0.f, 0.f, 0.f);
-        yv[ky][0] = ok && xlo ? r[-1] : 0.f;
-        yv[ky][1] = m.x;
-        yv[ky][2] = m.y;
-        yv[ky][3] = m.z;
-        yv[ky][4] = m.w;
-        yv[ky][5] = ok && xhi ? r[4] : 0.f;
-      }
+    for (int q = 0; q < 24; ++q) yv[q / 6][q % 6] = ny[q / 6][q % 6];
+    if (it + 1 < 4 * CO) load(it + 1, ny);          // in flight during this plane's products
+    const int oz = 2 * iz - 1 + (it & 3);
+    if (oz < 0 || oz >= DD) continue;
+    const float4* wk = sw + (it >> 2) * CIG * 16 + (it & 3) * 4;
 #pragma unroll
-      for (int ky = 0; ky < 4; ++ky) {
-        const int oy = 2 * iy - 1 + ky;
-        if (oy < 0 || oy >= DD) continue;
+    for (int ky = 0; ky < 4; ++ky) {
+      const int oy = 2 * iy - 1 + ky;
+      if (oy < 0 || oy >= DD) continue;
 #pragma unroll
-        for (int c = 0; c < CIG; ++c) {
-          const float4 w4 = sw[(co * CIG + c) * 16 + kz * 4 + ky];
-          if (xlo) acc[c][0] = fmaf(yv[ky][0], w4.x, acc[c][0]);
-          acc[c][1] = fmaf(yv[ky][2], w4.x, acc[c][1]);
-          acc[c][0] = fmaf(yv[ky][1], w4.y, acc[c][0]);
-          acc[c][1] = fmaf(yv[ky][3], w4.y, acc[c][1]);
-          acc[c][0] = fmaf(yv[ky][2], w4.z, acc[c][0]);
-          acc[c][1] = fmaf(yv[ky][4], w4.z, acc[c][1]);
-          acc[c][0] = fmaf(yv[ky][3], w4.w, acc[c][0]);
-          if (xhi) acc[c][1] = fmaf(yv[ky][5], w4.w, acc[c][1]);
-        }
+      for (int c = 0; c < CIG; ++c) {
+        const float4 w4 = wk[c * 16 + ky];
+        if (xlo) acc[c][0] = fmaf(yv[ky][0], w4.x, acc[c][0]);
+        acc[c][1] = fmaf(yv[ky][2], w4.x, acc[c][1]);
+        acc[c][0] = fmaf(yv[ky][1], w4.y, acc[c][0]);
+        acc[c][1] = fmaf(yv[ky][3], w4.y, acc[c][1]);
+        acc[c][0] = fmaf(yv[ky][2], w4.z, acc[c][0]);
+        acc[c][1] = fmaf(yv[ky][4], w4.z, acc[c][1]);
+        acc[c][0] = fmaf(yv[ky][3], w4.w, acc[c][0]);
+        if (xhi) acc[c][1] = fmaf(yv[ky][5], w4.w, acc[c][1]);
       }
     }
   }
@@ -378,55 +391,84 @@ __global__ void __launch_bounds__(kConvThreads) convT_bwd_data_kernel(const floa
 // Backward-weights, dW[ci][co][k] = sum_b sum_i x[b][ci][i] dy[b][co][2i - 1 + k], in two
 // fixed-order passes.  Pass 1: block (4 channels ci, co, kz; chunk) walks its chunk of the B D^3
 // input positions for the 16 taps of one kz plane; thread t takes positions t, t + 256, ... and keeps
-// the 4 x 16 tap sums in registers, so a position's 16 dy values (three loads per ky) serve 64 FMAs;
-// the block then sums the 256 threads' values tap by tap (thread order, through shared memory) into
-// part[chunk][ci][co][k].  Pass 2 sums the chunks in order.
+// the 4 x 16 tap sums in registers, so a position's 16 dy values (three loads per ky) serve 64 FMAs,
+// with the next position's loads in flight; the block then sums the 256 threads' values tap by tap
+// (thread order, through shared memory) into part[chunk][ci][co][k].  The blocks beyond the last chunk
+// take the bias: block (co, b) writes the tree sum of dy[b][co] to bpart[co][b].  Pass 2
+// (nn_final_sums_kernel) sums the chunks and the samples in order.
 constexpr int kBwdWThreads = 256;
 constexpr int kBwdWCi = 4;
 constexpr size_t kBwdWSmem = sizeof(float) * kBwdWThreads * (kBwdWCi * 16 + 1);
 template <int D, int CI, int CO>
 __global__ void __launch_bounds__(kBwdWThreads) convT_bwd_w_kernel(const float* __restrict__ x,
                                                                    const float* __restrict__ dy,
-                                                                   float* __restrict__ part, int B, int64_t chunk) {
+                                                                   float* __restrict__ part,
+                                                                   float* __restrict__ bpart, int B, int64_t chunk,
+                                                                   int nchunk) {
   extern __shared__ float red[];                    // [256][65]
-  constexpr int DD = 2 * D, V = D * D * D;
-  const int kz = blockIdx.x & 3, co = (blockIdx.x >> 2) % CO, ci0 = (blockIdx.x >> 2) / CO * kBwdWCi;
+  constexpr int DD = 2 * D, V = D * D * D, PB = CI / kBwdWCi * CO * 4;
+  if ((int)blockIdx.x >= PB * nchunk) {
+    const int q = blockIdx.x - PB * nchunk, co = q % CO, b = q / CO;
+    const float* yc = dy + ((int64_t)b * CO + co) * 8 * V;
+    float s = 0.f;
+#pragma unroll 16
+    for (int v = threadIdx.x; v < 8 * V; v += kBwdWThreads) s += yc[v];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    for (int st = kBwdWThreads / 2; st > 0; st >>= 1) {
+      if ((int)threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
+      __syncthreads();
+    }
+    if (threadIdx.x == 0) bpart[co * B + b] = red[0];
+    return;
+  }
+  const int pb = blockIdx.x % PB, ch = blockIdx.x / PB;
+  const int kz = pb & 3, co = (pb >> 2) % CO, ci0 = (pb >> 2) / CO * kBwdWCi;
   const int64_t total = (int64_t)B * V;
-  const int64_t p0 = (int64_t)blockIdx.y * chunk, p1 = min(total, p0 + chunk);
-  float acc[kBwdWCi][16];
-#pragma unroll
-  for (int k = 0; k < kBwdWCi * 16; ++k) acc[k >> 4][k & 15] = 0.f;
-  for (int64_t t = p0 + threadIdx.x; t < p1; t += kBwdWThreads) {
+  const int64_t p0 = (int64_t)ch * chunk, p1 = min(total, p0 + chunk);
+  struct Item {
+    float x[kBwdWCi], y[4][4];
+    bool ok, xlo, xhi, ylo, yhi;
+  };
+  auto load = [&](int64_t t, Item& v) {
     const int i = (int)(t % V);
     const int64_t bb = t / V;
     const int ix = i % D, iy = i / D % D, iz = i / (D * D);
     const int oz = 2 * iz - 1 + kz;
-    if (oz < 0 || oz >= DD) continue;
-    float xv[kBwdWCi];
+    v.ok = t < p1 && oz >= 0 && oz < DD;
+    v.xlo = ix > 0, v.xhi = ix + 1 < D, v.ylo = iy > 0, v.yhi = iy + 1 < D;
 #pragma unroll
-    for (int c = 0; c < kBwdWCi; ++c) xv[c] = x[(bb * CI + ci0 + c) * V + i];
+    for (int c = 0; c < kBwdWCi; ++c) v.x[c] = v.ok ? x[(bb * CI + ci0 + c) * V + i] : 0.f;
     const float* yc = dy + (((bb * CO + co) * DD + oz) * DD + 2 * iy) * DD + 2 * ix;
-    const bool xlo = ix > 0, xhi = ix + 1 < D;
-    float yv[4][4];
 #pragma unroll
     for (int ky = 0; ky < 4; ++ky) {
-      const bool ok = (ky != 0 || iy > 0) && (ky != 3 || iy + 1 < D);
+      const bool ok = v.ok && (ky != 0 || v.ylo) && (ky != 3 || v.yhi);
       const float* r = yc + (ky - 1) * DD;
       const float2 m = ok ? *reinterpret_cast<const float2*>(r) : make_float2(0.f, 0.f);
-      yv[ky][0] = ok && xlo ? r[-1] : 0.f;
-      yv[ky][1] = m.x;
-      yv[ky][2] = m.y;
-      yv[ky][3] = ok && xhi ? r[2] : 0.f;
+      v.y[ky][0] = ok && v.xlo ? r[-1] : 0.f;
+      v.y[ky][1] = m.x;
+      v.y[ky][2] = m.y;
+      v.y[ky][3] = ok && v.xhi ? r[2] : 0.f;
     }
+  };
+  float acc[kBwdWCi][16];
+#pragma unroll
+  for (int k = 0; k < kBwdWCi * 16; ++k) acc[k >> 4][k & 15] = 0.f;
+  Item next;
+  load(p0 + threadIdx.x, next);
+  for (int64_t t = p0 + threadIdx.x; t < p1; t += kBwdWThreads) {
+    const Item v = next;
+    load(t + kBwdWThreads, next);
+    if (!v.ok) continue;
 #pragma unroll
     for (int ky = 0; ky < 4; ++ky) {
-      if (!((ky != 0 || iy > 0) && (ky != 3 || iy + 1 < D))) continue;
+      if (!((ky != 0 || v.ylo) && (ky != 3 || v.yhi))) continue;
 #pragma unroll
       for (int c = 0; c < kBwdWCi; ++c) {
-        if (xlo) acc[c][ky * 4] = fmaf(xv[c], yv[ky][0], acc[c][ky * 4]);
-        acc[c][ky * 4 + 1] = fmaf(xv[c], yv[ky][1], acc[c][ky * 4 + 1]);
-        acc[c][ky * 4 + 2] = fmaf(xv[c], yv[ky][2], acc[c][ky * 4 + 2]);
-        if (xhi) acc[c][ky * 4 + 3] = fmaf(xv[c], yv[ky][3], acc[c][ky * 4 + 3]);
+        if (v.xlo) acc[c][ky * 4] = fmaf(v.x[c], v.y[ky][0], acc[c][ky * 4]);
+        acc[c][ky * 4 + 1] = fmaf(v.x[c], v.y[ky][1], acc[c][ky * 4 + 1]);
+        acc[c][ky * 4 + 2] = fmaf(v.x[c], v.y[ky][2], acc[c][ky * 4 + 2]);
+        if (v.xhi) acc[c][ky * 4 + 3] = fmaf(v.x[c], v.y[ky][3], acc[c][ky * 4 + 3]);
       }
     }
   }
@@ -439,54 +481,66 @@ __global__ void __launch_bounds__(kBwdWThreads) convT_bwd_w_kernel(const float* 
 #pragma unroll 16
     for (int q = 0; q < kBwdWThreads; ++q) sum += red[q * (NA + 1) + threadIdx.x];
     const int c = threadIdx.x >> 4;
-    part[(((int64_t)blockIdx.y * CI + ci0 + c) * CO + co) * 64 + kz * 16 + (threadIdx.x & 15)] = sum;
+    part[(((int64_t)ch * CI + ci0 + c) * CO + co) * 64 + kz * 16 + (threadIdx.x & 15)] = sum;
   }
 }
 
-// dw[q] = sum over chunks of part[chunk][q] (chunk order), q over Ci Co 64.
-__global__ void convT_bwd_w_final_kernel(const float* __restrict__ part, int nchunk, int64_t n, float* __restrict__ dw) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= n) return;
-  float s = 0.f;
-  for (int c = 0; c < nchunk; ++c) s += part[(int64_t)c * n + q];
-  dw[q] = s;
-}
-
-// per-channel sums of dy [B][Co][V] -> db [Co] in two fixed-order passes: block (co, b) writes
-// the tree sum of its (channel, sample) slab to part[co][b]; then db[co] = sum_b part[co][b].
-__global__ void chansum_kernel(const float* __restrict__ dy, int B, int Co, int64_t V, float* __restrict__ part) {
-  __shared__ float red[256];
-  const int co = blockIdx.x, b = blockIdx.y;
-  float s = 0.f;
-#pragma unroll 8
-  for (int64_t v = threadIdx.x; v < V; v += 256) s += dy[((int64_t)b * Co + co) * V + v];
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int st = 128; st > 0; st >>= 1) {
-    if ((int)threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
-    __syncthreads();
+// Every second-pass sum of a backward pass in one launch (eight launches of 3 to 7 us before, each
+// a chain of loads): output q of a segment is sum_{i < n} src[base(q) + i * stride] in i order.
+struct FinalSeg {
+  const float* src;
+  float* dst;
+  int count, n;          // outputs, terms per output
+  int64_t qs, is;        // src strides of the output and of the term
+};
+struct FinalSums {
+  FinalSeg seg[8];
+  int nseg;
+};
+__global__ void __launch_bounds__(128) nn_final_sums_kernel(FinalSums f) {
+  int q = blockIdx.x * 128 + threadIdx.x;
+  for (int k = 0; k < f.nseg; ++k) {
+    const FinalSeg& g = f.seg[k];
+    const int span = (g.count + 127) / 128 * 128;   // a block serves one segment
+    if (q >= span) {
+      q -= span;
+      continue;
+    }
+    if (q >= g.count) return;
+    const float* p = g.src + q * g.qs;
+    float s = 0.f;
+#pragma unroll 16
+    for (int i = 0; i < g.n; ++i) s += p[i * g.is];
+    g.dst[q] = s;
+    return;
   }
-  if (threadIdx.x == 0) part[co * B + b] = red[0];
 }
 
-__global__ void chansum_final_kernel(const float* __restrict__ part, int B, int Co, float* __restrict__ db) {
-  const int co = blockIdx.x * blockDim.x + threadIdx.x;
-  if (co >= Co) return;
-  float s = 0.f;
-  for (int b = 0; b < B; ++b) s += part[co * B + b];
-  db[co] = s;
-}
-
-// MSE: dy = 2 (y - t) / n, per-block partial sums of (y - t)^2 in FP64.
-__global__ void mse_kernel(const float* __restrict__ y, const float* __restrict__ t, int64_t n, float* __restrict__ dy,
-                           double* __restrict__ part) {
+// MSE: dy = 2 (y - t) / n, per-block partial sums of (y - t)^2 in FP64.  Block (j, b) takes elements
+// [4096 j, 4096 (j + 1)) of sample b, 16 per thread as float4s; the target of sample b is row idx[b] of t
+// (b without idx), so a minibatch's targets are read where they lie.
+constexpr int kMseChunk = 4096;
+__global__ void __launch_bounds__(256) mse_kernel(const float* __restrict__ y, const float* __restrict__ t,
+                                                  const int32_t* __restrict__ idx, int64_t width, float sc,
+                                                  float* __restrict__ dy, double* __restrict__ part) {
   __shared__ double red[256];
+  const int64_t b = blockIdx.y, o = (int64_t)blockIdx.x * kMseChunk + threadIdx.x * 4;
+  const float* yb = y + b * width + o;
+  const float* tb = t + (idx ? idx[b] : b) * width + o;
+  float* db = dy + b * width + o;
   double s = 0.0;
-  const float sc = 2.0f / (float)n;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const float d = y[i] - t[i];
-    dy[i] = sc * d;
-    s += (double)d * d;
+  float4 yv[4], tv[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    yv[u] = *reinterpret_cast<const float4*>(yb + u * 1024);
+    tv[u] = *reinterpret_cast<const float4*>(tb + u * 1024);
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const float d[4] = {yv[u].x - tv[u].x, yv[u].y - tv[u].y, yv[u].z - tv[u].z, yv[u].w - tv[u].w};
+    *reinterpret_cast<float4*>(db + u * 1024) = make_float4(sc * d[0], sc * d[1], sc * d[2], sc * d[3]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) s += (double)d[q] * d[q];
   }
   red[threadIdx.x] = s;
   __syncthreads();
@@ -494,12 +548,13 @@ __global__ void mse_kernel(const float* __restrict__ y, const float* __restrict_
     if ((int)threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
     __syncthreads();
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = red[0];
+  if (threadIdx.x == 0) part[b * gridDim.x + blockIdx.x] = red[0];
 }
 
 __global__ void sum_parts_kernel(const double* __restrict__ part, int n, double scale, double* __restrict__ out) {
   __shared__ double red[256];
   double s = 0.0;
+#pragma unroll 8
   for (int i = threadIdx.x; i < n; i += 256) s += part[i];
   red[threadIdx.x] = s;
   __syncthreads();
@@ -510,18 +565,48 @@ __global__ void sum_parts_kernel(const double* __restrict__ part, int n, double 
   if (threadIdx.x == 0) *out = red[0] * scale;
 }
 
-// Adam (Kingma & Ba) with bias correction; bc1 = 1 - b1^t, bc2 = 1 - b2^t.
-__global__ void adam_kernel(float* __restrict__ th, const float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, int64_t n, float lr, float b1, float b2, float eps, float bc1,
-                            float bc2) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    th[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+// Adam (Kingma & Ba) with bias correction; bc1 = 1 - b1^t, bc2 = 1 - b2^t.  HBM bound: four
+// parameters per thread, and the new W1 and W2 (the entries [0, n1) and [o2, o2 + n2)) leave their
+// BF16 copies on the way (a pass of their own read them again before).
+struct AdamArgs {
+  float lr, b1, b2, eps, bc1, bc2;
+  int64_t n, n1, o2, n2;
+};
+__device__ __forceinline__ void adam_update(float& th, float g, float& m, float& v, const AdamArgs& a) {
+  // the multiply-adds are spelled out so that the rounding does not hang on the compiler's choice
+  const float mi = fmaf(1.f - a.b1, g, a.b1 * m);
+  const float vi = fmaf((1.f - a.b2) * g, g, a.b2 * v);
+  m = mi;
+  v = vi;
+  th -= a.lr * (mi / a.bc1) / (sqrtf(vi / a.bc2) + a.eps);
+}
+__device__ __forceinline__ uint2 to_bf16x4(float4 v) {
+  const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+  return make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+}
+__global__ void __launch_bounds__(256) adam_kernel(float* __restrict__ th, const float* __restrict__ g,
+                                                   float* __restrict__ m, float* __restrict__ v,
+                                                   __nv_bfloat16* __restrict__ w1, __nv_bfloat16* __restrict__ w2,
+                                                   AdamArgs a) {
+  const int64_t i = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4;
+  if (i + 4 > a.n) {                                // the last, incomplete quadruple (all biases)
+    for (int64_t k = i; k < a.n; ++k) adam_update(th[k], g[k], m[k], v[k], a);
+    return;
   }
+  float4 t4 = *reinterpret_cast<float4*>(th + i), m4 = *reinterpret_cast<float4*>(m + i),
+         v4 = *reinterpret_cast<float4*>(v + i);
+  const float4 g4 = *reinterpret_cast<const float4*>(g + i);
+  adam_update(t4.x, g4.x, m4.x, v4.x, a);
+  adam_update(t4.y, g4.y, m4.y, v4.y, a);
+  adam_update(t4.z, g4.z, m4.z, v4.z, a);
+  adam_update(t4.w, g4.w, m4.w, v4.w, a);
+  *reinterpret_cast<float4*>(th + i) = t4;
+  *reinterpret_cast<float4*>(m + i) = m4;
+  *reinterpret_cast<float4*>(v + i) = v4;
+  if (i < a.n1)
+    *reinterpret_cast<uint2*>(w1 + i) = to_bf16x4(t4);
+  else if (i >= a.o2 && i < a.o2 + a.n2)
+    *reinterpret_cast<uint2*>(w2 + i - a.o2) = to_bf16x4(t4);
 }
 
 __global__ void to_bf16_kernel(const float* __restrict__ a, __nv_bfloat16* __restrict__ b, int64_t n) {
@@ -529,13 +614,13 @@ __global__ void to_bf16_kernel(const float* __restrict__ a, __nv_bfloat16* __res
     b[i] = __float2bfloat16_rn(a[i]);
 }
 
-__global__ void gather_rows_kernel(const float* __restrict__ src, const int32_t* __restrict__ idx, int n,
-                                   int64_t width, float* __restrict__ dst) {
-  const int64_t total = (int64_t)n * width;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = t / width, c = t % width;
-    dst[t] = src[(int64_t)idx[r] * width + c];
-  }
+// dst[r] = src[idx[r]], rows of `width` floats (blockIdx.y = r).
+__global__ void gather_rows_kernel(const float* __restrict__ src, const int32_t* __restrict__ idx, int64_t width,
+                                   float* __restrict__ dst) {
+  const float* p = src + (int64_t)idx[blockIdx.y] * width;
+  float* q = dst + (int64_t)blockIdx.y * width;
+  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < width; c += (int64_t)gridDim.x * blockDim.x)
+    q[c] = p[c];
 }
 
 // Mean over the 35 points of the order-4 barycentric lattice of each tet (points
@@ -633,10 +718,6 @@ void nn_dense_bwd_w(const float* dz, const float* x, float* dW, int B, int N, in
   GemmArgs g{N, K, nullptr, nullptr, dW, nullptr, N, K, B, B, false, false, false, false};
   gemm_launch<float, false, false, 64, 64, 4, 8>(dz, x, g, ws, ws_floats, s);
 }
-void nn_colsum(const float* dz, int B, int N, float* db, cudaStream_t s) {
-  note_launch(1);
-  colsum_kernel<<<(N + 31) / 32, 32, 0, s>>>(dz, B, N, db);
-}
 template <int D, int CI, int CO, bool RELU>
 static void conv_fwd(const float* x, const float* w, const float* b, float* y, int B, cudaStream_t s) {
   const int64_t n = (int64_t)B * D * D * (D / 2);
@@ -654,53 +735,84 @@ void nn_convT_fwd(int layer, const float* x, const float* w, const float* b, flo
     conv_fwd<16, 8, 2, false>(x, w, b, y, B, s);
 }
 
+// Chunks of the backward-weights sums of a layer: whole thread rounds, at most kConvChunks, as many as
+// make Ci x Co x chunks two per SM.  The count fixes the order of the sums.
+static int conv_chunks(int layer, int B, int64_t& chunk) {
+  constexpr int pairs[3] = {16 * 16, 16 * 8, 8 * 2}, vox[3] = {64, 512, 4096};
+  const int64_t total = (int64_t)B * vox[layer];
+  int nchunk = (int)std::min<int64_t>(kConvChunks, std::max<int64_t>(1, (2 * 152 + pairs[layer] - 1) / pairs[layer]));
+  chunk = (total + nchunk - 1) / nchunk;
+  chunk = (chunk + kBwdWThreads - 1) / kBwdWThreads * kBwdWThreads;
+  return (int)((total + chunk - 1) / chunk);
+}
+
 // CIG channels of dx per thread: fewer positions (small D) take fewer channels each, so that all
 // three layers launch 16k threads or more at batch 64.
-template <int D, int CI, int CO, int CIG>
-static void conv_bwd(const float* x, const float* w, const float* dy, float* dx, float* dw, float* db, int B,
-                     float* part, float* wpart, cudaStream_t s) {
+template <int LAYER, int D, int CI, int CO, int CIG>
+static void conv_bwd(const float* x, const float* w, const float* dy, float* dx, int B, float* bpart, float* wpart,
+                     cudaStream_t s) {
   const int64_t n = (int64_t)B * D * D * (D / 2);
   convT_bwd_data_kernel<D, CI, CO, CIG>
       <<<dim3((unsigned)((n + kConvThreads - 1) / kConvThreads), CI / CIG), kConvThreads, 0, s>>>(dy, w, x, dx, B);
-  // chunks of whole thread rounds, at most kConvChunks (the workspace holds kConvChunks x CI x CO x 64
-  // partial sums), as many as make CI x CO x chunks two per SM
-  const int64_t total = (int64_t)B * D * D * D;
-  int nchunk = (int)std::min<int64_t>(kConvChunks, std::max<int64_t>(1, (2 * 152 + CI * CO - 1) / (CI * CO)));
-  int64_t chunk = (total + nchunk - 1) / nchunk;
-  chunk = (chunk + kBwdWThreads - 1) / kBwdWThreads * kBwdWThreads;
-  nchunk = (int)((total + chunk - 1) / chunk);
+  int64_t chunk = 0;
+  const int nchunk = conv_chunks(LAYER, B, chunk);
   static const cudaError_t attr = cudaFuncSetAttribute(
       convT_bwd_w_kernel<D, CI, CO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBwdWSmem);
   (void)attr;   // a failure shows at the launch
-  convT_bwd_w_kernel<D, CI, CO>
-      <<<dim3(CI / kBwdWCi * CO * 4, nchunk), kBwdWThreads, kBwdWSmem, s>>>(x, dy, wpart, B, chunk);
-  const int64_t nw = (int64_t)CI * CO * 64;
-  convT_bwd_w_final_kernel<<<(unsigned)((nw + 255) / 256), 256, 0, s>>>(wpart, nchunk, nw, dw);
-  chansum_kernel<<<dim3(CO, B), 256, 0, s>>>(dy, B, CO, (int64_t)8 * D * D * D, part);
-  chansum_final_kernel<<<1, 32, 0, s>>>(part, B, CO, db);
+  convT_bwd_w_kernel<D, CI, CO><<<CI / kBwdWCi * CO * 4 * nchunk + CO * B, kBwdWThreads, kBwdWSmem, s>>>(
+      x, dy, wpart, bpart, B, chunk, nchunk);
 }
 
-void nn_convT_bwd(int layer, const float* x, const float* w, const float* dy, float* dx, float* dw, float* db, int B,
-                  float* part, float* wpart, cudaStream_t s) {
-  note_launch(5);
-  if (layer == 0)
-    conv_bwd<4, 16, 16, 2>(x, w, dy, dx, dw, db, B, part, wpart, s);
-  else if (layer == 1)
-    conv_bwd<8, 16, 8, 4>(x, w, dy, dx, dw, db, B, part, wpart, s);
-  else
-    conv_bwd<16, 8, 2, 8>(x, w, dy, dx, dw, db, B, part, wpart, s);
-}
-void nn_mse(const float* y, const float* t, int64_t n, float* dy, double* part, double* loss, cudaStream_t s) {
+// The partial sums of layer l start at these offsets of the bias and weight workspaces.
+static int64_t bpart_off(int l, int B) { return (l == 0 ? 0 : l == 1 ? 16 : 24) * (int64_t)B; }
+static int64_t wpart_off(int l) { return (int64_t)kConvChunks * 64 * (l == 0 ? 0 : l == 1 ? 256 : 384); }
+
+void nn_convT_bwd(int layer, const float* x, const float* w, const float* dy, float* dx, int B, float* bpart,
+                  float* wpart, cudaStream_t s) {
   note_launch(2);
-  const int nb = 256;
-  mse_kernel<<<nb, 256, 0, s>>>(y, t, n, dy, part);
-  sum_parts_kernel<<<1, 256, 0, s>>>(part, nb, 1.0 / (double)n, loss);
+  bpart += bpart_off(layer, B);
+  wpart += wpart_off(layer);
+  if (layer == 0)
+    conv_bwd<0, 4, 16, 16, 2>(x, w, dy, dx, B, bpart, wpart, s);
+  else if (layer == 1)
+    conv_bwd<1, 8, 16, 8, 4>(x, w, dy, dx, B, bpart, wpart, s);
+  else
+    conv_bwd<2, 16, 8, 2, 8>(x, w, dy, dx, B, bpart, wpart, s);
 }
-void nn_adam(float* th, const float* g, float* m, float* v, int64_t n, float lr, float b1, float b2, float eps, int step,
-             cudaStream_t s) {
+
+void nn_final_sums(int B, const float* bpart, const float* wpart, float* const dw[3], float* const db[3],
+                   const float* dz1, const float* dz2, int N, float* db1, float* db2, cudaStream_t s) {
   note_launch(1);
-  const float bc1 = 1.f - powf(b1, (float)step), bc2 = 1.f - powf(b2, (float)step);
-  adam_kernel<<<gsb(n), 256, 0, s>>>(th, g, m, v, n, lr, b1, b2, eps, bc1, bc2);
+  constexpr int co[3] = {16, 8, 2}, nw[3] = {16 * 16 * 64, 16 * 8 * 64, 8 * 2 * 64};
+  FinalSums f{};
+  int64_t blocks = 0;
+  auto add = [&](const float* src, float* dst, int count, int n, int64_t qs, int64_t is) {
+    f.seg[f.nseg++] = {src, dst, count, n, qs, is};
+    blocks += (count + 127) / 128;
+  };
+  for (int l = 0; l < 3; ++l) {
+    int64_t chunk = 0;
+    add(wpart + wpart_off(l), dw[l], nw[l], conv_chunks(l, B, chunk), 1, nw[l]);
+    add(bpart + bpart_off(l, B), db[l], co[l], B, B, 1);
+  }
+  add(dz2, db2, N, B, 1, N);
+  add(dz1, db1, N, B, 1, N);
+  nn_final_sums_kernel<<<(unsigned)blocks, 128, 0, s>>>(f);
+}
+
+void nn_mse(const float* y, const float* t, const int32_t* idx, int B, int64_t width, float* dy, double* part,
+            double* loss, cudaStream_t s) {
+  note_launch(2);
+  const int64_t n = B * width;
+  const int nb = (int)(width / kMseChunk);
+  mse_kernel<<<dim3(nb, B), 256, 0, s>>>(y, t, idx, width, 2.0f / (float)n, dy, part);
+  sum_parts_kernel<<<1, 256, 0, s>>>(part, nb * B, 1.0 / (double)n, loss);
+}
+void nn_adam(float* th, const float* g, float* m, float* v, void* w1, void* w2, int64_t n, int64_t n1, int64_t o2,
+             int64_t n2, float lr, float b1, float b2, float eps, int step, cudaStream_t s) {
+  note_launch(1);
+  const AdamArgs a{lr, b1, b2, eps, 1.f - powf(b1, (float)step), 1.f - powf(b2, (float)step), n, n1, o2, n2};
+  adam_kernel<<<(unsigned)((n + 1023) / 1024), 256, 0, s>>>(th, g, m, v, (__nv_bfloat16*)w1, (__nv_bfloat16*)w2, a);
 }
 void nn_to_bf16(const float* a, void* b, int64_t n, cudaStream_t s) {
   note_launch(1);
@@ -708,7 +820,8 @@ void nn_to_bf16(const float* a, void* b, int64_t n, cudaStream_t s) {
 }
 void nn_gather_rows(const float* src, const int32_t* idx, int n, int64_t width, float* dst, cudaStream_t s) {
   note_launch(1);
-  gather_rows_kernel<<<gsb((int64_t)n * width), 256, 0, s>>>(src, idx, n, width, dst);
+  gather_rows_kernel<<<dim3((unsigned)((width + 255) / 256 < 16 ? (width + 255) / 256 : 16), n), 256, 0, s>>>(
+      src, idx, width, dst);
 }
 void nn_grid_to_tets(const float* grid, int G, const double* box, const double* xyz, const int32_t* tets, int64_t T,
                      double* out, cudaStream_t s) {

@@ -177,12 +177,12 @@ struct NnState {
   float *x = nullptr, *h1 = nullptr, *h2 = nullptr, *g1 = nullptr,
         *g2 = nullptr, *y = nullptr, *t = nullptr;
   float* gws = nullptr;       // split-K partial sums of the dense layers [32][bcap][1024]
-  float* cpart = nullptr;     // per-(channel, sample) partial bias sums [bcap][16]
-  float* wpart = nullptr;     // partial weight-gradient sums of the decoder [kConvChunks][16][16][64]
+  float* cpart = nullptr;     // per-(channel, sample) partial bias sums of the decoder, 26 x bcap
+  float* wpart = nullptr;     // partial weight-gradient sums of the decoder, kConvChunks x 400 x 64
   float *dy = nullptr, *da2 = nullptr, *da1 = nullptr, *dz2 = nullptr, *dz1 = nullptr;
   double *part = nullptr, *loss = nullptr;
   float *data_x = nullptr, *data_t = nullptr;
-  int64_t data_n = 0;
+  double* losses = nullptr;   // per batch of an epoch
   int32_t* idx = nullptr;
   // parameter offsets (floats) in the flat layout W1 b1 W2 b2 C1 c1 C2 c2 C3 c3
   int64_t oW1, ob1, oW2, ob2, oC1, oc1, oC2, oc2, oC3, oc3;
@@ -372,15 +372,19 @@ T* upload_vec(Ctx* c, const std::vector<T>& h) {
 // Copies h into d, reallocating d only when its size changes (keeps the address, and so any
 // captured graph that names it, across repeated uploads of the same size).
 template <typename T>
-void upload_reuse(Ctx* c, T*& d, const std::vector<T>& h) {
-  const size_t bytes = std::max<size_t>(h.size() * sizeof(T), 16);
+void upload_reuse(Ctx* c, T*& d, const T* h, size_t n) {
+  const size_t bytes = std::max<size_t>(n * sizeof(T), 16);
   auto it = d ? c->allocs.find((void*)d) : c->allocs.end();
   if (!d || it == c->allocs.end() || it->second != bytes) {
     dfree(c, d);
     d = nullptr;
-    d = dalloc<T>(c, h.size());
+    d = dalloc<T>(c, n);
   }
-  if (!h.empty()) CK(cudaMemcpyAsync(d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice, c->stream));
+  if (n) CK(cudaMemcpyAsync(d, h, n * sizeof(T), cudaMemcpyHostToDevice, c->stream));
+}
+template <typename T>
+void upload_reuse(Ctx* c, T*& d, const std::vector<T>& h) {
+  upload_reuse(c, d, h.data(), h.size());
 }
 
 template <typename F>
@@ -3560,7 +3564,7 @@ static void nn_free(Ctx* c) {
                   (void*)n.y, (void*)n.t, (void*)n.dy, (void*)n.da2, (void*)n.da1,
                   (void*)n.dz2, (void*)n.dz1, (void*)n.part, (void*)n.loss,
                   (void*)n.gws, (void*)n.cpart, (void*)n.wpart,
-                  (void*)n.data_x, (void*)n.data_t, (void*)n.idx})
+                  (void*)n.data_x, (void*)n.data_t, (void*)n.idx, (void*)n.losses})
     dfree(c, p);
   n = NnState();
 }
@@ -3570,12 +3574,13 @@ static void nn_batch_buffers(Ctx* c, int B) {
   if (B <= n.bcap) return;
   for (void* p : {(void*)n.x, (void*)n.h1, (void*)n.h2, (void*)n.g1,
                   (void*)n.g2, (void*)n.y, (void*)n.t, (void*)n.dy, (void*)n.da2,
-                  (void*)n.da1, (void*)n.dz2, (void*)n.dz1, (void*)n.idx, (void*)n.gws,
-                  (void*)n.cpart, (void*)n.wpart})
+                  (void*)n.da1, (void*)n.dz2, (void*)n.dz1, (void*)n.gws,
+                  (void*)n.cpart, (void*)n.wpart, (void*)n.part})
     dfree(c, p);
-  n.wpart = dalloc<float>(c, (size_t)mwk::kConvChunks * 16 * 16 * 64);
+  n.wpart = dalloc<float>(c, (size_t)mwk::kConvChunks * 400 * 64);
   n.gws = dalloc<float>(c, (size_t)32 * B * kHid);
-  n.cpart = dalloc<float>(c, (size_t)16 * B);
+  n.cpart = dalloc<float>(c, (size_t)26 * B);
+  n.part = dalloc<double>(c, (size_t)(kOut / 4096) * B);
   n.x = dalloc<float>(c, (size_t)B * n.n_in);
   n.h1 = dalloc<float>(c, (size_t)B * kHid);
   n.h2 = dalloc<float>(c, (size_t)B * kHid);
@@ -3588,7 +3593,6 @@ static void nn_batch_buffers(Ctx* c, int B) {
   n.da1 = dalloc<float>(c, (size_t)B * 16 * 512);
   n.dz2 = dalloc<float>(c, (size_t)B * kHid);
   n.dz1 = dalloc<float>(c, (size_t)B * kHid);
-  n.idx = dalloc<int32_t>(c, (size_t)B);
   n.bcap = B;
 }
 
@@ -3620,8 +3624,8 @@ static void nn_forward(Ctx* c, int B) {
   mwk::nn_convT_fwd(2, n.g2, th + n.oC3, th + n.oc3, n.y, B, s);
 }
 
-// loss against n.t and gradient into n.grad
-static void nn_backward(Ctx* c, int B) {
+// mean squared error against the rows idx of t (row b without idx) into *loss, gradient into n.grad
+static void nn_backward(Ctx* c, int B, const float* t, const int32_t* idx, double* loss) {
   NnState& n = c->nn;
   const float* th = n.theta;
   float* g = n.grad;
@@ -3629,26 +3633,27 @@ static void nn_backward(Ctx* c, int B) {
   const double Bd = B, ni = n.n_in, H = kHid;
   {
     ProfScope ps(c, MW_K_NN_OTHER, 12.0 * Bd * kOut);
-    mwk::nn_mse(n.y, n.t, (int64_t)B * kOut, n.dy, n.part, n.loss, s);
+    mwk::nn_mse(n.y, t, idx, B, kOut, n.dy, n.part, loss, s);
   }
   {
     // backward-data and backward-weight of each transposed convolution (twice the forward
     // flops; the first layer's input gradient is the reshaped dh2), ReLU masks between them
     ProfScope ps(c, MW_K_NN_CONV, 4.0 * Bd * (kOut + 3 * 2 * 8 * 4096 + 3 * 2 * 16 * 512 + 2 * H),
                  4.0 * 64 * Bd * (16 * 16 * 64 + 16 * 8 * 512 + 8 * 2 * 4096));
-    mwk::nn_convT_bwd(2, n.g2, th + n.oC3, n.dy, n.da2, g + n.oC3, g + n.oc3, B, n.cpart, n.wpart, s);
-    mwk::nn_convT_bwd(1, n.g1, th + n.oC2, n.da2, n.da1, g + n.oC2, g + n.oc2, B, n.cpart, n.wpart, s);
-    mwk::nn_convT_bwd(0, n.h2, th + n.oC1, n.da1, n.dz2, g + n.oC1, g + n.oc1, B, n.cpart, n.wpart, s);
+    mwk::nn_convT_bwd(2, n.g2, th + n.oC3, n.dy, n.da2, B, n.cpart, n.wpart, s);
+    mwk::nn_convT_bwd(1, n.g1, th + n.oC2, n.da2, n.da1, B, n.cpart, n.wpart, s);
+    mwk::nn_convT_bwd(0, n.h2, th + n.oC1, n.da1, n.dz2, B, n.cpart, n.wpart, s);
   }
   // dW2 = dz2^T h1, dh1 = dz2 W2 (BF16 W2), dW1 = dz1^T x; bias sums and ReLU masks between
   ProfScope ps(c, MW_K_NN_GEMM, 4.0 * H * (H + ni) + 2.0 * H * H + 4.0 * Bd * (ni + 6 * H) + 8.0 * H,
                2.0 * Bd * H * (2 * H + ni));
   const size_t wsf = (size_t)32 * n.bcap * kHid;
   mwk::nn_dense_bwd_w(n.dz2, n.h1, g + n.oW2, B, kHid, kHid, n.gws, wsf, s);
-  mwk::nn_colsum(n.dz2, B, kHid, g + n.ob2, s);
   mwk::nn_dense_bwd_data(n.dz2, n.W2b, n.h1, n.dz1, B, kHid, kHid, n.gws, wsf, s);
   mwk::nn_dense_bwd_w(n.dz1, n.x, g + n.oW1, B, kHid, n.n_in, n.gws, wsf, s);
-  mwk::nn_colsum(n.dz1, B, kHid, g + n.ob1, s);
+  float* const dw[3] = {g + n.oC1, g + n.oC2, g + n.oC3};
+  float* const db[3] = {g + n.oc1, g + n.oc2, g + n.oc3};
+  mwk::nn_final_sums(B, n.cpart, n.wpart, dw, db, n.dz1, n.dz2, kHid, g + n.ob1, g + n.ob2, s);
 }
 
 mw_status mw_nn_init(mw_ctx* c, int32_t n_in, const float* theta) {
@@ -3678,7 +3683,6 @@ mw_status mw_nn_init(mw_ctx* c, int32_t n_in, const float* theta) {
     CK(cudaMemsetAsync(n.v, 0, sizeof(float) * n.np, c->stream));
     n.W1b = dalloc<uint16_t>(c, (size_t)kHid * n_in);
     n.W2b = dalloc<uint16_t>(c, (size_t)kHid * kHid);
-    n.part = dalloc<double>(c, 256);
     n.loss = dalloc<double>(c, 1);
     nn_refresh_bf16(c);
     check_launch("nn init");
@@ -3703,7 +3707,7 @@ mw_status mw_nn_loss_grad(mw_ctx* c, int64_t nsamp, const float* x, const float*
     CK(cudaMemcpyAsync(n.x, x, sizeof(float) * nsamp * n.n_in, cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemcpyAsync(n.t, t, sizeof(float) * nsamp * kOut, cudaMemcpyHostToDevice, c->stream));
     nn_forward(c, (int)nsamp);
-    nn_backward(c, (int)nsamp);
+    nn_backward(c, (int)nsamp, n.t, nullptr, n.loss);
     check_launch("nn loss/grad");
     CK(cudaMemcpyAsync(loss, n.loss, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     if (grad) CK(cudaMemcpyAsync(grad, n.grad, sizeof(float) * n.np, cudaMemcpyDeviceToHost, c->stream));
@@ -3726,13 +3730,20 @@ mw_status mw_nn_train(mw_ctx* c, const mw_nn_opts* o, int64_t nsamp, const float
     require(n.theta, MW_ESTATE, "network not initialised");
     require(o && nsamp >= 1 && x && t, MW_EINVAL, "bad training arguments");
     require(o->batch >= 1 && o->batch <= 4096 && o->epochs >= 0 && o->lr > 0, MW_EINVAL, "bad training options");
-    for (auto p : {(void*)n.data_x, (void*)n.data_t}) dfree(c, p);
-    n.data_x = upload(c, x, (size_t)nsamp * n.n_in);
-    n.data_t = upload(c, t, (size_t)nsamp * kOut);
-    n.data_n = nsamp;
     const int B = (int)std::min<int64_t>(o->batch, nsamp);
+    const int64_t nbatch = (nsamp + B - 1) / B;
+    // the resident training set, an epoch's order and its batches' losses
+    upload_reuse(c, n.data_x, x, (size_t)nsamp * n.n_in);
+    upload_reuse(c, n.data_t, t, (size_t)nsamp * kOut);
     nn_batch_buffers(c, B);
+    dfree(c, n.idx);
+    n.idx = nullptr;
+    n.idx = dalloc<int32_t>(c, (size_t)nsamp);
+    dfree(c, n.losses);
+    n.losses = nullptr;
+    n.losses = dalloc<double>(c, (size_t)nbatch);
     std::vector<int32_t> perm(nsamp);
+    std::vector<double> loss(nbatch);
     cudaEvent_t e0;
     CK(cudaEventCreate(&e0));
     CK(cudaEventRecord(e0, c->stream));
@@ -3743,32 +3754,33 @@ mw_status mw_nn_train(mw_ctx* c, const mw_nn_opts* o, int64_t nsamp, const float
         const int64_t j = (int64_t)(splitmix64_next(rs) % (uint64_t)(i + 1));
         std::swap(perm[i], perm[j]);
       }
-      double ep_loss = 0;
-      for (int64_t b0 = 0; b0 < nsamp; b0 += B) {
-        const int nb = (int)std::min<int64_t>(B, nsamp - b0);
-        CK(cudaMemcpyAsync(n.idx, perm.data() + b0, sizeof(int32_t) * nb, cudaMemcpyHostToDevice, c->stream));
+      CK(cudaMemcpyAsync(n.idx, perm.data(), sizeof(int32_t) * nsamp, cudaMemcpyHostToDevice, c->stream));
+      for (int64_t k = 0; k < nbatch; ++k) {
+        const int nb = (int)std::min<int64_t>(B, nsamp - k * B);
+        const int32_t* idx = n.idx + k * B;
         {
-          ProfScope ps(c, MW_K_NN_OTHER, 8.0 * nb * ((double)n.n_in + kOut));
-          mwk::nn_gather_rows(n.data_x, n.idx, nb, n.n_in, n.x, c->stream);
-          mwk::nn_gather_rows(n.data_t, n.idx, nb, kOut, n.t, c->stream);
+          ProfScope ps(c, MW_K_NN_OTHER, 8.0 * nb * (double)n.n_in);
+          mwk::nn_gather_rows(n.data_x, idx, nb, n.n_in, n.x, c->stream);
         }
         nn_forward(c, nb);
-        nn_backward(c, nb);
+        nn_backward(c, nb, n.data_t, idx, n.losses + k);
         n.step++;
         {
-          // Adam reads the parameters, gradient and both moments and writes three of them back;
-          // the BF16 copies of W1 and W2 are refreshed from the new parameters
+          // Adam reads the parameters, gradient and both moments and writes three of them and the
+          // BF16 copies of W1 and W2
           ProfScope ps(c, MW_K_NN_OTHER,
-                       28.0 * (double)n.np + 6.0 * (double)kHid * ((double)n.n_in + kHid));
-          mwk::nn_adam(n.theta, n.grad, n.m, n.v, n.np, o->lr, o->beta1, o->beta2, o->eps, n.step, c->stream);
-          nn_refresh_bf16(c);
+                       28.0 * (double)n.np + 2.0 * (double)kHid * ((double)n.n_in + kHid));
+          mwk::nn_adam(n.theta, n.grad, n.m, n.v, n.W1b, n.W2b, n.np, (int64_t)kHid * n.n_in, n.oW2,
+                       (int64_t)kHid * kHid, o->lr, o->beta1, o->beta2, o->eps, n.step, c->stream);
         }
-        double l = 0;
-        CK(cudaMemcpyAsync(&l, n.loss, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-        CK(cudaStreamSynchronize(c->stream));   // perm slice and loss are host memory
-        ep_loss += l * nb;
       }
       check_launch("nn train");
+      // one synchronisation per epoch (a host round trip per batch left the GPU idle between steps):
+      // perm and the losses are host memory
+      CK(cudaMemcpyAsync(loss.data(), n.losses, sizeof(double) * nbatch, cudaMemcpyDeviceToHost, c->stream));
+      CK(cudaStreamSynchronize(c->stream));
+      double ep_loss = 0;
+      for (int64_t k = 0; k < nbatch; ++k) ep_loss += loss[k] * (double)std::min<int64_t>(B, nsamp - k * B);
       if (st && st->epoch_loss) st->epoch_loss[ep] = ep_loss / (double)nsamp;
     }
     CK(cudaEventRecord(c->ev1, c->stream));
