@@ -1,18 +1,6 @@
-// K5 (ORAS setup) and the CUDA-core form of K4 (ORAS apply), Sec. IV-C.
-//
-// Setup, per subdomain s with n_s unknowns:
-//   1. dense local matrix  B_s = sum_{T in s} (K^T - k0^2 eps_T M^T)
-//                               + sum_{surface faces F of s} z_F B^F,
-//      z_F = i k0 sqrt(eps_F) on an interface face, eps_F the eps of the inside tet (first-order
-//      impedance transmission condition of Eq. m1 on the artificial boundary); on an outer face
-//      z_F = i k0 sqrt(eps_bg), or with face classes (waveguide ports) the global boundary's
-//      coefficient of that face (open, metal = 0, port = i beta_p); the rows and columns of
-//      metal edges are then those of the identity, as in the global matrix;
-//   2. in-place blocked Gauss-Jordan inversion without pivoting (the imaginary part of B_s is
-//      symmetric positive definite for lossy media, so every leading block is nonsingular);
-//   3. the owned rows of B_s^{-1} (restricted partition of unity, boolean D_s) are kept as
-//      W_s [n_own][n_s] in the apply precision.
-// Apply:  z[own_s] = W_s r[dofs_s]  for every s (owners partition the edges: no atomics).
+// Partial Gauss-Jordan of the multifrontal fronts (sparse form of K5) and the CUDA-core form of K4
+// (ORAS apply), Sec. IV-C.  Apply:  z[own_s] = W_s r[dofs_s]  for every s (owners partition the
+// edges: no atomics).
 #include "mw_internal.h"
 #include "k_oras.h"
 
@@ -29,92 +17,6 @@ template <>
 struct Tr<float2> {
   using S = float;
 };
-
-__device__ __forceinline__ double2 csqrt_principal(double a, double b) {
-  const double r = sqrt(a * a + b * b);
-  const double re = sqrt(0.5 * (r + a));
-  double im = sqrt(fmax(0.0, 0.5 * (r - a)));
-  if (b < 0.0) im = -im;
-  return make_double2(re, im);
-}
-
-// One warp per subdomain; tets then surface faces in list order, entries of one element by
-// different lanes (never the same matrix entry), elements in sequence (ordered by __syncwarp).
-// surf_tet codes: >= 0 inside tet of an interface face; -1 outer face with i k0 sqrt(eps_bg)
-// when zc is null, else -1 - c for an outer face of class c with coefficient zc[c].
-template <typename T>
-__global__ void local_assemble_kernel(const int32_t* __restrict__ sub_ids, const int64_t* __restrict__ dof_ptr,
-                                      const int32_t* __restrict__ dofs, const int64_t* __restrict__ tet_ptr,
-                                      const int32_t* __restrict__ tet_ids, const int32_t* __restrict__ tet_loc,
-                                      const int64_t* __restrict__ surf_ptr, const int32_t* __restrict__ surf_loc,
-                                      const int32_t* __restrict__ surf_tet, const double* __restrict__ Bsurf,
-                                      const double* __restrict__ KM, const double* __restrict__ eps, double k0,
-                                      double eps_bg_re, double eps_bg_im, const double2* __restrict__ zc,
-                                      const uint8_t* __restrict__ metal, const int64_t* __restrict__ ws_off,
-                                      T* __restrict__ ws) {
-  using Sc = typename Tr<T>::S;
-  const int b = blockIdx.x;
-  const int s = sub_ids[b];
-  const int lane = threadIdx.x;
-  const int64_t n = dof_ptr[s + 1] - dof_ptr[s];
-  T* A = ws + ws_off[b];
-  const double k0sq = k0 * k0;
-  for (int64_t q = tet_ptr[s]; q < tet_ptr[s + 1]; ++q) {
-    const int64_t t = tet_ids[q];
-    const int32_t* loc = tet_loc + 6 * q;
-    for (int e = lane; e < 36; e += 32) {
-      const int m = e / 6, nn = e % 6;
-      const int pk = mw::packed6(m, nn);
-      const double Kv = KM[42 * t + pk], Mv = KM[42 * t + 21 + pk];
-      const double re = Kv - (k0sq * eps[2 * t]) * Mv;
-      const double im = -(k0sq * eps[2 * t + 1]) * Mv;
-      T* p = A + (int64_t)loc[m] * n + loc[nn];
-      T v = *p;
-      v.x += (Sc)re;
-      v.y += (Sc)im;
-      *p = v;
-    }
-    __syncwarp();
-  }
-  const double2 sbg = csqrt_principal(eps_bg_re, eps_bg_im);
-  for (int64_t q = surf_ptr[s]; q < surf_ptr[s + 1]; ++q) {
-    if (lane < 9) {
-      const int m = lane / 3, nn = lane % 3;
-      const int32_t it = surf_tet[q];
-      const double Bv = Bsurf[6 * q + mw::packed3(m, nn)];
-      double re, im;
-      if (it < 0 && zc) {
-        const double2 z = zc[-1 - it];
-        re = z.x * Bv;
-        im = z.y * Bv;
-      } else {
-        const double2 sq = it >= 0 ? csqrt_principal(eps[2 * (int64_t)it], eps[2 * (int64_t)it + 1]) : sbg;
-        // i k0 sqrt(eps) = (-k0 Im sqrt, k0 Re sqrt)
-        re = (-k0 * sq.y) * Bv;
-        im = (k0 * sq.x) * Bv;
-      }
-      T* p = A + (int64_t)surf_loc[3 * q + m] * n + surf_loc[3 * q + nn];
-      T v = *p;
-      v.x += (Sc)re;
-      v.y += (Sc)im;
-      *p = v;
-    }
-    __syncwarp();
-  }
-  if (metal) {
-    const int32_t* gd = dofs + dof_ptr[s];
-    for (int64_t i = 0; i < n; ++i) {
-      if (!metal[gd[i]]) continue;
-      for (int64_t j = lane; j < n; j += 32) {
-        A[i * n + j] = T{0, 0};
-        A[j * n + i] = T{0, 0};
-      }
-      __syncwarp();
-      if (lane == 0) A[i * n + i] = T{1, 0};
-      __syncwarp();
-    }
-  }
-}
 
 constexpr int NB = 32;
 
@@ -324,27 +226,6 @@ __global__ void gj_colpanel_kernel(const int64_t* __restrict__ nmat, const int64
   }
 }
 
-// W_s[r][k] = Binv_s[own_local[r]][k], converted to the apply precision.
-template <typename T, typename U>
-__global__ void extract_owned_kernel(const int64_t* __restrict__ nmat, const int64_t* __restrict__ off,
-                                     const T* __restrict__ ws, const int32_t* __restrict__ sub_ids,
-                                     const int64_t* __restrict__ own_ptr, const int32_t* __restrict__ own_local,
-                                     const int64_t* __restrict__ w_off, U* __restrict__ W) {
-  using Su = decltype(U{}.x);
-  const int b = blockIdx.y;
-  const int s = sub_ids[b];
-  const int64_t n = nmat[b];
-  const int64_t nown = own_ptr[s + 1] - own_ptr[s];
-  const T* A = ws + off[b];
-  U* Ws = W + w_off[s];
-  const int64_t total = nown * n;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = e / n, k = e - r * n;
-    const T v = A[(int64_t)own_local[own_ptr[s] + r] * n + k];
-    Ws[e] = U{(Su)v.x, (Su)v.y};
-  }
-}
-
 // ---------------------------------------------------------------------------------------
 // CUDA-core apply: a block computes a 32-row tile of z[own rows of s] for all R columns.
 // ---------------------------------------------------------------------------------------
@@ -445,48 +326,9 @@ void gj_all(const OrasBatch& bt, T* ws, T* dinv, int32_t* status, cudaStream_t s
 
 }  // namespace
 
-void oras_local_assemble(const OrasBatch& bt, const OrasTopo& tp, const double* Bsurf, const double* KM,
-                         const double* eps, double k0, double ebr, double ebi, const double2* zc, const uint8_t* metal,
-                         int prec, void* ws, cudaStream_t s) {
-  note_launch(1);
-  if (prec == 0)
-    local_assemble_kernel<double2><<<bt.count, 32, 0, s>>>(bt.d_sub, tp.dof_ptr, tp.dofs, tp.tet_ptr, tp.tet_ids,
-                                                            tp.tet_loc, tp.surf_ptr, tp.surf_loc, tp.surf_tet, Bsurf,
-                                                            KM, eps, k0, ebr, ebi, zc, metal, bt.d_off, (double2*)ws);
-  else
-    local_assemble_kernel<float2><<<bt.count, 32, 0, s>>>(bt.d_sub, tp.dof_ptr, tp.dofs, tp.tet_ptr, tp.tet_ids,
-                                                           tp.tet_loc, tp.surf_ptr, tp.surf_loc, tp.surf_tet, Bsurf,
-                                                           KM, eps, k0, ebr, ebi, zc, metal, bt.d_off, (float2*)ws);
-}
-
-void oras_invert(const OrasBatch& bt, int prec, void* ws, void* dinv, int32_t* status, cudaStream_t s) {
-  if (prec == 0)
-    gj_all<double2>(bt, (double2*)ws, (double2*)dinv, status, s);
-  else
-    gj_all<float2>(bt, (float2*)ws, (float2*)dinv, status, s);
-}
-
 void partial_gj_f32(const OrasBatch& bt, const int64_t* lim, int64_t lim_max, float2* ws, float2* dinv,
                     int32_t* status, cudaStream_t s) {
   if (bt.count > 0 && lim_max > 0) gj_all<float2>(bt, ws, dinv, status, s, lim, lim_max);
-}
-
-void oras_extract(const OrasBatch& bt, const OrasTopo& tp, int ws_prec, const void* ws, int w_prec,
-                  const int64_t* w_off, void* W, cudaStream_t s) {
-  note_launch(1);
-  dim3 g(256, bt.count);
-  if (ws_prec == 0 && w_prec == 0)
-    extract_owned_kernel<double2, double2><<<g, 256, 0, s>>>(bt.d_n, bt.d_off, (const double2*)ws, bt.d_sub,
-                                                             tp.own_ptr, tp.own_local, w_off, (double2*)W);
-  else if (ws_prec == 0 && w_prec == 1)
-    extract_owned_kernel<double2, float2><<<g, 256, 0, s>>>(bt.d_n, bt.d_off, (const double2*)ws, bt.d_sub,
-                                                            tp.own_ptr, tp.own_local, w_off, (float2*)W);
-  else if (ws_prec == 1 && w_prec == 0)
-    extract_owned_kernel<float2, double2><<<g, 256, 0, s>>>(bt.d_n, bt.d_off, (const float2*)ws, bt.d_sub,
-                                                            tp.own_ptr, tp.own_local, w_off, (double2*)W);
-  else
-    extract_owned_kernel<float2, float2><<<g, 256, 0, s>>>(bt.d_n, bt.d_off, (const float2*)ws, bt.d_sub,
-                                                           tp.own_ptr, tp.own_local, w_off, (float2*)W);
 }
 
 void oras_apply_cc(const OrasTopo& tp, int n_tiles, const int32_t* tile_sub, const int32_t* tile_row0, int prec,

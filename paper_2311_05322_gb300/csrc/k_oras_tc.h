@@ -12,7 +12,7 @@ struct Subdomains;
 
 namespace mwk {
 struct OrasTopo;
-struct OrasBatch;
+struct InvBatch;
 
 // Pre-tiled BF16 layout of the owned-row inverses W_s (see k_oras_tc.cu).
 struct TcPlan {
@@ -37,7 +37,7 @@ bool tc_plan_build(TcPlan& p, const mw::Subdomains& sd, const std::function<void
 void tc_plan_free(TcPlan& p, const std::function<void(void*)>& dfree);
 size_t tc_w_bytes(const TcPlan& p);
 size_t tc_scratch_bytes(const TcPlan& p, int R);
-void tc_extract(const TcPlan& p, const OrasBatch& bt, const OrasTopo& tp, int ws_prec, const void* ws, void* W,
+void tc_extract(const TcPlan& p, const InvBatch& bt, const OrasTopo& tp, int ws_prec, const void* ws, void* W,
                 cudaStream_t s);
 struct MfTask;
 // Packs the FP32 blocks of tasks (A = src + a_off, [m][k], row stride lda, times the task's

@@ -17,6 +17,7 @@
 #include "k_adjoint.h"
 #include "k_mf.h"
 #include "k_nn.h"
+#include "k_inverse.h"
 #include "k_oras.h"
 #include "k_oras_tc.h"
 #include "mw_internal.h"
@@ -2660,13 +2661,11 @@ mw_status mw_setup_preconditioner(mw_ctx* c, int32_t n_sub, const int32_t* part,
     // W offsets (cc layouts) and apply tiles
     std::vector<int64_t> woff(n_sub + 1, 0);
     std::vector<int32_t> tsub, trow;
-    int64_t nmax = 0;
     for (int s = 0; s < n_sub; ++s) {
       const int64_t n = sd.dof_ptr[s + 1] - sd.dof_ptr[s], no = sd.own_ptr[s + 1] - sd.own_ptr[s];
       woff[s + 1] = woff[s] + n * no;
       p.sum_own_n += (double)n * no;
       p.sum_n += (double)n;
-      nmax = std::max(nmax, n);
       for (int64_t r0 = 0; r0 < no; r0 += 32) {
         tsub.push_back(s);
         trow.push_back((int32_t)r0);
@@ -2681,61 +2680,116 @@ mw_status mw_setup_preconditioner(mw_ctx* c, int32_t n_sub, const int32_t* part,
               MW_EINVAL, "BF16 tensor-core apply unavailable for this partition");
     const size_t wes = p.apply_prec == 0 ? sizeof(double2) : sizeof(float2);
     const size_t fes = p.factor_prec == 0 ? sizeof(double2) : sizeof(float2);
-    // workspace batches
+    // elimination order of every subdomain (unknowns not owned first, both parts padded to whole
+    // pivot blocks), and batches of subdomains whose matrices and panels fit the workspace
+    const int blk = mwk::inv_block(p.factor_prec);
+    auto pad = [&](int64_t n) { return (int32_t)((n + blk - 1) / blk * blk); };
+    std::vector<int32_t> np(n_sub), mn(n_sub), pos(sd.dofs.size());
+    auto ws_elems = [&](int s) { return (size_t)np[s] * np[s] + (size_t)2 * blk * np[s]; };
+    size_t total = 0, largest = 0;
+    for (int s = 0; s < n_sub; ++s) {
+      const int64_t n = sd.dof_ptr[s + 1] - sd.dof_ptr[s], no = sd.own_ptr[s + 1] - sd.own_ptr[s];
+      mn[s] = pad(n - no);
+      np[s] = mn[s] + pad(no);
+      require(np[s] <= (1 << 20), MW_EINVAL, "a subdomain is too large for a dense inverse");
+      int32_t a = 0, o = mn[s];
+      int64_t q = sd.own_ptr[s];
+      for (int64_t i = 0; i < n; ++i)
+        if (q < sd.own_ptr[s + 1] && sd.own_local[q] == i) {
+          pos[sd.dof_ptr[s] + i] = o++;
+          ++q;
+        } else {
+          pos[sd.dof_ptr[s] + i] = a++;
+        }
+      total += (ws_elems(s) * fes + 255) / 256 * 256;
+      largest = std::max(largest, ws_elems(s) * fes);
+    }
     size_t free_b = 0, total_b = 0;
     CK(cudaMemGetInfo(&free_b, &total_b));
-    size_t budget = std::min<size_t>((size_t)8 << 30, free_b / 4);
-    budget = std::max<size_t>(budget, (size_t)nmax * nmax * fes);
-    std::vector<int32_t> bsub;
-    std::vector<int64_t> bn, boff;
-    int32_t* d_status = dalloc<int32_t>(c, 1);
-    CK(cudaMemsetAsync(d_status, 0, sizeof(int32_t), c->stream));
-    void* ws = dalloc<unsigned char>(c, budget);
-    int32_t* d_bsub = dalloc<int32_t>(c, n_sub);
-    int64_t* d_bn = dalloc<int64_t>(c, n_sub);
-    int64_t* d_boff = dalloc<int64_t>(c, n_sub);
-    void* dinv = dalloc<unsigned char>(c, (size_t)n_sub * 32 * 32 * fes);
+    const size_t budget = std::max(largest, std::min({(size_t)8 << 30, free_b / 4, total}));
+    struct Batch {
+      std::vector<int32_t> sub, np, mn, prefix, tiles;
+      std::vector<int64_t> off, poff;
+      int np_max = 0, steps = 0;
+      size_t used = 0;
+      double flops = 0;
+    };
+    std::vector<Batch> batches;
+    for (int s = 0; s < n_sub; ++s) {
+      const size_t need = ws_elems(s) * fes;
+      if (batches.empty() || batches.back().used + need > budget) batches.emplace_back();
+      Batch& b = batches.back();
+      b.sub.push_back(s);
+      b.np.push_back(np[s]);
+      b.mn.push_back(mn[s]);
+      b.off.push_back((int64_t)(b.used / fes));
+      b.poff.push_back(b.off.back() + (int64_t)np[s] * np[s]);
+      b.used = (b.used + need + 255) / 256 * 256;
+      b.np_max = std::max(b.np_max, (int)np[s]);
+      // owned rows of the inverse of a complex symmetric matrix by block sweeps (8 real flops per
+      // complex multiply-add): n^2 m / 2 - m^3 / 6 + (n - m) (n^2 - m^2) / 2 of them, m not owned
+      const double n = (double)(sd.dof_ptr[s + 1] - sd.dof_ptr[s]), o = (double)(sd.own_ptr[s + 1] - sd.own_ptr[s]);
+      const double m = n - o;
+      b.flops += 8.0 * (n * n * m / 2 - m * m * m / 6 + o * (n * n - m * m) / 2);
+    }
+    size_t max_count = 0, max_prefix = 0;
+    for (Batch& b : batches) {
+      b.steps = b.np_max / blk;
+      for (int k = 0; k < b.steps; ++k) {
+        int64_t run = 0;
+        for (size_t i = 0; i < b.sub.size(); ++i) {
+          b.prefix.push_back((int32_t)run);
+          run += mwk::inv_update_tiles(b.np[i], b.mn[i], k * blk);
+        }
+        require(run < INT32_MAX, MW_EINVAL, "too many update tiles in one batch");
+        b.prefix.push_back((int32_t)run);
+        b.tiles.push_back((int32_t)run);
+      }
+      max_count = std::max(max_count, b.sub.size());
+      max_prefix = std::max(max_prefix, b.prefix.size());
+    }
+    // everything allocated for the factorisation alone
+    std::vector<void*> tmp;
+    auto scratch = [&](size_t bytes) {
+      tmp.push_back(dalloc<unsigned char>(c, bytes));
+      return tmp.back();
+    };
     p.W.assign(c->n_freq, nullptr);
     try {
+      int32_t* d_status = (int32_t*)scratch(sizeof(int32_t));
+      CK(cudaMemsetAsync(d_status, 0, sizeof(int32_t), c->stream));
+      void* ws = scratch(budget);
+      int32_t* d_pos = (int32_t*)scratch(sizeof(int32_t) * pos.size());
+      CK(cudaMemcpyAsync(d_pos, pos.data(), sizeof(int32_t) * pos.size(), cudaMemcpyHostToDevice, c->stream));
+      int32_t* d_i32 = (int32_t*)scratch(sizeof(int32_t) * 3 * max_count);
+      int64_t* d_i64 = (int64_t*)scratch(sizeof(int64_t) * 2 * max_count);
+      int32_t* d_prefix = (int32_t*)scratch(sizeof(int32_t) * max_prefix);
+      void* dinv = scratch(2 * max_count * blk * blk * fes);
       for (int f = 0; f < c->n_freq; ++f) {
         if (p.apply_prec == 2)
           p.W[f] = dalloc<unsigned char>(c, mwk::tc_w_bytes(p.tc));
         else
           p.W[f] = dalloc<unsigned char>(c, wes * std::max<int64_t>(woff[n_sub], 1));
         const double k0 = k0_of(c->freqs[f]);
-        int s = 0;
-        while (s < n_sub) {
-          bsub.clear();
-          bn.clear();
-          boff.clear();
-          size_t used = 0;
-          int64_t bmax = 0;
-          while (s < n_sub) {
-            const int64_t n = sd.dof_ptr[s + 1] - sd.dof_ptr[s];
-            const size_t need = (size_t)n * n * fes;
-            if (!bsub.empty() && used + need > budget) break;
-            bsub.push_back(s);
-            bn.push_back(n);
-            boff.push_back((int64_t)(used / fes));
-            used += need;
-            used = (used + 255) / 256 * 256;
-            bmax = std::max(bmax, n);
-            ++s;
-          }
-          const int cnt = (int)bsub.size();
-          CK(cudaMemcpyAsync(d_bsub, bsub.data(), sizeof(int32_t) * cnt, cudaMemcpyHostToDevice, c->stream));
-          CK(cudaMemcpyAsync(d_bn, bn.data(), sizeof(int64_t) * cnt, cudaMemcpyHostToDevice, c->stream));
-          CK(cudaMemcpyAsync(d_boff, boff.data(), sizeof(int64_t) * cnt, cudaMemcpyHostToDevice, c->stream));
-          mwk::OrasBatch bt{cnt, bmax, d_bsub, d_bn, d_boff};
-          CK(cudaMemsetAsync(ws, 0, used, c->stream));
+        for (const Batch& b : batches) {
+          const int cnt = (int)b.sub.size();
+          auto put = [&](void* d, const void* h, size_t bytes) {
+            CK(cudaMemcpyAsync(d, h, bytes, cudaMemcpyHostToDevice, c->stream));
+          };
+          put(d_i32, b.sub.data(), sizeof(int32_t) * cnt);
+          put(d_i32 + cnt, b.np.data(), sizeof(int32_t) * cnt);
+          put(d_i32 + 2 * cnt, b.mn.data(), sizeof(int32_t) * cnt);
+          put(d_i64, b.off.data(), sizeof(int64_t) * cnt);
+          put(d_i64 + cnt, b.poff.data(), sizeof(int64_t) * cnt);
+          put(d_prefix, b.prefix.data(), sizeof(int32_t) * b.prefix.size());
+          const mwk::InvBatch bt{cnt,   b.steps,     b.np_max, d_i32,    d_i32 + cnt,    d_i32 + 2 * cnt,
+                                 d_i64, d_i64 + cnt, d_pos,    d_prefix, b.tiles.data()};
+          CK(cudaMemsetAsync(ws, 0, b.used, c->stream));
           const double2* zc = c->d_zc ? c->d_zc + (size_t)f * (2 + c->n_port) : nullptr;
           mwk::oras_local_assemble(bt, p.topo(), p.Bsurf, c->d_KM, c->d_eps, k0, c->eps_bg[0], c->eps_bg[1], zc,
                                    c->d_metal, p.factor_prec, ws, c->stream);
           {
-            // in-place Gauss-Jordan inversion: n^3 complex multiply-adds (8 n^3 real flops)
-            double fl = 0;
-            for (int64_t n : bn) fl += 8.0 * (double)n * n * n;
-            ProfScope ps(c, MW_K_FACTOR, 0.0, fl);
+            ProfScope ps(c, MW_K_FACTOR, 0.0, b.flops);
             mwk::oras_invert(bt, p.factor_prec, ws, dinv, d_status, c->stream);
           }
           if (p.apply_prec == 2)
@@ -2751,21 +2805,11 @@ mw_status mw_setup_preconditioner(mw_ctx* c, int32_t n_sub, const int32_t* part,
       CK(cudaMemcpy(&st, d_status, sizeof(int32_t), cudaMemcpyDeviceToHost));
       require(st == 0, MW_ESINGULAR, "a subdomain matrix had a near-zero pivot");
     } catch (...) {
-      dfree(c, ws);
-      dfree(c, dinv);
-      dfree(c, d_status);
-      dfree(c, d_bsub);
-      dfree(c, d_bn);
-      dfree(c, d_boff);
+      for (void* q : tmp) dfree(c, q);
       release_prec(c);
       throw;
     }
-    dfree(c, ws);
-    dfree(c, dinv);
-    dfree(c, d_status);
-    dfree(c, d_bsub);
-    dfree(c, d_bn);
-    dfree(c, d_boff);
+    for (void* q : tmp) dfree(c, q);
     p.ready = true;
   });
 }
