@@ -2,6 +2,9 @@
 // index fastest ([E][R]), so the threads of one row read one contiguous span of X per nonzero.
 // Threads of a row split the R columns (CPL consecutive columns each); rows are spread over
 // the grid.  FP64 variant (FP64 arithmetic) and FP32 variant (FP32 arithmetic, FP32 accumulate).
+#include <algorithm>
+#include <type_traits>
+
 #include "mw_internal.h"
 
 namespace mwk {
@@ -86,6 +89,85 @@ __global__ void __launch_bounds__(512) spmm_kernel(const int64_t* __restrict__ r
 #pragma unroll
   for (int q = 0; q < CPL; ++q)
     if (c0 + q < R) yr[q] = acc[q];
+}
+
+// FP32 product with the matrix staged: a block takes ROWS consecutive rows, brings their nonzeros to shared
+// memory with coalesced loads, each as one 16-byte record {Re a, Im a, first element of its row of X}, and
+// then each group of 1 << lpr_log2 lanes computes whole rows: per term one broadcast 16-byte load of the
+// record, one address, one gather of VEC columns (CV times, spans of VEC << lpr_log2 columns apart) and the
+// FMAs.  Instruction issue and L1 wavefronts bound the product (ncu on spmm_kernel: issue 63 to 74 %,
+// wavefronts 67 %, L1 hits 58 %): a value load, an index load and their addresses per term and warp are
+// 21 instructions per term, this form spends about 11.  A row's last, short batch is masked, so no
+// gather waits for another.  The sums keep the canonical term order: the bits of spmm_kernel.
+template <typename XT, int VEC>
+struct alignas(VEC * sizeof(XT) > 16 ? 16 : VEC * sizeof(XT)) XPack {
+  XT v[VEC];
+};
+template <typename XT, int VEC, int CV>
+__global__ void __launch_bounds__(512, CV == 1 ? 4 : 1) spmm_staged_kernel(const int64_t* __restrict__ rp,
+                                                          const int32_t* __restrict__ ci,
+                                                          const float2* __restrict__ A, const XT* __restrict__ X,
+                                                          float2* __restrict__ Y, int64_t E, int R, int lpr_log2,
+                                                          int rows) {
+  constexpr int NB = VEC * CV >= 4 ? 2 : 4;
+  using Pack = XPack<XT, VEC>;
+  extern __shared__ float4 smem4[];
+  int* rs = reinterpret_cast<int*>(smem4);                       // [rows + 1], padded to 16 bytes
+  float4* rec = smem4 + (rows + 4) / 4;
+  const int64_t row0 = (int64_t)blockIdx.x * rows;
+  const int nrow = (int)min((int64_t)rows, E - row0);
+  const int64_t k0 = rp[row0];
+  const int n = (int)(rp[row0 + nrow] - k0);
+  for (int t = threadIdx.x; t <= nrow; t += blockDim.x) rs[t] = (int)(rp[row0 + t] - k0);
+  for (int q = threadIdx.x; q < n; q += blockDim.x) {
+    const float2 a = A[k0 + q];
+    rec[q] = make_float4(a.x, a.y, __int_as_float(ci[k0 + q] * R), 0.f);
+  }
+  __syncthreads();
+  const int c0 = (int)(threadIdx.x & ((1 << lpr_log2) - 1)) * VEC;
+  const int span = VEC << lpr_log2;
+  if (c0 >= R) return;
+  const XT* Xc = X + c0;
+  for (int r = threadIdx.x >> lpr_log2; r < nrow; r += blockDim.x >> lpr_log2) {
+    float2 acc[CV][VEC];
+#pragma unroll
+    for (int v = 0; v < CV; ++v)
+#pragma unroll
+      for (int q = 0; q < VEC; ++q) acc[v][q] = make_float2(0.f, 0.f);
+    const float4* p = rec + rs[r];
+    int left = rs[r + 1] - rs[r];
+    auto batch = [&](auto tag) {
+      constexpr bool full = decltype(tag)::value;
+      float4 a[NB];
+      Pack xv[NB][CV];
+#pragma unroll
+      for (int u = 0; u < NB; ++u)
+        if (full || u < left) {
+          a[u] = p[u];
+          const XT* xr = Xc + __float_as_int(a[u].z);
+#pragma unroll
+          for (int v = 0; v < CV; ++v)
+            if (CV == 1 || c0 + v * span < R) xv[u][v] = *reinterpret_cast<const Pack*>(xr + v * span);
+        }
+#pragma unroll
+      for (int u = 0; u < NB; ++u)
+        if (full || u < left)
+#pragma unroll
+          for (int v = 0; v < CV; ++v)
+            if (CV == 1 || c0 + v * span < R)
+#pragma unroll
+              for (int q = 0; q < VEC; ++q)
+                cmac(acc[v][q], make_float2(a[u].x, a[u].y), xval(xv[u][v].v[q]));
+    };
+    for (; left >= NB; left -= NB, p += NB) batch(std::true_type());
+    if (left > 0) batch(std::false_type());
+    float2* yr = Y + (row0 + r) * R + c0;
+#pragma unroll
+    for (int v = 0; v < CV; ++v)
+      if (CV == 1 || c0 + v * span < R)
+#pragma unroll
+        for (int q = 0; q < VEC; ++q) yr[v * span + q] = acc[v][q];
+  }
 }
 
 // r = b - A x in FP64 with per-block, per-column partial sums of |r|^2 (deterministic).  ZX: x = 0
@@ -177,6 +259,49 @@ void spmm_launch(const int64_t* rp, const int32_t* ci, const T* A, const T* X, T
   }
 }
 
+// Rows per block of the staged product by its thread count, and the shared memory of `nnz` records.
+inline int staged_rows(int threads) { return threads / 8; }
+inline size_t staged_smem(int rows, int nnz) { return 16 * (size_t)((rows + 4) / 4 + nnz); }
+
+template <typename XT, int VEC>
+void spmm_staged(const int64_t* rp, const int32_t* ci, const float2* A, const XT* X, float2* Y, int64_t E, int R,
+                 cudaStream_t s, int threads, size_t smem) {
+  const int packs = (R + VEC - 1) / VEC, rows = staged_rows(threads);
+  int l = 0;
+  while ((1 << l) < packs && l < 5) ++l;
+  const int cv = (packs + (1 << l) - 1) >> l;
+  const unsigned blocks = (unsigned)((E + rows - 1) / rows);
+  note_launch(1);
+  if (cv == 1)
+    spmm_staged_kernel<XT, VEC, 1><<<blocks, threads, smem, s>>>(rp, ci, A, X, Y, E, R, l, rows);
+  else if (cv == 2)
+    spmm_staged_kernel<XT, VEC, 2><<<blocks, threads, smem, s>>>(rp, ci, A, X, Y, E, R, l, rows);
+  else
+    spmm_staged_kernel<XT, VEC, 4><<<blocks, threads, smem, s>>>(rp, ci, A, X, Y, E, R, l, rows);
+}
+
+// The staged product when the records of a block fit 48 KB of shared memory and element offsets 31 bits;
+// win: the most nonzeros of 16, 32 and 64 consecutive rows (aligned).  A lane takes 4 neighbouring BF16
+// columns from 16 columns on (8 lanes per row at 32 columns: 126 us against 156 with one column per lane on
+// the 55x55x24 mesh), 2 above 32 columns (at 32 FP32 columns one and two columns per lane both take 160 us),
+// else one; always where the pack divides the row and its alignment.  Before: 224 us (FP32) and 222 us
+// (BF16) at 32 columns, 375 and 300 us at 64, 1,047 and 617 us at 128; the floor of the bytes is 55 us at 32.
+template <typename XT>
+bool spmm_staged_launch(const int64_t* rp, const int32_t* ci, const float2* A, const XT* X, float2* Y, int64_t E,
+                        int R, cudaStream_t s, int threads, const int* win) {
+  if (threads != 128 && threads != 256 && threads != 512) threads = 256;
+  const size_t smem = staged_smem(staged_rows(threads), win[threads == 128 ? 0 : threads == 256 ? 1 : 2]);
+  if ( R < 1 || R > 128 || smem > 48 * 1024 || E * R > INT32_MAX) return false;
+  const auto fits = [&](int vec) { return R % vec == 0 && (uintptr_t)X % (vec * sizeof(XT)) == 0; };
+  if (R >= 16 && sizeof(XT) == 4 && fits(4))
+    spmm_staged<XT, sizeof(XT) == 4 ? 4 : 2>(rp, ci, A, X, Y, E, R, s, threads, smem);
+  else if (R > 32 && fits(2))
+    spmm_staged<XT, 2>(rp, ci, A, X, Y, E, R, s, threads, smem);
+  else
+    spmm_staged<XT, 1>(rp, ci, A, X, Y, E, R, s, threads, smem);
+  return true;
+}
+
 // Halo-tiled FP32 SpMM.  One CTA takes one block of the SpMM plan (rows in Morton order whose
 // column set, the halo, holds at most kHaloMax edges; at most kHaloRows rows and kHaloNnz
 // nonzeros) and one chunk of kHaloCols columns.  Staging, all at the CTA's start:
@@ -255,7 +380,8 @@ void spmm_f64(const int64_t* rp, const int32_t* ci, const double2* A, const doub
   spmm_launch<double2>(rp, ci, A, X, Y, E, R, s, threads);
 }
 void spmm_f32(const int64_t* rp, const int32_t* ci, const float2* A, const float2* X, float2* Y, int64_t E, int R,
-              cudaStream_t s, int threads) {
+              cudaStream_t s, int threads, const int* win) {
+  if (spmm_staged_launch<float2>(rp, ci, A, X, Y, E, R, s, threads, win)) return;
   spmm_launch<float2>(rp, ci, A, X, Y, E, R, s, threads);
 }
 
@@ -275,7 +401,8 @@ bool spmm_halo_f32(const SpmmDev& p, const float2* A, const float2* X, float2* Y
 }
 
 void spmm_f32_bx(const int64_t* rp, const int32_t* ci, const float2* A, const void* X, float2* Y, int64_t E, int R,
-                 cudaStream_t s, int threads) {
+                 cudaStream_t s, int threads, const int* win) {
+  if (spmm_staged_launch<uint32_t>(rp, ci, A, (const uint32_t*)X, Y, E, R, s, threads, win)) return;
   if (threads != 128 && threads != 256 && threads != 512) threads = 256;
   if (R > 128) return;
   note_launch(1);
@@ -453,84 +580,104 @@ __device__ __forceinline__ void df_add(float& a_h, float& a_l, float b_h, float 
 // row alternate between two independent double-float accumulators (two dependency chains in
 // flight), joined by a double-float add at the end of the row.  ZX: x = 0 (the first outer step),
 // so every product and sum of a row is +0 and the row loop is skipped: the same r and norms.
-template <int CPL, bool ZX>
+//
+// A block takes tiles of `rows` consecutive rows in turn, their nonzeros staged in shared memory as in
+// spmm_staged_kernel; a row's lanes hold
+// columns lane, lane + 32, ... (CV of them) and keep NB gathers in flight.  With two terms in flight, loaded
+// from global memory per lane, it waited for loads most of the time.
+template <int CV, bool ZX>
 __global__ void __launch_bounds__(256) residual_df32_kernel(const int64_t* __restrict__ rp,
                                                             const int32_t* __restrict__ ci,
                                                             const float4* __restrict__ A, const float4* __restrict__ X,
                                                             const float4* __restrict__ Bdf, float2* __restrict__ Rv,
-                                                            double* __restrict__ part, int64_t E, int R, int tpr_log2) {
-  __shared__ double red[256 * CPL];
-  const int tpr = 1 << tpr_log2;
-  const int rows_per_block = 256 >> tpr_log2;
+                                                            double* __restrict__ part, int64_t E, int R, int tpr_log2,
+                                                            int rows, int cap) {
+  constexpr int NB = CV == 1 ? 4 : 2;               // even: the accumulators alternate by term
+  extern __shared__ float4 rsmem[];
+  float4* rec = rsmem;                              // [cap] values of the tile
+  int* col = reinterpret_cast<int*>(rec + (ZX ? 0 : cap));   // [cap] columns of the tile
+  int* rs = col + (ZX ? 0 : cap);                   // [rows + 1]
+  __shared__ double red[256 * CV];
+  const int tpr = 1 << tpr_log2, span = tpr;
+  const int groups = 256 >> tpr_log2;
   const int lane_c = threadIdx.x & (tpr - 1);
-  const int c0 = lane_c * CPL;
-  double nrm[CPL];
+  double nrm[CV];
 #pragma unroll
-  for (int q = 0; q < CPL; ++q) nrm[q] = 0.0;
-  for (int64_t row = (int64_t)blockIdx.x * rows_per_block + (threadIdx.x >> tpr_log2); row < E;
-       row += (int64_t)gridDim.x * rows_per_block) {
-    if (c0 >= R) continue;
-    float rh[CPL], rl[CPL], ih[CPL], il[CPL], rh2[CPL], rl2[CPL], ih2[CPL], il2[CPL];
-#pragma unroll
-    for (int q = 0; q < CPL; ++q) rh[q] = rl[q] = ih[q] = il[q] = rh2[q] = rl2[q] = ih2[q] = il2[q] = 0.f;
-    const int64_t kb = ZX ? 0 : rp[row], ke = ZX ? 0 : rp[row + 1];
-    int64_t k = kb;
-    for (; k + 1 < ke; k += 2) {
-      const float4 a = A[k], a2 = A[k + 1];
-      const float4* xr = X + (int64_t)ci[k] * R + c0;
-      const float4* xr2 = X + (int64_t)ci[k + 1] * R + c0;
-#pragma unroll
-      for (int q = 0; q < CPL; ++q)
-        if (c0 + q < R) {
-          const float4 x = xr[q], x2 = xr2[q];
-          df_mac(rh[q], rl[q], a.x, a.y, x.x, x.y);
-          df_mac(rh2[q], rl2[q], a2.x, a2.y, x2.x, x2.y);
-          df_mac(ih[q], il[q], a.x, a.y, x.z, x.w);
-          df_mac(ih2[q], il2[q], a2.x, a2.y, x2.z, x2.w);
-          df_mac(rh[q], rl[q], -a.z, -a.w, x.z, x.w);
-          df_mac(rh2[q], rl2[q], -a2.z, -a2.w, x2.z, x2.w);
-          df_mac(ih[q], il[q], a.z, a.w, x.x, x.y);
-          df_mac(ih2[q], il2[q], a2.z, a2.w, x2.x, x2.y);
-        }
-    }
-    if (k < ke) {
-      const float4 a = A[k];
-      const float4* xr = X + (int64_t)ci[k] * R + c0;
-#pragma unroll
-      for (int q = 0; q < CPL; ++q)
-        if (c0 + q < R) {
-          const float4 x = xr[q];
-          df_mac(rh[q], rl[q], a.x, a.y, x.x, x.y);
-          df_mac(ih[q], il[q], a.x, a.y, x.z, x.w);
-          df_mac(rh[q], rl[q], -a.z, -a.w, x.z, x.w);
-          df_mac(ih[q], il[q], a.z, a.w, x.x, x.y);
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < CPL; ++q) {
-      df_add(rh[q], rl[q], rh2[q], rl2[q]);
-      df_add(ih[q], il[q], ih2[q], il2[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < CPL; ++q)
-      if (c0 + q < R) {
-        const float4 bb = Bdf[row * R + c0 + q];
-        const float re = df_sub_round(bb.x, bb.y, rh[q], rl[q]);
-        const float im = df_sub_round(bb.z, bb.w, ih[q], il[q]);
-        Rv[row * R + c0 + q] = make_float2(re, im);
-        nrm[q] += (double)fmaf(re, re, __fmul_rn(im, im));
+  for (int v = 0; v < CV; ++v) nrm[v] = 0.0;
+  for (int64_t row0 = (int64_t)blockIdx.x * rows; row0 < E; row0 += (int64_t)gridDim.x * rows) {
+    const int nrow = (int)min((int64_t)rows, E - row0);
+    const int64_t k0 = ZX ? 0 : rp[row0];
+    if (!ZX) {
+      const int n = (int)(rp[row0 + nrow] - k0);
+      __syncthreads();                              // the previous tile has been read
+      for (int t = threadIdx.x; t <= nrow; t += 256) rs[t] = (int)(rp[row0 + t] - k0);
+      for (int q = threadIdx.x; q < n; q += 256) {
+        rec[q] = A[k0 + q];
+        col[q] = ci[k0 + q];
       }
+      __syncthreads();
+    }
+    if (lane_c >= R) continue;
+    for (int r = threadIdx.x >> tpr_log2; r < nrow; r += groups) {
+      float rh[CV], rl[CV], ih[CV], il[CV], rh2[CV], rl2[CV], ih2[CV], il2[CV];
+#pragma unroll
+      for (int v = 0; v < CV; ++v) rh[v] = rl[v] = ih[v] = il[v] = rh2[v] = rl2[v] = ih2[v] = il2[v] = 0.f;
+      if (!ZX) {
+        int k = rs[r];
+        for (int left = rs[r + 1] - k; left > 0; left -= NB, k += NB) {
+          float4 xv[NB][CV];
+#pragma unroll
+          for (int u = 0; u < NB; ++u)
+            if (u < left) {
+              const float4* xr = X + (int64_t)col[k + u] * R + lane_c;
+#pragma unroll
+              for (int v = 0; v < CV; ++v)
+                if (CV == 1 || lane_c + v * span < R) xv[u][v] = xr[v * span];
+            }
+#pragma unroll
+          for (int u = 0; u < NB; ++u)
+            if (u < left) {
+              const float4 a = rec[k + u];
+#pragma unroll
+              for (int v = 0; v < CV; ++v)
+                if (CV == 1 || lane_c + v * span < R) {
+                  const float4 x = xv[u][v];
+                  float& ph = u & 1 ? rh2[v] : rh[v];
+                  float& pl = u & 1 ? rl2[v] : rl[v];
+                  float& qh = u & 1 ? ih2[v] : ih[v];
+                  float& ql = u & 1 ? il2[v] : il[v];
+                  df_mac(ph, pl, a.x, a.y, x.x, x.y);
+                  df_mac(qh, ql, a.x, a.y, x.z, x.w);
+                  df_mac(ph, pl, -a.z, -a.w, x.z, x.w);
+                  df_mac(qh, ql, a.z, a.w, x.x, x.y);
+                }
+            }
+        }
+      }
+#pragma unroll
+      for (int v = 0; v < CV; ++v) {
+        const int c = lane_c + v * span;
+        if (CV > 1 && c >= R) continue;
+        df_add(rh[v], rl[v], rh2[v], rl2[v]);
+        df_add(ih[v], il[v], ih2[v], il2[v]);
+        const float4 bb = Bdf[(row0 + r) * R + c];
+        const float re = df_sub_round(bb.x, bb.y, rh[v], rl[v]);
+        const float im = df_sub_round(bb.z, bb.w, ih[v], il[v]);
+        Rv[(row0 + r) * R + c] = make_float2(re, im);
+        nrm[v] += (double)fmaf(re, re, __fmul_rn(im, im));
+      }
+    }
   }
 #pragma unroll
-  for (int q = 0; q < CPL; ++q) red[threadIdx.x * CPL + q] = nrm[q];
+  for (int v = 0; v < CV; ++v) red[v * 256 + threadIdx.x] = nrm[v];
   __syncthreads();
   if ((int)threadIdx.x < tpr) {
-    for (int q = 0; q < CPL; ++q) {
-      const int c = c0 + q;
+    for (int v = 0; v < CV; ++v) {
+      const int c = lane_c + v * span;
       if (c >= R) continue;
-      double s = 0.0;
-      for (int r = 0; r < rows_per_block; ++r) s += red[(r * tpr + lane_c) * CPL + q];
-      part[(int64_t)blockIdx.x * R + c] = s;
+      double sum = 0.0;
+      for (int r = 0; r < groups; ++r) sum += red[v * 256 + r * tpr + lane_c];
+      part[(int64_t)blockIdx.x * R + c] = sum;
     }
   }
 }
@@ -562,32 +709,34 @@ int residual_df(const int64_t* rp, const int32_t* ci, const float4* A, const flo
   return blocks;
 }
 
-int residual_df32(const int64_t* rp, const int32_t* ci, const float4* A, const float4* X, const float4* Bdf, float2* Rv,
-                  double* part, int64_t E, int R, cudaStream_t s, bool zero_x) {
-  note_launch(1);
-  Shape sh = shape_for(R);
-  const int blocks = 152 * 4;
-  switch (sh.cpl) {
-    case 1:
-      if (zero_x)
-        residual_df32_kernel<1, true><<<blocks, 256, 0, s>>>(rp, ci, A, X, Bdf, Rv, part, E, R, sh.tpr_log2);
-      else
-        residual_df32_kernel<1, false><<<blocks, 256, 0, s>>>(rp, ci, A, X, Bdf, Rv, part, E, R, sh.tpr_log2);
-      break;
-    case 2:
-      if (zero_x)
-        residual_df32_kernel<2, true><<<blocks, 256, 0, s>>>(rp, ci, A, X, Bdf, Rv, part, E, R, sh.tpr_log2);
-      else
-        residual_df32_kernel<2, false><<<blocks, 256, 0, s>>>(rp, ci, A, X, Bdf, Rv, part, E, R, sh.tpr_log2);
-      break;
-    default:
-      if (zero_x)
-        residual_df32_kernel<4, true><<<blocks, 256, 0, s>>>(rp, ci, A, X, Bdf, Rv, part, E, R, sh.tpr_log2);
-      else
-        residual_df32_kernel<4, false><<<blocks, 256, 0, s>>>(rp, ci, A, X, Bdf, Rv, part, E, R, sh.tpr_log2);
-      break;
-  }
+template <int CV>
+static int residual_df32_launch(const int64_t* rp, const int32_t* ci, const float4* A, const float4* X,
+                                const float4* Bdf, float2* Rv, double* part, int64_t E, int R, int l, const int* win,
+                                bool zero_x, cudaStream_t s) {
+  // tiles of 32 rows, of 16 where the nonzeros of 32 do not fit 200 KB (a row has at most kHaloMax)
+  constexpr int kCap = 10000;
+  static_assert(16 * kHaloMax <= kCap, "16 rows fit");
+  const int rows = win[1] <= kCap ? 32 : 16, cap = win[1] <= kCap ? win[1] : win[0];
+  const int blocks = (int)std::min<int64_t>(152 * 4, (E + rows - 1) / rows);
+  const size_t smem = (zero_x ? 0 : (size_t)cap * 20) + 4 * (rows + 1);
+  static const cudaError_t attr = cudaFuncSetAttribute(residual_df32_kernel<CV, false>,
+                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, kCap * 20 + 256);
+  (void)attr;   // a failure shows at the launch
+  if (zero_x)
+    residual_df32_kernel<CV, true><<<blocks, 256, smem, s>>>(rp, ci, A, X, Bdf, Rv, part, E, R, l, rows, cap);
+  else
+    residual_df32_kernel<CV, false><<<blocks, 256, smem, s>>>(rp, ci, A, X, Bdf, Rv, part, E, R, l, rows, cap);
   return blocks;
+}
+
+int residual_df32(const int64_t* rp, const int32_t* ci, const float4* A, const float4* X, const float4* Bdf, float2* Rv,
+                  double* part, int64_t E, int R, cudaStream_t s, const int* win, bool zero_x) {
+  note_launch(1);
+  int l = 0;
+  while ((1 << l) < R && l < 5) ++l;
+  if (R <= 32) return residual_df32_launch<1>(rp, ci, A, X, Bdf, Rv, part, E, R, l, win, zero_x, s);
+  if (R <= 64) return residual_df32_launch<2>(rp, ci, A, X, Bdf, Rv, part, E, R, l, win, zero_x, s);
+  return residual_df32_launch<4>(rp, ci, A, X, Bdf, Rv, part, E, R, l, win, zero_x, s);
 }
 
 }  // namespace mwk

@@ -237,6 +237,7 @@ struct Ctx {
           *d_tet_nb = nullptr;
   int8_t* d_sign = nullptr;
   int64_t *d_row = nullptr, *d_cptr = nullptr;
+  int row_win[3] = {0, 0, 0};      // most nonzeros of 16, 32, 64 aligned rows
   double *d_KM = nullptr, *d_vol = nullptr, *d_Bf = nullptr, *d_tikw = nullptr;
 
   int n_freq = 0;
@@ -1091,7 +1092,8 @@ int outer_residual(Ctx* c, int f, int wp, const double2* X, const double2* B, in
   if (wp == 0)
     return mwk::residual_f64(c->d_row, c->d_col, c->A64[f], X, B, w.r, w.npart, E, R, c->stream, zero_x);
   if (!zero_x) mwk::split_df(X, w.xdf, E * R, c->stream);
-  return mwk::residual_df32(c->d_row, c->d_col, c->Adf[f], w.xdf, w.bdf, w.r32, w.npart, E, R, c->stream, zero_x);
+  return mwk::residual_df32(c->d_row, c->d_col, c->Adf[f], w.xdf, w.bdf, w.r32, w.npart, E, R, c->stream, c->row_win,
+                            zero_x);
 }
 
 struct BlockStats {
@@ -1133,12 +1135,14 @@ bool spmm_halo_ok(Ctx* c, int R) {
 void spmm32(Ctx* c, int f, const float2* X, float2* Y, int R, int threads) {
   if (threads == kSpmmHaloShape && spmm_halo_ok(c, R) && mwk::spmm_halo_f32(c->spmm, c->A32b[f], X, Y, R, c->stream))
     return;
-  mwk::spmm_f32(c->d_row, c->d_col, c->A32[f], X, Y, c->topo.n_edge, R, c->stream, threads < 128 ? 256 : threads);
+  mwk::spmm_f32(c->d_row, c->d_col, c->A32[f], X, Y, c->topo.n_edge, R, c->stream, threads < 128 ? 256 : threads,
+                c->row_win);
 }
 // The same with X stored as complex BF16 pairs: the row-per-warp kernel (256 threads for the
 // halo shape, which has no BF16 form).
 void spmm32_bx(Ctx* c, int f, const void* X, float2* Y, int R, int threads) {
-  mwk::spmm_f32_bx(c->d_row, c->d_col, c->A32[f], X, Y, c->topo.n_edge, R, c->stream, threads < 128 ? 256 : threads);
+  mwk::spmm_f32_bx(c->d_row, c->d_col, c->A32[f], X, Y, c->topo.n_edge, R, c->stream, threads < 128 ? 256 : threads,
+                   c->row_win);
 }
 
 template <class Seg>
@@ -2178,6 +2182,12 @@ mw_status mw_set_mesh(mw_ctx* c, int64_t n_vert, const double* xyz, int64_t n_te
     c->d_sign = upload(c, t.tet_sign.data(), t.tet_sign.size());
     c->d_tet_edge = upload(c, t.tet_edge.data(), t.tet_edge.size());
     c->d_row = upload(c, t.row_ptr.data(), t.row_ptr.size());
+    for (int w = 0; w < 3; ++w) {
+      c->row_win[w] = 0;
+      for (int64_t r = 0; r < t.n_edge; r += 16 << w)
+        c->row_win[w] = std::max<int>(c->row_win[w],
+                                      (int)(t.row_ptr[std::min<int64_t>(r + (16 << w), t.n_edge)] - t.row_ptr[r]));
+    }
     c->d_col = upload(c, t.col_idx.data(), t.col_idx.size());
     c->d_cptr = upload(c, t.contrib_ptr.data(), t.contrib_ptr.size());
     c->d_contrib = upload(c, t.contrib.data(), t.contrib.size());
@@ -2301,7 +2311,8 @@ mw_status mw_apply_matrix(mw_ctx* c, int32_t f, int32_t prec, const void* x, voi
     if (prec == MW_PREC_FP64)
       mwk::spmm_f64(c->d_row, c->d_col, c->A64[f], (const double2*)x, (double2*)y, c->topo.n_edge, n_cols, c->stream);
     else if (prec == MW_PREC_FP32)
-      mwk::spmm_f32(c->d_row, c->d_col, c->A32[f], (const float2*)x, (float2*)y, c->topo.n_edge, n_cols, c->stream);
+      mwk::spmm_f32(c->d_row, c->d_col, c->A32[f], (const float2*)x, (float2*)y, c->topo.n_edge, n_cols, c->stream, 256,
+                    c->row_win);
     else if (prec == 4) {
       require(spmm_halo_ok(c, n_cols) && ((uintptr_t)x & 15) == 0, MW_EINVAL,
               "the halo-tiled SpMM takes an even column count up to 128 and a 16-byte aligned x");
@@ -2309,7 +2320,7 @@ mw_status mw_apply_matrix(mw_ctx* c, int32_t f, int32_t prec, const void* x, voi
               "halo-tiled SpMM: unsupported shape");
     }
     else if (prec == 5)
-      mwk::spmm_f32_bx(c->d_row, c->d_col, c->A32[f], x, (float2*)y, c->topo.n_edge, n_cols, c->stream);
+      mwk::spmm_f32_bx(c->d_row, c->d_col, c->A32[f], x, (float2*)y, c->topo.n_edge, n_cols, c->stream, 256, c->row_win);
     else if (prec == 3) {
       const int64_t n = c->topo.n_edge * (int64_t)n_cols;
       float4* xd = dalloc<float4>(c, n);

@@ -163,11 +163,13 @@ void reassemble(const int64_t* cptr, const int32_t* contrib, int64_t nnz, const 
                 const double* eps, double k0sq, double zb_re, double zb_im, const int32_t* fcls, const double2* zc,
                 const uint8_t* nzmask, double2* A64, float2* A32, cudaStream_t s);
 // K3 SpMM: Y = A X, [E][R] layout with leading dimension ld (>= R).
-// threads: block size, 128, 256 (default) or 512 (the result does not depend on it).
+// threads: block size, 128, 256 (default) or 512 (the result does not depend on it); win: the most
+// nonzeros of 16, 32 and 64 consecutive rows starting at a multiple of that count (sizes the staged
+// FP32 kernels' blocks).
 void spmm_f64(const int64_t* rp, const int32_t* ci, const double2* A, const double2* X, double2* Y, int64_t E,
               int R, cudaStream_t s, int threads = 256);
 void spmm_f32(const int64_t* rp, const int32_t* ci, const float2* A, const float2* X, float2* Y, int64_t E, int R,
-              cudaStream_t s, int threads = 256);
+              cudaStream_t s, int threads, const int* win);
 // Bounds of one block of the halo-tiled SpMM plan: columns (halo), rows and nonzeros.
 constexpr int kHaloMax = 480, kHaloRows = 512, kHaloNnz = 4096;
 // Device copy of mw::SpmmPlan (halo_max bounds every block's halo).
@@ -188,7 +190,7 @@ struct SpmmDev {
 bool spmm_halo_f32(const SpmmDev& p, const float2* A_blk, const float2* X, float2* Y, int R, cudaStream_t s);
 // Y = A X (FP32) with X stored as complex BF16 pairs [E][R] (real in the low half).
 void spmm_f32_bx(const int64_t* rp, const int32_t* ci, const float2* A, const void* X, float2* Y, int64_t E, int R,
-                 cudaStream_t s, int threads = 256);
+                 cudaStream_t s, int threads, const int* win);
 // A_blk[q] = A32[src[q]].
 void spmm_plan_values(const SpmmDev& p, const float2* A32, int64_t nnz, float2* A_blk, cudaStream_t s);
 // Split complex FP64 values into double-float (re_hi, re_lo, im_hi, im_lo).
@@ -200,7 +202,7 @@ int residual_df(const int64_t* rp, const int32_t* ci, const float4* A, const flo
 // The mixed solver's outer residual: b, A, x in double-float, r rounded to FP32 complex, partial
 // ||r||^2 (FP64) per block and column; returns the number of blocks.
 int residual_df32(const int64_t* rp, const int32_t* ci, const float4* A, const float4* X, const float4* Bdf,
-                  float2* Rv, double* part, int64_t E, int R, cudaStream_t s, bool zero_x = false);
+                  float2* Rv, double* part, int64_t E, int R, cudaStream_t s, const int* win, bool zero_x = false);
 // v0 = r / rnorm per column (0 for done columns) from an FP32 residual.
 void normalize_start32(const float2* r, const double* rnorm, const int32_t* done, int64_t E, int R, float2* v0,
                        cudaStream_t s);
