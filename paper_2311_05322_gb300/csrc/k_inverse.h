@@ -7,24 +7,23 @@
 
 namespace mwk {
 
-// Pivot block sizes of the FP32 and FP64 factorisations.
-constexpr int kInvBlock32 = 64, kInvBlock64 = 32;
-int inv_block(int prec);
+// Unknowns per pivot block, and the multiple to which a matrix is padded.
+constexpr int kInvBlock = 32, kInvPad = 64;
 
-// A batch of subdomains whose matrices share one workspace (positions: see k_inverse.cu).
+// A batch of subdomains whose matrices share one workspace (layout: see k_inverse.cu).
 struct InvBatch {
-  int count, steps, np_max;   // matrices, pivot blocks and order of the largest
+  int count, steps, np_max;   // matrices, pivot blocks and padded order of the largest
   const int32_t* d_sub;       // [count] subdomain ids
-  const int32_t* d_np;        // [count] padded order np (a multiple of the pivot block)
-  const int32_t* d_mn;        // [count] padded count of the unknowns not owned
+  const int32_t* d_n;         // [count] unknowns n
+  const int32_t* d_np;        // [count] n padded to a multiple of kInvPad
   const int64_t* d_off;       // [count] element offset of each matrix [np][np] in the workspace
-  const int64_t* d_poff;      // [count] element offset of its panel [2][block][np]
-  const int32_t* d_pos;       // position of every local unknown, at dof_ptr[s]
+  const int64_t* d_poff;      // [count] element offset of its panels [2][kInvBlock][np]
+  const int32_t* d_nsw;       // [steps][count] owned unknowns before the step's pivot block
   const int32_t* d_prefix;    // [steps][count + 1] running tile counts of the step's update
   const int32_t* h_tiles;     // [steps] their totals (host)
 };
-// Tiles of the update of pivot block kb in a matrix of order np with mn unknowns not owned.
-int64_t inv_update_tiles(int np, int mn, int kb);
+// Tiles of the update of pivot block kb in a matrix of n unknowns (padded np), nsw owned ones before it.
+int64_t inv_update_tiles(int n, int np, int nsw, int kb);
 
 // zc (optional): coefficients of the outer-face classes (surf_tet = -1 - class); metal
 // (optional, [E]): edges whose local rows and columns become those of the identity.  The workspace
@@ -32,8 +31,9 @@ int64_t inv_update_tiles(int np, int mn, int kb);
 void oras_local_assemble(const InvBatch& bt, const OrasTopo& tp, const double* Bsurf, const double* KM,
                          const double* eps, double k0, double eps_bg_re, double eps_bg_im, const double2* zc,
                          const uint8_t* metal, int prec, void* ws, cudaStream_t s);
-// dinv: 2 * count * block * block elements.
-void oras_invert(const InvBatch& bt, int prec, void* ws, void* dinv, int32_t* status, cudaStream_t s);
+// dinv: count * kInvBlock^2 elements.
+void oras_invert(const InvBatch& bt, const OrasTopo& tp, int prec, void* ws, void* dinv, int32_t* status,
+                 cudaStream_t s);
 void oras_extract(const InvBatch& bt, const OrasTopo& tp, int ws_prec, const void* ws, int w_prec,
                   const int64_t* w_off, void* W, cudaStream_t s);
 

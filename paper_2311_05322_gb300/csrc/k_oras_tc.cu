@@ -96,37 +96,37 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // One block per (subdomain of the batch, m tile, k tile); one 32-bit word per two dofs and plane.
 // ---------------------------------------------------------------------------------------
 template <typename T>
-__global__ void pack_w_kernel(InvBatch bt, const int64_t* __restrict__ dof_ptr, const int64_t* __restrict__ own_ptr,
+__global__ void pack_w_kernel(InvBatch bt, const int64_t* __restrict__ own_ptr, const int32_t* __restrict__ own_local,
                               const T* __restrict__ ws, const int64_t* __restrict__ sub_wtile,
                               const int32_t* __restrict__ sub_kt, uint8_t* __restrict__ W) {
   const int b = blockIdx.z;
   const int s = bt.d_sub[b];
-  const int np = bt.d_np[b], mn = bt.d_mn[b];
-  const int64_t n = dof_ptr[s + 1] - dof_ptr[s], nown = own_ptr[s + 1] - own_ptr[s];
+  const int64_t n = bt.d_n[b], np = bt.d_np[b];
+  const int64_t nown = own_ptr[s + 1] - own_ptr[s];
   const int mt = blockIdx.y, kt = blockIdx.x;
   const int KT = sub_kt[s];
   if (kt >= KT || (int64_t)mt * kTileM >= nown) return;
   const T* A = ws + bt.d_off[b];
-  const int32_t* pos = bt.d_pos + dof_ptr[s];
   uint8_t* tr = W + ((size_t)sub_wtile[s] + ((size_t)mt * KT + kt) * 2) * kATileBytes;
   uint8_t* ti = tr + kATileBytes;
   constexpr int kPairs = kTileKd / 2;
-  // entry (owned row q, unknown k) of -B_s^-1, of which the lower triangle is stored
-  auto entry = [&](int64_t q, int64_t k) {
-    const int p = mn + (int)q, c = pos[k];
-    const T v = A[(int64_t)max(p, c) * np + min(p, c)];
-    return make_float2((float)-v.x, (float)-v.y);
-  };
   for (int w = threadIdx.x; w < kTileM * kPairs; w += blockDim.x) {
     const int r = w / kPairs, kp = w % kPairs;
     const int64_t q = (int64_t)mt * kTileM + r, k = (int64_t)kt * kTileKd + 2 * kp;
-    float2 v0 = make_float2(0.f, 0.f), v1 = v0;
+    float re0 = 0.f, im0 = 0.f, re1 = 0.f, im1 = 0.f;
     if (q < nown) {
-      if (k < n) v0 = entry(q, k);
-      if (k + 1 < n) v1 = entry(q, k + 1);
+      const T* row = A + (int64_t)own_local[own_ptr[s] + q] * np;
+      if (k < n) {
+        re0 = (float)row[k].x;
+        im0 = (float)row[k].y;
+      }
+      if (k + 1 < n) {
+        re1 = (float)row[k + 1].x;
+        im1 = (float)row[k + 1].y;
+      }
     }
-    *reinterpret_cast<uint32_t*>(tr + swz(r, 2 * kp)) = pack_bf16(v0.x, v1.x);
-    *reinterpret_cast<uint32_t*>(ti + swz(r, 2 * kp)) = pack_bf16(v0.y, v1.y);
+    *reinterpret_cast<uint32_t*>(tr + swz(r, 2 * kp)) = pack_bf16(re0, re1);
+    *reinterpret_cast<uint32_t*>(ti + swz(r, 2 * kp)) = pack_bf16(im0, im1);
   }
 }
 
@@ -700,10 +700,10 @@ void tc_extract(const TcPlan& p, const InvBatch& bt, const OrasTopo& tp, int ws_
   const int mtmax = (bt.np_max + kTileM - 1) / kTileM;
   dim3 grid(ktmax, mtmax, bt.count);
   if (ws_prec == 0)
-    pack_w_kernel<double2><<<grid, 256, 0, s>>>(bt, tp.dof_ptr, tp.own_ptr, (const double2*)ws, p.sub_wtile,
+    pack_w_kernel<double2><<<grid, 256, 0, s>>>(bt, tp.own_ptr, tp.own_local, (const double2*)ws, p.sub_wtile,
                                                  p.sub_kt, (uint8_t*)W);
   else
-    pack_w_kernel<float2><<<grid, 256, 0, s>>>(bt, tp.dof_ptr, tp.own_ptr, (const float2*)ws, p.sub_wtile, p.sub_kt,
+    pack_w_kernel<float2><<<grid, 256, 0, s>>>(bt, tp.own_ptr, tp.own_local, (const float2*)ws, p.sub_wtile, p.sub_kt,
                                                 (uint8_t*)W);
 }
 

@@ -2691,27 +2691,16 @@ mw_status mw_setup_preconditioner(mw_ctx* c, int32_t n_sub, const int32_t* part,
               MW_EINVAL, "BF16 tensor-core apply unavailable for this partition");
     const size_t wes = p.apply_prec == 0 ? sizeof(double2) : sizeof(float2);
     const size_t fes = p.factor_prec == 0 ? sizeof(double2) : sizeof(float2);
-    // elimination order of every subdomain (unknowns not owned first, both parts padded to whole
-    // pivot blocks), and batches of subdomains whose matrices and panels fit the workspace
-    const int blk = mwk::inv_block(p.factor_prec);
-    auto pad = [&](int64_t n) { return (int32_t)((n + blk - 1) / blk * blk); };
-    std::vector<int32_t> np(n_sub), mn(n_sub), pos(sd.dofs.size());
+    // batches of subdomains whose matrices and panels fit the workspace
+    constexpr int blk = mwk::kInvBlock;
+    std::vector<int32_t> nn(n_sub), np(n_sub);
     auto ws_elems = [&](int s) { return (size_t)np[s] * np[s] + (size_t)2 * blk * np[s]; };
     size_t total = 0, largest = 0;
     for (int s = 0; s < n_sub; ++s) {
-      const int64_t n = sd.dof_ptr[s + 1] - sd.dof_ptr[s], no = sd.own_ptr[s + 1] - sd.own_ptr[s];
-      mn[s] = pad(n - no);
-      np[s] = mn[s] + pad(no);
-      require(np[s] <= (1 << 20), MW_EINVAL, "a subdomain is too large for a dense inverse");
-      int32_t a = 0, o = mn[s];
-      int64_t q = sd.own_ptr[s];
-      for (int64_t i = 0; i < n; ++i)
-        if (q < sd.own_ptr[s + 1] && sd.own_local[q] == i) {
-          pos[sd.dof_ptr[s] + i] = o++;
-          ++q;
-        } else {
-          pos[sd.dof_ptr[s] + i] = a++;
-        }
+      const int64_t n = sd.dof_ptr[s + 1] - sd.dof_ptr[s];
+      require(n <= (1 << 20), MW_EINVAL, "a subdomain is too large for a dense inverse");
+      nn[s] = (int32_t)n;
+      np[s] = (nn[s] + mwk::kInvPad - 1) / mwk::kInvPad * mwk::kInvPad;
       total += (ws_elems(s) * fes + 255) / 256 * 256;
       largest = std::max(largest, ws_elems(s) * fes);
     }
@@ -2719,7 +2708,7 @@ mw_status mw_setup_preconditioner(mw_ctx* c, int32_t n_sub, const int32_t* part,
     CK(cudaMemGetInfo(&free_b, &total_b));
     const size_t budget = std::max(largest, std::min({(size_t)8 << 30, free_b / 4, total}));
     struct Batch {
-      std::vector<int32_t> sub, np, mn, prefix, tiles;
+      std::vector<int32_t> sub, n, np, nsw, prefix, tiles;
       std::vector<int64_t> off, poff;
       int np_max = 0, steps = 0;
       size_t used = 0;
@@ -2731,26 +2720,30 @@ mw_status mw_setup_preconditioner(mw_ctx* c, int32_t n_sub, const int32_t* part,
       if (batches.empty() || batches.back().used + need > budget) batches.emplace_back();
       Batch& b = batches.back();
       b.sub.push_back(s);
+      b.n.push_back(nn[s]);
       b.np.push_back(np[s]);
-      b.mn.push_back(mn[s]);
       b.off.push_back((int64_t)(b.used / fes));
       b.poff.push_back(b.off.back() + (int64_t)np[s] * np[s]);
       b.used = (b.used + need + 255) / 256 * 256;
       b.np_max = std::max(b.np_max, (int)np[s]);
-      // owned rows of the inverse of a complex symmetric matrix by block sweeps (8 real flops per
-      // complex multiply-add): n^2 m / 2 - m^3 / 6 + (n - m) (n^2 - m^2) / 2 of them, m not owned
-      const double n = (double)(sd.dof_ptr[s + 1] - sd.dof_ptr[s]), o = (double)(sd.own_ptr[s + 1] - sd.own_ptr[s]);
-      const double m = n - o;
-      b.flops += 8.0 * (n * n * m / 2 - m * m * m / 6 + o * (n * n - m * m) / 2);
+      // Gauss-Jordan without the swept rows that are not owned: n^3 - m n^2 / 2 complex multiply-adds (8 real
+      // flops) with m unknowns not owned
+      const double n = nn[s], m = n - (double)(sd.own_ptr[s + 1] - sd.own_ptr[s]);
+      b.flops += 8.0 * n * n * (n - m / 2);
     }
     size_t max_count = 0, max_prefix = 0;
     for (Batch& b : batches) {
-      b.steps = b.np_max / blk;
+      for (int32_t n : b.n) b.steps = std::max(b.steps, (n + blk - 1) / blk);
+      std::vector<int64_t> next(b.sub.size());       // first owned unknown at or after the pivot block
+      for (size_t i = 0; i < b.sub.size(); ++i) next[i] = sd.own_ptr[b.sub[i]];
       for (int k = 0; k < b.steps; ++k) {
         int64_t run = 0;
         for (size_t i = 0; i < b.sub.size(); ++i) {
+          const int s = b.sub[i];
+          while (next[i] < sd.own_ptr[s + 1] && sd.own_local[next[i]] < k * blk) ++next[i];
+          b.nsw.push_back((int32_t)(next[i] - sd.own_ptr[s]));
           b.prefix.push_back((int32_t)run);
-          run += mwk::inv_update_tiles(b.np[i], b.mn[i], k * blk);
+          run += mwk::inv_update_tiles(b.n[i], b.np[i], b.nsw.back(), k * blk);
         }
         require(run < INT32_MAX, MW_EINVAL, "too many update tiles in one batch");
         b.prefix.push_back((int32_t)run);
@@ -2770,12 +2763,11 @@ mw_status mw_setup_preconditioner(mw_ctx* c, int32_t n_sub, const int32_t* part,
       int32_t* d_status = (int32_t*)scratch(sizeof(int32_t));
       CK(cudaMemsetAsync(d_status, 0, sizeof(int32_t), c->stream));
       void* ws = scratch(budget);
-      int32_t* d_pos = (int32_t*)scratch(sizeof(int32_t) * pos.size());
-      CK(cudaMemcpyAsync(d_pos, pos.data(), sizeof(int32_t) * pos.size(), cudaMemcpyHostToDevice, c->stream));
       int32_t* d_i32 = (int32_t*)scratch(sizeof(int32_t) * 3 * max_count);
       int64_t* d_i64 = (int64_t*)scratch(sizeof(int64_t) * 2 * max_count);
       int32_t* d_prefix = (int32_t*)scratch(sizeof(int32_t) * max_prefix);
-      void* dinv = scratch(2 * max_count * blk * blk * fes);
+      int32_t* d_nsw = (int32_t*)scratch(sizeof(int32_t) * max_prefix);
+      void* dinv = scratch(max_count * blk * blk * fes);
       for (int f = 0; f < c->n_freq; ++f) {
         if (p.apply_prec == 2)
           p.W[f] = dalloc<unsigned char>(c, mwk::tc_w_bytes(p.tc));
@@ -2788,20 +2780,21 @@ mw_status mw_setup_preconditioner(mw_ctx* c, int32_t n_sub, const int32_t* part,
             CK(cudaMemcpyAsync(d, h, bytes, cudaMemcpyHostToDevice, c->stream));
           };
           put(d_i32, b.sub.data(), sizeof(int32_t) * cnt);
-          put(d_i32 + cnt, b.np.data(), sizeof(int32_t) * cnt);
-          put(d_i32 + 2 * cnt, b.mn.data(), sizeof(int32_t) * cnt);
+          put(d_i32 + cnt, b.n.data(), sizeof(int32_t) * cnt);
+          put(d_i32 + 2 * cnt, b.np.data(), sizeof(int32_t) * cnt);
           put(d_i64, b.off.data(), sizeof(int64_t) * cnt);
           put(d_i64 + cnt, b.poff.data(), sizeof(int64_t) * cnt);
           put(d_prefix, b.prefix.data(), sizeof(int32_t) * b.prefix.size());
-          const mwk::InvBatch bt{cnt,   b.steps,     b.np_max, d_i32,    d_i32 + cnt,    d_i32 + 2 * cnt,
-                                 d_i64, d_i64 + cnt, d_pos,    d_prefix, b.tiles.data()};
+          put(d_nsw, b.nsw.data(), sizeof(int32_t) * b.nsw.size());
+          const mwk::InvBatch bt{cnt,   b.steps,     b.np_max, d_i32,    d_i32 + cnt,   d_i32 + 2 * cnt,
+                                 d_i64, d_i64 + cnt, d_nsw,    d_prefix, b.tiles.data()};
           CK(cudaMemsetAsync(ws, 0, b.used, c->stream));
           const double2* zc = c->d_zc ? c->d_zc + (size_t)f * (2 + c->n_port) : nullptr;
           mwk::oras_local_assemble(bt, p.topo(), p.Bsurf, c->d_KM, c->d_eps, k0, c->eps_bg[0], c->eps_bg[1], zc,
                                    c->d_metal, p.factor_prec, ws, c->stream);
           {
             ProfScope ps(c, MW_K_FACTOR, 0.0, b.flops);
-            mwk::oras_invert(bt, p.factor_prec, ws, dinv, d_status, c->stream);
+            mwk::oras_invert(bt, p.topo(), p.factor_prec, ws, dinv, d_status, c->stream);
           }
           if (p.apply_prec == 2)
             mwk::tc_extract(p.tc, bt, p.topo(), p.factor_prec, ws, p.W[f], c->stream);

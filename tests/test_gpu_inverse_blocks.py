@@ -1,6 +1,5 @@
-"""Dense subdomain inverses by block sweeps: sizes around the pivot blocks (64 in FP32, 32 in FP64) and
-the 128 x 64 update tiles, subdomains that own everything, little or nothing, against the oracle's
-exact subdomain solves (bars of the parity tests: 1e-11 FP64, 2e-5 FP32, 1e-2 BF16)."""
+"""Dense subdomain inverses: sizes around the 32-wide pivot blocks and the 64 x 64 update tiles,
+subdomains that own everything, little or nothing, against the oracle's exact subdomain solves (bars of the parity tests: 1e-11 FP64, 2e-5 FP32, 1e-2 BF16)."""
 import numpy as np
 import pytest
 
