@@ -385,67 +385,90 @@ __device__ __forceinline__ void cp_async16(void* s, const void* g) {
 
 // A_IJ -= C_I R_J on tiles of 64 active rows x 64 columns, 8 x 4 complex per thread.  FP32 (FP64) pipes bound
 // it: 1.05 MFLOP per 32 KB of operands and 64 KB of A read and written (FP32), 8 x 4 outputs per 6 shared-memory
-// loads of a warp's 128 multiply-adds.  The operands arrive in two cp.async groups; four blocks of 128 threads
-// per SM overlap one's loads and epilogue with the others' products.  The grid holds the tiles that exist: block
-// -> matrix by the step's prefix sums.  (4 x 4 outputs per thread, eight loads for 64 multiply-adds, over full
-// squares of the largest size, most of them empty: 30 TFLOP/s.)
+// loads of a warp's 128 multiply-adds.  Persistent blocks of 128 threads, three per SM (FP32), take every
+// gridDim-th of the step's tiles: the next tile's operands (two buffers, cp.async) and this tile's part of A (L2
+// prefetch) are on their way during the products, and the matrix of a tile is found by stepping on through the
+// prefix sums.  One block per tile waited for its search, its operands and A half of the time (FMA pipe 49 %).
+// (4 x 4 outputs per thread over full squares of the largest size, most of them empty: 30 TFLOP/s.)
 constexpr int kUp = 64;
+constexpr int kUpBlocks = 3;                        // per SM, by shared memory in FP32
 template <typename T>
-__global__ void __launch_bounds__(128, sizeof(T) == 8 ? 4 : 2) inv_update_kernel(InvBatch bt, OrasTopo tp,
-                                                                                 T* __restrict__ ws, int kb,
-                                                                                 const int32_t* __restrict__ nsws,
-                                                                                 const int32_t* __restrict__ prefix) {
+__global__ void __launch_bounds__(128, sizeof(T) == 8 ? kUpBlocks : 1) inv_update_kernel(
+    InvBatch bt, OrasTopo tp, T* __restrict__ ws, int kb, const int32_t* __restrict__ nsws,
+    const int32_t* __restrict__ prefix, int n_tiles) {
   constexpr int VEC = 16 / (int)sizeof(T);          // elements per 16-byte copy
-  constexpr int G = 2, QG = NB / G;                 // copy groups, k rows of each
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* Cs = reinterpret_cast<T*>(smem_raw);           // [q][64]
-  T* Rs = Cs + NB * kUp;                            // [q][64]
-  const int lane = threadIdx.x & 31;
-  // largest b with prefix[b] <= blockIdx.x (32-way search, every warp alike)
-  int lo = 0, hi = bt.count;
-  while (hi - lo > 1) {
-    const int step = (hi - lo + 31) / 32, q = lo + (lane + 1) * step;
-    const unsigned le = __ballot_sync(0xffffffffu, q < hi && prefix[q] <= (int)blockIdx.x);
-    const int k = __popc(le);
-    hi = min(hi, lo + (k + 1) * step);
-    lo += k * step;
-  }
-  const int b = lo;
-  const int np = bt.d_np[b], n = bt.d_n[b], nsw = nsws[b];
-  const int nj = np / kUp, idx = (int)blockIdx.x - prefix[b];
-  const int p0 = idx / nj * kUp, n0 = idx % nj * kUp;
-  const int count = nsw + max(0, n - kb - NB);
-  T* A = ws + bt.d_off[b];
-  const T* C = ws + bt.d_poff[b];
-  const T* Rp = C + (int64_t)NB * np;
   constexpr int CC = kUp / VEC;
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    for (int e = threadIdx.x; e < QG * 2 * CC; e += 128) {
-      const int q = g * QG + e / (2 * CC), c = e % (2 * CC);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int rows[kUp];
+  T* Sm = reinterpret_cast<T*>(smem_raw);           // two of {C [q][64], R [q][64]}
+  struct Tile {
+    int np, count, nsw, p0, n0;
+    T* A;
+    const T* C;
+    const int32_t* own;
+  };
+  int b = 0;
+  auto locate = [&](int t, Tile& x) {
+    while (prefix[b + 1] <= t) ++b;
+    const int s = bt.d_sub[b];
+    x.np = bt.d_np[b];
+    x.nsw = nsws[b];
+    x.count = x.nsw + max(0, bt.d_n[b] - kb - NB);
+    const int idx = t - prefix[b], nj = x.np / kUp;
+    x.p0 = idx / nj * kUp;
+    x.n0 = idx % nj * kUp;
+    x.A = ws + bt.d_off[b];
+    x.C = ws + bt.d_poff[b];
+    x.own = tp.own_local + tp.own_ptr[s];
+  };
+  auto fetch = [&](const Tile& x, int buf) {
+    T* Cs = Sm + (size_t)buf * 2 * NB * kUp;
+    for (int e = threadIdx.x; e < NB * 2 * CC; e += 128) {
+      const int q = e / (2 * CC), c = e % (2 * CC);
       if (c < CC) {
-        if (p0 + c * VEC < np) cp_async16(Cs + q * kUp + c * VEC, C + (int64_t)q * np + p0 + c * VEC);
+        if (x.p0 + c * VEC < x.np) cp_async16(Cs + q * kUp + c * VEC, x.C + (int64_t)q * x.np + x.p0 + c * VEC);
       } else {
-        cp_async16(Rs + q * kUp + (c - CC) * VEC, Rp + (int64_t)q * np + n0 + (c - CC) * VEC);
+        cp_async16(Cs + (NB + q) * kUp + (c - CC) * VEC, x.C + (int64_t)(NB + q) * x.np + x.n0 + (c - CC) * VEC);
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
-  }
-  const int tr = threadIdx.x / 16, tc = threadIdx.x % 16;     // rows 4 tr + 0..3 and + 32, columns 2 tc + 0..1 and + 32
-  T acc[8][4];
+  };
+  const int tr = threadIdx.x / 16, tc = threadIdx.x % 16;   // rows 4 tr + 0..3 and + 32, columns 2 tc + 0..1 and + 32
+  Tile cur, nxt;
+  locate(blockIdx.x, cur);
+  fetch(cur, 0);
+  for (int t = blockIdx.x, buf = 0; t < n_tiles; t += gridDim.x, buf ^= 1) {
+    const bool more = t + (int)gridDim.x < n_tiles;
+    {
+      // the tile's rows, and half a row of its part of A per thread into L2
+      const int p = cur.p0 + (int)threadIdx.x / 2;
+      const int row = p < cur.count ? active_row(cur.own, cur.nsw, kb, p) : -1;
+      if (!(threadIdx.x & 1)) rows[threadIdx.x / 2] = row;
+      if (row >= 0) {
+        const char* a =
+            reinterpret_cast<const char*>(cur.A + (int64_t)row * cur.np + cur.n0 + (threadIdx.x & 1) * (kUp / 2));
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = T{0, 0};
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    if (g == 0)
+        for (int o = 0; o < (int)sizeof(T) * kUp / 2; o += 128)
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(a + o));
+      }
+    }
+    if (more) {
+      locate(t + gridDim.x, nxt);
+      fetch(nxt, buf ^ 1);
       asm volatile("cp.async.wait_group 1;" ::: "memory");
-    else
+    } else {
       asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
     __syncthreads();
+    const T* Cs = Sm + (size_t)buf * 2 * NB * kUp;
+    const T* Rs = Cs + NB * kUp;
+    T acc[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = T{0, 0};
 #pragma unroll 2
-    for (int q = g * QG; q < (g + 1) * QG; ++q) {
+    for (int q = 0; q < NB; ++q) {
       T a[8], p[4];
 #pragma unroll
       for (int i = 0; i < 8; i += 2) load_pair(Cs + q * kUp + (i < 4 ? 0 : 32) + tr * 4 + i % 4, a[i], a[i + 1]);
@@ -456,21 +479,34 @@ __global__ void __launch_bounds__(128, sizeof(T) == 8 ? 4 : 2) inv_update_kernel
 #pragma unroll
         for (int j = 0; j < 4; ++j) cfma(acc[i][j], a[i], p[j]);
     }
-  }
-  const int32_t* own = tp.own_local + tp.own_ptr[bt.d_sub[b]];
+    // four rows at a time: all their loads of A in flight together
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int p = p0 + (i < 4 ? 0 : 32) + tr * 4 + i % 4;
-    if (p >= count) continue;
-    T* Ar = A + (int64_t)active_row(own, nsw, kb, p) * np;
+    for (int h = 0; h < 8; h += 4) {
+      T* Ar[4];
+      T u[4][4];
+      bool ok[4][2];
 #pragma unroll
-    for (int j = 0; j < 4; j += 2) {
-      const int c = n0 + (j < 2 ? 0 : 32) + tc * 2;
-      if (c >= kb && c < kb + NB) continue;         // pivot blocks start at multiples of 32: the pair is inside or outside
-      T u, w;
-      load_pair(Ar + c, u, w);
-      store_pair(Ar + c, T{u.x - acc[i][j].x, u.y - acc[i][j].y}, T{w.x - acc[i][j + 1].x, w.y - acc[i][j + 1].y});
+      for (int i = 0; i < 4; ++i) {
+        const int row = rows[h * 8 + tr * 4 + i];
+        Ar[i] = cur.A + (int64_t)row * cur.np + cur.n0 + tc * 2;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int c = cur.n0 + 32 * j + tc * 2;   // pivot blocks start at multiples of 32: the pair is inside or outside
+          ok[i][j] = row >= 0 && (c < kb || c >= kb + NB);
+          if (ok[i][j]) load_pair(Ar[i] + 32 * j, u[i][2 * j], u[i][2 * j + 1]);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          if (ok[i][j]) {
+            const T x = acc[h + i][2 * j], y = acc[h + i][2 * j + 1], v = u[i][2 * j], w = u[i][2 * j + 1];
+            store_pair(Ar[i] + 32 * j, T{v.x - x.x, v.y - x.y}, T{w.x - y.x, w.y - y.y});
+          }
     }
+    __syncthreads();                                // this buffer is filled again in the next round
+    cur = nxt;
   }
 }
 
@@ -492,7 +528,7 @@ __global__ void extract_owned_kernel(InvBatch bt, OrasTopo tp, const T* __restri
 
 template <typename T>
 void invert_all(const InvBatch& bt, const OrasTopo& tp, T* ws, T* dinv, int32_t* status, cudaStream_t st) {
-  constexpr size_t up_smem = sizeof(T) * NB * 2 * kUp;
+  constexpr size_t up_smem = sizeof(T) * NB * 2 * kUp * 2;
   constexpr size_t pa_smem = sizeof(T) * (NB * (kPan + 1) + NB * NB);
   static const cudaError_t attr[2] = {
       cudaFuncSetAttribute(inv_update_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)up_smem),
@@ -506,8 +542,9 @@ void invert_all(const InvBatch& bt, const OrasTopo& tp, T* ws, T* dinv, int32_t*
     inv_panel_kernel<T><<<dim3(2 * jt, bt.count), 256, pa_smem, st>>>(bt, tp, ws, kb, jt, dinv, nsws);
     if (bt.h_tiles[k] == 0) continue;
     note_launch(1);
-    inv_update_kernel<T><<<bt.h_tiles[k], 128, up_smem, st>>>(bt, tp, ws, kb, nsws,
-                                                             bt.d_prefix + (size_t)k * (bt.count + 1));
+    constexpr int blocks = 152 * (sizeof(T) == 8 ? kUpBlocks : 1);
+    inv_update_kernel<T><<<std::min(bt.h_tiles[k], blocks), 128, up_smem, st>>>(
+        bt, tp, ws, kb, nsws, bt.d_prefix + (size_t)k * (bt.count + 1), bt.h_tiles[k]);
   }
 }
 
