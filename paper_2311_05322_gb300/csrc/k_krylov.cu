@@ -736,9 +736,22 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 __device__ __forceinline__ double2 conjd(double2 a) { return make_double2(a.x, -a.y); }
 __device__ __forceinline__ double cabs2(double2 a) { return a.x * a.x + a.y * a.y; }
 
-// One thread per column: Hessenberg column j from h[0..j] and ||w||, previous rotations,
-// new rotation, residual estimate |g[j+1]| against the target.
-// One warp per column: the lanes sum the column's norm partials (fixed order: lane l takes parts
+// Adds a block's count of active columns (thread 0's `mine`) to state[0]; the launch's last block publishes the
+// total to the device word (read by the conditional graph nodes) and to the host's mapped word (read after
+// a synchronisation, no copy), and leaves the state zero for the next launch.
+__device__ __forceinline__ void publish_active(int mine, int32_t* state, int32_t* active, volatile int32_t* host) {
+  atomicAdd(&state[0], mine);
+  __threadfence();
+  if (atomicAdd(&state[1], 1) != (int)gridDim.x - 1) return;
+  const int total = atomicExch(&state[0], 0);
+  state[1] = 0;
+  *active = total;
+  *host = total;
+  __threadfence_system();
+}
+
+// Hessenberg column j from h[0..j] and ||w||, previous rotations, new rotation, residual estimate
+// |g[j+1]| against the target.  One warp per column: the lanes sum the column's norm partials (fixed order: lane l takes parts
 // l, l + 32, ..., then an xor-shuffle tree) and stage the new Hessenberg column and the stored
 // rotations in shared memory; lane 0 applies the rotations (a sequential chain) and forms the
 // new one; the lanes write the column back.
@@ -746,70 +759,80 @@ constexpr int kGivensWarps = 4;
 __global__ void __launch_bounds__(32 * kGivensWarps) givens_kernel(
     const double2* __restrict__ h, const double* __restrict__ npart, int nparts, int j, int m, int R,
     double2* __restrict__ H, double2* __restrict__ cs, double2* __restrict__ g, const double* __restrict__ target,
-    int32_t* __restrict__ done, int32_t* __restrict__ kcol, double* __restrict__ scale, int32_t* __restrict__ active) {
+    int32_t* __restrict__ done, int32_t* __restrict__ kcol, double* __restrict__ scale, int32_t* __restrict__ state,
+    int32_t* __restrict__ active, int32_t* __restrict__ host_active) {
+  __shared__ int go_on[kGivensWarps];
   __shared__ double2 hs_all[kGivensWarps][64], rc_all[kGivensWarps][64], rs_all[kGivensWarps][64];
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c = blockIdx.x * kGivensWarps + wib;
-  if (c >= R) return;
-  if (done[c]) {
-    if (lane == 0) scale[c] = 0.0;
-    return;
-  }
-  double2* hs = hs_all[wib];
-  double2* rc = rc_all[wib];
-  double2* rs = rs_all[wib];
-  double nn = 0.0;
-#pragma unroll 8
-  for (int p = lane; p < nparts; p += 32) nn += npart[(int64_t)p * R + c];
-  for (int off = 16; off > 0; off >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, off);
-  const double hn = sqrt(nn);
-  double2* Hc = H + ((int64_t)c * m + j) * (m + 1);
-  double2* csc = cs + (int64_t)c * 2 * m;
-  for (int i = lane; i <= j; i += 32) hs[i] = h[i * R + c];
-  for (int i = lane; i < j; i += 32) {
-    rc[i] = csc[2 * i];
-    rs[i] = csc[2 * i + 1];
-  }
-  __syncwarp();
+  const bool mine = c < R && !done[c];
   if (lane == 0) {
-    hs[j + 1] = make_double2(hn, 0.0);
-    for (int i = 0; i < j; ++i) {
-      const double2 ci = rc[i], si = rs[i];
-      const double2 a = hs[i], b = hs[i + 1];
-      hs[i] = cadd(cmul(ci, a), cmul(si, b));
-      hs[i + 1] = cadd(cmul(make_double2(-si.x, si.y), a), cmul(conjd(ci), b));  // -conj(s) a + conj(c) b
-    }
-    const double2 a = hs[j], b = hs[j + 1];
-    const double den = sqrt(cabs2(a) + cabs2(b));
-    double2 cj, sj;
-    if (den == 0.0) {
-      cj = make_double2(1.0, 0.0);
-      sj = make_double2(0.0, 0.0);
-    } else {
-      cj = make_double2(a.x / den, -a.y / den);   // conj(a)/den
-      sj = make_double2(b.x / den, -b.y / den);   // conj(b)/den
-    }
-    csc[2 * j] = cj;
-    csc[2 * j + 1] = sj;
-    hs[j] = make_double2(den, 0.0);
-    hs[j + 1] = make_double2(0.0, 0.0);
-    double2* gc = g + (int64_t)c * (m + 1);
-    const double2 gj = gc[j];
-    gc[j + 1] = cmul(make_double2(-sj.x, sj.y), gj);   // -conj(s) g_j
-    gc[j] = cmul(cj, gj);
-    const double res = sqrt(cabs2(gc[j + 1]));
-    const bool stop = (res <= target[c]) || (hn == 0.0) || (j + 1 >= m) || !(res == res);
-    kcol[c] = j + 1;
-    if (stop) {
-      done[c] = 1;
-      scale[c] = 0.0;
-    } else {
-      scale[c] = 1.0 / hn;
-      atomicAdd(active, 1);
-    }
+    go_on[wib] = 0;
+    if (c < R && !mine) scale[c] = 0.0;
   }
-  __syncwarp();
-  for (int i = lane; i <= j + 1; i += 32) Hc[i] = hs[i];
+  if (mine) {
+    double2* hs = hs_all[wib];
+    double2* rc = rc_all[wib];
+    double2* rs = rs_all[wib];
+    double nn = 0.0;
+#pragma unroll 8
+    for (int p = lane; p < nparts; p += 32) nn += npart[(int64_t)p * R + c];
+    for (int off = 16; off > 0; off >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, off);
+    const double hn = sqrt(nn);
+    double2* Hc = H + ((int64_t)c * m + j) * (m + 1);
+    double2* csc = cs + (int64_t)c * 2 * m;
+    for (int i = lane; i <= j; i += 32) hs[i] = h[i * R + c];
+    for (int i = lane; i < j; i += 32) {
+      rc[i] = csc[2 * i];
+      rs[i] = csc[2 * i + 1];
+    }
+    __syncwarp();
+    if (lane == 0) {
+      hs[j + 1] = make_double2(hn, 0.0);
+      for (int i = 0; i < j; ++i) {
+        const double2 ci = rc[i], si = rs[i];
+        const double2 a = hs[i], b = hs[i + 1];
+        hs[i] = cadd(cmul(ci, a), cmul(si, b));
+        hs[i + 1] = cadd(cmul(make_double2(-si.x, si.y), a), cmul(conjd(ci), b));  // -conj(s) a + conj(c) b
+      }
+      const double2 a = hs[j], b = hs[j + 1];
+      const double den = sqrt(cabs2(a) + cabs2(b));
+      double2 cj, sj;
+      if (den == 0.0) {
+        cj = make_double2(1.0, 0.0);
+        sj = make_double2(0.0, 0.0);
+      } else {
+        cj = make_double2(a.x / den, -a.y / den);   // conj(a)/den
+        sj = make_double2(b.x / den, -b.y / den);   // conj(b)/den
+      }
+      csc[2 * j] = cj;
+      csc[2 * j + 1] = sj;
+      hs[j] = make_double2(den, 0.0);
+      hs[j + 1] = make_double2(0.0, 0.0);
+      double2* gc = g + (int64_t)c * (m + 1);
+      const double2 gj = gc[j];
+      gc[j + 1] = cmul(make_double2(-sj.x, sj.y), gj);   // -conj(s) g_j
+      gc[j] = cmul(cj, gj);
+      const double res = sqrt(cabs2(gc[j + 1]));
+      const bool stop = (res <= target[c]) || (hn == 0.0) || (j + 1 >= m) || !(res == res);
+      kcol[c] = j + 1;
+      if (stop) {
+        done[c] = 1;
+        scale[c] = 0.0;
+      } else {
+        scale[c] = 1.0 / hn;
+        go_on[wib] = 1;
+      }
+    }
+    __syncwarp();
+    for (int i = lane; i <= j + 1; i += 32) Hc[i] = hs[i];
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int n = 0;
+    for (int w = 0; w < kGivensWarps; ++w) n += go_on[w];
+    publish_active(n, state, active, host_active);
+  }
 }
 
 template <typename T>
@@ -826,11 +849,12 @@ __global__ void scale_cols_kernel(T* __restrict__ v, const double* __restrict__ 
 }
 
 // Start of a cycle, one block per column: ||r|| from partials, per-column target and state; columns
-// already within tol of ||b|| are marked done, the others counted in *active (zeroed before).
+// already within tol of ||b|| are marked done, the others counted (publish_active).
 __global__ void __launch_bounds__(kColThreads) start_state_kernel(
     const double* __restrict__ npart, int nparts, int R, const double* __restrict__ bnorm, double tol,
     double inner_tol, int fp64_mode, double* __restrict__ rnorm, double2* __restrict__ g, double* __restrict__ target,
-    int32_t* __restrict__ done, int32_t* __restrict__ kcol, int m, int32_t* __restrict__ active) {
+    int32_t* __restrict__ done, int32_t* __restrict__ kcol, int m, int32_t* __restrict__ state,
+    int32_t* __restrict__ active, int32_t* __restrict__ host_active) {
   const int c = blockIdx.x;
   const double rn = sqrt(sum_column_parts(npart, nparts, R, c));
   double2* gc = g + (int64_t)c * (m + 1);
@@ -841,10 +865,10 @@ __global__ void __launch_bounds__(kColThreads) start_state_kernel(
   const bool conv = !(rn > goal);
   done[c] = conv ? 1 : 0;
   kcol[c] = 0;
-  if (!conv) atomicAdd(active, 1);
   // FP64 mode: aim a little below tol so the recomputed true residual passes;
   // mixed mode: reduce the residual by inner_tol (never below half the final goal).
   target[c] = fp64_mode ? 0.5 * goal : fmax(inner_tol * rn, 0.5 * goal);
+  publish_active(conv ? 0 : 1, state, active, host_active);
 }
 
 template <typename T>
@@ -861,10 +885,14 @@ __global__ void normalize_start_kernel(const double2* __restrict__ r, const doub
 }
 
 // v0 = r / |r| per column from an FP32 residual (mixed mode): the column scales are formed once
-// per block in shared memory, the column index advances with the grid stride.
+// per block in shared memory, the column index advances with the grid stride.  vscale (optional): the factors
+// of an unscaled basis; v0 is stored scaled, so its row of factors is set to one.
 __global__ void normalize_start32_kernel(const float2* __restrict__ r, const double* __restrict__ rnorm,
-                                         const int32_t* __restrict__ done, int64_t E, int R, float2* __restrict__ v0) {
+                                         const int32_t* __restrict__ done, int64_t E, int R, float2* __restrict__ v0,
+                                         double* __restrict__ vscale) {
   extern __shared__ float sc[];
+  if (vscale && blockIdx.x == 0)
+    for (int c = threadIdx.x; c < R; c += blockDim.x) vscale[c] = 1.0;
   for (int c = threadIdx.x; c < R; c += blockDim.x) sc[c] = done[c] ? 0.f : (float)(1.0 / rnorm[c]);
   __syncthreads();
   const int64_t n = E * R;
@@ -1011,10 +1039,13 @@ __global__ void __launch_bounds__(kBdThreads, 2)
       mbar_init(&empty[i], kBdConsumers / 32);   // one arrival per consumer warp
     }
     *abort_flag = 0;
-    int km = 0;
-    for (int c = 0; c < R; ++c) km = max(km, min(kcol[c], m));
-    kmax_s = km;
     mbar_init_fence();
+  }
+  if (tid >= 32 && tid < 64) {
+    int km = 0;
+    for (int c = tid - 32; c < R; c += 32) km = max(km, min(kcol[c], m));
+    km = __reduce_max_sync(0xffffffffu, km);
+    if (tid == 32) kmax_s = km;
   }
   for (int t = tid; t < R; t += kBdThreads) ks[t] = kcol[t];
   for (int t = tid; t < m * R; t += kBdThreads) {
@@ -1245,10 +1276,6 @@ int update_launch(const T* V, int64_t vstride, int nvec, const double2* h, T* w,
   return nb;
 }
 
-__global__ void fill_f64_kernel(double* __restrict__ x, int n, double v) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) x[i] = v;
-}
-
 // Deterministic pseudo-random fill in [-1, 1) (timing inputs of the launch-shape tuner).
 template <typename F>
 __global__ void fill_pattern_kernel(F* __restrict__ x, int64_t n, uint32_t seed, double scale) {
@@ -1274,10 +1301,6 @@ __global__ void set_step_conditions_kernel(StepHandles sh, const int32_t* __rest
 
 }  // namespace
 
-void fill_f64(double* x, int n, double v, cudaStream_t s) {
-  note_launch(1);
-  fill_f64_kernel<<<(n + 255) / 256 < 64 ? (n + 255) / 256 : 64, 256, 0, s>>>(x, n, v);
-}
 void fill_pattern_f32(float* x, int64_t n, uint32_t seed, cudaStream_t s, double scale) {
   note_launch(1);
   fill_pattern_kernel<float><<<gs_blocks(n), 256, 0, s>>>(x, n, seed, scale);
@@ -1339,11 +1362,11 @@ void reduce_cols(const double* part, int nparts, int R, double* out, cudaStream_
   reduce_cols_kernel<<<R, kColThreads, 0, s>>>(part, nparts, R, out);
 }
 void givens_step(const double2* h, const double* npart, int nparts, int j, int m, int R, double2* H, double2* cs,
-                 double2* gvec, double* target, int32_t* done, int32_t* kcol, double* scale, int32_t* active_count,
-                 cudaStream_t s) {
+                 double2* gvec, double* target, int32_t* done, int32_t* kcol, double* scale, int32_t* state,
+                 int32_t* active, int32_t* host_active, cudaStream_t s) {
   note_launch(1);
   givens_kernel<<<(R + kGivensWarps - 1) / kGivensWarps, 32 * kGivensWarps, 0, s>>>(
-      h, npart, nparts, j, m, R, H, cs, gvec, target, done, kcol, scale, active_count);
+      h, npart, nparts, j, m, R, H, cs, gvec, target, done, kcol, scale, state, active, host_active);
 }
 void scale_cols_f64(double2* v, const double* scale, int64_t E, int R, cudaStream_t s) {
   note_launch(1);
@@ -1355,10 +1378,10 @@ void scale_cols_f32(float2* v, const double* scale, int64_t E, int R, cudaStream
 }
 void start_state(const double* npart, int nparts, int R, const double* bnorm, double tol, double inner_tol,
                  int fp64_mode, double* rnorm, double2* gvec, double* target, int32_t* done, int32_t* kcol, int m,
-                 int32_t* active, cudaStream_t s) {
+                 int32_t* state, int32_t* active, int32_t* host_active, cudaStream_t s) {
   note_launch(1);
   start_state_kernel<<<R, kColThreads, 0, s>>>(npart, nparts, R, bnorm, tol, inner_tol, fp64_mode, rnorm, gvec, target,
-                                               done, kcol, m, active);
+                                               done, kcol, m, state, active, host_active);
 }
 void normalize_start_f64(const double2* r, const double* rnorm, const int32_t* done, int64_t E, int R, double2* v0,
                          cudaStream_t s) {
@@ -1371,9 +1394,9 @@ void normalize_start_f32(const double2* r, const double* rnorm, const int32_t* d
   normalize_start_kernel<float2><<<gs_blocks(E * R), 256, 0, s>>>(r, rnorm, done, E, R, v0);
 }
 void normalize_start32(const float2* r, const double* rnorm, const int32_t* done, int64_t E, int R, float2* v0,
-                       cudaStream_t s) {
+                       double* vscale, cudaStream_t s) {
   note_launch(1);
-  normalize_start32_kernel<<<gs_blocks(E * R), 256, sizeof(float) * R, s>>>(r, rnorm, done, E, R, v0);
+  normalize_start32_kernel<<<gs_blocks(E * R), 256, sizeof(float) * R, s>>>(r, rnorm, done, E, R, v0, vscale);
 }
 void solve_hessenberg(const double2* H, const double2* gvec, const int32_t* kcol, int m, int R, double2* y,
                       cudaStream_t s) {

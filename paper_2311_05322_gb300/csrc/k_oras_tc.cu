@@ -647,7 +647,8 @@ inline int rpad(int R) { return (R + 7) / 8 * 8; }
 
 }  // namespace
 
-bool tc_plan_build(TcPlan& p, const mw::Subdomains& sd, const std::function<void*(size_t)>& alloc, cudaStream_t s) {
+bool tc_plan_build(TcPlan& p, const mw::Subdomains& sd, const std::function<void*(size_t)>& alloc, int32_t* err,
+                   cudaStream_t s) {
   p = TcPlan();
   const int ns = sd.n_sub;
   std::vector<int32_t> mt_sub, mt_row0, sub_kt(ns), gt_sub, gt_kt;
@@ -700,8 +701,7 @@ bool tc_plan_build(TcPlan& p, const mw::Subdomains& sd, const std::function<void
   p.sub_kt = (int32_t*)up(sub_kt.data(), sizeof(int32_t) * ns);
   p.gt_sub = (int32_t*)up(gt_sub.data(), sizeof(int32_t) * std::max<size_t>(gt_sub.size(), 1));
   p.gt_kt = (int32_t*)up(gt_kt.data(), sizeof(int32_t) * std::max<size_t>(gt_kt.size(), 1));
-  p.err = (int32_t*)alloc(sizeof(int32_t));
-  cudaMemsetAsync(p.err, 0, sizeof(int32_t), s);
+  p.err = err;
   cudaStreamSynchronize(s);  // host vectors go out of scope
   p.max_kt = 0;
   for (int q = 0; q < ns; ++q) p.max_kt = std::max(p.max_kt, sub_kt[q]);
@@ -711,7 +711,7 @@ bool tc_plan_build(TcPlan& p, const mw::Subdomains& sd, const std::function<void
 
 void tc_plan_free(TcPlan& p, const std::function<void(void*)>& dfree) {
   for (void* q : {(void*)p.mt_sub, (void*)p.mt_row0, (void*)p.sub_wtile, (void*)p.sub_gtile, (void*)p.sub_kt,
-                  (void*)p.gt_sub, (void*)p.gt_kt, (void*)p.err})
+                  (void*)p.gt_sub, (void*)p.gt_kt})
     if (q) dfree(q);
   p = TcPlan();
 }

@@ -29,11 +29,13 @@ struct TcPlan {
   int32_t* sub_kt = nullptr;     // [n_sub] k tiles of s
   int32_t* gt_sub = nullptr;     // [n_ktiles_total] subdomain of each gathered-operand tile
   int32_t* gt_kt = nullptr;      // [n_ktiles_total] its k tile
-  int32_t* err = nullptr;        // device error word: nonzero after a timed-out wait
+  int32_t* err = nullptr;        // error word (mapped host memory): nonzero after a timed-out wait
   int max_kt = 0;
 };
 
-bool tc_plan_build(TcPlan& p, const mw::Subdomains& sd, const std::function<void*(size_t)>& alloc, cudaStream_t s);
+// err: device address of the error word, kept by the caller.
+bool tc_plan_build(TcPlan& p, const mw::Subdomains& sd, const std::function<void*(size_t)>& alloc, int32_t* err,
+                   cudaStream_t s);
 void tc_plan_free(TcPlan& p, const std::function<void(void*)>& dfree);
 size_t tc_w_bytes(const TcPlan& p);
 size_t tc_scratch_bytes(const TcPlan& p, int R);

@@ -32,7 +32,7 @@ void mwk::note_launch(int n) { g_launches.fetch_add(n, std::memory_order_relaxed
 namespace mwk {
 void start_state(const double* npart, int nparts, int R, const double* bnorm, double tol, double inner_tol,
                  int fp64_mode, double* rnorm, double2* gvec, double* target, int32_t* done, int32_t* kcol, int m,
-                 int32_t* active, cudaStream_t s);
+                 int32_t* state, int32_t* active, int32_t* host_active, cudaStream_t s);
 void normalize_start_f64(const double2* r, const double* rnorm, const int32_t* done, int64_t E, int R, double2* v0,
                          cudaStream_t s);
 void normalize_start_f32(const double2* r, const double* rnorm, const int32_t* done, int64_t E, int R, float2* v0,
@@ -125,7 +125,6 @@ struct Work {
   int64_t E = 0;
   int R = 0, m = 0, prec = -1;
   void *V = nullptr, *Z = nullptr;   // Krylov and preconditioned bases, vectors krylov_stride apart
-  int32_t* kerr = nullptr;     // bounded-wait error code of the streaming Gram-Schmidt kernel
   float4* xdf = nullptr;       // double-float copy of the iterate (mixed mode)
   float4* bdf = nullptr;       // double-float copy of the block's right-hand sides (mixed mode)
   float2* r32 = nullptr;       // outer residual rounded to FP32 (mixed mode)
@@ -133,8 +132,7 @@ struct Work {
   double2 *r = nullptr, *x = nullptr, *part = nullptr, *h = nullptr, *H = nullptr, *cs = nullptr, *g = nullptr,
           *y = nullptr, *bblk = nullptr;
   double *npart = nullptr, *target = nullptr, *rnorm = nullptr, *bnorm = nullptr, *scale = nullptr;
-  int32_t *done = nullptr, *kcol = nullptr, *active = nullptr;
-  int32_t* h_active = nullptr;  // pinned
+  int32_t *done = nullptr, *kcol = nullptr, *active = nullptr;   // active: [0] columns still active, [1..2] its counting
   double* h_vec = nullptr;      // pinned [R]
   int32_t* h_ivec = nullptr;    // pinned [R]
   void* tc_scratch = nullptr;   // BF16 gathered operand
@@ -220,8 +218,13 @@ struct CycleGraph {
   int64_t step_launches = 0;         // kernels inside one step's conditional bodies
 };
 
+// Words of the mapped host page that kernels write: columns still active, error codes of bounded waits in the
+// streaming Gram-Schmidt kernels and in the tensor-core apply.
+constexpr int kWordActive = 0, kWordKrylov = 1, kWordTc = 2, kWordCount = 3;
+
 struct Ctx {
   int device = 0;
+  int32_t *h_words = nullptr, *d_words = nullptr;   // the page on the host and on the device
   Profiler prof;
   NnState nn;
   cudaStream_t stream = nullptr;
@@ -423,9 +426,8 @@ void free_work(Ctx* c) {
   Work& w = c->work;
   for (void* p : {(void*)w.V, (void*)w.Z, (void*)w.xdf, (void*)w.r, (void*)w.x, (void*)w.part, (void*)w.h, (void*)w.H, (void*)w.cs,
                   (void*)w.g, (void*)w.y, (void*)w.npart, (void*)w.target, (void*)w.rnorm, (void*)w.bnorm,
-                  (void*)w.scale, (void*)w.done, (void*)w.kcol, (void*)w.active, (void*)w.bblk, (void*)w.kerr, (void*)w.bdf, (void*)w.r32, (void*)w.vscale, w.tc_scratch, w.mf_arena, w.mf_partial})
+                  (void*)w.scale, (void*)w.done, (void*)w.kcol, (void*)w.active, (void*)w.bblk, (void*)w.bdf, (void*)w.r32, (void*)w.vscale, w.tc_scratch, w.mf_arena, w.mf_partial})
     dfree(c, p);
-  if (w.h_active) cudaFreeHost(w.h_active);
   if (w.h_vec) cudaFreeHost(w.h_vec);
   if (w.h_ivec) cudaFreeHost(w.h_ivec);
   w = Work();
@@ -445,9 +447,7 @@ void ensure_work(Ctx* c, int R, int m, int prec) {
   const size_t nv = (size_t)krylov_stride(E, R);
   w.V = dalloc<unsigned char>(c, es * nv * (m + 1));
   w.Z = dalloc<unsigned char>(c, es * nv * m);
-  w.kerr = dalloc<int32_t>(c, 1);
   w.vscale = dalloc<double>(c, (size_t)(m + 1) * R);
-  CK(cudaMemsetAsync(w.kerr, 0, sizeof(int32_t), c->stream));
   w.r = dalloc<double2>(c, n);
   w.x = dalloc<double2>(c, n);
   if (prec == 1) {
@@ -469,8 +469,8 @@ void ensure_work(Ctx* c, int R, int m, int prec) {
   w.scale = dalloc<double>(c, R);
   w.done = dalloc<int32_t>(c, R);
   w.kcol = dalloc<int32_t>(c, R);
-  w.active = dalloc<int32_t>(c, 1);
-  CK(cudaMallocHost(&w.h_active, sizeof(int32_t)));
+  w.active = dalloc<int32_t>(c, 3);
+  CK(cudaMemsetAsync(w.active, 0, 3 * sizeof(int32_t), c->stream));
   CK(cudaMallocHost(&w.h_vec, sizeof(double) * R));
   CK(cudaMallocHost(&w.h_ivec, sizeof(int32_t) * R));
 }
@@ -984,7 +984,8 @@ void build_sparse_tc(Ctx* c, const std::vector<std::vector<mwk::MfTask>>& launch
     T.own_local = mf_up(c, m, fake.own_local);
     T.own_glob = mf_up(c, m, own_glob);
     T.c0_glob = mf_up(c, m, c0_glob);
-    require(mwk::tc_plan_build(T.plan, fake, [&](size_t b) { return (void*)dalloc<unsigned char>(c, b); }, c->stream),
+    require(mwk::tc_plan_build(T.plan, fake, [&](size_t b) { return (void*)dalloc<unsigned char>(c, b); },
+                               c->d_words + kWordTc, c->stream),
             MW_EINVAL, "tensor-core plan of the sparse sweeps");
     m.tc_scratch = std::max(m.tc_scratch, mwk::tc_scratch_bytes(T.plan, 128));
     T.W.assign(c->n_freq, nullptr);
@@ -1049,18 +1050,20 @@ struct ProfScope {
   }
 };
 
-// Reads the bounded-wait error word of the tensor-core preconditioner apply (after the work
-// that used it has completed on the stream) and turns a wait that ran out into MW_ETIMEOUT,
-// clearing the word for the next call.
+// After the stream has been synchronised: turns a bounded wait that ran out in a kernel (its code lies in a
+// mapped host word) into MW_ETIMEOUT, clearing the word for the next call.
+void check_wait_word(Ctx* c, int word, const char* what) {
+  volatile int32_t* w = c->h_words + word;
+  const int32_t e = *w;
+  if (e == 0) return;
+  *w = 0;
+  throw Fail{MW_ETIMEOUT, std::string(what) + ": bounded wait ran out (code " + std::to_string(e) + ")"};
+}
+// The same for the tensor-core preconditioner apply, after the work enqueued so far.
 void check_tc_wait(Ctx* c) {
-  if (!(c->prec.ready && c->prec.apply_prec == 2 && c->prec.tc.err)) return;
-  int32_t e = 0;
-  CK(cudaMemcpyAsync(&e, c->prec.tc.err, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
+  if (!(c->prec.ready && (c->prec.apply_prec == 2 || c->prec.apply_prec == 5))) return;
   CK(cudaStreamSynchronize(c->stream));
-  if (e != 0) {
-    CK(cudaMemsetAsync(c->prec.tc.err, 0, sizeof(int32_t), c->stream));
-    throw Fail{MW_ETIMEOUT, "tensor-core preconditioner apply: bounded wait ran out (code " + std::to_string(e) + ")"};
-  }
+  check_wait_word(c, kWordTc, c->prec.apply_prec == 2 ? "tensor-core preconditioner apply" : "tensor-core sparse sweep");
 }
 
 // Algorithmic bytes of one preconditioner apply on R columns: the owned-row inverses once,
@@ -1076,9 +1079,8 @@ double oras_bytes(Ctx* c, int R, bool zb = false) {
 }
 
 int read_active(Ctx* c) {
-  CK(cudaMemcpyAsync(c->work.h_active, c->work.active, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
-  return *c->work.h_active;
+  return *(volatile int32_t*)(c->h_words + kWordActive);
 }
 
 // r = b - A_f x with per-block partial norms: FP64 arithmetic into w.r in FP64 mode; in mixed
@@ -1167,24 +1169,24 @@ void arnoldi_step(Ctx* c, const CycleArgs& a, int j, Seg&& seg) {
   });
   seg(MW_K_CGS_DOTS, (double)a.es * E * R * (j + 2), [&] {
     const int np = a.wp == 0 ? mwk::cgs_dots_f64((const double2*)w.V, a.vstride, j + 1,
-                                                 (const double2*)a.Vp(w, j + 1), E, R, w.part, w.kerr, c->stream,
+                                                 (const double2*)a.Vp(w, j + 1), E, R, w.part, c->d_words + kWordKrylov, c->stream,
                                                  a.t.sh.dots_stages)
                              : mwk::cgs_dots_f32((const float2*)w.V, a.vstride, j + 1,
-                                                 (const float2*)a.Vp(w, j + 1), E, R, w.part, w.kerr, c->stream,
+                                                 (const float2*)a.Vp(w, j + 1), E, R, w.part, c->d_words + kWordKrylov, c->stream,
                                                  a.t.sh.dots_stages);
     mwk::reduce_h(w.part, np, j + 1, R, w.h, c->stream, vs);
   });
   int nu = 0;
   seg(MW_K_CGS_UPDATE, (double)a.es * E * R * (j + 3), [&] {
     nu = a.wp == 0 ? mwk::cgs_update_f64((const double2*)w.V, a.vstride, j + 1, w.h, (double2*)a.Vp(w, j + 1), E,
-                                         R, w.npart, c->stream, w.kerr, a.t.sh.update_stages, vs)
+                                         R, w.npart, c->stream, c->d_words + kWordKrylov, a.t.sh.update_stages, vs)
                    : mwk::cgs_update_f32((const float2*)w.V, a.vstride, j + 1, w.h, (float2*)a.Vp(w, j + 1), E,
-                                         R, w.npart, c->stream, w.kerr, a.t.sh.update_stages, vs);
+                                         R, w.npart, c->stream, c->d_words + kWordKrylov, a.t.sh.update_stages, vs);
   });
   seg(-1, 0.0, [&] {
-    CK(cudaMemsetAsync(w.active, 0, sizeof(int32_t), c->stream));
     mwk::givens_step(w.h, w.npart, nu, j, a.m, R, w.H, w.cs, w.g, w.target, w.done, w.kcol,
-                     vs ? w.vscale + (size_t)(j + 1) * R : w.scale, w.active, c->stream);
+                     vs ? w.vscale + (size_t)(j + 1) * R : w.scale, w.active + 1, w.active, c->d_words + kWordActive,
+                     c->stream);
     if (!vs) {
       if (a.wp == 0)
         mwk::scale_cols_f64((double2*)a.Vp(w, j + 1), w.scale, E, R, c->stream);
@@ -1200,8 +1202,8 @@ void cycle_start(Ctx* c, const CycleArgs& a) {
   if (a.wp == 0)
     mwk::normalize_start_f64(w.r, w.rnorm, w.done, a.E, a.R, (double2*)a.Vp(w, 0), c->stream);
   else
-    mwk::normalize_start32(w.r32, w.rnorm, w.done, a.E, a.R, (float2*)a.Vp(w, 0), c->stream);
-  if (a.lazy) mwk::fill_f64(w.vscale, a.R, 1.0, c->stream);   // V_0 is stored scaled
+    mwk::normalize_start32(w.r32, w.rnorm, w.done, a.E, a.R, (float2*)a.Vp(w, 0), a.lazy ? w.vscale : nullptr,
+                           c->stream);
 }
 
 // Least squares, x += Z y, and the per-column step counts into w.h_ivec (not yet synchronised).
@@ -1209,17 +1211,18 @@ void cycle_finish(Ctx* c, const CycleArgs& a) {
   Work& w = c->work;
   mwk::solve_hessenberg(w.H, w.g, w.kcol, a.m, a.R, w.y, c->stream);
   if (a.wp == 0)
-    mwk::update_x_f64((const double2*)a.Zp(w, 0), a.vstride, w.y, w.kcol, a.m, a.X, a.E, a.R, c->stream, w.kerr);
+    mwk::update_x_f64((const double2*)a.Zp(w, 0), a.vstride, w.y, w.kcol, a.m, a.X, a.E, a.R, c->stream, c->d_words + kWordKrylov);
   else
     if (a.zb)
-      mwk::update_x_bx(a.Zp(w, 0), a.vstride, w.y, w.kcol, a.m, a.X, a.E, a.R, c->stream, w.kerr);
+      mwk::update_x_bx(a.Zp(w, 0), a.vstride, w.y, w.kcol, a.m, a.X, a.E, a.R, c->stream, c->d_words + kWordKrylov);
     else
-      mwk::update_x_f32((const float2*)a.Zp(w, 0), a.vstride, w.y, w.kcol, a.m, a.X, a.E, a.R, c->stream, w.kerr);
+      mwk::update_x_f32((const float2*)a.Zp(w, 0), a.vstride, w.y, w.kcol, a.m, a.X, a.E, a.R, c->stream, c->d_words + kWordKrylov);
   check_launch("solution update");
   CK(cudaMemcpyAsync(w.h_ivec, w.kcol, sizeof(int32_t) * a.R, cudaMemcpyDeviceToHost, c->stream));
 }
 
-// Eager cycle: the host reads the active-column count after every step.  Returns the steps run.
+// Eager cycle: the host reads the active-column count after every step.  Returns the steps run; the per-column
+// counts are in w.h_ivec after the next synchronisation.
 int cycle_eager(Ctx* c, const CycleArgs& a, int max_steps) {
   cycle_start(c, a);
   int j = 0;
@@ -1237,7 +1240,6 @@ int cycle_eager(Ctx* c, const CycleArgs& a, int max_steps) {
     if (read_active(c) == 0 || j >= max_steps) break;
   }
   cycle_finish(c, a);
-  CK(cudaStreamSynchronize(c->stream));
   return j;
 }
 
@@ -1459,10 +1461,10 @@ Tuned autotune(Ctx* c, int R, int wp, int m, bool use_p) {
     for (int st = mwk::kCgsDotsMinStages; st <= mwk::kCgsDotsMaxStages; ++st) {
       const double ms = time_launch(c, [&] {
         if (wp == 0)
-          mwk::cgs_dots_f64((const double2*)w.V, vstride, nvec, (const double2*)Vp(nvec), E, R, w.part, w.kerr,
+          mwk::cgs_dots_f64((const double2*)w.V, vstride, nvec, (const double2*)Vp(nvec), E, R, w.part, c->d_words + kWordKrylov,
                             c->stream, st);
         else
-          mwk::cgs_dots_f32((const float2*)w.V, vstride, nvec, (const float2*)Vp(nvec), E, R, w.part, w.kerr,
+          mwk::cgs_dots_f32((const float2*)w.V, vstride, nvec, (const float2*)Vp(nvec), E, R, w.part, c->d_words + kWordKrylov,
                             c->stream, st);
       });
       t.t[MW_TUNE_DOTS].push_back({st, ms});
@@ -1474,10 +1476,10 @@ Tuned autotune(Ctx* c, int R, int wp, int m, bool use_p) {
       const double ms = time_launch(c, [&] {
         if (wp == 0)
           mwk::cgs_update_f64((const double2*)w.V, vstride, nvec, w.h, (double2*)Vp(nvec), E, R, w.npart, c->stream,
-                              w.kerr, st);
+                              c->d_words + kWordKrylov, st);
         else
           mwk::cgs_update_f32((const float2*)w.V, vstride, nvec, w.h, (float2*)Vp(nvec), E, R, w.npart, c->stream,
-                              w.kerr, st);
+                              c->d_words + kWordKrylov, st);
       });
       t.t[MW_TUNE_UPDATE].push_back({st, ms});
     }
@@ -1531,6 +1533,12 @@ BlockStats solve_block(Ctx* c, int f, int R, const double2* B, double2* X, const
   mwk::reduce_cols(w.npart, nb, R, w.bnorm, s);
   mwk::sqrt_inplace(w.bnorm, R, s);
   std::vector<int32_t> its(R, 0);
+  bool pending = false;   // a cycle's step counts are on their way to w.h_ivec
+  auto count_steps = [&] {
+    if (!pending) return;
+    for (int q = 0; q < R; ++q) its[q] += w.h_ivec[q];
+    pending = false;
+  };
   BlockStats st;
   const int max_outer = o.mode == MW_MODE_FP64 ? (o.max_it + m - 1) / m + 1 : std::max(1, o.max_outer);
   int total = 0;
@@ -1541,27 +1549,30 @@ BlockStats solve_block(Ctx* c, int f, int R, const double2* B, double2* X, const
                    outer == 0 ? 24.0 * E * R : (double)c->topo.nnz * 20 + 8.0 * (E + 1) + 3.0 * 16 * E * R);
       nb = outer_residual(c, f, wp, X, B, R, outer == 0);
     }
-    CK(cudaMemsetAsync(w.active, 0, sizeof(int32_t), s));
     mwk::start_state(w.npart, nb, R, w.bnorm, o.tol, o.inner_tol, wp == 0, w.rnorm, w.g, w.target, w.done, w.kcol,
-                     m, w.active, s);
+                     m, w.active + 1, w.active, c->d_words + kWordActive, s);
     check_launch("cycle start");
     st.outer++;
     st.have_relres = true;
-    if (read_active(c) == 0 || total >= o.max_it) break;
+    const int active = read_active(c);
+    count_steps();
+    if (active == 0 || total >= o.max_it) break;
     st.have_relres = false;
     // a cycle that may run all m steps is replayed from its captured graph
     const int steps = (c->graphs_on && o.max_it - total >= m) ? cycle_graph(c, a) : cycle_eager(c, a, o.max_it - total);
     total += steps;
     st.steps += steps;
-    for (int q = 0; q < R; ++q) its[q] += w.h_ivec[q];
+    pending = true;
   }
-  its_out = its;
   if (!st.have_relres) {
+    CK(cudaStreamSynchronize(s));
+    count_steps();
     // the loop ended after an update: measure the final residual
     nb = outer_residual(c, f, wp, X, B, R);
     mwk::reduce_cols(w.npart, nb, R, w.rnorm, s);
     mwk::sqrt_inplace(w.rnorm, R, s);
   }
+  its_out = its;
   return st;
 }
 
@@ -1660,24 +1671,7 @@ void solve_all(Ctx* c, const mw_solve_opts& o, int ncols, const std::vector<cons
   float ms = 0;
   CK(cudaEventElapsedTime(&ms, c->ev0, c->ev1));
   check_tc_wait(c);
-  if (c->prec.ready && c->prec.apply_prec == 5)
-    for (auto& L : c->prec.mf.tcl) {
-      if (!L.plan.err) continue;
-      int32_t e = 0;
-      CK(cudaMemcpy(&e, L.plan.err, sizeof(int32_t), cudaMemcpyDeviceToHost));
-      if (e != 0) {
-        CK(cudaMemsetAsync(L.plan.err, 0, sizeof(int32_t), s));
-        throw Fail{MW_ETIMEOUT, "tensor-core sparse sweep: bounded wait ran out (code " + std::to_string(e) + ")"};
-      }
-    }
-  if (c->work.kerr) {
-    int32_t e = 0;
-    CK(cudaMemcpy(&e, c->work.kerr, sizeof(int32_t), cudaMemcpyDeviceToHost));
-    if (e != 0) {
-      CK(cudaMemsetAsync(c->work.kerr, 0, sizeof(int32_t), s));
-      throw Fail{MW_ETIMEOUT, "streaming Gram-Schmidt dots: bounded wait ran out (code " + std::to_string(e) + ")"};
-    }
-  }
+  check_wait_word(c, kWordKrylov, "streaming Gram-Schmidt dots");
   int nconv = 0;
   double mx = 0;
   for (double r : rel_all) {
@@ -2057,6 +2051,10 @@ mw_status mw_create(mw_ctx** out, int device, void* stream) {
   c->device = device;
   c->stream = (cudaStream_t)stream;
   if (cudaEventCreate(&c->ev0) != cudaSuccess || cudaEventCreate(&c->ev1) != cudaSuccess) return MW_ECUDA;
+  if (cudaHostAlloc(&c->h_words, kWordCount * sizeof(int32_t), cudaHostAllocMapped) != cudaSuccess ||
+      cudaHostGetDevicePointer(&c->d_words, c->h_words, 0) != cudaSuccess)
+    return MW_ECUDA;
+  for (int i = 0; i < kWordCount; ++i) c->h_words[i] = 0;
   *out = c.release();
   return MW_OK;
 }
@@ -2071,6 +2069,7 @@ void mw_destroy(mw_ctx* c) {
   if (c->body_s) cudaStreamDestroy(c->body_s);
   if (c->ev0) cudaEventDestroy(c->ev0);
   if (c->ev1) cudaEventDestroy(c->ev1);
+  if (c->h_words) cudaFreeHost(c->h_words);
   delete c;
 }
 
@@ -2687,7 +2686,8 @@ mw_status mw_setup_preconditioner(mw_ctx* c, int32_t n_sub, const int32_t* part,
     p.tile_row0 = upload(c, trow.data(), trow.size());
     p.w_off = upload(c, woff.data(), woff.size());
     if (p.apply_prec == 2)
-      require(mwk::tc_plan_build(p.tc, sd, [&](size_t b) { return (void*)dalloc<unsigned char>(c, b); }, c->stream),
+      require(mwk::tc_plan_build(p.tc, sd, [&](size_t b) { return (void*)dalloc<unsigned char>(c, b); },
+                                 c->d_words + kWordTc, c->stream),
               MW_EINVAL, "BF16 tensor-core apply unavailable for this partition");
     const size_t wes = p.apply_prec == 0 ? sizeof(double2) : sizeof(float2);
     const size_t fes = p.factor_prec == 0 ? sizeof(double2) : sizeof(float2);

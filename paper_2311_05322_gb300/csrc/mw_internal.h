@@ -203,9 +203,9 @@ int residual_df(const int64_t* rp, const int32_t* ci, const float4* A, const flo
 // ||r||^2 (FP64) per block and column; returns the number of blocks.
 int residual_df32(const int64_t* rp, const int32_t* ci, const float4* A, const float4* X, const float4* Bdf,
                   float2* Rv, double* part, int64_t E, int R, cudaStream_t s, const int* win, bool zero_x = false);
-// v0 = r / rnorm per column (0 for done columns) from an FP32 residual.
+// v0 = r / rnorm per column (0 for done columns) from an FP32 residual; vscale[0 .. R) = 1 when given.
 void normalize_start32(const float2* r, const double* rnorm, const int32_t* done, int64_t E, int R, float2* v0,
-                       cudaStream_t s);
+                       double* vscale, cudaStream_t s);
 // r = b - A x (FP64) and per-column partial ||r||^2 into part[nblk][R]; returns nblk used.
 // zero_x: x is known to be 0 (the products are skipped; the same r and norms).
 int residual_f64(const int64_t* rp, const int32_t* ci, const double2* A, const double2* X, const double2* B,
@@ -241,13 +241,12 @@ int cgs_update_f64(const double2* V, int64_t vstride, int nvec, const double2* h
 int cgs_update_f32(const float2* V, int64_t vstride, int nvec, const double2* h, float2* w, int64_t E, int R,
                    double* npart, cudaStream_t s, int32_t* err = nullptr, int stages = 0,
                    const double* vscale = nullptr);
-// x[0..n) = v.
-void fill_f64(double* x, int n, double v, cudaStream_t s);
 int colnorm2_f64(const double2* x, int64_t E, int R, double* npart, cudaStream_t s);
-// Givens step for Arnoldi column j; see k_krylov.cu for the state layout.
+// Givens step for Arnoldi column j; see k_krylov.cu for the state layout.  state: two zeroed words of the
+// counting; active: device word, host_active: mapped host word, both set to the columns still active.
 void givens_step(const double2* h, const double* npart, int nparts, int j, int m, int R, double2* H,
                  double2* cs, double2* gvec, double* target, int32_t* done, int32_t* kcol, double* scale,
-                 int32_t* active_count, cudaStream_t s);
+                 int32_t* state, int32_t* active, int32_t* host_active, cudaStream_t s);
 void scale_cols_f64(double2* v, const double* scale, int64_t E, int R, cudaStream_t s);
 void scale_cols_f32(float2* v, const double* scale, int64_t E, int R, cudaStream_t s);
 void solve_hessenberg(const double2* H, const double2* gvec, const int32_t* kcol, int m, int R, double2* y,
