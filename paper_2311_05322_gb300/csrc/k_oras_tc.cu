@@ -71,14 +71,23 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
-  uint32_t r[8];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+// Eight columns of the four accumulator parts that one output value needs, with one wait.
+__device__ __forceinline__ void tmem_ld8x4(uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, float (&v)[4][8]) {
+  uint32_t r[32];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%32];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%33];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%34];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%24,%25,%26,%27,%28,%29,%30,%31}, [%35];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3)
+      : "memory");
 #pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < 32; ++i) v[i / 8][i % 8] = __uint_as_float(r[i]);
 }
 
 // Byte offset of (row, k) in a K-major, 128-byte-swizzled tile with 64 BF16 per row.
@@ -241,15 +250,11 @@ __global__ void __launch_bounds__(128, 8) gather_b_kernel(const int32_t* __restr
 // Apply, step 2: one CTA per 128-row output tile of one subdomain.
 // ---------------------------------------------------------------------------------------
 struct TcArgs {
-  const int32_t* mt_sub;
-  const int32_t* mt_row0;
-  const int64_t* sub_wtile;
-  const int64_t* sub_gtile;
-  const int32_t* sub_kt;
-  const int64_t* own_ptr;
+  const TcTile* tiles;
   const int32_t* own_glob;
   const int32_t* c0_glob;   // optional: row of z added to each output row (-1: none)
   int z_bf16;               // z holds complex BF16 pairs (4 bytes per value) instead of float2
+  int vec;                  // rows of z are whole, aligned 16-byte pieces
   const uint8_t* W;
   const uint8_t* Bt;
   float2* z;
@@ -293,6 +298,96 @@ __device__ __forceinline__ bool drain_ring(uint64_t* full_bar, RingPos p, int64_
   return ok;
 }
 
+// Rows that the copies of a tile move: whole 8-row swizzle groups that hold owned rows.  The other rows of A
+// feed only accumulator rows that the epilogue does not store.
+__device__ __forceinline__ uint32_t a_part_of(const TcTile& tl) { return (uint32_t)((tl.rows + 7) / 8) * 1024u; }
+
+// Epilogue of one accumulator row: z[og] = D (+ z[c0]), 8 columns at a time, the next C0 values on their way.
+// A thread owns a whole row, so its stores are 16 bytes where the rows allow it (vec): a warp's store then
+// touches each 32-byte sector twice, not four (FP32) or eight (BF16) times.
+struct EpiRow {
+  int64_t og = -1, c0 = -1;   // output row and row added to it; negative: none
+};
+__device__ __forceinline__ EpiRow epi_row(const TcArgs& a, const TcTile& tl, int row) {
+  EpiRow e;
+  if (row < tl.rows) {
+    e.og = (int64_t)a.own_glob[tl.own + row];
+    if (a.c0_glob) e.c0 = (int64_t)a.c0_glob[tl.own + row];
+  }
+  return e;
+}
+__device__ __forceinline__ void epi_fetch(const TcArgs& a, const float2* c0r, int cb, float2 (&v)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = make_float2(0.f, 0.f);
+  if (!c0r) return;
+  if (a.vec && !a.z_bf16) {
+#pragma unroll
+    for (int i = 0; i < 8; i += 2)
+      if (cb + i < a.R) {
+        const float4 t = *reinterpret_cast<const float4*>(c0r + cb + i);
+        v[i] = make_float2(t.x, t.y);
+        v[i + 1] = make_float2(t.z, t.w);
+      }
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if (cb + i < a.R) v[i] = c0r[cb + i];
+}
+__device__ __forceinline__ void epi_store(const TcArgs& a, int64_t og, int cb, const float2 (&v)[8]) {
+  if (a.z_bf16) {
+    uint32_t* zr = reinterpret_cast<uint32_t*>(a.z) + og * a.R + cb;
+    if (a.vec) {
+#pragma unroll
+      for (int i = 0; i < 8; i += 4)
+        if (cb + i < a.R)
+          *reinterpret_cast<uint4*>(zr + i) =
+              make_uint4(pack_bf16(v[i].x, v[i].y), pack_bf16(v[i + 1].x, v[i + 1].y),
+                         pack_bf16(v[i + 2].x, v[i + 2].y), pack_bf16(v[i + 3].x, v[i + 3].y));
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (cb + i < a.R) zr[i] = pack_bf16(v[i].x, v[i].y);
+    }
+    return;
+  }
+  float2* zr = a.z + og * a.R + cb;
+  if (a.vec) {
+#pragma unroll
+    for (int i = 0; i < 8; i += 2)
+      if (cb + i < a.R) *reinterpret_cast<float4*>(zr + i) = make_float4(v[i].x, v[i].y, v[i + 1].x, v[i + 1].y);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (cb + i < a.R) zr[i] = v[i];
+  }
+}
+// The accumulator at tmem (this warp's lanes) to z; every lane of the warp takes part in the reads.
+__device__ __forceinline__ void epi_tile(const TcArgs& a, uint32_t lanes, const EpiRow& e, bool valid,
+                                         float2 (&nxt)[8]) {
+  const float2* c0r = e.og >= 0 && e.c0 >= 0 ? a.z + e.c0 * a.R : nullptr;
+  const int Rp = a.N / 2;
+  for (int cb = 0; cb < Rp; cb += 8) {
+    // Re z = D1[c] - D2[Rp + c], Im z = D1[Rp + c] + D2[c] (plus the C0 row when given)
+    float2 cur[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) cur[i] = nxt[i];
+    if (cb + 8 < Rp) epi_fetch(a, c0r, cb + 8, nxt);
+    float d[4][8];   // Wr gr, Wr gi, Wi gr, Wi gi
+    tmem_ld8x4(lanes + (uint32_t)cb, lanes + (uint32_t)(Rp + cb), lanes + (uint32_t)(a.N + cb),
+               lanes + (uint32_t)(a.N + Rp + cb), d);
+    if (valid) {
+      float2 v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        v[i] = make_float2(d[0][i] - d[3][i], d[1][i] + d[2][i]);
+        if (c0r) v[i] = make_float2(v[i].x + cur[i].x, v[i].y + cur[i].y);
+      }
+      epi_store(a, e.og, cb, v);
+    }
+  }
+}
+
 __global__ void __launch_bounds__(kThreadsTc, 2) oras_tc_kernel(const TcArgs a) {
   extern __shared__ uint8_t dsm[];
   __shared__ __align__(8) uint64_t full_bar[8];
@@ -302,16 +397,14 @@ __global__ void __launch_bounds__(kThreadsTc, 2) oras_tc_kernel(const TcArgs a) 
   __shared__ int abort_flag;
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dsm) + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t = blockIdx.x;
-  const int s = a.mt_sub[t];
-  const int row0 = a.mt_row0[t];
-  const int KT = a.sub_kt[s];
+  const TcTile tl = a.tiles[blockIdx.x];
+  const int KT = tl.kt;
   const int S = a.stages;
   const uint32_t b_bytes = (uint32_t)a.N * 128u;
   const uint32_t a_bytes = 2u * kATileBytes;          // Wr and Wi tiles of one k tile
   const uint32_t stage_bytes = a_bytes + b_bytes;
-  const uint8_t* Wt = a.W + ((size_t)a.sub_wtile[s] + (size_t)(row0 / kTileM) * KT * 2) * kATileBytes;
-  const uint8_t* Bs = a.Bt + (size_t)a.sub_gtile[s] * b_bytes;
+  const uint8_t* Wt = a.W + (size_t)tl.w * kATileBytes;
+  const uint8_t* Bs = a.Bt + (size_t)tl.g * b_bytes;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < S; ++i) {
@@ -335,12 +428,8 @@ __global__ void __launch_bounds__(kThreadsTc, 2) oras_tc_kernel(const TcArgs a) 
 
   if (warp == 0) {
     if (lane == 0) {
-      // producer: bulk copies of (Wr and Wi tiles, B tile) per k tile.  In the last m tile of a
-      // subdomain only the 8-row swizzle groups that hold owned rows are copied: the other rows
-      // of A feed only accumulator rows that the epilogue does not store.
-      const int64_t nown_p = a.own_ptr[s + 1] - a.own_ptr[s];
-      const int rows_valid = (int)min((int64_t)kTileM, nown_p - (int64_t)row0);
-      const uint32_t a_part = (uint32_t)((rows_valid + 7) / 8) * 1024u;
+      // producer: bulk copies of (Wr and Wi tiles, B tile) per k tile
+      const uint32_t a_part = a_part_of(tl);
       int issued = 0;
       RingPos p;
       for (int kt = 0; kt < KT; ++kt, p.next(S)) {
@@ -386,53 +475,14 @@ __global__ void __launch_bounds__(kThreadsTc, 2) oras_tc_kernel(const TcArgs a) 
     // epilogue: warps 2..5 cover tensor-memory lane quadrants (warp % 4).  The output row, the C0
     // row and C0's first 8 columns are looked up while the MMAs run.
     const int quad = warp & 3;
-    const int row = quad * 32 + lane;
-    const int64_t nown = a.own_ptr[s + 1] - a.own_ptr[s];
-    const int64_t q = (int64_t)row0 + row;
-    const int64_t og = q < nown ? (int64_t)a.own_glob[a.own_ptr[s] + q] : -1;   // negative: skipped
-    const int64_t c0 = (og >= 0 && a.c0_glob) ? (int64_t)a.c0_glob[a.own_ptr[s] + q] : -1;
-    const float2* c0r = c0 >= 0 ? a.z + c0 * a.R : nullptr;
+    const EpiRow e = epi_row(a, tl, quad * 32 + lane);
     float2 nxt[8];
-    auto fetch_c0 = [&](int cb) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) nxt[i] = (c0r && cb + i < a.R) ? c0r[cb + i] : make_float2(0.f, 0.f);
-    };
-    fetch_c0(0);
+    epi_fetch(a, e.og >= 0 && e.c0 >= 0 ? a.z + e.c0 * a.R : nullptr, 0, nxt);
     bool ok = mbar_wait(&done_bar, 0);
     ok = __all_sync(0xffffffffu, ok);   // tcgen05.ld below is warp-collective
     if (!ok && lane == 0) atomicCAS(a.err, 0, 4);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const bool valid = ok && !abort_flag && og >= 0;
-    float2* zr = valid ? a.z + og * a.R : nullptr;
-    const int Rp = a.N / 2;
-    const uint32_t lanes = tmem + ((uint32_t)(quad * 32) << 16);
-    for (int cb = 0; cb < Rp; cb += 8) {
-      // Re z = D1[c] - D2[Rp + c], Im z = D1[Rp + c] + D2[c] (plus the C0 row when given)
-      float2 cur[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) cur[i] = nxt[i];
-      if (cb + 8 < Rp) fetch_c0(cb + 8);
-      float rr[8], ri[8], ir[8], ii[8];
-      if (ok) {
-        tmem_ld8(lanes + (uint32_t)cb, rr);                          // Wr gr
-        tmem_ld8(lanes + (uint32_t)(Rp + cb), ri);                   // Wr gi
-        tmem_ld8(lanes + (uint32_t)(a.N + cb), ir);                  // Wi gr
-        tmem_ld8(lanes + (uint32_t)(a.N + Rp + cb), ii);             // Wi gi
-      }
-      if (valid) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int col = cb + i;
-          if (col >= a.R) continue;
-          float2 v = make_float2(rr[i] - ii[i], ri[i] + ir[i]);
-          if (c0r) v = make_float2(v.x + cur[i].x, v.y + cur[i].y);
-          if (a.z_bf16)
-            reinterpret_cast<uint32_t*>(a.z)[og * a.R + col] = pack_bf16(v.x, v.y);
-          else
-            zr[col] = v;
-        }
-      }
-    }
+    if (ok) epi_tile(a, tmem + ((uint32_t)(quad * 32) << 16), e, !abort_flag && e.og >= 0, nxt);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -494,15 +544,14 @@ __global__ void __launch_bounds__(kThreadsTc, 2) oras_tc_persistent_kernel(const
     if (lane == 0) {
       int64_t it = 0;   // k tiles issued by this CTA
       RingPos p;        // ring position, running across its tiles
+      TcTile nxt = a.tiles[blockIdx.x];
       for (int t = blockIdx.x; t < n_tiles && !*abort_v; t += gridDim.x) {
-        const int s = a.mt_sub[t];
-        const int row0 = a.mt_row0[t];
-        const int KT = a.sub_kt[s];
-        const uint8_t* Wt = a.W + ((size_t)a.sub_wtile[s] + (size_t)(row0 / kTileM) * KT * 2) * kATileBytes;
-        const uint8_t* Bs = a.Bt + (size_t)a.sub_gtile[s] * b_bytes;
-        const int64_t nown_p = a.own_ptr[s + 1] - a.own_ptr[s];
-        const int rows_valid = (int)min((int64_t)kTileM, nown_p - (int64_t)row0);
-        const uint32_t a_part = (uint32_t)((rows_valid + 7) / 8) * 1024u;
+        const TcTile tl = nxt;
+        if (t + (int)gridDim.x < n_tiles) nxt = a.tiles[t + gridDim.x];
+        const int KT = tl.kt;
+        const uint8_t* Wt = a.W + (size_t)tl.w * kATileBytes;
+        const uint8_t* Bs = a.Bt + (size_t)tl.g * b_bytes;
+        const uint32_t a_part = a_part_of(tl);
         for (int kt = 0; kt < KT; ++kt, ++it, p.next(S)) {
           if (it >= S && !mbar_wait(&empty_bar[p.st], p.ph ^ 1u)) {
             atomicCAS(a.err, 0, 11);
@@ -521,8 +570,10 @@ __global__ void __launch_bounds__(kThreadsTc, 2) oras_tc_persistent_kernel(const
       const uint32_t idesc = idesc_bf16(a.N);
       RingPos p;
       int i = 0;   // tiles of this CTA
+      int kt_next = a.tiles[blockIdx.x].kt;
       for (int t = blockIdx.x; t < n_tiles && !*abort_v; t += gridDim.x, ++i) {
-        const int KT = a.sub_kt[a.mt_sub[t]];
+        const int KT = kt_next;
+        if (t + (int)gridDim.x < n_tiles) kt_next = a.tiles[t + gridDim.x].kt;
         const int buf = i & 1;
         if (i >= 2 && !mbar_wait(&acc_empty[buf], (uint32_t)(((i >> 1) + 1) & 1))) {
           atomicCAS(a.err, 0, 13);
@@ -560,25 +611,23 @@ __global__ void __launch_bounds__(kThreadsTc, 2) oras_tc_persistent_kernel(const
       if (!mbar_wait(&fin_bar, 0)) atomicCAS(a.err, 0, 15);
     }
   } else {
+    // A tile's record is read two tiles ahead and its row numbers one tile ahead: in line, that chain of
+    // dependent reads took longer than the copies of a tile with one to four k tiles (16 sparse subdomains of
+    // 44x44x17 cells, 16 columns: a solve's 15 applies 23.9 -> 21.2 ms with the 16-byte stores and the third stage).
     const int quad = warp & 3;
     const int row = quad * 32 + lane;
-    const int Rp = a.N / 2;
+    const int step = gridDim.x;
+    EpiRow e1 = epi_row(a, a.tiles[blockIdx.x], row);
+    TcTile t2;
+    if ((int)blockIdx.x + step < n_tiles) t2 = a.tiles[blockIdx.x + step];
     int i = 0;
-    for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, ++i) {
-      const int s = a.mt_sub[t];
-      const int row0 = a.mt_row0[t];
+    for (int t = blockIdx.x; t < n_tiles; t += step, ++i) {
       const int buf = i & 1;
-      const int64_t nown = a.own_ptr[s + 1] - a.own_ptr[s];
-      const int64_t q = (int64_t)row0 + row;
-      const int64_t og = q < nown ? (int64_t)a.own_glob[a.own_ptr[s] + q] : -1;
-      const int64_t c0 = (og >= 0 && a.c0_glob) ? (int64_t)a.c0_glob[a.own_ptr[s] + q] : -1;
-      const float2* c0r = c0 >= 0 ? a.z + c0 * a.R : nullptr;
+      const EpiRow e = e1;
       float2 nxt[8];
-      auto fetch_c0 = [&](int cb) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) nxt[j] = (c0r && cb + j < a.R) ? c0r[cb + j] : make_float2(0.f, 0.f);
-      };
-      fetch_c0(0);
+      epi_fetch(a, e.og >= 0 && e.c0 >= 0 ? a.z + e.c0 * a.R : nullptr, 0, nxt);
+      if (t + step < n_tiles) e1 = epi_row(a, t2, row);
+      if (t + 2 * step < n_tiles) t2 = a.tiles[t + 2 * step];
       bool ok = !*abort_v && mbar_wait(&acc_full[buf], (uint32_t)((i >> 1) & 1));
       ok = __all_sync(0xffffffffu, ok);   // tcgen05.ld below is warp-collective
       if (!ok) {
@@ -589,33 +638,7 @@ __global__ void __launch_bounds__(kThreadsTc, 2) oras_tc_persistent_kernel(const
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const bool valid = og >= 0;
-      float2* zr = valid ? a.z + og * a.R : nullptr;
-      const uint32_t lanes = tmem + (uint32_t)buf * a.tmem_cols + ((uint32_t)(quad * 32) << 16);
-      for (int cb = 0; cb < Rp; cb += 8) {
-        float2 cur[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) cur[j] = nxt[j];
-        if (cb + 8 < Rp) fetch_c0(cb + 8);
-        float rr[8], ri[8], ir[8], ii[8];
-        tmem_ld8(lanes + (uint32_t)cb, rr);
-        tmem_ld8(lanes + (uint32_t)(Rp + cb), ri);
-        tmem_ld8(lanes + (uint32_t)(a.N + cb), ir);
-        tmem_ld8(lanes + (uint32_t)(a.N + Rp + cb), ii);
-        if (valid) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const int col = cb + j;
-            if (col >= a.R) continue;
-            float2 v = make_float2(rr[j] - ii[j], ri[j] + ir[j]);
-            if (c0r) v = make_float2(v.x + cur[j].x, v.y + cur[j].y);
-            if (a.z_bf16)
-              reinterpret_cast<uint32_t*>(a.z)[og * a.R + col] = pack_bf16(v.x, v.y);
-            else
-              zr[col] = v;
-          }
-        }
-      }
+      epi_tile(a, tmem + (uint32_t)buf * a.tmem_cols + ((uint32_t)(quad * 32) << 16), e, e.og >= 0, nxt);
       // this warp's reads of the buffer are done: the MMA warp may overwrite it
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
@@ -651,7 +674,8 @@ bool tc_plan_build(TcPlan& p, const mw::Subdomains& sd, const std::function<void
                    cudaStream_t s) {
   p = TcPlan();
   const int ns = sd.n_sub;
-  std::vector<int32_t> mt_sub, mt_row0, sub_kt(ns), gt_sub, gt_kt;
+  std::vector<TcTile> tiles;
+  std::vector<int32_t> sub_kt(ns), gt_sub, gt_kt;
   std::vector<int64_t> sub_wtile(ns), sub_gtile(ns);
   int64_t wt = 0, gtile = 0;
   for (int q = 0; q < ns; ++q) {
@@ -681,12 +705,13 @@ bool tc_plan_build(TcPlan& p, const mw::Subdomains& sd, const std::function<void
   }
   if (n_mtiles <= 2 * 2 * 152)
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return sub_kt[a] > sub_kt[b]; });
-  for (int q : order)
-    for (int64_t r = 0; r < sd.own_ptr[q + 1] - sd.own_ptr[q]; r += kTileM) {
-      mt_sub.push_back(q);
-      mt_row0.push_back((int32_t)r);
-    }
-  p.n_mtiles = (int64_t)mt_sub.size();
+  for (int q : order) {
+    const int64_t nown = sd.own_ptr[q + 1] - sd.own_ptr[q];
+    for (int64_t r = 0; r < nown; r += kTileM)
+      tiles.push_back({sub_wtile[q] + r / kTileM * sub_kt[q] * 2, sub_gtile[q], sd.own_ptr[q] + r, sub_kt[q],
+                       (int32_t)std::min<int64_t>(kTileM, nown - r)});
+  }
+  p.n_mtiles = (int64_t)tiles.size();
   p.n_ktiles_total = gtile;
   p.w_tiles = wt;
   auto up = [&](const void* h, size_t bytes) {
@@ -694,10 +719,9 @@ bool tc_plan_build(TcPlan& p, const mw::Subdomains& sd, const std::function<void
     cudaMemcpyAsync(d, h, bytes, cudaMemcpyHostToDevice, s);
     return d;
   };
-  p.mt_sub = (int32_t*)up(mt_sub.data(), sizeof(int32_t) * std::max<size_t>(mt_sub.size(), 1));
-  p.mt_row0 = (int32_t*)up(mt_row0.data(), sizeof(int32_t) * std::max<size_t>(mt_row0.size(), 1));
+  if (tiles.empty()) tiles.resize(1);
+  p.tiles = (TcTile*)up(tiles.data(), sizeof(TcTile) * tiles.size());
   p.sub_wtile = (int64_t*)up(sub_wtile.data(), sizeof(int64_t) * ns);
-  p.sub_gtile = (int64_t*)up(sub_gtile.data(), sizeof(int64_t) * ns);
   p.sub_kt = (int32_t*)up(sub_kt.data(), sizeof(int32_t) * ns);
   p.gt_sub = (int32_t*)up(gt_sub.data(), sizeof(int32_t) * std::max<size_t>(gt_sub.size(), 1));
   p.gt_kt = (int32_t*)up(gt_kt.data(), sizeof(int32_t) * std::max<size_t>(gt_kt.size(), 1));
@@ -710,7 +734,7 @@ bool tc_plan_build(TcPlan& p, const mw::Subdomains& sd, const std::function<void
 }
 
 void tc_plan_free(TcPlan& p, const std::function<void(void*)>& dfree) {
-  for (void* q : {(void*)p.mt_sub, (void*)p.mt_row0, (void*)p.sub_wtile, (void*)p.sub_gtile, (void*)p.sub_kt,
+  for (void* q : {(void*)p.tiles, (void*)p.sub_wtile, (void*)p.sub_kt,
                   (void*)p.gt_sub, (void*)p.gt_kt})
     if (q) dfree(q);
   p = TcPlan();
@@ -756,9 +780,10 @@ int tc_stages(int N);
 size_t tc_smem_bytes(int N, int stages);
 
 int tc_stages(int N) {
-  // about 100 KB of stages per CTA so that two CTAs share an SM
+  // 110 KB of stages per CTA: two CTAs share the 228 KB of an SM (1 KB each for alignment and 1 KB reserved),
+  // with three stages up to 16 columns (100 KB gave two: 39.7 against 36.4 us per apply of 27 subdomains, 16 columns)
   const int stage = 2 * kATileBytes + N * 128;
-  int st = (100 * 1024) / stage;
+  int st = (110 * 1024) / stage;
   return st > 6 ? 6 : (st < 2 ? 2 : st);
 }
 
@@ -792,15 +817,11 @@ void oras_apply_tc(const TcPlan& p, const OrasTopo& tp, const void* W, const flo
   gather_b_kernel<<<(unsigned)std::max<int64_t>(gblocks, 1), 128, gsm, s>>>(
       p.gt_sub, p.gt_kt, tp.dof_ptr, tp.dofs, r, R, Rp, (uint8_t*)scratch, in_scale, p.n_ktiles_total);
   TcArgs a;
-  a.mt_sub = p.mt_sub;
-  a.mt_row0 = p.mt_row0;
-  a.sub_wtile = p.sub_wtile;
-  a.sub_gtile = p.sub_gtile;
-  a.sub_kt = p.sub_kt;
-  a.own_ptr = tp.own_ptr;
+  a.tiles = p.tiles;
   a.own_glob = tp.own_glob;
   a.c0_glob = c0_glob;
   a.z_bf16 = z_bf16 ? 1 : 0;
+  a.vec = R % (z_bf16 ? 4 : 2) == 0 && ((uintptr_t)z & 15) == 0;
   a.W = (const uint8_t*)W;
   a.Bt = (const uint8_t*)scratch;
   a.z = z;

@@ -14,6 +14,15 @@ namespace mwk {
 struct OrasTopo;
 struct InvBatch;
 
+// One 128-row output tile as the MMA kernels read it: everything a role needs in one 32-byte record.
+struct alignas(16) TcTile {
+  int64_t w;      // first W tile (Wr of k tile 0)
+  int64_t g;      // first gathered-operand tile
+  int64_t own;    // its first row in the owned-row lists
+  int32_t kt;     // k tiles
+  int32_t rows;   // rows that are owned, 1..128
+};
+
 // Pre-tiled BF16 layout of the owned-row inverses W_s (see k_oras_tc.cu).
 struct TcPlan {
   bool built = false;
@@ -22,10 +31,8 @@ struct TcPlan {
   int64_t n_ktiles_total = 0; // sum_s ceil(2 n_s / 64)
   int64_t w_tiles = 0;        // sum_s mtiles_s * ktiles_s (16 KB each)
   // device arrays
-  int32_t* mt_sub = nullptr;     // [n_mtiles] subdomain of each 128-row tile
-  int32_t* mt_row0 = nullptr;    // [n_mtiles] first owned row
+  TcTile* tiles = nullptr;       // [n_mtiles] output tiles in launch order
   int64_t* sub_wtile = nullptr;  // [n_sub] first W tile of s
-  int64_t* sub_gtile = nullptr;  // [n_sub] first gathered-operand k tile of s
   int32_t* sub_kt = nullptr;     // [n_sub] k tiles of s
   int32_t* gt_sub = nullptr;     // [n_ktiles_total] subdomain of each gathered-operand tile
   int32_t* gt_kt = nullptr;      // [n_ktiles_total] its k tile
