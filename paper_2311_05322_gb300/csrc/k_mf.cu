@@ -423,13 +423,6 @@ void mf_gemm(const MfTask* tasks, const MfTile* tiles, int n_tiles, const MfSpli
   }
 }
 
-void mf_reduce(const MfTask* tasks, const MfSplit* splits, int n_splits, const float2* partial, const int32_t* idx,
-               int R, float2* arena, cudaStream_t s) {
-  if (n_splits <= 0) return;
-  note_launch(1);
-  mf_reduce_kernel<<<n_splits, 256, 0, s>>>(tasks, splits, partial, idx, R, arena);
-}
-
 void mf_pull(const int64_t* out, const int64_t* ptr, const int64_t* src, int64_t n, const float2* in, int R,
              float2* arena, cudaStream_t s) {
   if (n <= 0) return;

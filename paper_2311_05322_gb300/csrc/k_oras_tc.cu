@@ -139,30 +139,31 @@ __global__ void pack_w_kernel(InvBatch bt, const int64_t* __restrict__ own_ptr, 
   }
 }
 
-// The same tiles from strided FP32 blocks: "subdomain" q of the plan stacks up to two products
-// with the same B, rows [0, m1) the product sign_1 A_1 of task first[q] and rows [m1, m1 + m2)
-// the product sign_2 A_2 of task second[q] (second[q] < 0: none); A_i [m_i][k] has row stride
-// lda_i at element a_off_i of src, both tasks have the same k, and the signs (+1 or -1) are
-// exact in BF16.  One block per (q, m tile, k tile).
+// The same tiles from strided FP32 blocks: output row i of the plan's "subdomain" q is row own_local[i] of the
+// stack of up to two products with the same B, the rows of sign_1 A_1 (task first[q]) and then those of
+// sign_2 A_2 (task second[q]; < 0: none); A_i [m_i][k] has row stride lda_i at element a_off_i of src, both
+// tasks have the same k, and the signs (+1 or -1) are exact in BF16.  One block per (q, m tile, k tile).
 __global__ void pack_w_stacked_kernel(const MfTask* __restrict__ tasks, const int32_t* __restrict__ first,
-                                      const int32_t* __restrict__ second, int q0,
+                                      const int32_t* __restrict__ second, const int64_t* __restrict__ own_ptr,
+                                      const int32_t* __restrict__ own_local, int q0,
                                       const int64_t* __restrict__ sub_wtile, const int32_t* __restrict__ sub_kt,
                                       const float2* __restrict__ src, uint8_t* __restrict__ W) {
   const int q = q0 + (int)blockIdx.z;
-  const MfTask t1 = tasks[first[q]];
-  const int j2 = second[q];
-  const int64_t m2 = j2 >= 0 ? tasks[j2].m : 0;
+  const int64_t o0 = own_ptr[q], nout = own_ptr[q + 1] - o0;
   const int mt = blockIdx.y, kt = blockIdx.x;
   const int KT = sub_kt[q];
-  if (kt >= KT || (int64_t)mt * kTileM >= t1.m + m2) return;
+  if (kt >= KT || (int64_t)mt * kTileM >= nout) return;
+  const MfTask t1 = tasks[first[q]];
+  const int j2 = second[q];
   uint8_t* tr = W + ((size_t)sub_wtile[q] + ((size_t)mt * KT + kt) * 2) * kATileBytes;
   uint8_t* ti = tr + kATileBytes;
   constexpr int kPairs = kTileKd / 2;
   for (int w = threadIdx.x; w < kTileM * kPairs; w += blockDim.x) {
     const int r = w / kPairs, kp = w % kPairs;
-    const int64_t row = (int64_t)mt * kTileM + r, k = (int64_t)kt * kTileKd + 2 * kp;
+    const int64_t o = (int64_t)mt * kTileM + r, k = (int64_t)kt * kTileKd + 2 * kp;
     float re0 = 0.f, im0 = 0.f, re1 = 0.f, im1 = 0.f;
-    if (row < t1.m + m2) {
+    if (o < nout) {
+      const int64_t row = own_local[o0 + o];
       const MfTask t = row < t1.m ? t1 : tasks[j2];
       const float2* a = src + t.a_off + (row < t1.m ? row : row - t1.m) * t.lda;
       if (k < t.k) {
@@ -246,13 +247,56 @@ __global__ void __launch_bounds__(128, 8) gather_b_kernel(const int32_t* __restr
   }
 }
 
+// The same tiles for the sparse sweeps, each operand row the sum of up to NS listed rows (in order, as the
+// multifrontal forward sweep assembles its right-hand sides): one block per tile, a thread takes 8 rows of a
+// column at a time, so a warp reads whole rows and writes one 16-byte piece per plane and row group.  Summing
+// here spares the front right-hand sides a pass through memory (written, read again by the gather and, for the
+// update rows, by the epilogue).
+template <int NS>
+__global__ void __launch_bounds__(256) gather_rows_kernel(const int32_t* __restrict__ src,
+                                                          const float2* __restrict__ in,
+                                                          const float2* __restrict__ arena, int R, int Rp,
+                                                          uint8_t* __restrict__ Bt) {
+  extern __shared__ __align__(16) uint8_t tsm[];
+  const int32_t* idx = src + (int64_t)blockIdx.x * kTileKd * NS;
+  for (int it = threadIdx.x; it < 8 * Rp; it += blockDim.x) {
+    const int c = it % Rp, g = it / Rp;
+    int32_t e[8 * NS];
+    const int4* ip = reinterpret_cast<const int4*>(idx + 8 * NS * g);
+#pragma unroll
+    for (int i = 0; i < 2 * NS; ++i) *reinterpret_cast<int4*>(e + 4 * i) = ip[i];
+    float2 v[8 * NS];
+#pragma unroll
+    for (int i = 0; i < 8 * NS; ++i) {
+      const float2* row = e[i] >= 0 ? arena + (int64_t)e[i] * R : in + (int64_t)(-2 - e[i]) * R;
+      v[i] = e[i] != -1 && c < R ? row[c] : make_float2(0.f, 0.f);
+    }
+    float2 t[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      t[j] = v[NS * j];
+#pragma unroll
+      for (int q = 1; q < NS; ++q) t[j] = make_float2(t[j].x + v[NS * j + q].x, t[j].y + v[NS * j + q].y);
+    }
+    *reinterpret_cast<uint4*>(tsm + swz(c, 8 * g)) = make_uint4(pack_bf16(t[0].x, t[1].x), pack_bf16(t[2].x, t[3].x),
+                                                                pack_bf16(t[4].x, t[5].x), pack_bf16(t[6].x, t[7].x));
+    *reinterpret_cast<uint4*>(tsm + swz(Rp + c, 8 * g)) =
+        make_uint4(pack_bf16(t[0].y, t[1].y), pack_bf16(t[2].y, t[3].y), pack_bf16(t[4].y, t[5].y),
+                   pack_bf16(t[6].y, t[7].y));
+  }
+  __syncthreads();
+  uint4* tile = reinterpret_cast<uint4*>(Bt + (size_t)blockIdx.x * 2 * Rp * 128);
+  for (int i = threadIdx.x; i < 16 * Rp; i += blockDim.x) tile[i] = reinterpret_cast<const uint4*>(tsm)[i];
+}
+
 // ---------------------------------------------------------------------------------------
 // Apply, step 2: one CTA per 128-row output tile of one subdomain.
 // ---------------------------------------------------------------------------------------
 struct TcArgs {
   const TcTile* tiles;
-  const int32_t* own_glob;
-  const int32_t* c0_glob;   // optional: row of z added to each output row (-1: none)
+  const int32_t* own_glob;  // dense applies: row of z per output row
+  const TcRow* rows;        // sparse sweeps (else null): z is the arena, z2 the result
+  float2* z2;
   int z_bf16;               // z holds complex BF16 pairs (4 bytes per value) instead of float2
   int vec;                  // rows of z are whole, aligned 16-byte pieces
   const uint8_t* W;
@@ -302,41 +346,53 @@ __device__ __forceinline__ bool drain_ring(uint64_t* full_bar, RingPos p, int64_
 // feed only accumulator rows that the epilogue does not store.
 __device__ __forceinline__ uint32_t a_part_of(const TcTile& tl) { return (uint32_t)((tl.rows + 7) / 8) * 1024u; }
 
-// Epilogue of one accumulator row: z[og] = D (+ z[c0]), 8 columns at a time, the next C0 values on their way.
-// A thread owns a whole row, so its stores are 16 bytes where the rows allow it (vec): a warp's store then
-// touches each 32-byte sector twice, not four (FP32) or eight (BF16) times.
-struct EpiRow {
-  int64_t og = -1, c0 = -1;   // output row and row added to it; negative: none
-};
-__device__ __forceinline__ EpiRow epi_row(const TcArgs& a, const TcTile& tl, int row) {
-  EpiRow e;
+// Epilogue of one accumulator row, 8 columns at a time, the next added values on their way.  A thread owns a
+// whole row, so its stores are 16 bytes where the rows allow it (vec): a warp's store then touches each 32-byte
+// sector twice, not four (FP32) or eight (BF16) times.
+__device__ __forceinline__ TcRow epi_row(const TcArgs& a, const TcTile& tl, int row) {
+  TcRow e{-1, -1, -1, -1};
   if (row < tl.rows) {
-    e.og = (int64_t)a.own_glob[tl.own + row];
-    if (a.c0_glob) e.c0 = (int64_t)a.c0_glob[tl.own + row];
+    if (a.rows) {
+      const int4 t = *reinterpret_cast<const int4*>(a.rows + tl.own + row);
+      e = TcRow{t.x, t.y, t.z, t.w};
+    } else {
+      e.out = a.own_glob[tl.own + row];
+    }
   }
   return e;
 }
-__device__ __forceinline__ void epi_fetch(const TcArgs& a, const float2* c0r, int cb, float2 (&v)[8]) {
+// v[i] = z[row][cb + i], 8 columns (zero past R)
+__device__ __forceinline__ void epi_load8(const TcArgs& a, int32_t row, int cb, float2 (&v)[8]) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) v[i] = make_float2(0.f, 0.f);
-  if (!c0r) return;
-  if (a.vec && !a.z_bf16) {
+  if (row < 0) return;
+  const float2* p = a.z + (int64_t)row * a.R + cb;
+  if (a.vec) {
 #pragma unroll
     for (int i = 0; i < 8; i += 2)
       if (cb + i < a.R) {
-        const float4 t = *reinterpret_cast<const float4*>(c0r + cb + i);
+        const float4 t = *reinterpret_cast<const float4*>(p + i);
         v[i] = make_float2(t.x, t.y);
         v[i + 1] = make_float2(t.z, t.w);
       }
-    return;
-  }
+  } else {
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
-    if (cb + i < a.R) v[i] = c0r[cb + i];
+    for (int i = 0; i < 8; ++i)
+      if (cb + i < a.R) v[i] = p[i];
+  }
 }
-__device__ __forceinline__ void epi_store(const TcArgs& a, int64_t og, int cb, const float2 (&v)[8]) {
-  if (a.z_bf16) {
-    uint32_t* zr = reinterpret_cast<uint32_t*>(a.z) + og * a.R + cb;
+struct EpiAdd {
+  float2 a[8], b[8];   // the two added rows' next 8 columns
+};
+__device__ __forceinline__ void epi_fetch(const TcArgs& a, const TcRow& e, int cb, EpiAdd& v) {
+  epi_load8(a, e.add0, cb, v.a);
+  epi_load8(a, e.add1, cb, v.b);
+}
+__device__ __forceinline__ void epi_store(const TcArgs& a, float2* z, int32_t row, bool bf16, int cb,
+                                          const float2 (&v)[8]) {
+  if (row < 0) return;
+  if (bf16) {
+    uint32_t* zr = reinterpret_cast<uint32_t*>(z) + (int64_t)row * a.R + cb;
     if (a.vec) {
 #pragma unroll
       for (int i = 0; i < 8; i += 4)
@@ -351,7 +407,7 @@ __device__ __forceinline__ void epi_store(const TcArgs& a, int64_t og, int cb, c
     }
     return;
   }
-  float2* zr = a.z + og * a.R + cb;
+  float2* zr = z + (int64_t)row * a.R + cb;
   if (a.vec) {
 #pragma unroll
     for (int i = 0; i < 8; i += 2)
@@ -362,29 +418,27 @@ __device__ __forceinline__ void epi_store(const TcArgs& a, int64_t og, int cb, c
       if (cb + i < a.R) zr[i] = v[i];
   }
 }
-// The accumulator at tmem (this warp's lanes) to z; every lane of the warp takes part in the reads.
-__device__ __forceinline__ void epi_tile(const TcArgs& a, uint32_t lanes, const EpiRow& e, bool valid,
-                                         float2 (&nxt)[8]) {
-  const float2* c0r = e.og >= 0 && e.c0 >= 0 ? a.z + e.c0 * a.R : nullptr;
+// The accumulator at lanes (this warp's) plus the added rows to the row's places; every lane of the warp takes
+// part in the reads.
+__device__ __forceinline__ void epi_tile(const TcArgs& a, uint32_t lanes, const TcRow& e, EpiAdd& nxt) {
   const int Rp = a.N / 2;
   for (int cb = 0; cb < Rp; cb += 8) {
-    // Re z = D1[c] - D2[Rp + c], Im z = D1[Rp + c] + D2[c] (plus the C0 row when given)
-    float2 cur[8];
+    // Re z = D1[c] - D2[Rp + c], Im z = D1[Rp + c] + D2[c]
+    float2 add[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) cur[i] = nxt[i];
-    if (cb + 8 < Rp) epi_fetch(a, c0r, cb + 8, nxt);
+    for (int i = 0; i < 8; ++i) add[i] = make_float2(nxt.a[i].x + nxt.b[i].x, nxt.a[i].y + nxt.b[i].y);
+    if (cb + 8 < Rp) epi_fetch(a, e, cb + 8, nxt);
     float d[4][8];   // Wr gr, Wr gi, Wi gr, Wi gi
     tmem_ld8x4(lanes + (uint32_t)cb, lanes + (uint32_t)(Rp + cb), lanes + (uint32_t)(a.N + cb),
                lanes + (uint32_t)(a.N + Rp + cb), d);
-    if (valid) {
-      float2 v[8];
+    float2 v[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        v[i] = make_float2(d[0][i] - d[3][i], d[1][i] + d[2][i]);
-        if (c0r) v[i] = make_float2(v[i].x + cur[i].x, v[i].y + cur[i].y);
-      }
-      epi_store(a, e.og, cb, v);
+    for (int i = 0; i < 8; ++i) {
+      v[i] = make_float2(d[0][i] - d[3][i], d[1][i] + d[2][i]);
+      if (e.add0 >= 0) v[i] = make_float2(v[i].x + add[i].x, v[i].y + add[i].y);
     }
+    epi_store(a, a.z, e.out, a.z_bf16, cb, v);
+    if (a.rows) epi_store(a, a.z2, e.z, false, cb, v);
   }
 }
 
@@ -475,14 +529,14 @@ __global__ void __launch_bounds__(kThreadsTc, 2) oras_tc_kernel(const TcArgs a) 
     // epilogue: warps 2..5 cover tensor-memory lane quadrants (warp % 4).  The output row, the C0
     // row and C0's first 8 columns are looked up while the MMAs run.
     const int quad = warp & 3;
-    const EpiRow e = epi_row(a, tl, quad * 32 + lane);
-    float2 nxt[8];
-    epi_fetch(a, e.og >= 0 && e.c0 >= 0 ? a.z + e.c0 * a.R : nullptr, 0, nxt);
+    const TcRow e = epi_row(a, tl, quad * 32 + lane);
+    EpiAdd nxt;
+    epi_fetch(a, e, 0, nxt);
     bool ok = mbar_wait(&done_bar, 0);
-    ok = __all_sync(0xffffffffu, ok);   // tcgen05.ld below is warp-collective
+    ok = __all_sync(0xffffffffu, ok && !*(volatile int*)&abort_flag);   // tcgen05.ld below is warp-collective
     if (!ok && lane == 0) atomicCAS(a.err, 0, 4);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (ok) epi_tile(a, tmem + ((uint32_t)(quad * 32) << 16), e, !abort_flag && e.og >= 0, nxt);
+    if (ok) epi_tile(a, tmem + ((uint32_t)(quad * 32) << 16), e, nxt);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -617,15 +671,15 @@ __global__ void __launch_bounds__(kThreadsTc, 2) oras_tc_persistent_kernel(const
     const int quad = warp & 3;
     const int row = quad * 32 + lane;
     const int step = gridDim.x;
-    EpiRow e1 = epi_row(a, a.tiles[blockIdx.x], row);
+    TcRow e1 = epi_row(a, a.tiles[blockIdx.x], row);
     TcTile t2;
     if ((int)blockIdx.x + step < n_tiles) t2 = a.tiles[blockIdx.x + step];
     int i = 0;
     for (int t = blockIdx.x; t < n_tiles; t += step, ++i) {
       const int buf = i & 1;
-      const EpiRow e = e1;
-      float2 nxt[8];
-      epi_fetch(a, e.og >= 0 && e.c0 >= 0 ? a.z + e.c0 * a.R : nullptr, 0, nxt);
+      const TcRow e = e1;
+      EpiAdd nxt;
+      epi_fetch(a, e, 0, nxt);
       if (t + step < n_tiles) e1 = epi_row(a, t2, row);
       if (t + 2 * step < n_tiles) t2 = a.tiles[t + 2 * step];
       bool ok = !*abort_v && mbar_wait(&acc_full[buf], (uint32_t)((i >> 1) & 1));
@@ -638,7 +692,7 @@ __global__ void __launch_bounds__(kThreadsTc, 2) oras_tc_persistent_kernel(const
         break;
       }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      epi_tile(a, tmem + (uint32_t)buf * a.tmem_cols + ((uint32_t)(quad * 32) << 16), e, e.og >= 0, nxt);
+      epi_tile(a, tmem + (uint32_t)buf * a.tmem_cols + ((uint32_t)(quad * 32) << 16), e, nxt);
       // this warp's reads of the buffer are done: the MMA warp may overwrite it
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
@@ -766,13 +820,15 @@ void tc_extract(const TcPlan& p, const InvBatch& bt, const OrasTopo& tp, int ws_
                                                 (uint8_t*)W);
 }
 
-void tc_pack_stacked(const TcPlan& p, const MfTask* tasks, const int32_t* first, const int32_t* second, int n,
-                     int ktmax, int mtmax, const float2* src, void* W, cudaStream_t s) {
+void tc_pack_stacked(const TcPlan& p, const MfTask* tasks, const int32_t* first, const int32_t* second,
+                     const int64_t* own_ptr, const int32_t* own_local, int n, int ktmax, int mtmax, const float2* src,
+                     void* W, cudaStream_t s) {
   for (int q0 = 0; q0 < n; q0 += 65535) {
     const int cnt = std::min(65535, n - q0);
     note_launch(1);
     dim3 grid((unsigned)std::max(ktmax, 1), (unsigned)std::max(mtmax, 1), (unsigned)cnt);
-    pack_w_stacked_kernel<<<grid, 256, 0, s>>>(tasks, first, second, q0, p.sub_wtile, p.sub_kt, src, (uint8_t*)W);
+    pack_w_stacked_kernel<<<grid, 256, 0, s>>>(tasks, first, second, own_ptr, own_local, q0, p.sub_wtile, p.sub_kt,
+                                               src, (uint8_t*)W);
   }
 }
 
@@ -798,33 +854,14 @@ int tc_max_stages(int R) {
   return st;
 }
 
-void oras_apply_tc(const TcPlan& p, const OrasTopo& tp, const void* W, const float2* r, float2* z, int R,
-                   void* scratch, cudaStream_t s, int stages, const double* in_scale, const int32_t* c0_glob,
-                   bool z_bf16, bool persistent) {
-  const int Rp = rpad(R);
-  const int N = 2 * Rp;
+// The MMA kernel over the plan's tiles, its operand tiles already in a.Bt.
+static void tc_mma(const TcPlan& p, TcArgs a, int R, int stages, bool persistent, cudaStream_t s) {
+  const int N = 2 * rpad(R);
   if (stages <= 0) stages = tc_stages(N);
   if (stages < tc_min_stages) stages = tc_min_stages;
   if (stages > tc_max_stages(R)) stages = tc_max_stages(R);
-  note_launch(2);
-  const size_t gsm = (size_t)N * 128;
-  static size_t gattr = 0;
-  if (gsm > 48 * 1024 && gsm > gattr) {
-    cudaFuncSetAttribute(gather_b_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm);
-    gattr = gsm;
-  }
-  const int64_t gblocks = std::min<int64_t>(p.n_ktiles_total, 152 * 8);    // one resident wave
-  gather_b_kernel<<<(unsigned)std::max<int64_t>(gblocks, 1), 128, gsm, s>>>(
-      p.gt_sub, p.gt_kt, tp.dof_ptr, tp.dofs, r, R, Rp, (uint8_t*)scratch, in_scale, p.n_ktiles_total);
-  TcArgs a;
+  note_launch(1);
   a.tiles = p.tiles;
-  a.own_glob = tp.own_glob;
-  a.c0_glob = c0_glob;
-  a.z_bf16 = z_bf16 ? 1 : 0;
-  a.vec = R % (z_bf16 ? 4 : 2) == 0 && ((uintptr_t)z & 15) == 0;
-  a.W = (const uint8_t*)W;
-  a.Bt = (const uint8_t*)scratch;
-  a.z = z;
   a.R = R;
   a.N = N;
   a.stages = stages;
@@ -858,6 +895,48 @@ void oras_apply_tc(const TcPlan& p, const OrasTopo& tp, const void* W, const flo
   oras_tc_kernel<<<(unsigned)p.n_mtiles, kThreadsTc, smem, s>>>(a);
 }
 
+void oras_apply_tc(const TcPlan& p, const OrasTopo& tp, const void* W, const float2* r, float2* z, int R,
+                   void* scratch, cudaStream_t s, int stages, const double* in_scale, bool z_bf16) {
+  const int Rp = rpad(R);
+  note_launch(1);
+  const size_t gsm = (size_t)2 * Rp * 128;
+  static size_t gattr = 0;
+  if (gsm > 48 * 1024 && gsm > gattr) {
+    cudaFuncSetAttribute(gather_b_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm);
+    gattr = gsm;
+  }
+  const int64_t gblocks = std::min<int64_t>(p.n_ktiles_total, 152 * 8);    // one resident wave
+  gather_b_kernel<<<(unsigned)std::max<int64_t>(gblocks, 1), 128, gsm, s>>>(
+      p.gt_sub, p.gt_kt, tp.dof_ptr, tp.dofs, r, R, Rp, (uint8_t*)scratch, in_scale, p.n_ktiles_total);
+  TcArgs a{};
+  a.own_glob = tp.own_glob;
+  a.z_bf16 = z_bf16 ? 1 : 0;
+  a.vec = R % (z_bf16 ? 4 : 2) == 0 && ((uintptr_t)z & 15) == 0;
+  a.W = (const uint8_t*)W;
+  a.Bt = (const uint8_t*)scratch;
+  a.z = z;
+  tc_mma(p, a, R, stages, false, s);
+}
+
+void tc_sweep(const TcPlan& p, const TcRow* rows, const int32_t* src, int n_src, const void* W, const float2* in,
+              float2* arena, float2* z, int R, void* scratch, cudaStream_t s, bool persistent) {
+  const int Rp = rpad(R);
+  note_launch(1);
+  const unsigned blocks = (unsigned)p.n_ktiles_total, threads = (unsigned)std::min(8 * Rp, 256);
+  const size_t gsm = (size_t)2 * Rp * 128;   // at most 32 KB
+  if (n_src == 3)
+    gather_rows_kernel<3><<<blocks, threads, gsm, s>>>(src, in, arena, R, Rp, (uint8_t*)scratch);
+  else
+    gather_rows_kernel<1><<<blocks, threads, gsm, s>>>(src, in, arena, R, Rp, (uint8_t*)scratch);
+  TcArgs a{};
+  a.rows = rows;
+  a.vec = R % 2 == 0 && (((uintptr_t)arena | (uintptr_t)z) & 15) == 0;
+  a.W = (const uint8_t*)W;
+  a.Bt = (const uint8_t*)scratch;
+  a.z = arena;
+  a.z2 = z;
+  tc_mma(p, a, R, 0, persistent, s);
+}
 
 // ---------------------------------------------------------------------------------------
 // Fixed scratch for the preconditioner apply that allocates nothing.

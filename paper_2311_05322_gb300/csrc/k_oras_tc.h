@@ -51,22 +51,30 @@ void tc_extract(const TcPlan& p, const InvBatch& bt, const OrasTopo& tp, int ws_
 struct MfTask;
 // Packs the FP32 blocks of tasks (A = src + a_off, [m][k], row stride lda, times the task's
 // sign) into the plan's BF16 tiles for n plan "subdomains" that each stack up to two products
-// with the same B (same k): subdomain q is task first[q] over task second[q] (rows of the second
-// after those of the first; second[q] < 0: the first alone); ktmax / mtmax: the largest tile
-// counts of the stacked products.
-void tc_pack_stacked(const TcPlan& p, const MfTask* tasks, const int32_t* first, const int32_t* second, int n,
-                     int ktmax, int mtmax, const float2* src, void* W, cudaStream_t s);
+// with the same B (same k): subdomain q is task first[q] over task second[q] (second[q] < 0: the
+// first alone), and its output row i (own_ptr[q] <= i < own_ptr[q + 1]) is row own_local[i] of the
+// stack; ktmax / mtmax: the largest tile counts.
+void tc_pack_stacked(const TcPlan& p, const MfTask* tasks, const int32_t* first, const int32_t* second,
+                     const int64_t* own_ptr, const int32_t* own_local, int n, int ktmax, int mtmax, const float2* src,
+                     void* W, cudaStream_t s);
+// Where an output row of a sweep goes: row out of the arena and row z of the result (-1: neither), after the
+// arena rows add0 and add1 (-1: none) have been added.
+struct alignas(16) TcRow {
+  int32_t out, add0, add1, z;
+};
+// One launch of the sparse sweeps: the plan's products with operand rows from src, n_src (1 or 3) entries per
+// row, summed in order (>= 0: that arena row, -1: nothing, else row -2 - src of in); 64 rows per k tile, in
+// the order of the plan's k tiles.  in and z do not overlap.
+// persistent: CTAs loop over the output tiles with one copy ring and double-buffered accumulators (for plans
+// of many short tiles; up to 64 columns, else the one-tile-per-CTA kernel runs); the same bits either way.
+void tc_sweep(const TcPlan& p, const TcRow* rows, const int32_t* src, int n_src, const void* W, const float2* in,
+              float2* arena, float2* z, int R, void* scratch, cudaStream_t s, bool persistent);
 // stages: shared-memory pipeline depth of the MMA kernel (0 = default; the result does not depend
 // on it, only the speed).  in_scale (may be null): per-column factor of r (z = M^{-1}(r * in_scale)).
-// Output row q of "subdomain" s goes to z row own_glob[own_ptr[s] + q] (skipped when negative);
-// c0_glob (may be null) lists, per output row, a row of z added to it (-1: none).  z_bf16: z is
-// written as complex BF16 pairs (real in the low half), 4 bytes per value, row stride R values.
-// persistent: CTAs loop over the output tiles with one copy ring and double-buffered
-// accumulators (for plans of many short tiles; up to 64 columns, else the one-tile-per-CTA
-// kernel runs); the same bits either way.
+// z_bf16: z is written as complex BF16 pairs (real in the low half), 4 bytes per value, row stride R values.
 void oras_apply_tc(const TcPlan& p, const OrasTopo& tp, const void* W, const float2* r, float2* z, int R,
                    void* scratch, cudaStream_t s, int stages = 0, const double* in_scale = nullptr,
-                   const int32_t* c0_glob = nullptr, bool z_bf16 = false, bool persistent = false);
+                   bool z_bf16 = false);
 // Pipeline depths the MMA kernel accepts for R columns: [tc_min_stages, tc_max_stages(R)].
 constexpr int tc_min_stages = 2;
 int tc_max_stages(int R);

@@ -74,11 +74,11 @@ struct Prec {
   struct Mf {
     mw::Multifrontal sym;
     std::vector<void*> allocs;       // every device table below
-    int64_t *f = nullptr, *ws_off = nullptr, *fac_off = nullptr, *piv_ptr = nullptr, *child_ptr = nullptr,
-            *inv_off = nullptr, *rhs_row = nullptr, *w_row = nullptr, *own_row = nullptr, *asm_ptr = nullptr,
+    int64_t *f = nullptr, *ws_off = nullptr, *fac_off = nullptr, *child_ptr = nullptr,
+            *inv_off = nullptr, *own_row = nullptr, *asm_ptr = nullptr,
             *asm_target = nullptr, *sh_f = nullptr, *sh_off = nullptr, *sh_lim = nullptr;
-    int32_t *p = nullptr, *preal = nullptr, *piv_glob = nullptr, *child = nullptr, *inv = nullptr, *idx = nullptr,
-            *asm_code = nullptr, *sh_nodes = nullptr, *h_nodes = nullptr;
+    int32_t *p = nullptr, *child = nullptr, *inv = nullptr, *idx = nullptr,
+            *asm_code = nullptr, *sh_nodes = nullptr;
     mwk::MfTask* tasks = nullptr;
     mwk::MfTile* tiles = nullptr;
     mwk::MfSplit* splits = nullptr;
@@ -91,29 +91,20 @@ struct Prec {
     std::vector<int64_t> sh_ptr;     // [(n_sub * (H + 1)) + 1] node ranges per (subdomain, height)
     std::vector<int64_t> sh_fmax, sh_pmax, sh_emax;
     std::vector<int64_t> h_ptr;      // [H + 2] node ranges per height (all subdomains)
-    std::vector<int64_t> h_fmax;
     std::vector<int64_t> fwd_tiles, bwd_tiles;  // [H + 2] tile ranges per height
     int64_t arena_rows = 0, ws_max = 0, n_own = 0, max_sh = 0;
     std::vector<void*> fac;          // factors per frequency (FP32 complex; freed after BF16 packing)
     // BF16 tensor-core sweeps (apply_prec 5): one plan per launch (height x direction), whose
-    // "subdomains" are the launch's products with K > 0; outputs go to partial slots that
-    // mf_reduce turns into C = C0 + sign * A B
+    // "subdomains" are the launch's products (see build_sparse_tc)
     struct TcLaunch {
       mwk::TcPlan plan;
-      int64_t *dof_ptr = nullptr, *own_ptr = nullptr;
-      int32_t *dofs = nullptr, *own_local = nullptr, *own_glob = nullptr;
-      int32_t* c0_glob = nullptr;    // per output row: arena row of C0, or -1
-      mwk::MfTask* tasks = nullptr;  // products with K > 0 (plan order), then those with K = 0
-      mwk::MfSplit* splits = nullptr;
-      int32_t *pk_first = nullptr, *pk_second = nullptr;   // tasks stacked in each plan "subdomain"
-      int n_tc = 0, n_splits = 0, ktmax = 0, mtmax = 0;
-      // the plan's B rows are rows of the input vector (the leaves' pivot entries), not arena
-      // rows: the launch gathers straight from the input and the leaves' pull is skipped
-      bool from_input = false;
+      mwk::TcRow* rows = nullptr;    // where each output row of the plan goes and what is added to it
+      int32_t* src = nullptr;        // n_src entries per operand row, 64 rows per k tile (see tc_sweep)
+      int n_src = 1;
       std::vector<void*> W;          // BF16 tiles per frequency
     };
     std::vector<TcLaunch> tcl;       // [2 (H + 1)]: forward heights, then backward heights
-    int64_t tc_slots = 0;            // partial slots of the largest tensor-core launch
+    double tc_entries = 0.0;         // factor entries that the sweeps read
     size_t tc_scratch = 0;           // gathered-operand bytes of the largest plan at 128 columns
   } mf;
   mwk::OrasTopo topo() const {
@@ -491,9 +482,8 @@ void ensure_prec_scratch(Ctx* c, int R) {
       w.mf_arena = dalloc<unsigned char>(c, need);
       w.mf_bytes = need;
     }
-    const int64_t slots = std::max<int64_t>({p.mf.max_slots, p.mf.tc_slots, (int64_t)1});
-    const size_t pneed = (size_t)slots * mwk::kMfTileRows * R * sizeof(float2);
-    if (w.mf_pbytes < pneed) {
+    const size_t pneed = (size_t)std::max<int64_t>(p.mf.max_slots, 1) * mwk::kMfTileRows * R * sizeof(float2);
+    if (p.apply_prec == 4 && w.mf_pbytes < pneed) {
       dfree(c, w.mf_partial);
       w.mf_partial = nullptr;
       w.mf_partial = dalloc<unsigned char>(c, pneed);
@@ -530,25 +520,9 @@ void apply_sparse(Ctx* c, int f, const float2* v, float2* z, int R) {
   float2* partial = (float2*)w.mf_partial;
   const int H = m.sym.max_height;
   if (c->prec.apply_prec == 5) {
-    auto run = [&](Prec::Mf::TcLaunch& L) {
-      if (L.n_tc > 0) {
-        // C = C0 + (sign A) B straight from the MMA epilogue into the arena
-        const mwk::OrasTopo tp{L.dof_ptr, L.dofs, L.own_ptr, L.own_local, L.own_glob, nullptr, nullptr, nullptr,
-                               nullptr, nullptr, nullptr};
-        mwk::oras_apply_tc(L.plan, tp, L.W[f], L.from_input ? v : arena, arena, R, w.tc_scratch, s, 0, nullptr,
-                           L.c0_glob, false, c->sweep_persistent != 0);
-      }
-      // products with K = 0: C = C0
-      if (L.n_splits > 0) mwk::mf_reduce(L.tasks, L.splits, L.n_splits, partial, m.idx, R, arena, s);
-    };
-    for (int h = 0; h <= H; ++h) {
-      if (!m.tcl[h].from_input)
-        mwk::mf_pull(m.pull_out + m.pull_h[h], m.pull_ptr + m.pull_h[h], m.pull_src, m.pull_h[h + 1] - m.pull_h[h],
-                     v, R, arena, s);
-      run(m.tcl[h]);
-    }
-    for (int h = H; h >= 0; --h) run(m.tcl[H + 1 + h]);
-    mwk::mf_owned(c->prec.own_glob, m.own_row, m.n_own, arena, R, z, s);
+    for (Prec::Mf::TcLaunch& L : m.tcl)
+      if (L.plan.n_mtiles > 0)
+        mwk::tc_sweep(L.plan, L.rows, L.src, L.n_src, L.W[f], v, arena, z, R, w.tc_scratch, s, c->sweep_persistent != 0);
     return;
   }
   const float2* fac = (const float2*)m.fac[f];
@@ -573,8 +547,7 @@ T* mf_up(Ctx* c, Prec::Mf& m, const std::vector<T>& h) {
   return d;
 }
 
-void build_sparse_tc(Ctx* c, const std::vector<std::vector<mwk::MfTask>>& launches, const std::vector<int32_t>& idx,
-                     const std::vector<int32_t>& leaf_in);
+void build_sparse_tc(Ctx* c);
 
 // Symbolic factorisation on the host, device tables, then the numeric factorisation of every
 // subdomain for every frequency (FP32 fronts in a workspace, partial Gauss-Jordan per height).
@@ -614,13 +587,9 @@ void setup_sparse(Ctx* c) {
   std::vector<int32_t> h_nodes, sh_nodes;
   std::vector<int64_t> sh_f, sh_off, sh_lim;
   m.h_ptr.assign(1, 0);
-  m.h_fmax.assign(H + 1, 0);
   for (int h = 0; h <= H; ++h) {
     for (int k = 0; k < N; ++k)
-      if (y.height[k] == h) {
-        h_nodes.push_back(k);
-        m.h_fmax[h] = std::max(m.h_fmax[h], y.f[k]);
-      }
+      if (y.height[k] == h) h_nodes.push_back(k);
     m.h_ptr.push_back((int64_t)h_nodes.size());
   }
   // pull lists of the front right-hand sides: row r of node k sums its input entry (a real
@@ -628,7 +597,8 @@ void setup_sparse(Ctx* c) {
   // leaf receive nothing (they are zero), so they are not listed, and its w product has no C0.
   std::vector<int64_t> pull_out, pull_ptr(1, 0), pull_src;
   m.pull_h.assign(1, 0);
-  for (int h = 0; h <= H; ++h) {
+  const bool f32_sweeps = P.apply_prec == 4;   // the BF16 sweeps have tables of their own
+  for (int h = 0; h <= H && f32_sweeps; ++h) {
     for (int64_t q = m.h_ptr[h]; q < m.h_ptr[h + 1]; ++q) {
       const int k = h_nodes[q];
       const bool leaf = y.child_ptr[k + 1] == y.child_ptr[k];
@@ -675,9 +645,7 @@ void setup_sparse(Ctx* c) {
   std::vector<mwk::MfTask> tasks;
   std::vector<mwk::MfTile> tiles;
   std::vector<mwk::MfSplit> splits;
-  std::vector<std::vector<mwk::MfTask>> launches;   // forward heights, then backward heights
   auto emit_launch = [&](const std::vector<mwk::MfTask>& tl) {
-    launches.push_back(tl);
     int64_t row_tiles = 0;
     for (const auto& t : tl) row_tiles += (t.m + 63) / 64;
     const int64_t want = row_tiles >= kMfTargetCtas ? 1 : (kMfTargetCtas + row_tiles - 1) / std::max<int64_t>(row_tiles, 1);
@@ -704,7 +672,7 @@ void setup_sparse(Ctx* c) {
   };
   m.fwd_tiles.assign(1, 0);
   m.fwd_splits.assign(1, 0);
-  for (int h = 0; h <= H; ++h) {
+  for (int h = 0; h <= H && f32_sweeps; ++h) {
     std::vector<mwk::MfTask> tl;
     for (int64_t q = m.h_ptr[h]; q < m.h_ptr[h + 1]; ++q) {
       const int k = h_nodes[q];
@@ -720,7 +688,7 @@ void setup_sparse(Ctx* c) {
   }
   m.bwd_tiles.assign(1, m.fwd_tiles.back());
   m.bwd_splits.assign(1, m.fwd_splits.back());
-  for (int h = 0; h <= H; ++h) {
+  for (int h = 0; h <= H && f32_sweeps; ++h) {
     std::vector<mwk::MfTask> tl;
     for (int64_t q = m.h_ptr[h]; q < m.h_ptr[h + 1]; ++q) {
       const int k = h_nodes[q];
@@ -801,11 +769,8 @@ void setup_sparse(Ctx* c) {
   m.f = mf_up(c, m, y.f);
   m.ws_off = mf_up(c, m, y.ws_off);
   m.fac_off = mf_up(c, m, y.fac_off);
-  m.piv_ptr = mf_up(c, m, y.piv_ptr);
   m.child_ptr = mf_up(c, m, y.child_ptr);
   m.inv_off = mf_up(c, m, y.inv_off);
-  m.rhs_row = mf_up(c, m, rhs_row);
-  m.w_row = mf_up(c, m, w_row);
   m.own_row = mf_up(c, m, own_row);
   m.pull_out = mf_up(c, m, pull_out);
   m.pull_ptr = mf_up(c, m, pull_ptr);
@@ -816,14 +781,11 @@ void setup_sparse(Ctx* c) {
   m.sh_off = mf_up(c, m, sh_off);
   m.sh_lim = mf_up(c, m, sh_lim);
   m.p = mf_up(c, m, pp);
-  m.preal = mf_up(c, m, y.preal);
-  m.piv_glob = mf_up(c, m, piv_glob);
   m.child = mf_up(c, m, y.child);
   m.inv = mf_up(c, m, y.inv);
   m.idx = mf_up(c, m, idx);
   m.asm_code = mf_up(c, m, y.asm_code);
   m.sh_nodes = mf_up(c, m, sh_nodes);
-  m.h_nodes = mf_up(c, m, h_nodes);
   m.tasks = mf_up(c, m, tasks);
   m.tiles = mf_up(c, m, tiles);
   m.splits = mf_up(c, m, splits);
@@ -875,128 +837,155 @@ void setup_sparse(Ctx* c) {
   dfree(c, ws);
   dfree(c, dinv);
   dfree(c, status);
-  if (P.apply_prec == 5) {
-    // input row of each arena row that the leaves' pull fills (-1: an identity-padded pivot,
-    // zero; -2: not such a row)
-    std::vector<int32_t> leaf_in((size_t)rows, -2);
-    for (int64_t i = m.pull_h[0]; i < m.pull_h[1]; ++i) {
-      const int64_t n_src = pull_ptr[i + 1] - pull_ptr[i];
-      if (n_src == 0)
-        leaf_in[pull_out[i]] = -1;
-      else if (n_src == 1 && pull_src[pull_ptr[i]] < 0)
-        leaf_in[pull_out[i]] = (int32_t)(-pull_src[pull_ptr[i]] - 1);
-    }
-    build_sparse_tc(c, launches, idx, leaf_in);
-  }
+  if (P.apply_prec == 5) build_sparse_tc(c);
 }
 
-// BF16 tensor-core form of the sweeps: per launch, a tile plan whose "subdomains" are the
-// products with K > 0 (inputs: the arena rows of B; outputs: the arena rows of C, with the
-// arena rows of C0 added in the MMA epilogue), the BF16 tiles of their FP32 factor blocks times
-// the product's sign for every frequency, and one reduction split per 64-row tile of the
-// products with K = 0 (C = C0).  The FP32 factors are then freed.
-void build_sparse_tc(Ctx* c, const std::vector<std::vector<mwk::MfTask>>& launches, const std::vector<int32_t>& idx,
-                     const std::vector<int32_t>& leaf_in) {
+// BF16 tensor-core form of the sweeps.  The vector arena holds w (u rows per node) and x (the dofs of each
+// subdomain), and one plan per height and direction holds as "subdomains" that launch's products:
+//   forward:  [TL; BL] rhs(p) of a node, stacked: the t rows to their x rows, the w rows plus the children's w
+//             mapped to them; rhs(p) = the pivots' input rows plus the children's w is summed where the
+//             operand is gathered;
+//   backward: x(p) -= TR x(u), and x(owned) straight to z.
+// A row of t or x is computed only if it is owned or enters another row that is: most subdomain dofs outside
+// the owned region (the overlap) are leaves that nothing reads.  With the sums and the scatter inside the
+// launches (no separate right-hand-side, copy and owned-row passes) and those rows left out, an apply of 16
+// subdomains of 25,052 unknowns, 16 columns, takes 34 launches and 0.77 ms (55 and 1.05 ms with them).  The FP32
+// factors are freed after packing.
+void build_sparse_tc(Ctx* c) {
   Prec& P = c->prec;
   Prec::Mf& m = P.mf;
+  const mw::Multifrontal& y = m.sym;
+  const mw::Subdomains& sd = P.sd;
+  const int N = y.n_nodes, H = y.max_height, S = sd.n_sub;
   const char* bad = "internal: sparse tensor-core table out of range";
-  m.tcl.resize(launches.size());
-  for (size_t L = 0; L < launches.size(); ++L) {
+  std::vector<int64_t> w_row(N), x_row(S);
+  int64_t rows = 0;
+  for (int k = 0; k < N; ++k) { w_row[k] = rows; rows += y.u[k]; }
+  for (int s = 0; s < S; ++s) { x_row[s] = rows; rows += sd.dof_ptr[s + 1] - sd.dof_ptr[s]; }
+  m.arena_rows = rows;
+  // z row of each subdomain dof (-1: not owned), and whether its x is needed or read by a product
+  std::vector<int32_t> z_row(sd.dofs.size(), -1);
+  std::vector<uint8_t> need(sd.dofs.size(), 0), read(sd.dofs.size(), 0), live(N, 0);
+  for (int s = 0; s < S; ++s)
+    for (int64_t q = sd.own_ptr[s]; q < sd.own_ptr[s + 1]; ++q) {
+      const int64_t d = sd.dof_ptr[s] + sd.own_local[q];
+      z_row[d] = sd.dofs[d];
+      need[d] = 1;
+    }
+  for (int k = 0; k < N; ++k) {   // children come before their parents
+    require(y.parent[k] < 0 || y.parent[k] > k, MW_EINVAL, bad);
+    require(y.child_ptr[k + 1] - y.child_ptr[k] <= 2, MW_EINVAL, bad);
+    const int64_t d0 = sd.dof_ptr[y.sub[k]];
+    for (int64_t q = y.piv_ptr[k]; q < y.piv_ptr[k + 1]; ++q) live[k] |= need[d0 + y.piv_loc[q]];
+    if (!live[k]) continue;
+    for (int64_t q = y.upd_ptr[k]; q < y.upd_ptr[k + 1]; ++q) need[d0 + y.upd_loc[q]] = read[d0 + y.upd_loc[q]] = 1;
+  }
+  m.tc_entries = 0.0;
+  m.tcl.resize(2 * (H + 1));
+  for (int L = 0; L < 2 * (H + 1); ++L) {
     Prec::Mf::TcLaunch& T = m.tcl[L];
-    std::vector<mwk::MfTask> ord;
-    for (const auto& t : launches[L])
-      if (t.k > 0) ord.push_back(t);
-    T.n_tc = (int)ord.size();
-    for (const auto& t : launches[L])
-      if (t.k <= 0) ord.push_back(t);
-    auto b_row_of = [&](const mwk::MfTask& t, int64_t i) {
-      return t.b_idx >= 0 ? (int64_t)idx[t.b_idx + i] : t.b_row + i;
-    };
-    // the first forward launch (the leaves) reads its B rows from the input when every one of
-    // them is a leaf pivot row that the pull would only copy
-    T.from_input = L == 0 && T.n_tc > 0;
-    for (int q = 0; q < T.n_tc && T.from_input; ++q)
-      for (int64_t i = 0; i < ord[q].k && T.from_input; ++i) {
-        const int64_t row = b_row_of(ord[q], i);
-        T.from_input = row >= 0 && row < (int64_t)leaf_in.size() && leaf_in[row] >= -1;
-      }
-    // plan "subdomains": consecutive products with the same B (the forward t and w products of
-    // a front) are stacked, so B is gathered once and their rows share the MMA tiles
-    mw::Subdomains fake;
+    const bool fwd = L <= H;
+    const int h = fwd ? L : 2 * H + 1 - L;
+    T.n_src = fwd && h > 0 ? 3 : 1;
+    mw::Subdomains fake;   // the plan's shape: operand rows and output rows of each product
     fake.dof_ptr.assign(1, 0);
     fake.own_ptr.assign(1, 0);
-    std::vector<int32_t> own_glob, c0_glob, first, second;
-    std::vector<mwk::MfSplit> sp;
-    int64_t slot = 0;
-    for (int q = 0; q < T.n_tc;) {
-      const mwk::MfTask& t = ord[q];
-      int q2 = -1;
-      if (q + 1 < T.n_tc) {
-        const mwk::MfTask& u = ord[q + 1];
-        if (u.k == t.k && u.b_idx == t.b_idx && (t.b_idx >= 0 || u.b_row == t.b_row)) q2 = q + 1;
+    std::vector<mwk::MfTask> tasks;
+    std::vector<mwk::TcRow> out;
+    std::vector<int32_t> src, first, second;
+    int ktmax = 0, mtmax = 0;
+    for (int k = 0; k < N; ++k) {
+      if (y.height[k] != h) continue;
+      const int64_t p = y.p[k], u = y.u[k], ff = y.f[k], d0 = sd.dof_ptr[y.sub[k]], x0 = x_row[y.sub[k]];
+      if (!fwd && (u == 0 || !live[k])) continue;
+      const size_t out0 = out.size();
+      // rows of t (forward; x itself at a root, which has no update dofs) or x (backward)
+      for (int32_t i = 0; i < y.preal[k]; ++i) {
+        const int32_t loc = y.piv_loc[y.piv_ptr[k] + i];
+        if (!need[d0 + loc]) continue;
+        const int32_t xr = (int32_t)(x0 + loc), zr = z_row[d0 + loc];
+        fake.own_local.push_back(i);
+        if (fwd && u > 0)
+          out.push_back({xr, -1, -1, -1});
+        else
+          out.push_back({read[d0 + loc] ? xr : -1, fwd ? -1 : xr, -1, zr});
       }
-      first.push_back(q);
-      second.push_back(q2);
-      for (int64_t i = 0; i < t.k; ++i) {
-        const int64_t row = b_row_of(t, i);
-        require(row >= 0 && row < m.arena_rows, MW_EINVAL, bad);
-        if (T.from_input) {
-          const int32_t in = leaf_in[row];
-          require(in >= -1 && in < c->topo.n_edge, MW_EINVAL, bad);
-          fake.dofs.push_back(in);
-        } else {
-          fake.dofs.push_back((int32_t)row);
+      int32_t ch[2] = {-1, -1};
+      for (int64_t q = y.child_ptr[k]; q < y.child_ptr[k + 1]; ++q) ch[q - y.child_ptr[k]] = y.child[q];
+      auto child_row = [&](int q, int64_t r) -> int32_t {   // arena row of child q's w entry for front row r
+        const int32_t a = ch[q] >= 0 ? y.inv[y.inv_off[ch[q]] + r] : -1;
+        return a >= 0 ? (int32_t)(w_row[ch[q]] + a) : -1;
+      };
+      for (int32_t i = 0; fwd && i < u; ++i) {
+        const int32_t a = child_row(0, p + i), b = child_row(1, p + i);
+        fake.own_local.push_back((int32_t)p + i);
+        out.push_back({(int32_t)(w_row[k] + i), a >= 0 ? a : b, a >= 0 ? b : -1, -1});
+      }
+      if (out.size() == out0) continue;
+      for (size_t i = out0; i < out.size(); ++i)
+        for (int32_t r : {out[i].out, out[i].add0, out[i].add1, out[i].z < 0 ? -1 : 0})
+          require(r >= -1 && r < rows && out[i].z >= -1 && out[i].z < c->topo.n_edge, MW_EINVAL, bad);
+      // operand rows, in whole k tiles; a node without pivots has one empty tile (its w rows are the sums alone)
+      const int64_t K = fwd ? p : u;
+      const int64_t kt = std::max<int64_t>((K + 63) / 64, 1);
+      for (int64_t i = 0; i < 64 * kt; ++i) {
+        if (!fwd) {
+          src.push_back(i < u ? (int32_t)(x0 + y.upd_loc[y.upd_ptr[k] + i]) : -1);
+          continue;
         }
+        const bool piv = i < y.preal[k];
+        src.push_back(piv ? -2 - sd.dofs[d0 + y.piv_loc[y.piv_ptr[k] + i]] : -1);
+        for (int q = 0; q < 2 && h > 0; ++q) src.push_back(i < p ? child_row(q, i) : -1);
       }
-      fake.dof_ptr.push_back((int64_t)fake.dofs.size());
-      int64_t r_out = 0;
-      for (int qq : {q, q2}) {
-        if (qq < 0) continue;
-        const mwk::MfTask& tt = ord[qq];
-        for (int64_t r = 0; r < tt.m; ++r, ++r_out) {
-          const int64_t crow = tt.c_idx >= 0 ? (int64_t)idx[tt.c_idx + r] : tt.c_row + r;
-          const int64_t c0 = tt.c0_row >= 0 ? tt.c0_row + r : -1;
-          require(crow >= -1 && crow < m.arena_rows && c0 >= -1 && c0 < m.arena_rows, MW_EINVAL, bad);
-          fake.own_local.push_back((int32_t)r_out);
-          own_glob.push_back((int32_t)crow);
-          c0_glob.push_back((int32_t)c0);
-        }
+      // stacked factor blocks: pivot rows, then (forward) update rows
+      first.push_back((int32_t)tasks.size());
+      if (fwd) {
+        tasks.push_back({y.fac_off[k], std::max<int64_t>(ff, 1), p, p, 0, -1, 0, -1, -1, 1.f, 0});
+        second.push_back((int32_t)tasks.size());
+        tasks.push_back({y.fac_off[k] + p * ff, std::max<int64_t>(p, 1), u, p, 0, -1, 0, -1, -1, 1.f, 0});
+      } else {
+        second.push_back(-1);
+        tasks.push_back({y.fac_off[k] + p, ff, p, u, 0, -1, 0, -1, -1, -1.f, 0});
       }
-      fake.own_ptr.push_back((int64_t)fake.own_local.size());
-      T.ktmax = std::max<int>(T.ktmax, (int)((t.k + 63) / 64));
-      T.mtmax = std::max<int>(T.mtmax, (int)((r_out + 127) / 128));
-      q += q2 >= 0 ? 2 : 1;
+      fake.dof_ptr.push_back(fake.dof_ptr.back() + 64 * kt);
+      fake.own_ptr.push_back((int64_t)out.size());
+      m.tc_entries += (double)K * (double)(out.size() - out0);
+      ktmax = std::max(ktmax, (int)kt);
+      mtmax = std::max(mtmax, (int)((out.size() - out0 + 127) / 128));
     }
     fake.n_sub = (int)first.size();
-    for (int q = T.n_tc; q < (int)ord.size(); ++q)
-      for (int64_t r0 = 0; r0 < ord[q].m; r0 += mwk::kMfTileRows) sp.push_back({q, (int32_t)r0, 0, 0});
-    require(slot * mwk::kMfTileRows < INT32_MAX, MW_EINVAL, bad);
-    m.tc_slots = std::max<int64_t>(m.tc_slots, slot);
-    T.n_splits = (int)sp.size();
-    T.tasks = mf_up(c, m, ord);
-    T.splits = mf_up(c, m, sp);
-    if (T.n_tc == 0) continue;
-    T.pk_first = mf_up(c, m, first);
-    T.pk_second = mf_up(c, m, second);
-    T.dof_ptr = mf_up(c, m, fake.dof_ptr);
-    T.dofs = mf_up(c, m, fake.dofs);
-    T.own_ptr = mf_up(c, m, fake.own_ptr);
-    T.own_local = mf_up(c, m, fake.own_local);
-    T.own_glob = mf_up(c, m, own_glob);
-    T.c0_glob = mf_up(c, m, c0_glob);
+    if (fake.n_sub == 0) continue;
+    for (int32_t r : src) require(r >= 0 ? r < rows : -2 - r < c->topo.n_edge, MW_EINVAL, bad);
+    T.rows = mf_up(c, m, out);
+    T.src = mf_up(c, m, src);
     require(mwk::tc_plan_build(T.plan, fake, [&](size_t b) { return (void*)dalloc<unsigned char>(c, b); },
                                c->d_words + kWordTc, c->stream),
             MW_EINVAL, "tensor-core plan of the sparse sweeps");
     m.tc_scratch = std::max(m.tc_scratch, mwk::tc_scratch_bytes(T.plan, 128));
-    T.W.assign(c->n_freq, nullptr);
-    for (int f = 0; f < c->n_freq; ++f) {
-      T.W[f] = dalloc<unsigned char>(c, std::max<size_t>(mwk::tc_w_bytes(T.plan), 16));
-      mwk::tc_pack_stacked(T.plan, T.tasks, T.pk_first, T.pk_second, fake.n_sub, T.ktmax, T.mtmax,
-                           (const float2*)m.fac[f], T.W[f], c->stream);
+    std::vector<void*> tmp;
+    auto temp = [&](const auto& v) {
+      auto* d = upload_vec(c, v);
+      tmp.push_back(d);
+      return d;
+    };
+    try {
+      const mwk::MfTask* d_tasks = temp(tasks);
+      const int32_t *d_first = temp(first), *d_second = temp(second), *d_local = temp(fake.own_local);
+      const int64_t* d_own = temp(fake.own_ptr);
+      T.W.assign(c->n_freq, nullptr);
+      for (int f = 0; f < c->n_freq; ++f) {
+        T.W[f] = dalloc<unsigned char>(c, std::max<size_t>(mwk::tc_w_bytes(T.plan), 16));
+        mwk::tc_pack_stacked(T.plan, d_tasks, d_first, d_second, d_own, d_local, fake.n_sub, ktmax, mtmax,
+                             (const float2*)m.fac[f], T.W[f], c->stream);
+      }
+      check_launch("sparse tensor-core packing");
+      CK(cudaStreamSynchronize(c->stream));
+    } catch (...) {
+      for (void* q : tmp) dfree(c, q);
+      throw;
     }
-    check_launch("sparse tensor-core packing");
+    for (void* q : tmp) dfree(c, q);
   }
-  CK(cudaStreamSynchronize(c->stream));
   for (void*& q : m.fac) {
     dfree(c, q);
     q = nullptr;
@@ -1015,7 +1004,7 @@ void apply_prec(Ctx* c, int f, int work_prec, const void* v, void* z, int R, int
     Work& w = c->work;
     ensure_prec_scratch(c, R);
     mwk::oras_apply_tc(p.tc, p.topo(), p.W[f], (const float2*)v, (float2*)z, R, w.tc_scratch, s, stages, in_scale,
-                       nullptr, z_bf16);
+                       z_bf16);
   } else {
     const int need = work_prec;  // 0 FP64, 1 FP32
     require(p.apply_prec == need, MW_EINVAL,
@@ -1072,7 +1061,7 @@ void check_tc_wait(Ctx* c) {
 double oras_bytes(Ctx* c, int R, bool zb = false) {
   const Prec& p = c->prec;
   if (p.apply_prec == 4) return 8.0 * (double)p.mf.sym.fac_total + 8.0 * R * (p.sum_n + (double)c->topo.n_edge);
-  if (p.apply_prec == 5) return 4.0 * (double)p.mf.sym.fac_total + 8.0 * R * (p.sum_n + (double)c->topo.n_edge);
+  if (p.apply_prec == 5) return 4.0 * p.mf.tc_entries + 8.0 * R * (p.sum_n + (double)c->topo.n_edge);
   const double wb = p.apply_prec == 0 ? 16.0 : (p.apply_prec == 1 ? 8.0 : 4.0);
   const double vb = p.apply_prec == 0 ? 16.0 : 8.0;
   return wb * p.sum_own_n + vb * R * (double)p.sum_n + (zb ? 4.0 : vb) * R * (double)c->topo.n_edge;
