@@ -18,6 +18,7 @@
 
 #include "mw_async.cuh"
 #include "mw_internal.h"
+#include "mw_reduce.cuh"
 
 namespace mwk {
 namespace {
@@ -64,6 +65,19 @@ inline Shape shape_for(int R) {
 constexpr int kDotThreads = 512;
 constexpr int kDotWarps = kDotThreads / 32;
 constexpr int kDotVecPerWarp = 4;   // nvec <= 64 = 16 warps x 4
+
+// Sums (x, y) over the lanes that agree in the bits below tpr.  An FP64 add of a warp takes an SM 16 cycles
+// whatever its lanes, so the first exchange leaves x with one half of the lanes and y with the other, and each
+// further level costs one add, not two (the sums of a butterfly, pair by pair).  Valid in lanes below tpr.
+__device__ __forceinline__ double2 sum_lanes_pair(double2 v, int lane, int tpr) {
+  if (tpr == 32) return v;
+  const bool hi = (lane & tpr) != 0;
+  const double got = __shfl_xor_sync(0xffffffffu, hi ? v.x : v.y, tpr);
+  double mine = (hi ? v.y : v.x) + got;
+  for (int off = 2 * tpr; off < 32; off <<= 1) mine += __shfl_xor_sync(0xffffffffu, mine, off);
+  const double y = __shfl_xor_sync(0xffffffffu, mine, tpr);
+  return make_double2(mine, y);
+}
 
 template <typename T, int CPL>
 __global__ void __launch_bounds__(kDotThreads) cgs_dots_kernel(const T* __restrict__ V, int64_t vstride, int nvec,
@@ -138,17 +152,10 @@ __global__ void __launch_bounds__(kDotThreads) cgs_dots_kernel(const T* __restri
   }
   // reduce over the rows of the warp (lanes with equal column)
 #pragma unroll
-  for (int a = 0; a < kDotVecPerWarp; ++a) {
+  for (int a = 0; a < kDotVecPerWarp; ++a)
+    if (a < nmine)
 #pragma unroll
-    for (int q = 0; q < CPL; ++q) {
-      double x = acc[a][q].x, y = acc[a][q].y;
-      for (int off = tpr; off < 32; off <<= 1) {
-        x += __shfl_xor_sync(0xffffffffu, x, off);
-        y += __shfl_xor_sync(0xffffffffu, y, off);
-      }
-      acc[a][q] = make_double2(x, y);
-    }
-  }
+      for (int q = 0; q < CPL; ++q) acc[a][q] = sum_lanes_pair(acc[a][q], lane, tpr);
   if (S == 1) {
     if (lrow == 0 && active_c) {
 #pragma unroll
@@ -397,7 +404,23 @@ __global__ void __launch_bounds__(kBdThreads, 2)
 // tree through shared memory.  The loads' latency bounds it: a warp per entry, one strided load at
 // a time, took 7 us (304 parts) to 80 us (9,728 parts).
 // With vscale (the basis kept unscaled, V_i = vscale[i][c] * Vu_i), h[i][c] is scaled by it.
-constexpr int kRhEntries = 8;
+// Up to kRhWarpEntries entries a warp alone takes each: one warp per SM then shares its FP64 unit with nobody.
+constexpr int kRhEntries = 8, kRhWarpEntries = 512;
+__global__ void __launch_bounds__(32) reduce_h_warp_kernel(const double2* __restrict__ part, int nparts, int n,
+                                                           double2* __restrict__ h,
+                                                           const double* __restrict__ vscale) {
+  const int t = blockIdx.x, lane = threadIdx.x;
+  const double sc = vscale ? vscale[t] : 1.0;
+  double2 s = make_double2(0.0, 0.0);
+#pragma unroll 8
+  for (int p = lane; p < nparts; p += 32) {
+    const double2 v = part[(int64_t)p * n + t];
+    s.x += v.x;
+    s.y += v.y;
+  }
+  s = sum_lanes_pair(s, lane, 1);
+  if (lane == 0) h[t] = make_double2(s.x * sc, s.y * sc);
+}
 __global__ void __launch_bounds__(256) reduce_h_kernel(const double2* __restrict__ part, int nparts, int nvec, int R,
                                                        double2* __restrict__ h, const double* __restrict__ vscale) {
   __shared__ double2 red[32][kRhEntries];
@@ -489,18 +512,7 @@ __global__ void __launch_bounds__(kThreads) cgs_update_kernel(const T* __restric
         }
     }
   }
-#pragma unroll
-  for (int q = 0; q < CPL; ++q) red[threadIdx.x * CPL + q] = nrm[q];
-  __syncthreads();
-  if ((int)threadIdx.x < tpr) {
-    for (int q = 0; q < CPL; ++q) {
-      const int c = c0 + q;
-      if (c >= R) continue;
-      double s = 0.0;
-      for (int r = 0; r < rows_per_block; ++r) s += red[(r * tpr + lc) * CPL + q];
-      npart[(int64_t)blockIdx.x * R + c] = s;
-    }
-  }
+  store_column_norms(nrm, red, tpr, c0, 1, R, npart + (int64_t)blockIdx.x * R);
 }
 
 // Streaming form of the update for 16 <= R <= 128 with 16-byte aligned vectors, on the tiles,
@@ -693,17 +705,7 @@ __global__ void __launch_bounds__(kThreads) colnorm2_kernel(const T* __restrict_
           const T v = x[row * R + c0 + q];
           nrm[q] += (double)v.x * v.x + (double)v.y * v.y;
         }
-#pragma unroll
-  for (int q = 0; q < CPL; ++q) red[threadIdx.x * CPL + q] = nrm[q];
-  __syncthreads();
-  if ((int)threadIdx.x < tpr)
-    for (int q = 0; q < CPL; ++q) {
-      const int c = c0 + q;
-      if (c >= R) continue;
-      double s = 0.0;
-      for (int r = 0; r < rows_per_block; ++r) s += red[(r * tpr + lc) * CPL + q];
-      npart[(int64_t)blockIdx.x * R + c] = s;
-    }
+  store_column_norms(nrm, red, tpr, c0, 1, R, npart + (int64_t)blockIdx.x * R);
 }
 
 // Sum of part[p][c] over the parts of one column by a block of kColThreads threads (thread t takes
@@ -736,103 +738,113 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 __device__ __forceinline__ double2 conjd(double2 a) { return make_double2(a.x, -a.y); }
 __device__ __forceinline__ double cabs2(double2 a) { return a.x * a.x + a.y * a.y; }
 
-// Adds a block's count of active columns (thread 0's `mine`) to state[0]; the launch's last block publishes the
-// total to the device word (read by the conditional graph nodes) and to the host's mapped word (read after
-// a synchronisation, no copy), and leaves the state zero for the next launch.
+// Adds a block's count of active columns (thread 0's `mine`) to *state, which also counts the blocks in its low
+// 16 bits, so one atomic tells the launch's last block the total (at most 128 columns and blocks).  That block
+// publishes it to the device word (read by the conditional graph nodes) and to the host's mapped word (read
+// after a synchronisation, no copy) and leaves the state zero for the next launch.
 __device__ __forceinline__ void publish_active(int mine, int32_t* state, int32_t* active, volatile int32_t* host) {
-  atomicAdd(&state[0], mine);
-  __threadfence();
-  if (atomicAdd(&state[1], 1) != (int)gridDim.x - 1) return;
-  const int total = atomicExch(&state[0], 0);
-  state[1] = 0;
+  const int32_t old = atomicAdd(state, (mine << 16) | 1);
+  if ((old & 0xffff) != (int)gridDim.x - 1) return;
+  const int total = (old >> 16) + mine;
+  *state = 0;
   *active = total;
   *host = total;
-  __threadfence_system();
 }
 
 // Hessenberg column j from h[0..j] and ||w||, previous rotations, new rotation, residual estimate
-// |g[j+1]| against the target.  One warp per column: the lanes sum the column's norm partials (fixed order: lane l takes parts
-// l, l + 32, ..., then an xor-shuffle tree) and stage the new Hessenberg column and the stored
-// rotations in shared memory; lane 0 applies the rotations (a sequential chain) and forms the
-// new one; the lanes write the column back.
-constexpr int kGivensWarps = 4;
-__global__ void __launch_bounds__(32 * kGivensWarps) givens_kernel(
+// |g[j+1]| against the target.  One warp per column and block, every operand loaded before anything waits.  An
+// FP64 instruction of a warp takes an SM 16 cycles, so columns do not share an SM, and the lanes take what is
+// not a chain: the previous rotations (c_i complex, s_i real: the subdiagonal entries are norms) give
+//   a_0 = h_0, a_{i+1} = conj(c_i) h_{i+1} - s_i a_i   (the only chain: one complex FMA by a real per step)
+//   H_i = c_i a_i + s_i h_{i+1}
+// and the square roots and quotients of ||w|| and of the new rotation run side by side in two lanes.  Four columns
+// to a block and one lane doing all of it took 15 us at 8 columns.
+__global__ void __launch_bounds__(32) givens_kernel(
     const double2* __restrict__ h, const double* __restrict__ npart, int nparts, int j, int m, int R,
     double2* __restrict__ H, double2* __restrict__ cs, double2* __restrict__ g, const double* __restrict__ target,
     int32_t* __restrict__ done, int32_t* __restrict__ kcol, double* __restrict__ scale, int32_t* __restrict__ state,
     int32_t* __restrict__ active, int32_t* __restrict__ host_active) {
-  __shared__ int go_on[kGivensWarps];
-  __shared__ double2 hs_all[kGivensWarps][64], rc_all[kGivensWarps][64], rs_all[kGivensWarps][64];
-  const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int c = blockIdx.x * kGivensWarps + wib;
-  const bool mine = c < R && !done[c];
-  if (lane == 0) {
-    go_on[wib] = 0;
-    if (c < R && !mine) scale[c] = 0.0;
+  __shared__ double2 hs[64], qs[64];
+  __shared__ double rs[64];
+  const int c = blockIdx.x, lane = threadIdx.x;
+  double2* gc = g + (int64_t)c * (m + 1);
+  double2* csc = cs + (int64_t)c * 2 * m;
+  const int was_done = done[c];
+  const double2 gj = gc[j];
+  const double goal = target[c];
+  double2 hv[2], cv[2];
+  double sv[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int i = lane + 32 * k;
+    hv[k] = i <= j ? h[i * R + c] : make_double2(0.0, 0.0);
+    cv[k] = i < j ? csc[2 * i] : make_double2(0.0, 0.0);
+    sv[k] = i < j ? csc[2 * i + 1].x : 0.0;
   }
-  if (mine) {
-    double2* hs = hs_all[wib];
-    double2* rc = rc_all[wib];
-    double2* rs = rs_all[wib];
-    double nn = 0.0;
+  double nn = 0.0;
 #pragma unroll 8
-    for (int p = lane; p < nparts; p += 32) nn += npart[(int64_t)p * R + c];
-    for (int off = 16; off > 0; off >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, off);
-    const double hn = sqrt(nn);
-    double2* Hc = H + ((int64_t)c * m + j) * (m + 1);
-    double2* csc = cs + (int64_t)c * 2 * m;
-    for (int i = lane; i <= j; i += 32) hs[i] = h[i * R + c];
-    for (int i = lane; i < j; i += 32) {
-      rc[i] = csc[2 * i];
-      rs[i] = csc[2 * i + 1];
-    }
-    __syncwarp();
+  for (int p = lane; p < nparts; p += 32) nn += npart[(int64_t)p * R + c];
+  if (was_done) {
     if (lane == 0) {
-      hs[j + 1] = make_double2(hn, 0.0);
-      for (int i = 0; i < j; ++i) {
-        const double2 ci = rc[i], si = rs[i];
-        const double2 a = hs[i], b = hs[i + 1];
-        hs[i] = cadd(cmul(ci, a), cmul(si, b));
-        hs[i + 1] = cadd(cmul(make_double2(-si.x, si.y), a), cmul(conjd(ci), b));  // -conj(s) a + conj(c) b
-      }
-      const double2 a = hs[j], b = hs[j + 1];
-      const double den = sqrt(cabs2(a) + cabs2(b));
-      double2 cj, sj;
-      if (den == 0.0) {
-        cj = make_double2(1.0, 0.0);
-        sj = make_double2(0.0, 0.0);
-      } else {
-        cj = make_double2(a.x / den, -a.y / den);   // conj(a)/den
-        sj = make_double2(b.x / den, -b.y / den);   // conj(b)/den
-      }
-      csc[2 * j] = cj;
-      csc[2 * j + 1] = sj;
-      hs[j] = make_double2(den, 0.0);
-      hs[j + 1] = make_double2(0.0, 0.0);
-      double2* gc = g + (int64_t)c * (m + 1);
-      const double2 gj = gc[j];
-      gc[j + 1] = cmul(make_double2(-sj.x, sj.y), gj);   // -conj(s) g_j
-      gc[j] = cmul(cj, gj);
-      const double res = sqrt(cabs2(gc[j + 1]));
-      const bool stop = (res <= target[c]) || (hn == 0.0) || (j + 1 >= m) || !(res == res);
-      kcol[c] = j + 1;
-      if (stop) {
-        done[c] = 1;
-        scale[c] = 0.0;
-      } else {
-        scale[c] = 1.0 / hn;
-        go_on[wib] = 1;
-      }
+      scale[c] = 0.0;
+      publish_active(0, state, active, host_active);
     }
-    __syncwarp();
-    for (int i = lane; i <= j + 1; i += 32) Hc[i] = hs[i];
+    return;
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int n = 0;
-    for (int w = 0; w < kGivensWarps; ++w) n += go_on[w];
-    publish_active(n, state, active, host_active);
+  for (int off = 16; off > 0; off >>= 1) nn += __shfl_xor_sync(0xffffffffu, nn, off);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    hs[lane + 32 * k] = hv[k];
+    rs[lane + 32 * k] = sv[k];
   }
+  __syncwarp();
+  double2 b[2];   // h_{i+1}
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int i = lane + 32 * k;
+    if (32 * k >= j) continue;
+    b[k] = i < j ? hs[i + 1] : make_double2(0.0, 0.0);
+    qs[i] = cmul(conjd(cv[k]), b[k]);
+  }
+  __syncwarp();
+  double2 a = hs[0], mine[2];
+  for (int i = 0; i < j; ++i) {
+    if (i == lane) mine[0] = a;
+    if (i == lane + 32) mine[1] = a;
+    const double2 q = qs[i];
+    const double si = rs[i];
+    a = make_double2(fma(-si, a.x, q.x), fma(-si, a.y, q.y));
+  }
+  double2* Hc = H + ((int64_t)c * m + j) * (m + 1);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int i = lane + 32 * k;
+    if (i < j) {
+      const double2 t = cmul(cv[k], mine[k]);
+      Hc[i] = make_double2(fma(sv[k], b[k].x, t.x), fma(sv[k], b[k].y, t.y));
+    }
+  }
+  // lane 0: ||w|| and its inverse; the others: the rotation's norm and its inverse
+  const double root = sqrt(lane == 0 ? nn : cabs2(a) + nn);
+  const double inv = root == 0.0 ? 0.0 : 1.0 / root;
+  const double hn = __shfl_sync(0xffffffffu, root, 0), den = __shfl_sync(0xffffffffu, root, 1);
+  const double iden = __shfl_sync(0xffffffffu, inv, 1);
+  if (lane != 0) return;
+  const double2 cj = den == 0.0 ? make_double2(1.0, 0.0) : make_double2(a.x * iden, -a.y * iden);   // conj(a)/den
+  const double sj = hn * iden;
+  csc[2 * j] = cj;
+  csc[2 * j + 1] = make_double2(sj, 0.0);
+  Hc[j] = make_double2(den, 0.0);
+  Hc[j + 1] = make_double2(0.0, 0.0);
+  const double2 gn = make_double2(-sj * gj.x, -sj * gj.y);
+  gc[j + 1] = gn;
+  gc[j] = cmul(cj, gj);
+  const double res = sqrt(cabs2(gn));
+  const bool stop = (res <= goal) || (hn == 0.0) || (j + 1 >= m) || !(res == res);
+  kcol[c] = j + 1;
+  scale[c] = stop ? 0.0 : inv;
+  if (stop) done[c] = 1;
+  publish_active(stop ? 0 : 1, state, active, host_active);
 }
 
 template <typename T>
@@ -911,7 +923,8 @@ __global__ void normalize_start32_kernel(const float2* __restrict__ r, const dou
 
 // Back substitution R y = g (R upper triangular after the rotations), one warp per column: the
 // triangle is brought to shared memory (packed by columns, 33 KB at 63 steps) with all lanes, then
-// column by column y_i = s_i / R_ii and the lanes subtract R_li y_i from s_l, l < i.  A thread per
+// column by column y_i = s_i / R_ii and the lanes subtract R_li y_i from s_l, l < i.  The inverses of the
+// diagonal are formed first, by all lanes: a quotient per step in the chain took 26 us at 12 steps.  A thread per
 // column waited for one H entry at a time: 9 us at 3 steps, 27 us at 12.
 __global__ void __launch_bounds__(32) hessenberg_solve_kernel(const double2* __restrict__ H,
                                                               const double2* __restrict__ g,
@@ -931,12 +944,15 @@ __global__ void __launch_bounds__(32) hessenberg_solve_kernel(const double2* __r
     for (int i = lane; i <= l; i += 32) tri[(l * (l + 1)) / 2 + i] = Hl[i];
   }
   __syncwarp();
+  for (int i = lane; i < k; i += 32) {
+    double2* d = tri + (i * (i + 1)) / 2 + i;
+    const double dd = cabs2(*d);
+    *d = dd > 0.0 ? make_double2(d->x / dd, -d->y / dd) : make_double2(0.0, 0.0);
+  }
+  __syncwarp();
   for (int i = k - 1; i >= 0; --i) {
     const double2* Ri = tri + (i * (i + 1)) / 2;
-    const double2 d = Ri[i], s = sv[i];
-    const double dd = cabs2(d);
-    const double2 yi = dd > 0.0 ? make_double2((s.x * d.x + s.y * d.y) / dd, (s.y * d.x - s.x * d.y) / dd)
-                                : make_double2(0.0, 0.0);
+    const double2 yi = cmul(sv[i], Ri[i]);
     if (lane == 0) yc[i] = yi;
     for (int l = lane; l < i; l += 32) {
       const double2 p = cmul(Ri[l], yi);
@@ -1329,7 +1345,10 @@ int cgs_dots_f32(const float2* V, int64_t vstride, int nvec, const float2* w, in
 void reduce_h(const double2* part, int nparts, int nvec, int R, double2* h, cudaStream_t s, const double* vscale) {
   note_launch(1);
   const int n = nvec * R;
-  reduce_h_kernel<<<(n + kRhEntries - 1) / kRhEntries, 256, 0, s>>>(part, nparts, nvec, R, h, vscale);
+  if (n <= kRhWarpEntries)
+    reduce_h_warp_kernel<<<n, 32, 0, s>>>(part, nparts, n, h, vscale);
+  else
+    reduce_h_kernel<<<(n + kRhEntries - 1) / kRhEntries, 256, 0, s>>>(part, nparts, nvec, R, h, vscale);
 }
 int cgs_update_f64(const double2* V, int64_t vstride, int nvec, const double2* h, double2* w, int64_t E, int R,
                    double* npart, cudaStream_t s, int32_t* err, int stages, const double* vscale) {
@@ -1365,7 +1384,7 @@ void givens_step(const double2* h, const double* npart, int nparts, int j, int m
                  double2* gvec, double* target, int32_t* done, int32_t* kcol, double* scale, int32_t* state,
                  int32_t* active, int32_t* host_active, cudaStream_t s) {
   note_launch(1);
-  givens_kernel<<<(R + kGivensWarps - 1) / kGivensWarps, 32 * kGivensWarps, 0, s>>>(
+  givens_kernel<<<R, 32, 0, s>>>(
       h, npart, nparts, j, m, R, H, cs, gvec, target, done, kcol, scale, state, active, host_active);
 }
 void scale_cols_f64(double2* v, const double* scale, int64_t E, int R, cudaStream_t s) {

@@ -6,6 +6,7 @@
 #include <type_traits>
 
 #include "mw_internal.h"
+#include "mw_reduce.cuh"
 
 namespace mwk {
 namespace {
@@ -207,18 +208,7 @@ __global__ void __launch_bounds__(256) residual_kernel(const int64_t* __restrict
         nrm[q] += r.x * r.x + r.y * r.y;
       }
   }
-#pragma unroll
-  for (int q = 0; q < CPL; ++q) red[threadIdx.x * CPL + q] = nrm[q];
-  __syncthreads();
-  if ((int)threadIdx.x < tpr) {
-    for (int q = 0; q < CPL; ++q) {
-      const int c = c0 + q;
-      if (c >= R) continue;
-      double s = 0.0;
-      for (int r = 0; r < rows_per_block; ++r) s += red[(r * tpr + lane_c) * CPL + q];
-      part[(int64_t)blockIdx.x * R + c] = s;
-    }
-  }
+  store_column_norms(nrm, red, tpr, c0, 1, R, part + (int64_t)blockIdx.x * R);
 }
 
 struct Shape {
@@ -563,18 +553,7 @@ __global__ void __launch_bounds__(256) residual_df_kernel(const int64_t* __restr
         nrm[q] += r.x * r.x + r.y * r.y;
       }
   }
-#pragma unroll
-  for (int q = 0; q < CPL; ++q) red[threadIdx.x * CPL + q] = nrm[q];
-  __syncthreads();
-  if ((int)threadIdx.x < tpr) {
-    for (int q = 0; q < CPL; ++q) {
-      const int c = c0 + q;
-      if (c >= R) continue;
-      double s = 0.0;
-      for (int r = 0; r < rows_per_block; ++r) s += red[(r * tpr + lane_c) * CPL + q];
-      part[(int64_t)blockIdx.x * R + c] = s;
-    }
-  }
+  store_column_norms(nrm, red, tpr, c0, 1, R, part + (int64_t)blockIdx.x * R);
 }
 
 // (b_h + b_l) - (y_h + y_l) rounded to FP32: the high parts' difference with its exact error
@@ -690,18 +669,7 @@ __global__ void __launch_bounds__(256) residual_df32_kernel(const int64_t* __res
       }
     }
   }
-#pragma unroll
-  for (int v = 0; v < CV; ++v) red[v * 256 + threadIdx.x] = nrm[v];
-  __syncthreads();
-  if ((int)threadIdx.x < tpr) {
-    for (int v = 0; v < CV; ++v) {
-      const int c = lane_c + v * span;
-      if (c >= R) continue;
-      double sum = 0.0;
-      for (int r = 0; r < groups; ++r) sum += red[v * 256 + r * tpr + lane_c];
-      part[(int64_t)blockIdx.x * R + c] = sum;
-    }
-  }
+  store_column_norms(nrm, red, tpr, lane_c, span, R, part + (int64_t)blockIdx.x * R);
 }
 
 }  // namespace

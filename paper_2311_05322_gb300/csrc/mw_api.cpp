@@ -123,7 +123,7 @@ struct Work {
   double2 *r = nullptr, *x = nullptr, *part = nullptr, *h = nullptr, *H = nullptr, *cs = nullptr, *g = nullptr,
           *y = nullptr, *bblk = nullptr;
   double *npart = nullptr, *target = nullptr, *rnorm = nullptr, *bnorm = nullptr, *scale = nullptr;
-  int32_t *done = nullptr, *kcol = nullptr, *active = nullptr;   // active: [0] columns still active, [1..2] its counting
+  int32_t *done = nullptr, *kcol = nullptr, *active = nullptr;   // active: [0] columns still active, [1] its counting
   double* h_vec = nullptr;      // pinned [R]
   int32_t* h_ivec = nullptr;    // pinned [R]
   void* tc_scratch = nullptr;   // BF16 gathered operand
@@ -460,8 +460,8 @@ void ensure_work(Ctx* c, int R, int m, int prec) {
   w.scale = dalloc<double>(c, R);
   w.done = dalloc<int32_t>(c, R);
   w.kcol = dalloc<int32_t>(c, R);
-  w.active = dalloc<int32_t>(c, 3);
-  CK(cudaMemsetAsync(w.active, 0, 3 * sizeof(int32_t), c->stream));
+  w.active = dalloc<int32_t>(c, 2);
+  CK(cudaMemsetAsync(w.active, 0, 2 * sizeof(int32_t), c->stream));
   CK(cudaMallocHost(&w.h_vec, sizeof(double) * R));
   CK(cudaMallocHost(&w.h_ivec, sizeof(int32_t) * R));
 }
