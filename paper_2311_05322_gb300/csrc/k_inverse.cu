@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "k_inverse.h"
+#include "mw_chain.cuh"
 #include "mw_internal.h"
 
 namespace mwk {
@@ -199,6 +200,7 @@ constexpr int NB = kInvBlock;
 template <typename T>
 __global__ void __launch_bounds__(256) inv_diag_kernel(InvBatch bt, const T* __restrict__ ws, int kb,
                                                        T* __restrict__ Dinv, int32_t* __restrict__ status) {
+  chain_wait();
   using Sc = typename Tr<T>::S;
   constexpr int R = NB / 16;
   __shared__ T row[2][NB], col[2][NB];
@@ -289,6 +291,7 @@ constexpr int kPan = 64;
 template <typename T>
 __global__ void __launch_bounds__(256) inv_panel_kernel(InvBatch bt, OrasTopo tp, T* __restrict__ ws, int kb, int jt,
                                                         const T* __restrict__ Dinv, const int32_t* __restrict__ nsws) {
+  chain_wait();
   extern __shared__ unsigned char smem_raw[];
   T* Ps = reinterpret_cast<T*>(smem_raw);           // [q][64 + 1]
   T* Ds = Ps + NB * (kPan + 1);                     // [NB][NB]
@@ -396,6 +399,7 @@ template <typename T>
 __global__ void __launch_bounds__(128, sizeof(T) == 8 ? kUpBlocks : 1) inv_update_kernel(
     InvBatch bt, OrasTopo tp, T* __restrict__ ws, int kb, const int32_t* __restrict__ nsws,
     const int32_t* __restrict__ prefix, int n_tiles) {
+  chain_wait();
   constexpr int VEC = 16 / (int)sizeof(T);          // elements per 16-byte copy
   constexpr int CC = kUp / VEC;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -538,13 +542,13 @@ void invert_all(const InvBatch& bt, const OrasTopo& tp, T* ws, T* dinv, int32_t*
     const int kb = k * NB, jt = (bt.np_max + kPan - 1) / kPan;
     const int32_t* nsws = bt.d_nsw + (size_t)k * bt.count;
     note_launch(2);
-    inv_diag_kernel<T><<<bt.count, 256, 0, st>>>(bt, ws, kb, dinv, status);
-    inv_panel_kernel<T><<<dim3(2 * jt, bt.count), 256, pa_smem, st>>>(bt, tp, ws, kb, jt, dinv, nsws);
+    launch_chained(inv_diag_kernel<T>, bt.count, 256, 0, st, bt, ws, kb, dinv, status);
+    launch_chained(inv_panel_kernel<T>, dim3(2 * jt, bt.count), 256, pa_smem, st, bt, tp, ws, kb, jt, dinv, nsws);
     if (bt.h_tiles[k] == 0) continue;
     note_launch(1);
     constexpr int blocks = 152 * (sizeof(T) == 8 ? kUpBlocks : 1);
-    inv_update_kernel<T><<<std::min(bt.h_tiles[k], blocks), 128, up_smem, st>>>(
-        bt, tp, ws, kb, nsws, bt.d_prefix + (size_t)k * (bt.count + 1), bt.h_tiles[k]);
+    launch_chained(inv_update_kernel<T>, std::min(bt.h_tiles[k], blocks), 128, up_smem, st, bt, tp, ws, kb, nsws,
+        bt.d_prefix + (size_t)k * (bt.count + 1), bt.h_tiles[k]);
   }
 }
 

@@ -17,6 +17,7 @@
 #include <cstdint>
 
 #include "mw_async.cuh"
+#include "mw_chain.cuh"
 #include "mw_internal.h"
 #include "mw_reduce.cuh"
 
@@ -83,6 +84,7 @@ template <typename T, int CPL>
 __global__ void __launch_bounds__(kDotThreads) cgs_dots_kernel(const T* __restrict__ V, int64_t vstride, int nvec,
                                                             const T* __restrict__ w, int64_t E, int R, int tpr_log2,
                                                             int S, double2* __restrict__ part) {
+  chain_wait();
   using Sc = typename Traits<T>::S;
   // rows in flight per thread: the same bytes per thread for every CPL and precision
   constexpr int kUnroll = (16 / CPL) / (sizeof(T) / 8) > 0 ? (16 / CPL) / (sizeof(T) / 8) : 1;
@@ -231,6 +233,7 @@ template <typename T>
 __global__ void __launch_bounds__(kBdThreads, 2)
     cgs_dots_bulk_kernel(const T* __restrict__ V, int64_t vstride, int nvec, const T* __restrict__ w, int64_t E,
                          int R, int G, int VG, int NS, double2* __restrict__ part, int32_t* __restrict__ err) {
+  chain_wait();
   using Sc = typename Traits<T>::S;
   constexpr int RPT = bd_rows<T>();
   constexpr int kStageElems = kBdStageBytes / (int)sizeof(T);
@@ -409,6 +412,7 @@ constexpr int kRhEntries = 8, kRhWarpEntries = 512;
 __global__ void __launch_bounds__(32) reduce_h_warp_kernel(const double2* __restrict__ part, int nparts, int n,
                                                            double2* __restrict__ h,
                                                            const double* __restrict__ vscale) {
+  chain_wait();
   const int t = blockIdx.x, lane = threadIdx.x;
   const double sc = vscale ? vscale[t] : 1.0;
   double2 s = make_double2(0.0, 0.0);
@@ -423,6 +427,7 @@ __global__ void __launch_bounds__(32) reduce_h_warp_kernel(const double2* __rest
 }
 __global__ void __launch_bounds__(256) reduce_h_kernel(const double2* __restrict__ part, int nparts, int nvec, int R,
                                                        double2* __restrict__ h, const double* __restrict__ vscale) {
+  chain_wait();
   __shared__ double2 red[32][kRhEntries];
   const int e = threadIdx.x % kRhEntries, lane = threadIdx.x / kRhEntries;
   const int n = nvec * R;
@@ -467,6 +472,7 @@ __global__ void __launch_bounds__(kThreads) cgs_update_kernel(const T* __restric
                                                               int64_t E, int R, int tpr_log2,
                                                               double* __restrict__ npart,
                                                               const double* __restrict__ vscale) {
+  chain_wait();
   using Sc = typename Traits<T>::S;
   extern __shared__ unsigned char smem_raw[];
   T* hs = reinterpret_cast<T*>(smem_raw);                          // [nvec][R]
@@ -528,6 +534,7 @@ __global__ void __launch_bounds__(kBdThreads, 2)
     cgs_update_bulk_kernel(const T* __restrict__ V, int64_t vstride, int nvec, const double2* __restrict__ h,
                            T* __restrict__ w, int64_t E, int R, int G, int NS, double* __restrict__ npart,
                            int32_t* __restrict__ err, const double* __restrict__ vscale) {
+  chain_wait();
   using Sc = typename Traits<T>::S;
   constexpr int RPT = bd_rows<T>();
   constexpr int kStageElems = kBdStageBytes / (int)sizeof(T);
@@ -688,6 +695,7 @@ inline size_t bu_smem_bytes(int R, int nvec, int NS) {
 template <typename T, int CPL>
 __global__ void __launch_bounds__(kThreads) colnorm2_kernel(const T* __restrict__ x, int64_t E, int R, int tpr_log2,
                                                             double* __restrict__ npart) {
+  chain_wait();
   __shared__ double red[kThreads * CPL];
   const int tpr = 1 << tpr_log2;
   const int rows_per_block = kThreads >> tpr_log2;
@@ -728,6 +736,7 @@ __device__ __forceinline__ double sum_column_parts(const double* __restrict__ pa
 
 __global__ void __launch_bounds__(kColThreads) reduce_cols_kernel(const double* __restrict__ part, int nparts, int R,
                                                                   double* __restrict__ out) {
+  chain_wait();
   const double s = sum_column_parts(part, nparts, R, blockIdx.x);
   if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
@@ -764,6 +773,7 @@ __global__ void __launch_bounds__(32) givens_kernel(
     double2* __restrict__ H, double2* __restrict__ cs, double2* __restrict__ g, const double* __restrict__ target,
     int32_t* __restrict__ done, int32_t* __restrict__ kcol, double* __restrict__ scale, int32_t* __restrict__ state,
     int32_t* __restrict__ active, int32_t* __restrict__ host_active) {
+  chain_wait();
   __shared__ double2 hs[64], qs[64];
   __shared__ double rs[64];
   const int c = blockIdx.x, lane = threadIdx.x;
@@ -849,6 +859,7 @@ __global__ void __launch_bounds__(32) givens_kernel(
 
 template <typename T>
 __global__ void scale_cols_kernel(T* __restrict__ v, const double* __restrict__ sc, int64_t E, int R) {
+  chain_wait();
   using Sc = typename Traits<T>::S;
   const int64_t n = E * R;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -867,6 +878,7 @@ __global__ void __launch_bounds__(kColThreads) start_state_kernel(
     double inner_tol, int fp64_mode, double* __restrict__ rnorm, double2* __restrict__ g, double* __restrict__ target,
     int32_t* __restrict__ done, int32_t* __restrict__ kcol, int m, int32_t* __restrict__ state,
     int32_t* __restrict__ active, int32_t* __restrict__ host_active) {
+  chain_wait();
   const int c = blockIdx.x;
   const double rn = sqrt(sum_column_parts(npart, nparts, R, c));
   double2* gc = g + (int64_t)c * (m + 1);
@@ -886,6 +898,7 @@ __global__ void __launch_bounds__(kColThreads) start_state_kernel(
 template <typename T>
 __global__ void normalize_start_kernel(const double2* __restrict__ r, const double* __restrict__ rnorm,
                                        const int32_t* __restrict__ done, int64_t E, int R, T* __restrict__ v0) {
+  chain_wait();
   using Sc = typename Traits<T>::S;
   const int64_t n = E * R;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -902,6 +915,7 @@ __global__ void normalize_start_kernel(const double2* __restrict__ r, const doub
 __global__ void normalize_start32_kernel(const float2* __restrict__ r, const double* __restrict__ rnorm,
                                          const int32_t* __restrict__ done, int64_t E, int R, float2* __restrict__ v0,
                                          double* __restrict__ vscale) {
+  chain_wait();
   extern __shared__ float sc[];
   if (vscale && blockIdx.x == 0)
     for (int c = threadIdx.x; c < R; c += blockDim.x) vscale[c] = 1.0;
@@ -930,6 +944,7 @@ __global__ void __launch_bounds__(32) hessenberg_solve_kernel(const double2* __r
                                                               const double2* __restrict__ g,
                                                               const int32_t* __restrict__ kcol, int m, int R,
                                                               double2* __restrict__ y) {
+  chain_wait();
   extern __shared__ double2 tri[];                  // [k (k + 1) / 2] triangle, then [k] right-hand side
   const int c = blockIdx.x, lane = threadIdx.x;
   const int k = kcol[c];
@@ -967,6 +982,7 @@ __global__ void __launch_bounds__(32) hessenberg_solve_kernel(const double2* __r
 template <typename T>
 __global__ void update_x_kernel(const T* __restrict__ Z, int64_t zstride, const double2* __restrict__ y,
                                 const int32_t* __restrict__ kcol, int m, double2* __restrict__ x, int64_t E, int R) {
+  chain_wait();
   using Sc = typename Traits<T>::S;
   const int64_t n = E * R;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -993,6 +1009,7 @@ __global__ void update_x_kernel(const T* __restrict__ Z, int64_t zstride, const 
 // the correction is formed in FP32 from the widened values and added to x in FP64.
 __global__ void update_x_bx_kernel(const uint32_t* __restrict__ Z, int64_t zstride, const double2* __restrict__ y,
                                    const int32_t* __restrict__ kcol, int m, double2* __restrict__ x, int64_t E, int R) {
+  chain_wait();
   const int64_t n = E * R;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const int c = (int)(i % R);
@@ -1036,6 +1053,7 @@ __global__ void __launch_bounds__(kBdThreads, 2)
     update_x_bulk_kernel(const ZT* __restrict__ Z, int64_t zstride, const double2* __restrict__ y,
                          const int32_t* __restrict__ kcol, int m, double2* __restrict__ x, int64_t E, int R, int G,
                          int NS, int32_t* __restrict__ err) {
+  chain_wait();
   using Sc = typename Traits<T>::S;
   constexpr int RPT = bd_rows<T>();
   constexpr int kStageElems = kBdStageBytes / (int)sizeof(ZT);
@@ -1190,8 +1208,8 @@ bool update_x_bulk(const ZT* Z, int64_t zstride, const double2* y, const int32_t
   }
   int NS = kBdStages;
   while (NS > 2 && ux_smem_bytes(R, m, NS) > (size_t)226 * 1024) --NS;
-  update_x_bulk_kernel<T, ZT><<<152 * 2, kBdThreads, ux_smem_bytes(R, m, NS), s>>>(Z, zstride, y, kcol, m, x, E, R,
-                                                                                  kBdConsumers / R, NS, err);
+  launch_chained(update_x_bulk_kernel<T, ZT>, 152 * 2, kBdThreads, ux_smem_bytes(R, m, NS), s, Z, zstride, y,
+      kcol, m, x, E, R, kBdConsumers / R, NS, err);
   return true;
 }
 
@@ -1218,8 +1236,8 @@ int dots_launch(const T* V, int64_t vstride, int nvec, const T* w, int64_t E, in
     const int VG = std::min(64, 2048 / R);
     const int nb = 152 * 2;
     const int NS = stages >= 2 && stages <= kBdMaxStages ? stages : kBdStages;
-    cgs_dots_bulk_kernel<T>
-        <<<nb, kBdThreads, bd_smem_bytes(R, NS, sizeof(T)), s>>>(V, vstride, nvec, w, E, R, G, VG, NS, part, err);
+    launch_chained(cgs_dots_bulk_kernel<T>, nb, kBdThreads, bd_smem_bytes(R, NS, sizeof(T)), s, V, vstride, nvec,
+        w, E, R, G, VG, NS, part, err);
     return nb;
   }
   Shape sh = shape_for(R);
@@ -1230,13 +1248,16 @@ int dots_launch(const T* V, int64_t vstride, int nvec, const T* w, int64_t E, in
   const int nb = (int)std::min<int64_t>(kBlocks, (E + chunk - 1) / chunk);
   switch (sh.cpl) {
     case 1:
-      cgs_dots_kernel<T, 1><<<nb, kDotThreads, 0, s>>>(V, vstride, nvec, w, E, R, sh.tpr_log2, S, part);
+      launch_chained(cgs_dots_kernel<T, 1>, nb, kDotThreads, 0, s, V, vstride, nvec, w, E, R, sh.tpr_log2, S,
+          part);
       break;
     case 2:
-      cgs_dots_kernel<T, 2><<<nb, kDotThreads, 0, s>>>(V, vstride, nvec, w, E, R, sh.tpr_log2, S, part);
+      launch_chained(cgs_dots_kernel<T, 2>, nb, kDotThreads, 0, s, V, vstride, nvec, w, E, R, sh.tpr_log2, S,
+          part);
       break;
     default:
-      cgs_dots_kernel<T, 4><<<nb, kDotThreads, 0, s>>>(V, vstride, nvec, w, E, R, sh.tpr_log2, S, part);
+      launch_chained(cgs_dots_kernel<T, 4>, nb, kDotThreads, 0, s, V, vstride, nvec, w, E, R, sh.tpr_log2, S,
+          part);
       break;
   }
   return nb;
@@ -1259,8 +1280,8 @@ int update_launch(const T* V, int64_t vstride, int nvec, const double2* h, T* w,
     while (NS > 2 && bu_smem_bytes(R, nvec, NS) > (size_t)226 * 1024) --NS;
     const int G = kBdConsumers / R;
     const int nb = 152 * 2;
-    cgs_update_bulk_kernel<T>
-        <<<nb, kBdThreads, bu_smem_bytes(R, nvec, NS), s>>>(V, vstride, nvec, h, w, E, R, G, NS, npart, err, vscale);
+    launch_chained(cgs_update_bulk_kernel<T>, nb, kBdThreads, bu_smem_bytes(R, nvec, NS), s, V, vstride, nvec, h,
+        w, E, R, G, NS, npart, err, vscale);
     return nb;
   }
   Shape sh = shape_for(R);
@@ -1277,16 +1298,16 @@ int update_launch(const T* V, int64_t vstride, int nvec, const double2* h, T* w,
   const int nb = (int)std::min<int64_t>(kBlocks, (E + rows_per_block - 1) / rows_per_block);
   switch (sh.cpl) {
     case 1:
-      cgs_update_kernel<T, 1>
-          <<<nb, kThreads, smem, s>>>(V, vstride, nvec, h, w, E, R, sh.tpr_log2, npart, vscale);
+      launch_chained(cgs_update_kernel<T, 1>, nb, kThreads, smem, s, V, vstride, nvec, h, w, E, R, sh.tpr_log2,
+          npart, vscale);
       break;
     case 2:
-      cgs_update_kernel<T, 2>
-          <<<nb, kThreads, smem, s>>>(V, vstride, nvec, h, w, E, R, sh.tpr_log2, npart, vscale);
+      launch_chained(cgs_update_kernel<T, 2>, nb, kThreads, smem, s, V, vstride, nvec, h, w, E, R, sh.tpr_log2,
+          npart, vscale);
       break;
     default:
-      cgs_update_kernel<T, 4>
-          <<<nb, kThreads, smem, s>>>(V, vstride, nvec, h, w, E, R, sh.tpr_log2, npart, vscale);
+      launch_chained(cgs_update_kernel<T, 4>, nb, kThreads, smem, s, V, vstride, nvec, h, w, E, R, sh.tpr_log2,
+          npart, vscale);
       break;
   }
   return nb;
@@ -1346,9 +1367,10 @@ void reduce_h(const double2* part, int nparts, int nvec, int R, double2* h, cuda
   note_launch(1);
   const int n = nvec * R;
   if (n <= kRhWarpEntries)
-    reduce_h_warp_kernel<<<n, 32, 0, s>>>(part, nparts, n, h, vscale);
+    launch_chained(reduce_h_warp_kernel, n, 32, 0, s, part, nparts, n, h, vscale);
   else
-    reduce_h_kernel<<<(n + kRhEntries - 1) / kRhEntries, 256, 0, s>>>(part, nparts, nvec, R, h, vscale);
+    launch_chained(reduce_h_kernel, (n + kRhEntries - 1) / kRhEntries, 256, 0, s, part, nparts, nvec, R, h,
+        vscale);
 }
 int cgs_update_f64(const double2* V, int64_t vstride, int nvec, const double2* h, double2* w, int64_t E, int R,
                    double* npart, cudaStream_t s, int32_t* err, int stages, const double* vscale) {
@@ -1365,81 +1387,83 @@ int colnorm2_f64(const double2* x, int64_t E, int R, double* npart, cudaStream_t
   const int nb = (int)std::min<int64_t>(kBlocks, (E + rows_per_block - 1) / rows_per_block);
   switch (sh.cpl) {
     case 1:
-      colnorm2_kernel<double2, 1><<<nb, kThreads, 0, s>>>(x, E, R, sh.tpr_log2, npart);
+      launch_chained(colnorm2_kernel<double2, 1>, nb, kThreads, 0, s, x, E, R, sh.tpr_log2, npart);
       break;
     case 2:
-      colnorm2_kernel<double2, 2><<<nb, kThreads, 0, s>>>(x, E, R, sh.tpr_log2, npart);
+      launch_chained(colnorm2_kernel<double2, 2>, nb, kThreads, 0, s, x, E, R, sh.tpr_log2, npart);
       break;
     default:
-      colnorm2_kernel<double2, 4><<<nb, kThreads, 0, s>>>(x, E, R, sh.tpr_log2, npart);
+      launch_chained(colnorm2_kernel<double2, 4>, nb, kThreads, 0, s, x, E, R, sh.tpr_log2, npart);
       break;
   }
   return nb;
 }
 void reduce_cols(const double* part, int nparts, int R, double* out, cudaStream_t s) {
   note_launch(1);
-  reduce_cols_kernel<<<R, kColThreads, 0, s>>>(part, nparts, R, out);
+  launch_chained(reduce_cols_kernel, R, kColThreads, 0, s, part, nparts, R, out);
 }
 void givens_step(const double2* h, const double* npart, int nparts, int j, int m, int R, double2* H, double2* cs,
                  double2* gvec, double* target, int32_t* done, int32_t* kcol, double* scale, int32_t* state,
                  int32_t* active, int32_t* host_active, cudaStream_t s) {
   note_launch(1);
-  givens_kernel<<<R, 32, 0, s>>>(
-      h, npart, nparts, j, m, R, H, cs, gvec, target, done, kcol, scale, state, active, host_active);
+  launch_chained(givens_kernel, R, 32, 0, s, h, npart, nparts, j, m, R, H, cs, gvec, target, done, kcol, scale,
+      state, active, host_active);
 }
 void scale_cols_f64(double2* v, const double* scale, int64_t E, int R, cudaStream_t s) {
   note_launch(1);
-  scale_cols_kernel<double2><<<gs_blocks(E * R), 256, 0, s>>>(v, scale, E, R);
+  launch_chained(scale_cols_kernel<double2>, gs_blocks(E * R), 256, 0, s, v, scale, E, R);
 }
 void scale_cols_f32(float2* v, const double* scale, int64_t E, int R, cudaStream_t s) {
   note_launch(1);
-  scale_cols_kernel<float2><<<gs_blocks(E * R), 256, 0, s>>>(v, scale, E, R);
+  launch_chained(scale_cols_kernel<float2>, gs_blocks(E * R), 256, 0, s, v, scale, E, R);
 }
 void start_state(const double* npart, int nparts, int R, const double* bnorm, double tol, double inner_tol,
                  int fp64_mode, double* rnorm, double2* gvec, double* target, int32_t* done, int32_t* kcol, int m,
                  int32_t* state, int32_t* active, int32_t* host_active, cudaStream_t s) {
   note_launch(1);
-  start_state_kernel<<<R, kColThreads, 0, s>>>(npart, nparts, R, bnorm, tol, inner_tol, fp64_mode, rnorm, gvec, target,
-                                               done, kcol, m, state, active, host_active);
+  launch_chained(start_state_kernel, R, kColThreads, 0, s, npart, nparts, R, bnorm, tol, inner_tol, fp64_mode,
+      rnorm, gvec, target, done, kcol, m, state, active, host_active);
 }
 void normalize_start_f64(const double2* r, const double* rnorm, const int32_t* done, int64_t E, int R, double2* v0,
                          cudaStream_t s) {
   note_launch(1);
-  normalize_start_kernel<double2><<<gs_blocks(E * R), 256, 0, s>>>(r, rnorm, done, E, R, v0);
+  launch_chained(normalize_start_kernel<double2>, gs_blocks(E * R), 256, 0, s, r, rnorm, done, E, R, v0);
 }
 void normalize_start_f32(const double2* r, const double* rnorm, const int32_t* done, int64_t E, int R, float2* v0,
                          cudaStream_t s) {
   note_launch(1);
-  normalize_start_kernel<float2><<<gs_blocks(E * R), 256, 0, s>>>(r, rnorm, done, E, R, v0);
+  launch_chained(normalize_start_kernel<float2>, gs_blocks(E * R), 256, 0, s, r, rnorm, done, E, R, v0);
 }
 void normalize_start32(const float2* r, const double* rnorm, const int32_t* done, int64_t E, int R, float2* v0,
                        double* vscale, cudaStream_t s) {
   note_launch(1);
-  normalize_start32_kernel<<<gs_blocks(E * R), 256, sizeof(float) * R, s>>>(r, rnorm, done, E, R, v0, vscale);
+  launch_chained(normalize_start32_kernel, gs_blocks(E * R), 256, sizeof(float) * R, s, r, rnorm, done, E, R, v0,
+      vscale);
 }
 void solve_hessenberg(const double2* H, const double2* gvec, const int32_t* kcol, int m, int R, double2* y,
                       cudaStream_t s) {
   note_launch(1);
   const size_t smem = sizeof(double2) * (m * (m + 1) / 2 + m);   // 33 KB at the largest m = 63
-  hessenberg_solve_kernel<<<R, 32, smem, s>>>(H, gvec, kcol, m, R, y);
+  launch_chained(hessenberg_solve_kernel, R, 32, smem, s, H, gvec, kcol, m, R, y);
 }
 void update_x_f64(const double2* Z, int64_t zstride, const double2* y, const int32_t* kcol, int m, double2* x,
                   int64_t E, int R, cudaStream_t s, int32_t* err) {
   note_launch(1);
   if (update_x_bulk<double2>(Z, zstride, y, kcol, m, x, E, R, err, s)) return;
-  update_x_kernel<double2><<<gs_blocks(E * R), 256, 0, s>>>(Z, zstride, y, kcol, m, x, E, R);
+  launch_chained(update_x_kernel<double2>, gs_blocks(E * R), 256, 0, s, Z, zstride, y, kcol, m, x, E, R);
 }
 void update_x_bx(const void* Z, int64_t zstride, const double2* y, const int32_t* kcol, int m, double2* x, int64_t E,
                  int R, cudaStream_t s, int32_t* err) {
   note_launch(1);
   if (update_x_bulk<float2, uint32_t>((const uint32_t*)Z, zstride, y, kcol, m, x, E, R, err, s)) return;
-  update_x_bx_kernel<<<gs_blocks(E * R), 256, 0, s>>>((const uint32_t*)Z, zstride, y, kcol, m, x, E, R);
+  launch_chained(update_x_bx_kernel, gs_blocks(E * R), 256, 0, s, (const uint32_t*)Z, zstride, y, kcol, m, x, E,
+      R);
 }
 void update_x_f32(const float2* Z, int64_t zstride, const double2* y, const int32_t* kcol, int m, double2* x,
                   int64_t E, int R, cudaStream_t s, int32_t* err) {
   note_launch(1);
   if (update_x_bulk<float2>(Z, zstride, y, kcol, m, x, E, R, err, s)) return;
-  update_x_kernel<float2><<<gs_blocks(E * R), 256, 0, s>>>(Z, zstride, y, kcol, m, x, E, R);
+  launch_chained(update_x_kernel<float2>, gs_blocks(E * R), 256, 0, s, Z, zstride, y, kcol, m, x, E, R);
 }
 
 }  // namespace mwk

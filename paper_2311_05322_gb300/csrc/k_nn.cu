@@ -9,6 +9,7 @@
 #include <algorithm>
 
 #include "k_nn.h"
+#include "mw_chain.cuh"
 #include "mw_internal.h"
 
 namespace mwk {
@@ -103,6 +104,7 @@ struct TileIo {
 template <typename TB, bool AK, bool BK, int TM, int TN, int RM, int RN>
 __global__ void __launch_bounds__((TM / RM) * (TN / RN)) gemm_kernel(const float* __restrict__ A,
                                                                      const TB* __restrict__ B, GemmArgs g) {
+  chain_wait();
   constexpr int NT = (TM / RM) * (TN / RN);
   __shared__ __align__(16) float As[2][TK * TM];
   __shared__ __align__(16) float Bs[2][TK * TN];
@@ -179,6 +181,7 @@ __global__ void __launch_bounds__((TM / RM) * (TN / RN)) gemm_kernel(const float
 
 // C = sum_z P[z] (z ascending), then the epilogue of gemm_kernel.
 __global__ void gemm_reduce_kernel(const float* __restrict__ P, int nz, GemmArgs g) {
+  chain_wait();
   const int64_t MN = (int64_t)g.M * g.N;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < MN; i += (int64_t)gridDim.x * blockDim.x) {
     float v = 0.f;
@@ -210,6 +213,7 @@ __global__ void __launch_bounds__(kConvThreads) convT_fwd_kernel(const float* __
                                                                  const float* __restrict__ w,
                                                                  const float* __restrict__ bias,
                                                                  float* __restrict__ y, int B) {
+  chain_wait();
   constexpr int COG = kConvCog, DD = 2 * D;
   __shared__ float4 sw[CI * COG * 16];              // [ci][co][kz][ky] of kx quadruples
   const int co0 = blockIdx.y * COG;
@@ -316,6 +320,7 @@ __global__ void __launch_bounds__(kConvThreads) convT_bwd_data_kernel(const floa
                                                                       const float* __restrict__ w,
                                                                       const float* __restrict__ act,
                                                                       float* __restrict__ dx, int B) {
+  chain_wait();
   constexpr int DD = 2 * D;
   __shared__ float4 sw[CO * CIG * 16];              // [co][ci][kz][ky] of kx quadruples
   const int ci0 = blockIdx.y * CIG;
@@ -405,6 +410,7 @@ __global__ void __launch_bounds__(kBwdWThreads) convT_bwd_w_kernel(const float* 
                                                                    float* __restrict__ part,
                                                                    float* __restrict__ bpart, int B, int64_t chunk,
                                                                    int nchunk) {
+  chain_wait();
   extern __shared__ float red[];                    // [256][65]
   constexpr int DD = 2 * D, V = D * D * D, PB = CI / kBwdWCi * CO * 4;
   if ((int)blockIdx.x >= PB * nchunk) {
@@ -498,6 +504,7 @@ struct FinalSums {
   int nseg;
 };
 __global__ void __launch_bounds__(128) nn_final_sums_kernel(FinalSums f) {
+  chain_wait();
   int q = blockIdx.x * 128 + threadIdx.x;
   for (int k = 0; k < f.nseg; ++k) {
     const FinalSeg& g = f.seg[k];
@@ -523,6 +530,7 @@ constexpr int kMseChunk = 4096;
 __global__ void __launch_bounds__(256) mse_kernel(const float* __restrict__ y, const float* __restrict__ t,
                                                   const int32_t* __restrict__ idx, int64_t width, float sc,
                                                   float* __restrict__ dy, double* __restrict__ part) {
+  chain_wait();
   __shared__ double red[256];
   const int64_t b = blockIdx.y, o = (int64_t)blockIdx.x * kMseChunk + threadIdx.x * 4;
   const float* yb = y + b * width + o;
@@ -552,6 +560,7 @@ __global__ void __launch_bounds__(256) mse_kernel(const float* __restrict__ y, c
 }
 
 __global__ void sum_parts_kernel(const double* __restrict__ part, int n, double scale, double* __restrict__ out) {
+  chain_wait();
   __shared__ double red[256];
   double s = 0.0;
 #pragma unroll 8
@@ -588,6 +597,7 @@ __global__ void __launch_bounds__(256) adam_kernel(float* __restrict__ th, const
                                                    float* __restrict__ m, float* __restrict__ v,
                                                    __nv_bfloat16* __restrict__ w1, __nv_bfloat16* __restrict__ w2,
                                                    AdamArgs a) {
+  chain_wait();
   const int64_t i = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4;
   if (i + 4 > a.n) {                                // the last, incomplete quadruple (all biases)
     for (int64_t k = i; k < a.n; ++k) adam_update(th[k], g[k], m[k], v[k], a);
@@ -610,6 +620,7 @@ __global__ void __launch_bounds__(256) adam_kernel(float* __restrict__ th, const
 }
 
 __global__ void to_bf16_kernel(const float* __restrict__ a, __nv_bfloat16* __restrict__ b, int64_t n) {
+  chain_wait();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     b[i] = __float2bfloat16_rn(a[i]);
 }
@@ -617,6 +628,7 @@ __global__ void to_bf16_kernel(const float* __restrict__ a, __nv_bfloat16* __res
 // dst[r] = src[idx[r]], rows of `width` floats (blockIdx.y = r).
 __global__ void gather_rows_kernel(const float* __restrict__ src, const int32_t* __restrict__ idx, int64_t width,
                                    float* __restrict__ dst) {
+  chain_wait();
   const float* p = src + (int64_t)idx[blockIdx.y] * width;
   float* q = dst + (int64_t)blockIdx.y * width;
   for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < width; c += (int64_t)gridDim.x * blockDim.x)
@@ -630,6 +642,7 @@ __global__ void gather_rows_kernel(const float* __restrict__ src, const int32_t*
 __global__ void grid_to_tets_kernel(const float* __restrict__ grid, int G, double lx, double ly, double lz, double hx,
                                     double hy, double hz, const double* __restrict__ xyz,
                                     const int32_t* __restrict__ tets, int64_t T, double* __restrict__ out) {
+  chain_wait();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= T) return;
   double v[4][3];
@@ -695,10 +708,10 @@ static void gemm_launch(const float* A, const TB* B, GemmArgs g, float* ws, size
   g.vc = al(z > 1 ? ws : g.C, g.N, 4);
   note_launch(z > 1 ? 2 : 1);
   const dim3 grid((g.N + TN - 1) / TN, (g.M + TM - 1) / TM, z);
-  gemm_kernel<TB, AK, BK, TM, TN, RM, RN><<<grid, (TM / RM) * (TN / RN), 0, s>>>(A, B, g);
+  launch_chained(gemm_kernel<TB, AK, BK, TM, TN, RM, RN>, grid, (TM / RM) * (TN / RN), 0, s, A, B, g);
   if (z == 1) return;
   const int64_t MN = (int64_t)g.M * g.N;
-  gemm_reduce_kernel<<<(int)std::min<int64_t>((MN + 255) / 256, 152 * 8), 256, 0, s>>>(ws, z, g);
+  launch_chained(gemm_reduce_kernel, (int)std::min<int64_t>((MN + 255) / 256, 152 * 8), 256, 0, s, ws, z, g);
 }
 
 // 32 x 32 tiles with 4 x 4 outputs per thread where the batch is the tile's short side (512 CTAs of
@@ -721,8 +734,8 @@ void nn_dense_bwd_w(const float* dz, const float* x, float* dW, int B, int N, in
 template <int D, int CI, int CO, bool RELU>
 static void conv_fwd(const float* x, const float* w, const float* b, float* y, int B, cudaStream_t s) {
   const int64_t n = (int64_t)B * D * D * (D / 2);
-  convT_fwd_kernel<D, CI, CO, RELU>
-      <<<dim3((unsigned)((n + kConvThreads - 1) / kConvThreads), CO / kConvCog), kConvThreads, 0, s>>>(x, w, b, y, B);
+  launch_chained(convT_fwd_kernel<D, CI, CO, RELU>, dim3((unsigned)((n + kConvThreads - 1) / kConvThreads),
+      CO / kConvCog), kConvThreads, 0, s, x, w, b, y, B);
 }
 
 void nn_convT_fwd(int layer, const float* x, const float* w, const float* b, float* y, int B, cudaStream_t s) {
@@ -752,15 +765,15 @@ template <int LAYER, int D, int CI, int CO, int CIG>
 static void conv_bwd(const float* x, const float* w, const float* dy, float* dx, int B, float* bpart, float* wpart,
                      cudaStream_t s) {
   const int64_t n = (int64_t)B * D * D * (D / 2);
-  convT_bwd_data_kernel<D, CI, CO, CIG>
-      <<<dim3((unsigned)((n + kConvThreads - 1) / kConvThreads), CI / CIG), kConvThreads, 0, s>>>(dy, w, x, dx, B);
+  launch_chained(convT_bwd_data_kernel<D, CI, CO, CIG>, dim3((unsigned)((n + kConvThreads - 1) / kConvThreads),
+      CI / CIG), kConvThreads, 0, s, dy, w, x, dx, B);
   int64_t chunk = 0;
   const int nchunk = conv_chunks(LAYER, B, chunk);
   static const cudaError_t attr = cudaFuncSetAttribute(
       convT_bwd_w_kernel<D, CI, CO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBwdWSmem);
   (void)attr;   // a failure shows at the launch
-  convT_bwd_w_kernel<D, CI, CO><<<CI / kBwdWCi * CO * 4 * nchunk + CO * B, kBwdWThreads, kBwdWSmem, s>>>(
-      x, dy, wpart, bpart, B, chunk, nchunk);
+  launch_chained(convT_bwd_w_kernel<D, CI, CO>, CI / kBwdWCi * CO * 4 * nchunk + CO * B, kBwdWThreads, kBwdWSmem,
+      s, x, dy, wpart, bpart, B, chunk, nchunk);
 }
 
 // The partial sums of layer l start at these offsets of the bias and weight workspaces.
@@ -797,7 +810,7 @@ void nn_final_sums(int B, const float* bpart, const float* wpart, float* const d
   }
   add(dz2, db2, N, B, 1, N);
   add(dz1, db1, N, B, 1, N);
-  nn_final_sums_kernel<<<(unsigned)blocks, 128, 0, s>>>(f);
+  launch_chained(nn_final_sums_kernel, (unsigned)blocks, 128, 0, s, f);
 }
 
 void nn_mse(const float* y, const float* t, const int32_t* idx, int B, int64_t width, float* dy, double* part,
@@ -805,29 +818,30 @@ void nn_mse(const float* y, const float* t, const int32_t* idx, int B, int64_t w
   note_launch(2);
   const int64_t n = B * width;
   const int nb = (int)(width / kMseChunk);
-  mse_kernel<<<dim3(nb, B), 256, 0, s>>>(y, t, idx, width, 2.0f / (float)n, dy, part);
-  sum_parts_kernel<<<1, 256, 0, s>>>(part, nb * B, 1.0 / (double)n, loss);
+  launch_chained(mse_kernel, dim3(nb, B), 256, 0, s, y, t, idx, width, 2.0f / (float)n, dy, part);
+  launch_chained(sum_parts_kernel, 1, 256, 0, s, part, nb * B, 1.0 / (double)n, loss);
 }
 void nn_adam(float* th, const float* g, float* m, float* v, void* w1, void* w2, int64_t n, int64_t n1, int64_t o2,
              int64_t n2, float lr, float b1, float b2, float eps, int step, cudaStream_t s) {
   note_launch(1);
   const AdamArgs a{lr, b1, b2, eps, 1.f - powf(b1, (float)step), 1.f - powf(b2, (float)step), n, n1, o2, n2};
-  adam_kernel<<<(unsigned)((n + 1023) / 1024), 256, 0, s>>>(th, g, m, v, (__nv_bfloat16*)w1, (__nv_bfloat16*)w2, a);
+  launch_chained(adam_kernel, (unsigned)((n + 1023) / 1024), 256, 0, s, th, g, m, v, (__nv_bfloat16*)w1,
+      (__nv_bfloat16*)w2, a);
 }
 void nn_to_bf16(const float* a, void* b, int64_t n, cudaStream_t s) {
   note_launch(1);
-  to_bf16_kernel<<<gsb(n), 256, 0, s>>>(a, (__nv_bfloat16*)b, n);
+  launch_chained(to_bf16_kernel, gsb(n), 256, 0, s, a, (__nv_bfloat16*)b, n);
 }
 void nn_gather_rows(const float* src, const int32_t* idx, int n, int64_t width, float* dst, cudaStream_t s) {
   note_launch(1);
-  gather_rows_kernel<<<dim3((unsigned)((width + 255) / 256 < 16 ? (width + 255) / 256 : 16), n), 256, 0, s>>>(
-      src, idx, width, dst);
+  launch_chained(gather_rows_kernel, dim3((unsigned)((width + 255) / 256 < 16 ? (width + 255) / 256 : 16), n),
+      256, 0, s, src, idx, width, dst);
 }
 void nn_grid_to_tets(const float* grid, int G, const double* box, const double* xyz, const int32_t* tets, int64_t T,
                      double* out, cudaStream_t s) {
   note_launch(1);
-  grid_to_tets_kernel<<<(unsigned)((T + 127) / 128), 128, 0, s>>>(grid, G, box[0], box[1], box[2], box[3], box[4],
-                                                                   box[5], xyz, tets, T, out);
+  launch_chained(grid_to_tets_kernel, (unsigned)((T + 127) / 128), 128, 0, s, grid, G, box[0], box[1], box[2],
+      box[3], box[4], box[5], xyz, tets, T, out);
 }
 
 }  // namespace mwk

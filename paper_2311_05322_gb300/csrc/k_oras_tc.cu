@@ -32,6 +32,7 @@
 #include "k_oras_tc.h"
 #include "k_mf.h"
 #include "mw_async.cuh"
+#include "mw_chain.cuh"
 #include "mw_internal.h"
 
 namespace mwk {
@@ -192,6 +193,7 @@ __global__ void __launch_bounds__(128, 8) gather_b_kernel(const int32_t* __restr
                                                        const float2* __restrict__ r, int R, int Rp,
                                                        uint8_t* __restrict__ Bt, const double* __restrict__ cscale,
                                                        int64_t ntiles) {
+  chain_wait();
   // Blocks of 4 warps walk the tiles with a grid stride.  Per tile (64 dofs), warp w takes dofs
   // 16w .. 16w+15 and lane c the columns c, c + 32, ...: the dof indices come in one coalesced
   // load and are handed out by shuffles, the 16 values of a lane are independent loads, and each
@@ -257,6 +259,7 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const int32_t* __restr
                                                           const float2* __restrict__ in,
                                                           const float2* __restrict__ arena, int R, int Rp,
                                                           uint8_t* __restrict__ Bt) {
+  chain_wait();
   extern __shared__ __align__(16) uint8_t tsm[];
   const int32_t* idx = src + (int64_t)blockIdx.x * kTileKd * NS;
   for (int it = threadIdx.x; it < 8 * Rp; it += blockDim.x) {
@@ -451,14 +454,10 @@ __global__ void __launch_bounds__(kThreadsTc, 2) oras_tc_kernel(const TcArgs a) 
   __shared__ int abort_flag;
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dsm) + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const TcTile tl = a.tiles[blockIdx.x];
-  const int KT = tl.kt;
   const int S = a.stages;
   const uint32_t b_bytes = (uint32_t)a.N * 128u;
   const uint32_t a_bytes = 2u * kATileBytes;          // Wr and Wi tiles of one k tile
   const uint32_t stage_bytes = a_bytes + b_bytes;
-  const uint8_t* Wt = a.W + (size_t)tl.w * kATileBytes;
-  const uint8_t* Bs = a.Bt + (size_t)tl.g * b_bytes;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < S; ++i) {
@@ -479,6 +478,11 @@ __global__ void __launch_bounds__(kThreadsTc, 2) oras_tc_kernel(const TcArgs a) 
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_base;
+  chain_wait();   // the set-up above and the tensor memory are this block's own
+  const TcTile tl = a.tiles[blockIdx.x];
+  const int KT = tl.kt;
+  const uint8_t* Wt = a.W + (size_t)tl.w * kATileBytes;
+  const uint8_t* Bs = a.Bt + (size_t)tl.g * b_bytes;
 
   if (warp == 0) {
     if (lane == 0) {
@@ -593,6 +597,7 @@ __global__ void __launch_bounds__(kThreadsTc, 2) oras_tc_persistent_kernel(const
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_base;
+  chain_wait();   // the set-up above and the tensor memory are this block's own
 
   if (warp == 0) {
     if (lane == 0) {
@@ -880,7 +885,8 @@ static void tc_mma(const TcPlan& p, TcArgs a, int R, int stages, bool persistent
       pattr = smem;
     }
     const int grid = (int)std::min<int64_t>(p.n_mtiles, (int64_t)per_sm * 152);
-    oras_tc_persistent_kernel<<<(unsigned)std::max(grid, 1), kThreadsTc, smem, s>>>(a, (int)p.n_mtiles);
+    launch_chained(oras_tc_persistent_kernel, (unsigned)std::max(grid, 1), kThreadsTc, smem, s, a,
+        (int)p.n_mtiles);
     return;
   }
   // two CTAs of an SM must fit their tensor memory (512 columns per SM): above 256 columns the
@@ -892,7 +898,7 @@ static void tc_mma(const TcPlan& p, TcArgs a, int R, int stages, bool persistent
     cudaFuncSetAttribute(oras_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     attr = smem;
   }
-  oras_tc_kernel<<<(unsigned)p.n_mtiles, kThreadsTc, smem, s>>>(a);
+  launch_chained(oras_tc_kernel, (unsigned)p.n_mtiles, kThreadsTc, smem, s, a);
 }
 
 void oras_apply_tc(const TcPlan& p, const OrasTopo& tp, const void* W, const float2* r, float2* z, int R,
@@ -906,8 +912,8 @@ void oras_apply_tc(const TcPlan& p, const OrasTopo& tp, const void* W, const flo
     gattr = gsm;
   }
   const int64_t gblocks = std::min<int64_t>(p.n_ktiles_total, 152 * 8);    // one resident wave
-  gather_b_kernel<<<(unsigned)std::max<int64_t>(gblocks, 1), 128, gsm, s>>>(
-      p.gt_sub, p.gt_kt, tp.dof_ptr, tp.dofs, r, R, Rp, (uint8_t*)scratch, in_scale, p.n_ktiles_total);
+  launch_chained(gather_b_kernel, (unsigned)std::max<int64_t>(gblocks, 1), 128, gsm, s, p.gt_sub, p.gt_kt,
+      tp.dof_ptr, tp.dofs, r, R, Rp, (uint8_t*)scratch, in_scale, p.n_ktiles_total);
   TcArgs a{};
   a.own_glob = tp.own_glob;
   a.z_bf16 = z_bf16 ? 1 : 0;
@@ -925,9 +931,9 @@ void tc_sweep(const TcPlan& p, const TcRow* rows, const int32_t* src, int n_src,
   const unsigned blocks = (unsigned)p.n_ktiles_total, threads = (unsigned)std::min(8 * Rp, 256);
   const size_t gsm = (size_t)2 * Rp * 128;   // at most 32 KB
   if (n_src == 3)
-    gather_rows_kernel<3><<<blocks, threads, gsm, s>>>(src, in, arena, R, Rp, (uint8_t*)scratch);
+    launch_chained(gather_rows_kernel<3>, blocks, threads, gsm, s, src, in, arena, R, Rp, (uint8_t*)scratch);
   else
-    gather_rows_kernel<1><<<blocks, threads, gsm, s>>>(src, in, arena, R, Rp, (uint8_t*)scratch);
+    launch_chained(gather_rows_kernel<1>, blocks, threads, gsm, s, src, in, arena, R, Rp, (uint8_t*)scratch);
   TcArgs a{};
   a.rows = rows;
   a.vec = R % 2 == 0 && (((uintptr_t)arena | (uintptr_t)z) & 15) == 0;

@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "mw_chain.cuh"
 #include "mw_internal.h"
 #include "mw_reduce.cuh"
 
@@ -49,6 +50,7 @@ template <typename T, int CPL, typename XT = T>
 __global__ void __launch_bounds__(512) spmm_kernel(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
                                                    const T* __restrict__ A, const XT* __restrict__ X, T* __restrict__ Y,
                                                    int64_t E, int R, int tpr_log2) {
+  chain_wait();
   constexpr int NB = 8 / CPL;
   const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t row = g >> tpr_log2;
@@ -110,6 +112,7 @@ __global__ void __launch_bounds__(512, CV == 1 ? 4 : 1) spmm_staged_kernel(const
                                                           const float2* __restrict__ A, const XT* __restrict__ X,
                                                           float2* __restrict__ Y, int64_t E, int R, int lpr_log2,
                                                           int rows) {
+  chain_wait();
   constexpr int NB = VEC * CV >= 4 ? 2 : 4;
   using Pack = XPack<XT, VEC>;
   extern __shared__ float4 smem4[];
@@ -178,6 +181,7 @@ __global__ void __launch_bounds__(256) residual_kernel(const int64_t* __restrict
                                                        const double2* __restrict__ A, const double2* __restrict__ X,
                                                        const double2* __restrict__ B, double2* __restrict__ Rv,
                                                        double* __restrict__ part, int64_t E, int R, int tpr_log2) {
+  chain_wait();
   __shared__ double red[256 * CPL];
   const int tpr = 1 << tpr_log2;
   const int rows_per_block = 256 >> tpr_log2;
@@ -238,13 +242,13 @@ void spmm_launch(const int64_t* rp, const int32_t* ci, const T* A, const T* X, T
   const int blocks = (int)((nthr + threads - 1) / threads);
   switch (sh.cpl) {
     case 1:
-      spmm_kernel<T, 1><<<blocks, threads, 0, s>>>(rp, ci, A, X, Y, E, R, sh.tpr_log2);
+      launch_chained(spmm_kernel<T, 1>, blocks, threads, 0, s, rp, ci, A, X, Y, E, R, sh.tpr_log2);
       break;
     case 2:
-      spmm_kernel<T, 2><<<blocks, threads, 0, s>>>(rp, ci, A, X, Y, E, R, sh.tpr_log2);
+      launch_chained(spmm_kernel<T, 2>, blocks, threads, 0, s, rp, ci, A, X, Y, E, R, sh.tpr_log2);
       break;
     default:
-      spmm_kernel<T, 4><<<blocks, threads, 0, s>>>(rp, ci, A, X, Y, E, R, sh.tpr_log2);
+      launch_chained(spmm_kernel<T, 4>, blocks, threads, 0, s, rp, ci, A, X, Y, E, R, sh.tpr_log2);
       break;
   }
 }
@@ -263,11 +267,11 @@ void spmm_staged(const int64_t* rp, const int32_t* ci, const float2* A, const XT
   const unsigned blocks = (unsigned)((E + rows - 1) / rows);
   note_launch(1);
   if (cv == 1)
-    spmm_staged_kernel<XT, VEC, 1><<<blocks, threads, smem, s>>>(rp, ci, A, X, Y, E, R, l, rows);
+    launch_chained(spmm_staged_kernel<XT, VEC, 1>, blocks, threads, smem, s, rp, ci, A, X, Y, E, R, l, rows);
   else if (cv == 2)
-    spmm_staged_kernel<XT, VEC, 2><<<blocks, threads, smem, s>>>(rp, ci, A, X, Y, E, R, l, rows);
+    launch_chained(spmm_staged_kernel<XT, VEC, 2>, blocks, threads, smem, s, rp, ci, A, X, Y, E, R, l, rows);
   else
-    spmm_staged_kernel<XT, VEC, 4><<<blocks, threads, smem, s>>>(rp, ci, A, X, Y, E, R, l, rows);
+    launch_chained(spmm_staged_kernel<XT, VEC, 4>, blocks, threads, smem, s, rp, ci, A, X, Y, E, R, l, rows);
 }
 
 // The staged product when the records of a block fit 48 KB of shared memory and element offsets 31 bits;
@@ -402,13 +406,13 @@ void spmm_f32_bx(const int64_t* rp, const int32_t* ci, const float2* A, const vo
   const uint32_t* Xb = (const uint32_t*)X;
   switch (sh.cpl) {
     case 1:
-      spmm_kernel<float2, 1, uint32_t><<<blocks, threads, 0, s>>>(rp, ci, A, Xb, Y, E, R, sh.tpr_log2);
+      launch_chained(spmm_kernel<float2, 1, uint32_t>, blocks, threads, 0, s, rp, ci, A, Xb, Y, E, R, sh.tpr_log2);
       break;
     case 2:
-      spmm_kernel<float2, 2, uint32_t><<<blocks, threads, 0, s>>>(rp, ci, A, Xb, Y, E, R, sh.tpr_log2);
+      launch_chained(spmm_kernel<float2, 2, uint32_t>, blocks, threads, 0, s, rp, ci, A, Xb, Y, E, R, sh.tpr_log2);
       break;
     default:
-      spmm_kernel<float2, 4, uint32_t><<<blocks, threads, 0, s>>>(rp, ci, A, Xb, Y, E, R, sh.tpr_log2);
+      launch_chained(spmm_kernel<float2, 4, uint32_t>, blocks, threads, 0, s, rp, ci, A, Xb, Y, E, R, sh.tpr_log2);
       break;
   }
 }
@@ -426,21 +430,21 @@ int residual_f64(const int64_t* rp, const int32_t* ci, const double2* A, const d
   switch (sh.cpl) {
     case 1:
       if (zero_x)
-        residual_kernel<1, true><<<blocks, 256, 0, s>>>(rp, ci, A, X, B, Rv, part, E, R, sh.tpr_log2);
+        launch_chained(residual_kernel<1, true>, blocks, 256, 0, s, rp, ci, A, X, B, Rv, part, E, R, sh.tpr_log2);
       else
-        residual_kernel<1, false><<<blocks, 256, 0, s>>>(rp, ci, A, X, B, Rv, part, E, R, sh.tpr_log2);
+        launch_chained(residual_kernel<1, false>, blocks, 256, 0, s, rp, ci, A, X, B, Rv, part, E, R, sh.tpr_log2);
       break;
     case 2:
       if (zero_x)
-        residual_kernel<2, true><<<blocks, 256, 0, s>>>(rp, ci, A, X, B, Rv, part, E, R, sh.tpr_log2);
+        launch_chained(residual_kernel<2, true>, blocks, 256, 0, s, rp, ci, A, X, B, Rv, part, E, R, sh.tpr_log2);
       else
-        residual_kernel<2, false><<<blocks, 256, 0, s>>>(rp, ci, A, X, B, Rv, part, E, R, sh.tpr_log2);
+        launch_chained(residual_kernel<2, false>, blocks, 256, 0, s, rp, ci, A, X, B, Rv, part, E, R, sh.tpr_log2);
       break;
     default:
       if (zero_x)
-        residual_kernel<4, true><<<blocks, 256, 0, s>>>(rp, ci, A, X, B, Rv, part, E, R, sh.tpr_log2);
+        launch_chained(residual_kernel<4, true>, blocks, 256, 0, s, rp, ci, A, X, B, Rv, part, E, R, sh.tpr_log2);
       else
-        residual_kernel<4, false><<<blocks, 256, 0, s>>>(rp, ci, A, X, B, Rv, part, E, R, sh.tpr_log2);
+        launch_chained(residual_kernel<4, false>, blocks, 256, 0, s, rp, ci, A, X, B, Rv, part, E, R, sh.tpr_log2);
       break;
   }
   return blocks;
@@ -494,6 +498,7 @@ __device__ __forceinline__ void split_double(double v, float& hi, float& lo) {
 
 // A_df[k] = (re_hi, re_lo, im_hi, im_lo) of a complex FP64 value.
 __global__ void split_df_kernel(const double2* __restrict__ a, float4* __restrict__ o, int64_t n) {
+  chain_wait();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const double2 v = a[i];
     float4 r;
@@ -593,6 +598,7 @@ __global__ void __launch_bounds__(256) residual_df32_kernel(const int64_t* __res
                                                             const float4* __restrict__ Bdf, float2* __restrict__ Rv,
                                                             double* __restrict__ part, int64_t E, int R, int tpr_log2,
                                                             int rows, int cap) {
+  chain_wait();
   constexpr int NB = CV == 1 ? 4 : 2;               // even: the accumulators alternate by term
   extern __shared__ float4 rsmem[];
   float4* rec = rsmem;                              // [cap] values of the tile
@@ -677,7 +683,7 @@ __global__ void __launch_bounds__(256) residual_df32_kernel(const int64_t* __res
 void split_df(const double2* a, float4* o, int64_t n, cudaStream_t s) {
   note_launch(1);
   int64_t b = (n + 255) / 256;
-  split_df_kernel<<<(int)(b < 152 * 16 ? (b > 0 ? b : 1) : 152 * 16), 256, 0, s>>>(a, o, n);
+  launch_chained(split_df_kernel, (int)(b < 152 * 16 ? (b > 0 ? b : 1) : 152 * 16), 256, 0, s, a, o, n);
 }
 
 int residual_df(const int64_t* rp, const int32_t* ci, const float4* A, const float4* X, const double2* B, double2* Rv,
@@ -713,9 +719,11 @@ static int residual_df32_launch(const int64_t* rp, const int32_t* ci, const floa
                                                        cudaFuncAttributeMaxDynamicSharedMemorySize, kCap * 20 + 256);
   (void)attr;   // a failure shows at the launch
   if (zero_x)
-    residual_df32_kernel<CV, true><<<blocks, 256, smem, s>>>(rp, ci, A, X, Bdf, Rv, part, E, R, l, rows, cap);
+    launch_chained(residual_df32_kernel<CV, true>, blocks, 256, smem, s, rp, ci, A, X, Bdf, Rv, part, E, R, l,
+        rows, cap);
   else
-    residual_df32_kernel<CV, false><<<blocks, 256, smem, s>>>(rp, ci, A, X, Bdf, Rv, part, E, R, l, rows, cap);
+    launch_chained(residual_df32_kernel<CV, false>, blocks, 256, smem, s, rp, ci, A, X, Bdf, Rv, part, E, R, l,
+        rows, cap);
   return blocks;
 }
 
