@@ -18,6 +18,7 @@
 
 #include "mw_async.cuh"
 #include "mw_chain.cuh"
+#include "mw_df.cuh"
 #include "mw_internal.h"
 #include "mw_reduce.cuh"
 
@@ -1005,60 +1006,118 @@ __global__ void update_x_kernel(const T* __restrict__ Z, int64_t zstride, const 
   }
 }
 
-// The same update with Z stored as complex BF16 pairs (4 bytes per value, real in the low half):
-// the correction is formed in FP32 from the widened values and added to x in FP64.
-__global__ void update_x_bx_kernel(const uint32_t* __restrict__ Z, int64_t zstride, const double2* __restrict__ y,
-                                   const int32_t* __restrict__ kcol, int m, double2* __restrict__ x, int64_t E, int R) {
-  chain_wait();
-  const int64_t n = E * R;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(i % R);
-    const int k = kcol[c];
-    float dr = 0.f, di = 0.f;
-    for (int l = 0; l < k; ++l) {
-      const uint32_t u = Z[(int64_t)l * zstride + i];
-      const float zx = __uint_as_float(u << 16), zy = __uint_as_float(u & 0xffff0000u);
-      const double2 yy = y[(int64_t)c * m + l];
-      const float yr = (float)yy.x, yi = (float)yy.y;
-      dr = fmaf(yr, zx, dr);
-      dr = fmaf(-yi, zy, dr);
-      di = fmaf(yr, zy, di);
-      di = fmaf(yi, zx, di);
-    }
-    double2 xv = x[i];
-    xv.x += (double)dr;
-    xv.y += (double)di;
-    x[i] = xv;
-  }
-}
-
-// Stored value of Z widened to the arithmetic type: itself, or a complex BF16 pair (real in the
-// low half) as complex FP32.
+// Value of an FP32 basis: itself, or a complex BF16 pair (real in the low half).
 __device__ __forceinline__ float2 zval(float2 v) { return v; }
-__device__ __forceinline__ double2 zval(double2 v) { return v; }
 __device__ __forceinline__ float2 zval(uint32_t u) {
   return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
+}
+
+// x += Z y for FP32 bases (stored FP32 or BF16): the correction in FP32, added to x in FP64, and x's double-float
+// copy (which the outer residual reads) written on the way; a pass of its own read all of x again.  Memory
+// bound: x in, x and its copy out, kmax vectors of Z.  A thread takes VEC neighbouring columns of U rows, so that
+// its x values and U loads of Z per vector are in flight together; a ring of bulk copies into shared memory, whose
+// consumers then waited for x, took 980 us for 525,329 rows of 64 columns and 7 BF16 vectors, and the copy 250 us
+// more; this takes 603.  Columns past their kcol take no part in a term (their Z is stale).
+constexpr int kUxRows = 4;
+template <typename ZT, int VEC>
+__global__ void __launch_bounds__(256) update_x32_kernel(const ZT* __restrict__ Z, int64_t zstride,
+                                                         const double2* __restrict__ y,
+                                                         const int32_t* __restrict__ kcol, int m,
+                                                         double2* __restrict__ x, float4* __restrict__ xdf, int64_t E,
+                                                         int R) {
+  chain_wait();
+  extern __shared__ __align__(16) float2 ux_y[];   // [kmax][R]
+  __shared__ int kmax_s;
+  struct alignas(sizeof(ZT) * VEC) ZV {
+    ZT v[VEC];
+  };
+  if (threadIdx.x < 32) {
+    int km = 0;
+    for (int c = threadIdx.x; c < R; c += 32) km = max(km, min(kcol[c], m));
+    km = __reduce_max_sync(0xffffffffu, km);
+    if (threadIdx.x == 0) kmax_s = km;
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < kmax_s * R; t += 256) {
+    const int l = t / R, c = t - l * R;
+    const double2 v = y[(int64_t)c * m + l];
+    ux_y[t] = make_float2((float)v.x, (float)v.y);
+  }
+  __syncthreads();
+  const int tpr = R / VEC, rpb = 256 / tpr;
+  const int lr = threadIdx.x / tpr, c = threadIdx.x % tpr * VEC;
+  if (lr >= rpb) return;
+  int kc[VEC], kt = 0;
+#pragma unroll
+  for (int v = 0; v < VEC; ++v) {
+    kc[v] = min(kcol[c + v], m);
+    kt = max(kt, kc[v]);
+  }
+  for (int64_t row0 = (int64_t)blockIdx.x * rpb * kUxRows + lr; row0 < E; row0 += (int64_t)gridDim.x * rpb * kUxRows) {
+    double2 xv[kUxRows][VEC];
+    float2 d[kUxRows][VEC];
+    const ZT* zp[kUxRows];
+#pragma unroll
+    for (int u = 0; u < kUxRows; ++u) {
+      const int64_t row = min(row0 + (int64_t)u * rpb, E - 1);   // rows past the end repeat the last one, unstored
+      zp[u] = Z + row * R + c;
+#pragma unroll
+      for (int v = 0; v < VEC; ++v) {
+        xv[u][v] = x[row * R + c + v];
+        d[u][v] = make_float2(0.f, 0.f);
+      }
+    }
+#pragma unroll 4
+    for (int l = 0; l < kt; ++l) {
+      ZV z[kUxRows];
+#pragma unroll
+      for (int u = 0; u < kUxRows; ++u) z[u] = *reinterpret_cast<const ZV*>(zp[u] + (int64_t)l * zstride);
+#pragma unroll
+      for (int v = 0; v < VEC; ++v) {
+        const float2 yy = ux_y[l * R + c + v];
+        if (l < kc[v])
+#pragma unroll
+          for (int u = 0; u < kUxRows; ++u) {
+            const float2 zz = zval(z[u].v[v]);
+            d[u][v].x = fmaf(yy.x, zz.x, d[u][v].x);
+            d[u][v].x = fmaf(-yy.y, zz.y, d[u][v].x);
+            d[u][v].y = fmaf(yy.x, zz.y, d[u][v].y);
+            d[u][v].y = fmaf(yy.y, zz.x, d[u][v].y);
+          }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kUxRows; ++u) {
+      const int64_t row = row0 + (int64_t)u * rpb;
+      if (row >= E) break;
+#pragma unroll
+      for (int v = 0; v < VEC; ++v) {
+        double2 t = xv[u][v];
+        t.x += (double)d[u][v].x;
+        t.y += (double)d[u][v].y;
+        x[row * R + c + v] = t;
+        xdf[row * R + c + v] = split_df2(t);
+      }
+    }
+  }
 }
 
 // Streaming form of the solution update for 16 <= R <= 128 with 16-byte aligned bases, on the tiles,
 // ring and thread map of cgs_dots_bulk_kernel: the producer streams Z_0 .. Z_{kmax-1} per tile
 // (kmax = the largest kcol of the block); consumer (c, g) forms the correction of its rows of
 // column c in the basis precision with the operations of update_x_kernel, in the same order
-// (bit-identical x), and adds it to x in FP64.  y is staged in shared memory as T.  ZT is the
-// stored type of Z: T, or uint32_t for complex BF16 pairs (T = float2; the widened values enter
-// the same operations as update_x_bx_kernel's, bit-identical to it); the tiles keep
-// bd_rows<T>() rows per row group, so BF16 tiles fill half a stage.
-template <typename T, typename ZT = T>
+// (bit-identical x), and adds it to x in FP64.  y is staged in shared memory as T.
+template <typename T>
 __global__ void __launch_bounds__(kBdThreads, 2)
-    update_x_bulk_kernel(const ZT* __restrict__ Z, int64_t zstride, const double2* __restrict__ y,
+    update_x_bulk_kernel(const T* __restrict__ Z, int64_t zstride, const double2* __restrict__ y,
                          const int32_t* __restrict__ kcol, int m, double2* __restrict__ x, int64_t E, int R, int G,
                          int NS, int32_t* __restrict__ err) {
   chain_wait();
   using Sc = typename Traits<T>::S;
   constexpr int RPT = bd_rows<T>();
-  constexpr int kStageElems = kBdStageBytes / (int)sizeof(ZT);
+  constexpr int kStageElems = kBdStageBytes / (int)sizeof(T);
   extern __shared__ __align__(128) uint8_t ux_smem[];
-  ZT* stage = reinterpret_cast<ZT*>(ux_smem);
+  T* stage = reinterpret_cast<T*>(ux_smem);
   T* ys = reinterpret_cast<T*>(ux_smem + (size_t)NS * kBdStageBytes);   // [m][R]
   int32_t* ks = reinterpret_cast<int32_t*>(ys + (size_t)m * R);          // [R]
   uint64_t* full = reinterpret_cast<uint64_t*>(ks + ((R + 3) & ~3));
@@ -1103,7 +1162,7 @@ __global__ void __launch_bounds__(kBdThreads, 2)
     for (int64_t t = t0; t < t1 && !stop; ++t) {
       const int64_t r0 = t * TR;
       const int64_t rows = E - r0 < TR ? E - r0 : (int64_t)TR;
-      const uint32_t bytes = (uint32_t)((rows * R * (int64_t)sizeof(ZT)) & ~(int64_t)15);
+      const uint32_t bytes = (uint32_t)((rows * R * (int64_t)sizeof(T)) & ~(int64_t)15);
       for (int l = 0; l < kmax; ++l) {
         if (it >= NS && !mbar_wait(&empty[st], ph ^ 1u)) {
           atomicCAS(err, 0, 31);
@@ -1113,7 +1172,7 @@ __global__ void __launch_bounds__(kBdThreads, 2)
           stop = true;
           break;
         }
-        const ZT* src = Z + (int64_t)l * zstride + r0 * R;
+        const T* src = Z + (int64_t)l * zstride + r0 * R;
         if (bytes > 0) {
           mbar_expect_tx(&full[st], bytes);
           bulk_g2s(stage + (size_t)st * kStageElems, src, bytes, &full[st]);
@@ -1143,7 +1202,7 @@ __global__ void __launch_bounds__(kBdThreads, 2)
   for (int64_t t = t0; t < t1; ++t) {
     const int64_t r0 = t * TR;
     const int64_t rows = E - r0 < TR ? E - r0 : (int64_t)TR;
-    const int64_t ncop = ((rows * R * (int64_t)sizeof(ZT)) & ~(int64_t)15) / (int64_t)sizeof(ZT);
+    const int64_t ncop = ((rows * R * (int64_t)sizeof(T)) & ~(int64_t)15) / (int64_t)sizeof(T);
     Sc dr[RPT], di[RPT];
 #pragma unroll
     for (int k = 0; k < RPT; ++k) dr[k] = di[k] = 0;
@@ -1153,15 +1212,15 @@ __global__ void __launch_bounds__(kBdThreads, 2)
         *abort_flag = 1;
       }
       if (act && l < kc) {
-        const ZT* sm = stage + (size_t)st * kStageElems;
-        const ZT* gl = Z + (int64_t)l * zstride + r0 * R;
+        const T* sm = stage + (size_t)st * kStageElems;
+        const T* gl = Z + (int64_t)l * zstride + r0 * R;
         const T yy = ys[l * R + c];
 #pragma unroll
         for (int k = 0; k < RPT; ++k) {
           const int row = k * G + g;
           const int f = row * R + c;
           if (row < rows) {
-            const T z = zval(f < ncop ? sm[f] : gl[f]);
+            const T z = f < ncop ? sm[f] : gl[f];
             dr[k] = fma(yy.x, z.x, dr[k]);
             dr[k] = fma(-yy.y, z.y, dr[k]);
             di[k] = fma(yy.x, z.y, di[k]);
@@ -1195,20 +1254,20 @@ inline size_t ux_smem_bytes(int R, int m, int NS) {
   return (size_t)NS * kBdStageBytes + (size_t)m * R * 16 + ((R + 3) & ~3) * 4 + 2 * NS * sizeof(uint64_t) + 16;
 }
 
-template <typename T, typename ZT = T>
-bool update_x_bulk(const ZT* Z, int64_t zstride, const double2* y, const int32_t* kcol, int m, double2* x, int64_t E,
+template <typename T>
+bool update_x_bulk(const T* Z, int64_t zstride, const double2* y, const int32_t* kcol, int m, double2* x, int64_t E,
                    int R, int32_t* err, cudaStream_t s) {
-  const bool aligned = ((uintptr_t)Z % 16 == 0) && ((zstride * sizeof(ZT)) % 16 == 0);
+  const bool aligned = ((uintptr_t)Z % 16 == 0) && ((zstride * sizeof(T)) % 16 == 0);
   if (!err || !aligned || R < 16 || R > 128 || m < 1) return false;
   static bool attr = false;   // one per instantiation
   if (!attr) {
     // 226 KB: the kernel's static shared memory shares the 227 KB per block
-    attr = cudaFuncSetAttribute(update_x_bulk_kernel<T, ZT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    attr = cudaFuncSetAttribute(update_x_bulk_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 226 * 1024) == cudaSuccess;
   }
   int NS = kBdStages;
   while (NS > 2 && ux_smem_bytes(R, m, NS) > (size_t)226 * 1024) --NS;
-  launch_chained(update_x_bulk_kernel<T, ZT>, 152 * 2, kBdThreads, ux_smem_bytes(R, m, NS), s, Z, zstride, y,
+  launch_chained(update_x_bulk_kernel<T>, 152 * 2, kBdThreads, ux_smem_bytes(R, m, NS), s, Z, zstride, y,
       kcol, m, x, E, R, kBdConsumers / R, NS, err);
   return true;
 }
@@ -1452,18 +1511,32 @@ void update_x_f64(const double2* Z, int64_t zstride, const double2* y, const int
   if (update_x_bulk<double2>(Z, zstride, y, kcol, m, x, E, R, err, s)) return;
   launch_chained(update_x_kernel<double2>, gs_blocks(E * R), 256, 0, s, Z, zstride, y, kcol, m, x, E, R);
 }
-void update_x_bx(const void* Z, int64_t zstride, const double2* y, const int32_t* kcol, int m, double2* x, int64_t E,
-                 int R, cudaStream_t s, int32_t* err) {
+template <typename ZT>
+static void update_x32(const ZT* Z, int64_t zstride, const double2* y, const int32_t* kcol, int m, double2* x,
+                       float4* xdf, int64_t E, int R, cudaStream_t s) {
   note_launch(1);
-  if (update_x_bulk<float2, uint32_t>((const uint32_t*)Z, zstride, y, kcol, m, x, E, R, err, s)) return;
-  launch_chained(update_x_bx_kernel, gs_blocks(E * R), 256, 0, s, (const uint32_t*)Z, zstride, y, kcol, m, x, E,
-      R);
+  const size_t smem = sizeof(float2) * m * R;   // at most 63 KB
+  auto go = [&](auto kernel, int vec) {
+    static bool attr[3] = {};
+    if (smem > 48 * 1024 && !attr[vec])
+      attr[vec] = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024) == cudaSuccess;
+    const int64_t rows = (int64_t)(256 / (R / vec)) * kUxRows;
+    launch_chained(kernel, (unsigned)std::min<int64_t>((E + rows - 1) / rows, 152 * 4), 256, smem, s, Z, zstride, y,
+                   kcol, m, x, xdf, E, R);
+  };
+  // pairs of columns where a pair of Z values is one aligned load
+  if (R % 2 == 0 && zstride % 2 == 0 && (uintptr_t)Z % (2 * sizeof(ZT)) == 0)
+    go(update_x32_kernel<ZT, 2>, 2);
+  else
+    go(update_x32_kernel<ZT, 1>, 1);
+}
+void update_x_bx(const void* Z, int64_t zstride, const double2* y, const int32_t* kcol, int m, double2* x, float4* xdf,
+                 int64_t E, int R, cudaStream_t s) {
+  update_x32((const uint32_t*)Z, zstride, y, kcol, m, x, xdf, E, R, s);
 }
 void update_x_f32(const float2* Z, int64_t zstride, const double2* y, const int32_t* kcol, int m, double2* x,
-                  int64_t E, int R, cudaStream_t s, int32_t* err) {
-  note_launch(1);
-  if (update_x_bulk<float2>(Z, zstride, y, kcol, m, x, E, R, err, s)) return;
-  launch_chained(update_x_kernel<float2>, gs_blocks(E * R), 256, 0, s, Z, zstride, y, kcol, m, x, E, R);
+                  float4* xdf, int64_t E, int R, cudaStream_t s) {
+  update_x32(Z, zstride, y, kcol, m, x, xdf, E, R, s);
 }
 
 }  // namespace mwk

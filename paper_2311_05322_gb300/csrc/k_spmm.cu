@@ -6,6 +6,7 @@
 #include <type_traits>
 
 #include "mw_chain.cuh"
+#include "mw_df.cuh"
 #include "mw_internal.h"
 #include "mw_reduce.cuh"
 
@@ -476,35 +477,11 @@ __device__ __forceinline__ void df_mac(float& s_h, float& s_l, float a_h, float 
   s_h = t;
 }
 
-// v = hi + lo with hi the nearest float (ties to even) and lo the nearest float to v - hi, from the bits of v: the
-// significand's upper 24 bits rounded, and the signed remainder (29 bits) converted and scaled.  The same
-// values as conversions and a subtraction in FP64, whose pipe (1/64 of the FP32 rate) bounded this pass at a
-// third of the copy bandwidth.  Zeros, and exponents whose parts would not be normal floats, take that way.
-__device__ __forceinline__ void split_double(double v, float& hi, float& lo) {
-  const long long b = __double_as_longlong(v);
-  const int e = (int)(b >> 52 & 0x7ff) - 1023;
-  if (e < -90 || e > 126) {
-    hi = __double2float_rn(v);
-    lo = __double2float_rn(v - (double)hi);
-    return;
-  }
-  const long long m = (b & 0xfffffffffffffll) | 0x10000000000000ll;      // 53 bits, value m 2^(e - 52)
-  const int up = (int)((m + 0xfffffffll + (m >> 29 & 1)) >> 29);          // 24 bits (or 2^24)
-  const int rem = (int)(m - ((long long)up << 29));
-  const float s = __int_as_float((e + 127 - 23) << 23 | (int)(b >> 32 & 0x80000000ll));
-  hi = (float)up * s;                                                     // exact
-  lo = (float)rem * s * 0x1p-29f;                                         // the conversion rounds, the scaling is exact
-}
-
 // A_df[k] = (re_hi, re_lo, im_hi, im_lo) of a complex FP64 value.
 __global__ void split_df_kernel(const double2* __restrict__ a, float4* __restrict__ o, int64_t n) {
   chain_wait();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double2 v = a[i];
-    float4 r;
-    split_double(v.x, r.x, r.y);
-    split_double(v.y, r.z, r.w);
-    o[i] = r;
+    o[i] = split_df2(a[i]);
   }
 }
 

@@ -1075,14 +1075,13 @@ int read_active(Ctx* c) {
 // r = b - A_f x with per-block partial norms: FP64 arithmetic into w.r in FP64 mode; in mixed
 // mode double-float arithmetic on the FP32 pipes (same accuracy class) with b taken from w.bdf
 // (split once per block solve) and r rounded to FP32 into w.r32, which is all the inner solver's
-// start vector needs.
+// start vector needs; x comes from its double-float copy w.xdf, which the solution update keeps.
 // zero_x: X is known to be 0 (the first outer step), so r = b without the products.
 int outer_residual(Ctx* c, int f, int wp, const double2* X, const double2* B, int R, bool zero_x = false) {
   Work& w = c->work;
   const int64_t E = c->topo.n_edge;
   if (wp == 0)
     return mwk::residual_f64(c->d_row, c->d_col, c->A64[f], X, B, w.r, w.npart, E, R, c->stream, zero_x);
-  if (!zero_x) mwk::split_df(X, w.xdf, E * R, c->stream);
   return mwk::residual_df32(c->d_row, c->d_col, c->Adf[f], w.xdf, w.bdf, w.r32, w.npart, E, R, c->stream, c->row_win,
                             zero_x);
 }
@@ -1203,9 +1202,9 @@ void cycle_finish(Ctx* c, const CycleArgs& a) {
     mwk::update_x_f64((const double2*)a.Zp(w, 0), a.vstride, w.y, w.kcol, a.m, a.X, a.E, a.R, c->stream, c->d_words + kWordKrylov);
   else
     if (a.zb)
-      mwk::update_x_bx(a.Zp(w, 0), a.vstride, w.y, w.kcol, a.m, a.X, a.E, a.R, c->stream, c->d_words + kWordKrylov);
+      mwk::update_x_bx(a.Zp(w, 0), a.vstride, w.y, w.kcol, a.m, a.X, w.xdf, a.E, a.R, c->stream);
     else
-      mwk::update_x_f32((const float2*)a.Zp(w, 0), a.vstride, w.y, w.kcol, a.m, a.X, a.E, a.R, c->stream, c->d_words + kWordKrylov);
+      mwk::update_x_f32((const float2*)a.Zp(w, 0), a.vstride, w.y, w.kcol, a.m, a.X, w.xdf, a.E, a.R, c->stream);
   check_launch("solution update");
   CK(cudaMemcpyAsync(w.h_ivec, w.kcol, sizeof(int32_t) * a.R, cudaMemcpyDeviceToHost, c->stream));
 }

@@ -255,11 +255,10 @@ void solve_hessenberg(const double2* H, const double2* gvec, const int32_t* kcol
 void update_x_f64(const double2* Z, int64_t zstride, const double2* y, const int32_t* kcol, int m, double2* x,
                   int64_t E, int R, cudaStream_t s, int32_t* err = nullptr);
 void update_x_f32(const float2* Z, int64_t zstride, const double2* y, const int32_t* kcol, int m, double2* x,
-                  int64_t E, int R, cudaStream_t s, int32_t* err = nullptr);
-// The same with Z stored as complex BF16 pairs [E][R] per vector (real in the low half), vectors
-// zstride values apart.
-void update_x_bx(const void* Z, int64_t zstride, const double2* y, const int32_t* kcol, int m, double2* x, int64_t E,
-                 int R, cudaStream_t s, int32_t* err);
+                  float4* xdf, int64_t E, int R, cudaStream_t s);
+// Z as complex BF16 pairs.  Both also leave the double-float copy of the new x in xdf.
+void update_x_bx(const void* Z, int64_t zstride, const double2* y, const int32_t* kcol, int m, double2* x, float4* xdf,
+                 int64_t E, int R, cudaStream_t s);
 void reduce_cols(const double* part, int nparts, int R, double* out, cudaStream_t s);
 
 // layout conversions
