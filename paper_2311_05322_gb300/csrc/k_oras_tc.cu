@@ -192,8 +192,9 @@ __global__ void __launch_bounds__(128, 8) gather_b_kernel(const int32_t* __restr
                                                        const int32_t* __restrict__ dofs,
                                                        const float2* __restrict__ r, int R, int Rp,
                                                        uint8_t* __restrict__ Bt, const double* __restrict__ cscale,
-                                                       int64_t ntiles) {
+                                                       int64_t ntiles, const int32_t* __restrict__ go) {
   chain_wait();
+  if (go && *go == 0) return;
   // Blocks of 4 warps walk the tiles with a grid stride.  Per tile (64 dofs), warp w takes dofs
   // 16w .. 16w+15 and lane c the columns c, c + 32, ...: the dof indices come in one coalesced
   // load and are handed out by shuffles, the 16 values of a lane are independent loads, and each
@@ -308,6 +309,7 @@ struct TcArgs {
   int R, N, stages;
   uint32_t tmem_cols;
   int32_t* err;
+  const int32_t* go;        // optional: zero when the kernel starts: nothing is done
 };
 
 // Position in a ring of S stages: the stage and the parity of its current round.  Running counters: a
@@ -479,12 +481,15 @@ __global__ void __launch_bounds__(kThreadsTc, 2) oras_tc_kernel(const TcArgs a) 
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_base;
   chain_wait();   // the set-up above and the tensor memory are this block's own
+  const bool go = !a.go || *a.go != 0;
   const TcTile tl = a.tiles[blockIdx.x];
   const int KT = tl.kt;
   const uint8_t* Wt = a.W + (size_t)tl.w * kATileBytes;
   const uint8_t* Bs = a.Bt + (size_t)tl.g * b_bytes;
 
-  if (warp == 0) {
+  if (!go) {
+    // launched ahead of a step that is not taken
+  } else if (warp == 0) {
     if (lane == 0) {
       // producer: bulk copies of (Wr and Wi tiles, B tile) per k tile
       const uint32_t a_part = a_part_of(tl);
@@ -903,7 +908,8 @@ static void tc_mma(const TcPlan& p, TcArgs a, int R, int stages, bool persistent
 }
 
 void oras_apply_tc(const TcPlan& p, const OrasTopo& tp, const void* W, const float2* r, float2* z, int R,
-                   void* scratch, cudaStream_t s, int stages, const double* in_scale, bool z_bf16) {
+                   void* scratch, cudaStream_t s, int stages, const double* in_scale, bool z_bf16,
+                   const int32_t* go) {
   const int Rp = rpad(R);
   note_launch(1);
   const size_t gsm = (size_t)2 * Rp * 128;
@@ -914,10 +920,11 @@ void oras_apply_tc(const TcPlan& p, const OrasTopo& tp, const void* W, const flo
   }
   const int64_t gblocks = std::min<int64_t>(p.n_ktiles_total, 152 * 8);    // one resident wave
   launch_chained(gather_b_kernel, (unsigned)std::max<int64_t>(gblocks, 1), 128, gsm, s, p.gt_sub, p.gt_kt,
-      tp.dof_ptr, tp.dofs, r, R, Rp, (uint8_t*)scratch, in_scale, p.n_ktiles_total);
+      tp.dof_ptr, tp.dofs, r, R, Rp, (uint8_t*)scratch, in_scale, p.n_ktiles_total, go);
   TcArgs a{};
   a.own_glob = tp.own_glob;
   a.z_bf16 = z_bf16 ? 1 : 0;
+  a.go = go;
   a.vec = R % (z_bf16 ? 4 : 2) == 0 && ((uintptr_t)z & 15) == 0;
   a.W = (const uint8_t*)W;
   a.Bt = (const uint8_t*)scratch;

@@ -72,9 +72,10 @@ void tc_sweep(const TcPlan& p, const TcRow* rows, const int32_t* src, int n_src,
 // stages: shared-memory pipeline depth of the MMA kernel (0 = default; the result does not depend
 // on it, only the speed).  in_scale (may be null): per-column factor of r (z = M^{-1}(r * in_scale)).
 // z_bf16: z is written as complex BF16 pairs (real in the low half), 4 bytes per value, row stride R values.
+// go (may be null): device word; zero when the kernels start: nothing is done.
 void oras_apply_tc(const TcPlan& p, const OrasTopo& tp, const void* W, const float2* r, float2* z, int R,
                    void* scratch, cudaStream_t s, int stages = 0, const double* in_scale = nullptr,
-                   bool z_bf16 = false);
+                   bool z_bf16 = false, const int32_t* go = nullptr);
 // Pipeline depths the MMA kernel accepts for R columns: [tc_min_stages, tc_max_stages(R)].
 constexpr int tc_min_stages = 2;
 int tc_max_stages(int R);

@@ -112,8 +112,9 @@ __global__ void __launch_bounds__(512, CV == 1 ? 4 : 1) spmm_staged_kernel(const
                                                           const int32_t* __restrict__ ci,
                                                           const float2* __restrict__ A, const XT* __restrict__ X,
                                                           float2* __restrict__ Y, int64_t E, int R, int lpr_log2,
-                                                          int rows) {
+                                                          int rows, const int32_t* __restrict__ go) {
   chain_wait();
+  if (go && *go == 0) return;   // launched ahead of a step that is not taken
   constexpr int NB = VEC * CV >= 4 ? 2 : 4;
   using Pack = XPack<XT, VEC>;
   extern __shared__ float4 smem4[];
@@ -260,7 +261,7 @@ inline size_t staged_smem(int rows, int nnz) { return 16 * (size_t)((rows + 4) /
 
 template <typename XT, int VEC>
 void spmm_staged(const int64_t* rp, const int32_t* ci, const float2* A, const XT* X, float2* Y, int64_t E, int R,
-                 cudaStream_t s, int threads, size_t smem) {
+                 cudaStream_t s, int threads, size_t smem, const int32_t* go) {
   const int packs = (R + VEC - 1) / VEC, rows = staged_rows(threads);
   int l = 0;
   while ((1 << l) < packs && l < 5) ++l;
@@ -268,11 +269,11 @@ void spmm_staged(const int64_t* rp, const int32_t* ci, const float2* A, const XT
   const unsigned blocks = (unsigned)((E + rows - 1) / rows);
   note_launch(1);
   if (cv == 1)
-    launch_chained(spmm_staged_kernel<XT, VEC, 1>, blocks, threads, smem, s, rp, ci, A, X, Y, E, R, l, rows);
+    launch_chained(spmm_staged_kernel<XT, VEC, 1>, blocks, threads, smem, s, rp, ci, A, X, Y, E, R, l, rows, go);
   else if (cv == 2)
-    launch_chained(spmm_staged_kernel<XT, VEC, 2>, blocks, threads, smem, s, rp, ci, A, X, Y, E, R, l, rows);
+    launch_chained(spmm_staged_kernel<XT, VEC, 2>, blocks, threads, smem, s, rp, ci, A, X, Y, E, R, l, rows, go);
   else
-    launch_chained(spmm_staged_kernel<XT, VEC, 4>, blocks, threads, smem, s, rp, ci, A, X, Y, E, R, l, rows);
+    launch_chained(spmm_staged_kernel<XT, VEC, 4>, blocks, threads, smem, s, rp, ci, A, X, Y, E, R, l, rows, go);
 }
 
 // The staged product when the records of a block fit 48 KB of shared memory and element offsets 31 bits;
@@ -283,17 +284,17 @@ void spmm_staged(const int64_t* rp, const int32_t* ci, const float2* A, const XT
 // (BF16) at 32 columns, 375 and 300 us at 64, 1,047 and 617 us at 128; the floor of the bytes is 55 us at 32.
 template <typename XT>
 bool spmm_staged_launch(const int64_t* rp, const int32_t* ci, const float2* A, const XT* X, float2* Y, int64_t E,
-                        int R, cudaStream_t s, int threads, const int* win) {
+                        int R, cudaStream_t s, int threads, const int* win, const int32_t* go) {
   if (threads != 128 && threads != 256 && threads != 512) threads = 256;
   const size_t smem = staged_smem(staged_rows(threads), win[threads == 128 ? 0 : threads == 256 ? 1 : 2]);
   if ( R < 1 || R > 128 || smem > 48 * 1024 || E * R > INT32_MAX) return false;
   const auto fits = [&](int vec) { return R % vec == 0 && (uintptr_t)X % (vec * sizeof(XT)) == 0; };
   if (R >= 16 && sizeof(XT) == 4 && fits(4))
-    spmm_staged<XT, sizeof(XT) == 4 ? 4 : 2>(rp, ci, A, X, Y, E, R, s, threads, smem);
+    spmm_staged<XT, sizeof(XT) == 4 ? 4 : 2>(rp, ci, A, X, Y, E, R, s, threads, smem, go);
   else if (R > 32 && fits(2))
-    spmm_staged<XT, 2>(rp, ci, A, X, Y, E, R, s, threads, smem);
+    spmm_staged<XT, 2>(rp, ci, A, X, Y, E, R, s, threads, smem, go);
   else
-    spmm_staged<XT, 1>(rp, ci, A, X, Y, E, R, s, threads, smem);
+    spmm_staged<XT, 1>(rp, ci, A, X, Y, E, R, s, threads, smem, go);
   return true;
 }
 
@@ -375,8 +376,8 @@ void spmm_f64(const int64_t* rp, const int32_t* ci, const double2* A, const doub
   spmm_launch<double2>(rp, ci, A, X, Y, E, R, s, threads);
 }
 void spmm_f32(const int64_t* rp, const int32_t* ci, const float2* A, const float2* X, float2* Y, int64_t E, int R,
-              cudaStream_t s, int threads, const int* win) {
-  if (spmm_staged_launch<float2>(rp, ci, A, X, Y, E, R, s, threads, win)) return;
+              cudaStream_t s, int threads, const int* win, const int32_t* go) {
+  if (spmm_staged_launch<float2>(rp, ci, A, X, Y, E, R, s, threads, win, go)) return;
   spmm_launch<float2>(rp, ci, A, X, Y, E, R, s, threads);
 }
 
@@ -396,8 +397,8 @@ bool spmm_halo_f32(const SpmmDev& p, const float2* A, const float2* X, float2* Y
 }
 
 void spmm_f32_bx(const int64_t* rp, const int32_t* ci, const float2* A, const void* X, float2* Y, int64_t E, int R,
-                 cudaStream_t s, int threads, const int* win) {
-  if (spmm_staged_launch<uint32_t>(rp, ci, A, (const uint32_t*)X, Y, E, R, s, threads, win)) return;
+                 cudaStream_t s, int threads, const int* win, const int32_t* go) {
+  if (spmm_staged_launch<uint32_t>(rp, ci, A, (const uint32_t*)X, Y, E, R, s, threads, win, go)) return;
   if (threads != 128 && threads != 256 && threads != 512) threads = 256;
   if (R > 128) return;
   note_launch(1);

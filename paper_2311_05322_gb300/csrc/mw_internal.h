@@ -168,8 +168,10 @@ void reassemble(const int64_t* cptr, const int32_t* contrib, int64_t nnz, const 
 // FP32 kernels' blocks).
 void spmm_f64(const int64_t* rp, const int32_t* ci, const double2* A, const double2* X, double2* Y, int64_t E,
               int R, cudaStream_t s, int threads = 256);
+// go (may be null): device word; zero when the kernel starts: nothing is done (only the staged product looks).
 void spmm_f32(const int64_t* rp, const int32_t* ci, const float2* A, const float2* X, float2* Y, int64_t E, int R,
-              cudaStream_t s, int threads, const int* win);
+              cudaStream_t s, int threads, const int* win,
+              const int32_t* go = nullptr);
 // Bounds of one block of the halo-tiled SpMM plan: columns (halo), rows and nonzeros.
 constexpr int kHaloMax = 480, kHaloRows = 512, kHaloNnz = 4096;
 // Device copy of mw::SpmmPlan (halo_max bounds every block's halo).
@@ -190,7 +192,8 @@ struct SpmmDev {
 bool spmm_halo_f32(const SpmmDev& p, const float2* A_blk, const float2* X, float2* Y, int R, cudaStream_t s);
 // Y = A X (FP32) with X stored as complex BF16 pairs [E][R] (real in the low half).
 void spmm_f32_bx(const int64_t* rp, const int32_t* ci, const float2* A, const void* X, float2* Y, int64_t E, int R,
-                 cudaStream_t s, int threads, const int* win);
+                 cudaStream_t s, int threads, const int* win,
+                 const int32_t* go = nullptr);
 // A_blk[q] = A32[src[q]].
 void spmm_plan_values(const SpmmDev& p, const float2* A32, int64_t nnz, float2* A_blk, cudaStream_t s);
 // Split complex FP64 values into double-float (re_hi, re_lo, im_hi, im_lo).
