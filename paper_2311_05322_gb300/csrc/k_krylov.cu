@@ -712,7 +712,8 @@ __global__ void __launch_bounds__(kThreads) colnorm2_kernel(const T* __restrict_
       for (int q = 0; q < CPL; ++q)
         if (c0 + q < R) {
           const T v = x[row * R + c0 + q];
-          nrm[q] += (double)v.x * v.x + (double)v.y * v.y;
+          // zeros, most of a right-hand side, add nothing: warps full of them skip the slow FP64 operations
+          if (v.x != 0 || v.y != 0) nrm[q] += (double)v.x * v.x + (double)v.y * v.y;
         }
   store_column_norms(nrm, red, tpr, c0, 1, R, npart + (int64_t)blockIdx.x * R);
 }
