@@ -19,6 +19,10 @@ namespace mwk {
 
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Lets the next launch's blocks in before this launch ends (the one use: the gather lets the MMA kernel in, whose
+// blocks then set up and start copies that do not depend on the gather).
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 template <typename... P, typename... A>
 inline void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
