@@ -7,8 +7,8 @@
 // calls it (also those with nothing to do), so a launch never completes before its predecessor, and a launch that
 // is not chained keeps the stream's usual order.  In a captured stream the launches are ordinary ones.
 //
-// A kernel's blocks come in as the last blocks of its predecessor leave; they are not let in earlier
-// (griddepcontrol.launch_dependents): blocks that wait on an SM take the place of working ones where a kernel
+// A kernel's blocks come in as the last blocks of its predecessor leave; but for the MMA kernel behind its gather
+// (chain_next) they are not let in earlier: blocks that wait on an SM take the place of working ones where a kernel
 // counts on an even spread over the SMs.  Subdomain inverses of 30x30x13 cells: 228 ms with ordinary launches,
 // 226 ms so, 349 ms let in early; its gradient evaluation 14.1, 13.4 and 13.8 ms; sphere 12^3 solve 1.91, 1.61 and
 // 1.64 ms; 16 sparse subdomains 17.6, 15.9 and 16.7 ms; training epochs at 2048 inputs 16.2, 14.1 and 17.0 ms.
