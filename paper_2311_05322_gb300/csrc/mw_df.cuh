@@ -7,7 +7,7 @@ namespace mwk {
 // v = hi + lo with hi the nearest float (ties to even) and lo the nearest float to v - hi, from the bits of v: the
 // significand's upper 24 bits rounded, and the signed remainder (29 bits) converted and scaled.  The same
 // values as conversions and a subtraction in FP64, whose pipe (1/64 of the FP32 rate) bounded this pass at a
-// third of the copy bandwidth.  Exponents whose parts would not be normal floats take that way.
+// third of the copy bandwidth.  Exponents outside [-90, 126], where a part or its scale may not be exact, take that way.
 __device__ __forceinline__ void split_double(double v, float& hi, float& lo) {
   const long long b = __double_as_longlong(v);
   const int e = (int)(b >> 52 & 0x7ff) - 1023;
@@ -26,7 +26,9 @@ __device__ __forceinline__ void split_double(double v, float& hi, float& lo) {
   const int rem = (int)(m - ((long long)up << 29));
   const float s = __int_as_float((e + 127 - 23) << 23 | (int)(b >> 32 & 0x80000000ll));
   hi = (float)up * s;                                                     // exact
-  lo = (float)rem * s * 0x1p-29f;                                         // the conversion rounds, the scaling is exact
+  // the conversion rounds, the scaling is exact: s 2^-29 is a power of two, at least 2^-142 (denormals are on).  rem s
+  // alone, with |rem| up to 2^28, would overflow from exponent 123 on.
+  lo = (float)rem * (s * 0x1p-29f);
 }
 
 // (re_hi, re_lo, im_hi, im_lo) of a complex FP64 value.

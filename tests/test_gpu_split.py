@@ -34,3 +34,26 @@ def test_split_product_against_fp64(scale):
     bound = 2.0 ** -44 * (A.abs() @ x.abs()) + 2.0 ** -148 * A.abs().sum(1, keepdim=True)
     assert torch.all((y.cpu() - ref).abs() <= bound)
     c.close()
+
+
+@pytest.mark.parametrize("exponent", [121, 122, 123, 124, 125, 126, 127])
+def test_split_near_the_largest_floats(exponent):
+    """Values of one binade up to the largest floats, on a mesh whose matrix entries are small enough for their
+    products: both parts are ordinary floats, so the bound is the one above without its denormal term."""
+    from paper_2311_05322_gb300 import mw
+    h = 2.0 ** 30
+    m = kuhn_mesh(5, 4, 3, lo=(-2 * h, -1.5 * h, -h), hi=(2 * h, 1.5 * h, h))
+    c = mw.Context(0)
+    E = c.set_mesh(m.xyz, m.tets).n_edge
+    c.assemble([1e7 / h], np.tile([EPS_MATCHING.real, EPS_MATCHING.imag], (m.n_tet, 1)), EPS_MATCHING)
+    _, _, _, rp, ci = c.get_topology()
+    A = torch.sparse_csr_tensor(torch.from_numpy(rp), torch.from_numpy(ci.astype(np.int64)),
+                                torch.from_numpy(c.get_matrix(0)), (E, E)).to_dense()
+    rng = np.random.default_rng(exponent)
+    part = lambda: rng.uniform(1.0, 1.99, (E, 3)) * rng.choice([-1.0, 1.0], (E, 3))
+    x = torch.from_numpy((part() + 1j * part()) * 2.0 ** exponent)
+    y = torch.empty((E, 3), dtype=torch.complex128, device="cuda")
+    c.apply_matrix(0, 3, x.cuda(), y, 3)
+    torch.cuda.synchronize()
+    c.close()
+    assert torch.all((y.cpu() - A @ x).abs() <= 2.0 ** -44 * (A.abs() @ x.abs()))
