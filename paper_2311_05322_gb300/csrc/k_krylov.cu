@@ -1516,10 +1516,10 @@ template <typename ZT>
 static void update_x32(const ZT* Z, int64_t zstride, const double2* y, const int32_t* kcol, int m, double2* x,
                        float4* xdf, int64_t E, int R, cudaStream_t s) {
   note_launch(1);
-  const size_t smem = sizeof(float2) * m * R;   // at most 63 KB
+  const size_t smem = sizeof(float2) * m * R;   // at most 63 KB, with the kernel's static memory on top
   auto go = [&](auto kernel, int vec) {
     static bool attr[3] = {};
-    if (smem > 48 * 1024 && !attr[vec])
+    if (!attr[vec])
       attr[vec] = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024) == cudaSuccess;
     const int64_t rows = (int64_t)(256 / (R / vec)) * kUxRows;
     launch_chained(kernel, (unsigned)std::min<int64_t>((E + rows - 1) / rows, 152 * 4), 256, smem, s, Z, zstride, y,
