@@ -31,6 +31,7 @@
 #include "k_inverse.h"
 #include "mw_chain.cuh"
 #include "mw_internal.h"
+#include "mw_smem.h"
 
 namespace mwk {
 namespace {
@@ -534,10 +535,9 @@ template <typename T>
 void invert_all(const InvBatch& bt, const OrasTopo& tp, T* ws, T* dinv, int32_t* status, cudaStream_t st) {
   constexpr size_t up_smem = sizeof(T) * NB * 2 * kUp * 2;
   constexpr size_t pa_smem = sizeof(T) * (NB * (kPan + 1) + NB * NB);
-  static const cudaError_t attr[2] = {
-      cudaFuncSetAttribute(inv_update_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)up_smem),
-      cudaFuncSetAttribute(inv_panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pa_smem)};
-  (void)attr;   // a failure shows at the launch
+  static SmemLimit update_limit, panel_limit;
+  update_limit.raise(inv_update_kernel<T>, up_smem);
+  panel_limit.raise(inv_panel_kernel<T>, pa_smem);
   for (int k = 0; k < bt.steps; ++k) {
     const int kb = k * NB, jt = (bt.np_max + kPan - 1) / kPan;
     const int32_t* nsws = bt.d_nsw + (size_t)k * bt.count;

@@ -21,6 +21,7 @@
 #include "mw_df.cuh"
 #include "mw_internal.h"
 #include "mw_reduce.cuh"
+#include "mw_smem.h"
 
 namespace mwk {
 namespace {
@@ -1260,12 +1261,8 @@ bool update_x_bulk(const T* Z, int64_t zstride, const double2* y, const int32_t*
                    int R, int32_t* err, cudaStream_t s) {
   const bool aligned = ((uintptr_t)Z % 16 == 0) && ((zstride * sizeof(T)) % 16 == 0);
   if (!err || !aligned || R < 16 || R > 128 || m < 1) return false;
-  static bool attr = false;   // one per instantiation
-  if (!attr) {
-    // 226 KB: the kernel's static shared memory shares the 227 KB per block
-    attr = cudaFuncSetAttribute(update_x_bulk_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                226 * 1024) == cudaSuccess;
-  }
+  static SmemLimit limit;   // one per instantiation
+  limit.raise(update_x_bulk_kernel<T>, 226 * 1024);   // its static shared memory shares the 227 KB per block
   int NS = kBdStages;
   while (NS > 2 && ux_smem_bytes(R, m, NS) > (size_t)226 * 1024) --NS;
   launch_chained(update_x_bulk_kernel<T>, 152 * 2, kBdThreads, ux_smem_bytes(R, m, NS), s, Z, zstride, y,
@@ -1284,14 +1281,8 @@ int dots_launch(const T* V, int64_t vstride, int nvec, const T* w, int64_t E, in
   note_launch(1);
   const bool aligned = ((uintptr_t)V % 16 == 0) && ((uintptr_t)w % 16 == 0) && ((vstride * sizeof(T)) % 16 == 0);
   if (err && aligned && R >= 16 && R <= 128 && nvec >= 1) {
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(cgs_dots_bulk_kernel<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)kBdMaxSmem);
-      cudaFuncSetAttribute(cgs_dots_bulk_kernel<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)kBdMaxSmem);
-      attr = true;
-    }
+    static SmemLimit limit;
+    limit.raise(cgs_dots_bulk_kernel<T>, kBdMaxSmem);
     const int G = kBdConsumers / R;
     const int VG = std::min(64, 2048 / R);
     const int nb = 152 * 2;
@@ -1329,13 +1320,8 @@ int update_launch(const T* V, int64_t vstride, int nvec, const double2* h, T* w,
   note_launch(1);
   const bool aligned = ((uintptr_t)V % 16 == 0) && ((uintptr_t)w % 16 == 0) && ((vstride * sizeof(T)) % 16 == 0);
   if (err && aligned && R >= 16 && R <= 128 && nvec >= 1) {
-    static bool attr = false;
-    if (!attr) {
-      attr = cudaFuncSetAttribute(cgs_update_bulk_kernel<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  226 * 1024) == cudaSuccess &&
-             cudaFuncSetAttribute(cgs_update_bulk_kernel<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  226 * 1024) == cudaSuccess;
-    }
+    static SmemLimit limit;
+    limit.raise(cgs_update_bulk_kernel<T>, 226 * 1024);
     int NS = stages >= 2 && stages <= kBdMaxStages ? stages : kBdStages;
     while (NS > 2 && bu_smem_bytes(R, nvec, NS) > (size_t)226 * 1024) --NS;
     const int G = kBdConsumers / R;
@@ -1346,26 +1332,23 @@ int update_launch(const T* V, int64_t vstride, int nvec, const double2* h, T* w,
   }
   Shape sh = shape_for(R);
   const size_t smem = sizeof(T) * nvec * R + 16 + sizeof(double) * kThreads * sh.cpl;
-  static bool attr = false;
-  if (!attr) {
-    const int mx = 200 * 1024;
-    cudaFuncSetAttribute(cgs_update_kernel<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    cudaFuncSetAttribute(cgs_update_kernel<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    cudaFuncSetAttribute(cgs_update_kernel<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx);
-    attr = true;
-  }
+  static SmemLimit limit[3];
+  constexpr size_t mx = 200 * 1024;
   const int rows_per_block = kThreads >> sh.tpr_log2;
   const int nb = (int)std::min<int64_t>(kBlocks, (E + rows_per_block - 1) / rows_per_block);
   switch (sh.cpl) {
     case 1:
+      limit[0].raise(cgs_update_kernel<T, 1>, mx);
       launch_chained(cgs_update_kernel<T, 1>, nb, kThreads, smem, s, V, vstride, nvec, h, w, E, R, sh.tpr_log2,
           npart, vscale);
       break;
     case 2:
+      limit[1].raise(cgs_update_kernel<T, 2>, mx);
       launch_chained(cgs_update_kernel<T, 2>, nb, kThreads, smem, s, V, vstride, nvec, h, w, E, R, sh.tpr_log2,
           npart, vscale);
       break;
     default:
+      limit[2].raise(cgs_update_kernel<T, 4>, mx);
       launch_chained(cgs_update_kernel<T, 4>, nb, kThreads, smem, s, V, vstride, nvec, h, w, E, R, sh.tpr_log2,
           npart, vscale);
       break;
@@ -1517,10 +1500,9 @@ static void update_x32(const ZT* Z, int64_t zstride, const double2* y, const int
                        float4* xdf, int64_t E, int R, cudaStream_t s) {
   note_launch(1);
   const size_t smem = sizeof(float2) * m * R;   // at most 63 KB, with the kernel's static memory on top
+  static SmemLimit limit[3];
   auto go = [&](auto kernel, int vec) {
-    static bool attr[3] = {};
-    if (!attr[vec])
-      attr[vec] = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024) == cudaSuccess;
+    limit[vec].raise(kernel, 64 * 1024);
     const int64_t rows = (int64_t)(256 / (R / vec)) * kUxRows;
     launch_chained(kernel, (unsigned)std::min<int64_t>((E + rows - 1) / rows, 152 * 4), 256, smem, s, Z, zstride, y,
                    kcol, m, x, xdf, E, R);

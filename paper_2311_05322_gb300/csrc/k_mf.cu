@@ -18,6 +18,7 @@
 
 #include "k_mf.h"
 #include "mw_internal.h"
+#include "mw_smem.h"
 
 namespace mwk {
 namespace {
@@ -410,11 +411,8 @@ void mf_gemm(const MfTask* tasks, const MfTile* tiles, int n_tiles, const MfSpli
              const float2* fac, const int32_t* idx, int R, float2* arena, float2* partial, cudaStream_t s) {
   if (n_tiles <= 0) return;
   note_launch(1);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(mf_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMfSmem);
-    attr = true;
-  }
+  static SmemLimit limit;
+  limit.raise(mf_gemm_kernel, kMfSmem);
   dim3 g((unsigned)n_tiles, (unsigned)((R + kMfCols - 1) / kMfCols));
   mf_gemm_kernel<<<g, kMfThreads, kMfSmem, s>>>(tasks, tiles, fac, idx, R, arena, partial);
   if (n_splits > 0) {

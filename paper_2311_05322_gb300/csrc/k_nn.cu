@@ -11,6 +11,7 @@
 #include "k_nn.h"
 #include "mw_chain.cuh"
 #include "mw_internal.h"
+#include "mw_smem.h"
 
 namespace mwk {
 namespace {
@@ -769,9 +770,8 @@ static void conv_bwd(const float* x, const float* w, const float* dy, float* dx,
       CI / CIG), kConvThreads, 0, s, dy, w, x, dx, B);
   int64_t chunk = 0;
   const int nchunk = conv_chunks(LAYER, B, chunk);
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      convT_bwd_w_kernel<D, CI, CO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBwdWSmem);
-  (void)attr;   // a failure shows at the launch
+  static SmemLimit limit;
+  limit.raise(convT_bwd_w_kernel<D, CI, CO>, kBwdWSmem);
   launch_chained(convT_bwd_w_kernel<D, CI, CO>, CI / kBwdWCi * CO * 4 * nchunk + CO * B, kBwdWThreads, kBwdWSmem,
       s, x, dy, wpart, bpart, B, chunk, nchunk);
 }

@@ -2,6 +2,7 @@
 // (ORAS apply), Sec. IV-C.  Apply:  z[own_s] = W_s r[dofs_s]  for every s (owners partition the
 // edges: no atomics).
 #include "mw_internal.h"
+#include "mw_smem.h"
 #include "k_oras.h"
 
 namespace mwk {
@@ -307,11 +308,8 @@ void gj_all(const OrasBatch& bt, T* ws, T* dinv, int32_t* status, cudaStream_t s
   const int nb = bt.count;
   const int64_t nmax = bt.nmax;
   const size_t smem = sizeof(T) * 2 * 64 * NB;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(gj_update_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr_set = true;
-  }
+  static SmemLimit limit;
+  limit.raise(gj_update_kernel<T>, smem);
   const int64_t kend = lim ? lim_max : nmax;
   for (int64_t kb = 0; kb < kend; kb += NB) {
     note_launch(4);

@@ -34,6 +34,7 @@
 #include "mw_async.cuh"
 #include "mw_chain.cuh"
 #include "mw_internal.h"
+#include "mw_smem.h"
 
 namespace mwk {
 namespace {
@@ -895,14 +896,17 @@ int tc_stages(int N) {
   return st > 6 ? 6 : (st < 2 ? 2 : st);
 }
 
+// Most dynamic shared memory of an MMA block: 1 KB of the 227 KB is left for its static shared memory.
+constexpr size_t kTcMaxSmem = (size_t)226 * 1024;
+
 size_t tc_smem_bytes(int N, int stages) { return (size_t)stages * (2 * kATileBytes + N * 128) + 1024; }
 
 
 int tc_max_stages(int R) {
-  // the kernel holds 8 stage barriers; 1 KB of the 227 KB is left for its static shared memory
+  // the kernel holds 8 stage barriers
   const int N = 2 * rpad(R);
   int st = tc_min_stages;
-  while (st < 8 && tc_smem_bytes(N, st + 1) <= (size_t)226 * 1024) ++st;
+  while (st < 8 && tc_smem_bytes(N, st + 1) <= kTcMaxSmem) ++st;
   return st;
 }
 
@@ -927,11 +931,8 @@ static void tc_mma(const TcPlan& p, TcArgs a, int R, int stages, bool persistent
     const int per_sm = 4 * cols <= 512 ? 2 : 1;
     size_t smem = tc_smem_bytes(N, stages);
     if (per_sm == 1 && smem < (size_t)120 * 1024) smem = (size_t)120 * 1024;
-    static size_t pattr = 0;
-    if (smem > pattr) {
-      cudaFuncSetAttribute(oras_tc_persistent_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      pattr = smem;
-    }
+    static SmemLimit limit;
+    limit.raise(oras_tc_persistent_kernel, kTcMaxSmem);
     const int grid = (int)std::min<int64_t>(p.n_mtiles, (int64_t)per_sm * 152);
     launch_chained(oras_tc_persistent_kernel, (unsigned)std::max(grid, 1), kThreadsTc, smem, s, a,
         (int)p.n_mtiles);
@@ -941,11 +942,8 @@ static void tc_mma(const TcPlan& p, TcArgs a, int R, int stages, bool persistent
   // shared-memory request keeps one CTA per SM
   size_t smem = tc_smem_bytes(N, stages);
   if (cols > 256 && smem < (size_t)120 * 1024) smem = (size_t)120 * 1024;
-  static size_t attr = 0;
-  if (smem > attr) {
-    cudaFuncSetAttribute(oras_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr = smem;
-  }
+  static SmemLimit limit;
+  limit.raise(oras_tc_kernel, kTcMaxSmem);
   launch_chained(oras_tc_kernel, (unsigned)p.n_mtiles, kThreadsTc, smem, s, a);
 }
 
@@ -954,12 +952,7 @@ void oras_apply_tc(const TcPlan& p, const OrasTopo& tp, const void* W, const flo
                    const int32_t* go) {
   const int Rp = rpad(R);
   note_launch(1);
-  const size_t gsm = (size_t)2 * Rp * 128;
-  static size_t gattr = 0;
-  if (gsm > 48 * 1024 && gsm > gattr) {
-    cudaFuncSetAttribute(gather_b_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm);
-    gattr = gsm;
-  }
+  const size_t gsm = (size_t)2 * Rp * 128;   // at most 32 KB
   const int64_t gblocks = std::min<int64_t>(p.n_ktiles_total, 152 * 8);    // one resident wave
   // the MMA kernel comes in while the gather runs where it has at most two waves of blocks: 27 subdomains, 16 columns
   // 33.9 -> 32.3 us; 731 tiles lost 0.4 % of a gradient evaluation

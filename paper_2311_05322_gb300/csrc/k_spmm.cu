@@ -9,6 +9,7 @@
 #include "mw_df.cuh"
 #include "mw_internal.h"
 #include "mw_reduce.cuh"
+#include "mw_smem.h"
 
 namespace mwk {
 namespace {
@@ -384,11 +385,8 @@ void spmm_f32(const int64_t* rp, const int32_t* ci, const float2* A, const float
 bool spmm_halo_f32(const SpmmDev& p, const float2* A, const float2* X, float2* Y, int R, cudaStream_t s) {
   if (!p.n_block || p.halo_max > kHaloMax || R < 2 || R > 128 || (R & 1) || ((uintptr_t)X & 15)) return false;
   const size_t smem = kHaloSmem;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(spmm_halo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    attr = true;
-  }
+  static SmemLimit limit;
+  limit.raise(spmm_halo_kernel, smem);
   const int nchunk = (R + kHaloCols - 1) / kHaloCols;
   note_launch(1);
   spmm_halo_kernel<<<(unsigned)(p.n_block * nchunk), kHaloThreads, smem, s>>>(p.blk_row, p.blk_halo, p.halo, p.rows,
@@ -693,9 +691,8 @@ static int residual_df32_launch(const int64_t* rp, const int32_t* ci, const floa
   const int rows = win[1] <= kCap ? 32 : 16, cap = win[1] <= kCap ? win[1] : win[0];
   const int blocks = (int)std::min<int64_t>(152 * 4, (E + rows - 1) / rows);
   const size_t smem = (zero_x ? 0 : (size_t)cap * 20) + 4 * (rows + 1);
-  static const cudaError_t attr = cudaFuncSetAttribute(residual_df32_kernel<CV, false>,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, kCap * 20 + 256);
-  (void)attr;   // a failure shows at the launch
+  static SmemLimit limit;
+  limit.raise(residual_df32_kernel<CV, false>, kCap * 20 + 256);
   if (zero_x)
     launch_chained(residual_df32_kernel<CV, true>, blocks, 256, smem, s, rp, ci, A, X, Bdf, Rv, part, E, R, l,
         rows, cap);
