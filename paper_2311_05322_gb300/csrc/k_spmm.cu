@@ -51,8 +51,9 @@ __device__ __forceinline__ float2 xval(uint32_t u) {
 template <typename T, int CPL, typename XT = T>
 __global__ void __launch_bounds__(512) spmm_kernel(const int64_t* __restrict__ rp, const int32_t* __restrict__ ci,
                                                    const T* __restrict__ A, const XT* __restrict__ X, T* __restrict__ Y,
-                                                   int64_t E, int R, int tpr_log2) {
+                                                   int64_t E, int R, int tpr_log2, const int32_t* __restrict__ go) {
   chain_wait();
+  if (go && *go == 0) return;   // launched ahead of a step that is not taken
   constexpr int NB = 8 / CPL;
   const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t row = g >> tpr_log2;
@@ -233,7 +234,7 @@ inline Shape shape_for(int R) {
 
 template <typename T>
 void spmm_launch(const int64_t* rp, const int32_t* ci, const T* A, const T* X, T* Y, int64_t E, int R,
-                 cudaStream_t s, int threads) {
+                 cudaStream_t s, int threads, const int32_t* go = nullptr) {
   if (threads != 128 && threads != 256 && threads != 512) threads = 256;
   note_launch(1);
   Shape sh = shape_for(R);
@@ -245,13 +246,13 @@ void spmm_launch(const int64_t* rp, const int32_t* ci, const T* A, const T* X, T
   const int blocks = (int)((nthr + threads - 1) / threads);
   switch (sh.cpl) {
     case 1:
-      launch_chained(spmm_kernel<T, 1>, blocks, threads, 0, s, rp, ci, A, X, Y, E, R, sh.tpr_log2);
+      launch_chained(spmm_kernel<T, 1>, blocks, threads, 0, s, rp, ci, A, X, Y, E, R, sh.tpr_log2, go);
       break;
     case 2:
-      launch_chained(spmm_kernel<T, 2>, blocks, threads, 0, s, rp, ci, A, X, Y, E, R, sh.tpr_log2);
+      launch_chained(spmm_kernel<T, 2>, blocks, threads, 0, s, rp, ci, A, X, Y, E, R, sh.tpr_log2, go);
       break;
     default:
-      launch_chained(spmm_kernel<T, 4>, blocks, threads, 0, s, rp, ci, A, X, Y, E, R, sh.tpr_log2);
+      launch_chained(spmm_kernel<T, 4>, blocks, threads, 0, s, rp, ci, A, X, Y, E, R, sh.tpr_log2, go);
       break;
   }
 }
@@ -323,7 +324,8 @@ __global__ void __launch_bounds__(kHaloThreads, 2)
                      const int32_t* __restrict__ halo, const int32_t* __restrict__ rows,
                      const int64_t* __restrict__ rptr, const uint16_t* __restrict__ lcol,
                      const float2* __restrict__ A, const float2* __restrict__ X, float2* __restrict__ Y, int R,
-                     int nchunk) {
+                     int nchunk, const int32_t* __restrict__ go) {
+  if (go && *go == 0) return;   // launched ahead of a step that is not taken
   extern __shared__ float4 smem4[];
   float2* sX = reinterpret_cast<float2*>(smem4);
   float2* sA = sX + (size_t)kHaloMax * kHaloCols;
@@ -379,10 +381,11 @@ void spmm_f64(const int64_t* rp, const int32_t* ci, const double2* A, const doub
 void spmm_f32(const int64_t* rp, const int32_t* ci, const float2* A, const float2* X, float2* Y, int64_t E, int R,
               cudaStream_t s, int threads, const int* win, const int32_t* go) {
   if (spmm_staged_launch<float2>(rp, ci, A, X, Y, E, R, s, threads, win, go)) return;
-  spmm_launch<float2>(rp, ci, A, X, Y, E, R, s, threads);
+  spmm_launch<float2>(rp, ci, A, X, Y, E, R, s, threads, go);
 }
 
-bool spmm_halo_f32(const SpmmDev& p, const float2* A, const float2* X, float2* Y, int R, cudaStream_t s) {
+bool spmm_halo_f32(const SpmmDev& p, const float2* A, const float2* X, float2* Y, int R, cudaStream_t s,
+                   const int32_t* go) {
   if (!p.n_block || p.halo_max > kHaloMax || R < 2 || R > 128 || (R & 1) || ((uintptr_t)X & 15)) return false;
   const size_t smem = kHaloSmem;
   static SmemLimit limit;
@@ -390,7 +393,7 @@ bool spmm_halo_f32(const SpmmDev& p, const float2* A, const float2* X, float2* Y
   const int nchunk = (R + kHaloCols - 1) / kHaloCols;
   note_launch(1);
   spmm_halo_kernel<<<(unsigned)(p.n_block * nchunk), kHaloThreads, smem, s>>>(p.blk_row, p.blk_halo, p.halo, p.rows,
-                                                                           p.rptr, p.lcol, A, X, Y, R, nchunk);
+                                                                           p.rptr, p.lcol, A, X, Y, R, nchunk, go);
   return true;
 }
 
@@ -406,13 +409,13 @@ void spmm_f32_bx(const int64_t* rp, const int32_t* ci, const float2* A, const vo
   const uint32_t* Xb = (const uint32_t*)X;
   switch (sh.cpl) {
     case 1:
-      launch_chained(spmm_kernel<float2, 1, uint32_t>, blocks, threads, 0, s, rp, ci, A, Xb, Y, E, R, sh.tpr_log2);
+      launch_chained(spmm_kernel<float2, 1, uint32_t>, blocks, threads, 0, s, rp, ci, A, Xb, Y, E, R, sh.tpr_log2, go);
       break;
     case 2:
-      launch_chained(spmm_kernel<float2, 2, uint32_t>, blocks, threads, 0, s, rp, ci, A, Xb, Y, E, R, sh.tpr_log2);
+      launch_chained(spmm_kernel<float2, 2, uint32_t>, blocks, threads, 0, s, rp, ci, A, Xb, Y, E, R, sh.tpr_log2, go);
       break;
     default:
-      launch_chained(spmm_kernel<float2, 4, uint32_t>, blocks, threads, 0, s, rp, ci, A, Xb, Y, E, R, sh.tpr_log2);
+      launch_chained(spmm_kernel<float2, 4, uint32_t>, blocks, threads, 0, s, rp, ci, A, Xb, Y, E, R, sh.tpr_log2, go);
       break;
   }
 }

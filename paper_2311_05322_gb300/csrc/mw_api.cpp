@@ -1126,7 +1126,8 @@ bool spmm_halo_ok(Ctx* c, int R) {
   return c->spmm.n_block > 0 && R >= 2 && R <= 128 && R % 2 == 0 && (int)c->A32b.size() == c->n_freq;
 }
 void spmm32(Ctx* c, int f, const float2* X, float2* Y, int R, int threads, const int32_t* go = nullptr) {
-  if (threads == kSpmmHaloShape && spmm_halo_ok(c, R) && mwk::spmm_halo_f32(c->spmm, c->A32b[f], X, Y, R, c->stream))
+  if (threads == kSpmmHaloShape && spmm_halo_ok(c, R) &&
+      mwk::spmm_halo_f32(c->spmm, c->A32b[f], X, Y, R, c->stream, go))
     return;
   mwk::spmm_f32(c->d_row, c->d_col, c->A32[f], X, Y, c->topo.n_edge, R, c->stream, threads < 128 ? 256 : threads,
                 c->row_win, go);

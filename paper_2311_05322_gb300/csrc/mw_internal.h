@@ -168,7 +168,7 @@ void reassemble(const int64_t* cptr, const int32_t* contrib, int64_t nnz, const 
 // FP32 kernels' blocks).
 void spmm_f64(const int64_t* rp, const int32_t* ci, const double2* A, const double2* X, double2* Y, int64_t E,
               int R, cudaStream_t s, int threads = 256);
-// go (may be null): device word; zero when the kernel starts: nothing is done (only the staged product looks).
+// go (may be null): device word; zero when the kernel starts: Y is left alone.  The same in every FP32 form below.
 void spmm_f32(const int64_t* rp, const int32_t* ci, const float2* A, const float2* X, float2* Y, int64_t E, int R,
               cudaStream_t s, int threads, const int* win,
               const int32_t* go = nullptr);
@@ -189,7 +189,8 @@ struct SpmmDev {
 // Y = A X with the halo-tiled kernel; A_blk holds the FP32 values in the plan's blocked order.
 // Returns false (nothing launched) when the shape is not supported: R odd or above 128, or X
 // not 16-byte aligned.  Bit-identical to spmm_f32.
-bool spmm_halo_f32(const SpmmDev& p, const float2* A_blk, const float2* X, float2* Y, int R, cudaStream_t s);
+bool spmm_halo_f32(const SpmmDev& p, const float2* A_blk, const float2* X, float2* Y, int R, cudaStream_t s,
+                   const int32_t* go = nullptr);
 // Y = A X (FP32) with X stored as complex BF16 pairs [E][R] (real in the low half).
 void spmm_f32_bx(const int64_t* rp, const int32_t* ci, const float2* A, const void* X, float2* Y, int64_t E, int R,
                  cudaStream_t s, int threads, const int* win,
