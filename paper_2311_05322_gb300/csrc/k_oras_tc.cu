@@ -343,10 +343,11 @@ __device__ __forceinline__ void copy_stage(uint8_t* sa, const uint8_t* w, uint32
   bulk_g2s(sa + 2u * kATileBytes, b, b_bytes, bar);
 }
 
-// The first turns of the ring.  W and the tile records were written by a set-up that the host has waited for, so
-// their copies start before this launch's predecessor, the gather, has completed (in short launches and in the
-// sweeps it lets this launch in when it starts: 16 sparse subdomains, 15 applies of 17 launches 15.6 -> 15.4 ms);
-// ring_open issues them and returns their count, ring_join adds the B tiles once they are there and
+// The first turns of the ring.  Their copies of W start before this launch's predecessor, the gather, has completed
+// (in short launches and in the sweeps it lets this launch in when it starts: 16 sparse subdomains, 15 applies of 17
+// launches 15.6 -> 15.4 ms).  Nothing but the host orders these reads of W and of the tile records behind the set-up
+// that wrote them: it synchronises the stream after packing W and after uploading the records.
+// ring_open issues the copies and returns their count, ring_join adds the B tiles once they are there and
 // leaves the position of the next turn.
 __device__ __forceinline__ int ring_open(uint8_t* base, uint32_t stage_bytes, const uint8_t* Wt, uint32_t a_part,
                                          uint32_t b_bytes, int KT, int S, uint64_t* full_bar) {
@@ -833,7 +834,7 @@ bool tc_plan_build(TcPlan& p, const mw::Subdomains& sd, const std::function<void
   p.gt_sub = (int32_t*)up(gt_sub.data(), sizeof(int32_t) * std::max<size_t>(gt_sub.size(), 1));
   p.gt_kt = (int32_t*)up(gt_kt.data(), sizeof(int32_t) * std::max<size_t>(gt_kt.size(), 1));
   p.err = err;
-  cudaStreamSynchronize(s);  // host vectors go out of scope
+  cudaStreamSynchronize(s);  // host vectors go out of scope, and ring_open reads the records without waiting
   p.max_kt = 0;
   for (int q = 0; q < ns; ++q) p.max_kt = std::max(p.max_kt, sub_kt[q]);
   p.built = true;

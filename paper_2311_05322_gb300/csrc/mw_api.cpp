@@ -980,6 +980,8 @@ void build_sparse_tc(Ctx* c) {
                              (const float2*)m.fac[f], T.W[f], c->stream);
       }
       check_launch("sparse tensor-core packing");
+      // before the tables are freed, and before any sweep is launched: the MMA kernel's first copies of W (ring_open)
+      // do not wait for earlier launches
       CK(cudaStreamSynchronize(c->stream));
     } catch (...) {
       for (void* q : tmp) dfree(c, q);
@@ -2816,7 +2818,8 @@ mw_status mw_setup_preconditioner(mw_ctx* c, int32_t n_sub, const int32_t* part,
           else
             mwk::oras_extract(bt, p.topo(), p.factor_prec, ws, p.apply_prec, p.w_off, p.W[f], c->stream);
           check_launch("oras setup");
-          // host vectors must outlive the async copies
+          // Host vectors must outlive the async copies, and W must be complete before any apply is launched: the
+          // MMA kernel's first copies of W (ring_open) do not wait for earlier launches.
           CK(cudaStreamSynchronize(c->stream));
         }
       }
