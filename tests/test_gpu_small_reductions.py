@@ -56,3 +56,33 @@ def test_column_norms_scale_with_the_column(n_cols, mode):
     xs = x.cpu().numpy() / s[:, None]
     assert np.linalg.norm(xs - xs[0]) <= 1e-12 * np.linalg.norm(xs)
     assert np.all(np.abs(st["relres"] - st["relres"].ravel()[0]) <= 1e-12)
+
+
+@pytest.mark.parametrize("n_cols", [1, 2, 3, 5, 9, 17, 32, 33, 65, 128])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_reported_residuals_of_unfinished_solves(n_cols, mode):
+    """||b - A x|| / ||b|| of columns with different supports after a few steps, against norms formed from the
+    returned x on the CPU.  A lost row or warp moves them by its share, far above the bars: FP64 sums 1e-10;
+    mixed mode rounds each residual entry to FP32 and sums its square from there, 4 * 2^-24."""
+    from paper_2311_05322_gb300 import mw
+    m = kuhn_mesh(7, 6, 5, lo=(-0.03, -0.025, -0.02), hi=(0.03, 0.025, 0.02))
+    c = mw.Context(0)
+    E = c.set_mesh(m.xyz, m.tets).n_edge
+    c.assemble([1e9], np.tile([EPS_MATCHING.real, EPS_MATCHING.imag], (m.n_tet, 1)), EPS_MATCHING)
+    _, _, _, rp, ci = c.get_topology()
+    A = torch.sparse_csr_tensor(torch.from_numpy(rp), torch.from_numpy(ci.astype(np.int64)),
+                                torch.from_numpy(c.get_matrix(0)), (E, E)).to_dense().numpy()
+    rng = np.random.default_rng(100 * n_cols + mode)
+    B = rng.normal(size=(n_cols, E)) + 1j * rng.normal(size=(n_cols, E))
+    for q in range(n_cols):                 # every (1 + q % 5)-th row from a place of its own
+        keep = np.zeros(E, bool)
+        keep[37 * q % (E // 2)::1 + q % 5] = True
+        B[q, ~keep] = 0.0
+    b = torch.from_numpy(B).cuda()
+    x = torch.empty_like(b)
+    st = c.solve_rhs(n_cols, b, x, mw.solve_opts(mode=mode, restart=4, tol=1e-12, inner_tol=1e-1, max_it=4, max_outer=1,
+                                                 use_precond=0), allow_noconv=True)
+    c.close()
+    true = np.linalg.norm(B.T - A @ x.cpu().numpy().T, axis=0) / np.linalg.norm(B, axis=1)
+    assert np.all(true > 1e-3) and len(np.unique(np.round(true, 9))) == n_cols
+    assert np.all(np.abs(st["relres"].ravel() - true) <= (4 * 2.0 ** -24 if mode else 1e-10) * true)
