@@ -27,8 +27,6 @@ namespace mwk {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
-constexpr int kMaxVecPerWarp = 8;   // restart m <= 63 => nvec <= 64 = 8 warps x 8
 constexpr int kChunk = 16;          // FP32 rows summed before promotion to FP64
 constexpr int kBlocks = 152 * 4;
 

@@ -835,8 +835,6 @@ bool tc_plan_build(TcPlan& p, const mw::Subdomains& sd, const std::function<void
   p.gt_kt = (int32_t*)up(gt_kt.data(), sizeof(int32_t) * std::max<size_t>(gt_kt.size(), 1));
   p.err = err;
   cudaStreamSynchronize(s);  // host vectors go out of scope, and ring_open reads the records without waiting
-  p.max_kt = 0;
-  for (int q = 0; q < ns; ++q) p.max_kt = std::max(p.max_kt, sub_kt[q]);
   p.built = true;
   return true;
 }

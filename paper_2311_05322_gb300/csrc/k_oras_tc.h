@@ -37,7 +37,6 @@ struct TcPlan {
   int32_t* gt_sub = nullptr;     // [n_ktiles_total] subdomain of each gathered-operand tile
   int32_t* gt_kt = nullptr;      // [n_ktiles_total] its k tile
   int32_t* err = nullptr;        // error word (mapped host memory): nonzero after a timed-out wait
-  int max_kt = 0;
 };
 
 // err: device address of the error word, kept by the caller.

@@ -289,7 +289,7 @@ bool spmm_staged_launch(const int64_t* rp, const int32_t* ci, const float2* A, c
                         int R, cudaStream_t s, int threads, const int* win, const int32_t* go) {
   if (threads != 128 && threads != 256 && threads != 512) threads = 256;
   const size_t smem = staged_smem(staged_rows(threads), win[threads == 128 ? 0 : threads == 256 ? 1 : 2]);
-  if ( R < 1 || R > 128 || smem > 48 * 1024 || E * R > INT32_MAX) return false;
+  if (R < 1 || R > 128 || smem > 48 * 1024 || E * R > INT32_MAX) return false;
   const auto fits = [&](int vec) { return R % vec == 0 && (uintptr_t)X % (vec * sizeof(XT)) == 0; };
   if (R >= 16 && sizeof(XT) == 4 && fits(4))
     spmm_staged<XT, sizeof(XT) == 4 ? 4 : 2>(rp, ci, A, X, Y, E, R, s, threads, smem, go);

@@ -570,6 +570,7 @@ void setup_sparse(Ctx* c) {
   for (int s = 0; s < S; ++s) { x_row[s] = rows; rows += sd.dof_ptr[s + 1] - sd.dof_ptr[s]; }
   require(rows < INT32_MAX, MW_EINVAL, "sparse preconditioner too large");
   m.arena_rows = rows;
+  const bool f32_sweeps = P.apply_prec == 4;   // the BF16 sweeps have tables of their own
   // pivots as global edges (forward input) and as arena rows of x; update dofs as arena rows of x
   std::vector<int32_t> piv_glob(y.piv_loc.size()), idx;
   std::vector<int64_t> bidx(N, -1), cidx(N, -1);
@@ -577,6 +578,7 @@ void setup_sparse(Ctx* c) {
     const int sub = y.sub[k];
     const int64_t d0 = sd.dof_ptr[sub];
     for (int64_t q = y.piv_ptr[k]; q < y.piv_ptr[k + 1]; ++q) piv_glob[q] = sd.dofs[d0 + y.piv_loc[q]];
+    if (!f32_sweeps) continue;
     bidx[k] = (int64_t)idx.size();
     for (int64_t q = y.upd_ptr[k]; q < y.upd_ptr[k + 1]; ++q) idx.push_back((int32_t)(x_row[sub] + y.upd_loc[q]));
     cidx[k] = (int64_t)idx.size();
@@ -598,7 +600,6 @@ void setup_sparse(Ctx* c) {
   // leaf receive nothing (they are zero), so they are not listed, and its w product has no C0.
   std::vector<int64_t> pull_out, pull_ptr(1, 0), pull_src;
   m.pull_h.assign(1, 0);
-  const bool f32_sweeps = P.apply_prec == 4;   // the BF16 sweeps have tables of their own
   for (int h = 0; h <= H && f32_sweeps; ++h) {
     for (int64_t q = m.h_ptr[h]; q < m.h_ptr[h + 1]; ++q) {
       const int k = h_nodes[q];
@@ -701,8 +702,8 @@ void setup_sparse(Ctx* c) {
     m.bwd_splits.push_back((int64_t)splits.size());
   }
   // owned rows of x
-  std::vector<int64_t> own_row(sd.own_local.size());
-  for (int s = 0; s < S; ++s)
+  std::vector<int64_t> own_row(f32_sweeps ? sd.own_local.size() : 0);
+  for (int s = 0; s < S && f32_sweeps; ++s)
     for (int64_t q = sd.own_ptr[s]; q < sd.own_ptr[s + 1]; ++q) own_row[q] = x_row[s] + sd.own_local[q];
   m.n_own = (int64_t)own_row.size();
   // every index the kernels will follow, checked against its buffer before the first launch
