@@ -128,8 +128,8 @@ mw_status mw_set_graphs(mw_ctx* ctx, int32_t enable);
  *                  (only with a BF16 preconditioner in mixed mode);
  *   dots_stages    ring depth of the streaming Gram-Schmidt dots, 2..6 (16..128 columns);
  *   update_stages  ring depth of the streaming Gram-Schmidt update, 2..6 (16..128 columns);
- *   spmm_threads   threads per block of the row-per-warp SpMM, 128 / 256 / 512, or 1 for the
- *                  halo-tiled SpMM (FP32, even column counts).
+ *   spmm_threads   threads per block of the SpMM, 128 / 256 / 512, or 1 for the halo-tiled SpMM
+ *                  (FP32, even column counts).
  * None of these changes a result bit: the same arithmetic runs in the same order.  The choice is
  * kept per shape until the mesh or preconditioner changes.  Solves tune each new shape before
  * their timed phase while automatic tuning is on (mw_set_autotune, default on); mw_autotune

@@ -721,7 +721,8 @@ __global__ void __launch_bounds__(kThreadsTc, 2) oras_tc_persistent_kernel(const
   } else {
     // A tile's record is read two tiles ahead and its row numbers one tile ahead: in line, that chain of
     // dependent reads took longer than the copies of a tile with one to four k tiles (16 sparse subdomains of
-    // 44x44x17 cells, 16 columns: a solve's 15 applies 23.9 -> 21.2 ms with the 16-byte stores and the third stage).
+    // 44x44x17 cells, 32 columns, two ring stages: a solve of 15 applies 23.9 -> 21.2 ms together with the 16-byte
+    // stores).
     const int quad = warp & 3;
     const int row = quad * 32 + lane;
     const int step = gridDim.x;

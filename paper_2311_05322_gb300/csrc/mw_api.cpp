@@ -851,8 +851,8 @@ void setup_sparse(Ctx* c) {
 // A row of t or x is computed only if it is owned or enters another row that is: most subdomain dofs outside
 // the owned region (the overlap) are leaves that nothing reads.  With the sums and the scatter inside the
 // launches (no separate right-hand-side, copy and owned-row passes) and those rows left out, an apply of 16
-// subdomains of 25,052 unknowns, 16 columns, takes 34 launches and 0.77 ms (55 and 1.05 ms with them).  The FP32
-// factors are freed after packing.
+// subdomains of 25,052 unknowns, 32 columns, takes 34 launches and 0.77 ms (55 and 1.05 ms with them; 0.67 ms with
+// chained launches).  The FP32 factors are freed after packing.
 void build_sparse_tc(Ctx* c) {
   Prec& P = c->prec;
   Prec::Mf& m = P.mf;
@@ -1123,7 +1123,7 @@ struct CycleArgs {
 // Arnoldi step j as segments (preconditioner apply, SpMM, Gram-Schmidt dots, Gram-Schmidt
 // update, Givens and scaling); seg(cls, bytes, fn) runs fn, which launches on c->stream.
 // FP32 SpMM of frequency f: the halo-tiled kernel for launch shape kSpmmHaloShape (when the
-// shape allows it), else the row-per-warp kernel with `threads` per block.  Both sum every row
+// shape allows it), else the staged or the row-per-warp kernel with `threads` per block.  All sum every row
 // in the same order, so the choice never changes a result bit.
 bool spmm_halo_ok(Ctx* c, int R) {
   return c->spmm.n_block > 0 && R >= 2 && R <= 128 && R % 2 == 0 && (int)c->A32b.size() == c->n_freq;
@@ -1135,8 +1135,7 @@ void spmm32(Ctx* c, int f, const float2* X, float2* Y, int R, int threads, const
   mwk::spmm_f32(c->d_row, c->d_col, c->A32[f], X, Y, c->topo.n_edge, R, c->stream, threads < 128 ? 256 : threads,
                 c->row_win, go);
 }
-// The same with X stored as complex BF16 pairs: the row-per-warp kernel (256 threads for the
-// halo shape, which has no BF16 form).
+// The same with X stored as complex BF16 pairs (256 threads for the halo shape, which has no BF16 form).
 void spmm32_bx(Ctx* c, int f, const void* X, float2* Y, int R, int threads, const int32_t* go = nullptr) {
   mwk::spmm_f32_bx(c->d_row, c->d_col, c->A32[f], X, Y, c->topo.n_edge, R, c->stream, threads < 128 ? 256 : threads,
                    c->row_win, go);
