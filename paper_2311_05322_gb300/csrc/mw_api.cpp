@@ -349,6 +349,24 @@ void dfree(Ctx* c, void* p) {
   cudaFree(p);
 }
 
+// Device buffers of one call, given back when it ends, also by an exception.
+struct Temps {
+  Ctx* c;
+  std::vector<void*> v;
+  explicit Temps(Ctx* ctx) : c(ctx) { v.reserve(4); }
+  Temps(const Temps&) = delete;
+  ~Temps() {
+    for (void* p : v) dfree(c, p);
+  }
+  template <typename T>
+  T* get(size_t n) {
+    v.push_back(nullptr);
+    T* p = dalloc<T>(c, n);
+    v.back() = p;
+    return p;
+  }
+};
+
 template <typename T>
 T* upload(Ctx* c, const T* h, size_t n) {
   T* d = dalloc<T>(c, n);
@@ -2339,14 +2357,13 @@ mw_status mw_apply_matrix(mw_ctx* c, int32_t f, int32_t prec, const void* x, voi
       mwk::spmm_f32_bx(c->d_row, c->d_col, c->A32[f], x, (float2*)y, c->topo.n_edge, n_cols, c->stream, 256, c->row_win);
     else if (prec == 3) {
       const int64_t n = c->topo.n_edge * (int64_t)n_cols;
-      float4* xd = dalloc<float4>(c, n);
-      double* part = dalloc<double>(c, (size_t)152 * 4 * n_cols);
+      Temps tmp(c);
+      float4* xd = tmp.get<float4>(n);
+      double* part = tmp.get<double>((size_t)152 * 4 * n_cols);
       mwk::split_df((const double2*)x, xd, n, c->stream);
       mwk::residual_df(c->d_row, c->d_col, c->Adf[f], xd, nullptr, (double2*)y, part, c->topo.n_edge, n_cols,
                        c->stream);
       CK(cudaStreamSynchronize(c->stream));
-      dfree(c, xd);
-      dfree(c, part);
     } else
       throw Fail{MW_EINVAL, "apply_matrix precision must be FP64 (0), FP32 (1) or double-float (3)"};
     check_launch("spmm");
@@ -2845,15 +2862,14 @@ mw_status mw_apply_preconditioner(mw_ctx* c, int32_t f, const void* r, void* z, 
       CK(cudaMemsetAsync(z, 0, sizeof(double2) * n, c->stream));
       apply_prec(c, f, 0, r, z, n_cols);
     } else {
-      float2* a = dalloc<float2>(c, n);
-      float2* b = dalloc<float2>(c, n);
+      Temps tmp(c);
+      float2* a = tmp.get<float2>(n);
+      float2* b = tmp.get<float2>(n);
       mwk::cast_f64_to_f32((const double2*)r, a, n, c->stream);
       CK(cudaMemsetAsync(b, 0, sizeof(float2) * n, c->stream));
       apply_prec(c, f, 1, a, b, n_cols);
       mwk::cast_f32_to_f64(b, (double2*)z, n, c->stream);
       CK(cudaStreamSynchronize(c->stream));
-      dfree(c, a);
-      dfree(c, b);
     }
     check_launch("apply preconditioner");
     check_tc_wait(c);
@@ -2887,13 +2903,13 @@ mw_status mw_solve(mw_ctx* c, const mw_solve_opts* opts, void* fields, double* S
       for (int f = 0; f < c->n_freq; ++f)
         mwk::transpose_out(c->Xf[f], (double2*)fields + (int64_t)f * c->n_src * E, E, c->n_src, c->stream);
     if (S) {
-      double2* dS = dalloc<double2>(c, (size_t)c->n_freq * c->n_src * c->n_src);
+      Temps tmp(c);
+      double2* dS = tmp.get<double2>((size_t)c->n_freq * c->n_src * c->n_src);
       for (int f = 0; f < c->n_freq; ++f)
         mwk::s_project(c->Xf[f], c->d_q_ptr, c->d_q_edge, c->d_q_w, c->d_q_norm, c->n_src,
                        dS + (size_t)f * c->n_src * c->n_src, c->stream);
       CK(cudaMemcpyAsync(S, dS, sizeof(double2) * c->n_freq * c->n_src * c->n_src, cudaMemcpyDeviceToHost, c->stream));
       CK(cudaStreamSynchronize(c->stream));
-      dfree(c, dS);
     }
     check_launch("solve outputs");
     CK(cudaStreamSynchronize(c->stream));
@@ -2911,9 +2927,10 @@ mw_status mw_solve_rhs(mw_ctx* c, const mw_solve_opts* opts, int32_t n_cols, con
     const int64_t E = c->topo.n_edge;
     std::vector<double2*> Bi(c->n_freq), Xi(c->n_freq);
     std::vector<const double2*> Bc(c->n_freq);
+    Temps tmp(c);
     for (int f = 0; f < c->n_freq; ++f) {
-      Bi[f] = dalloc<double2>(c, E * n_cols);
-      Xi[f] = dalloc<double2>(c, E * n_cols);
+      Bi[f] = tmp.get<double2>(E * n_cols);
+      Xi[f] = tmp.get<double2>(E * n_cols);
       mwk::transpose_in((const double2*)b + (int64_t)f * n_cols * E, Bi[f], E, n_cols, c->stream);
       Bc[f] = Bi[f];
     }
@@ -2922,23 +2939,13 @@ mw_status mw_solve_rhs(mw_ctx* c, const mw_solve_opts* opts, int32_t n_cols, con
     try {
       solve_all(c, o, n_cols, Bc, Xi, stats);
     } catch (const Fail& e) {
-      if (e.code != MW_ENOCONV) {
-        for (int f = 0; f < c->n_freq; ++f) {
-          dfree(c, Bi[f]);
-          dfree(c, Xi[f]);
-        }
-        throw;
-      }
+      if (e.code != MW_ENOCONV) throw;
       conv = e.code;
       msg = e.msg;
     }
     for (int f = 0; f < c->n_freq; ++f)
       mwk::transpose_out(Xi[f], (double2*)x + (int64_t)f * n_cols * E, E, n_cols, c->stream);
     CK(cudaStreamSynchronize(c->stream));
-    for (int f = 0; f < c->n_freq; ++f) {
-      dfree(c, Bi[f]);
-      dfree(c, Xi[f]);
-    }
     if (conv != MW_OK) throw Fail{conv, msg};
   });
 }
@@ -2958,15 +2965,15 @@ mw_status mw_tikhonov(mw_ctx* c, const double* eps_r, double* R_out, double* gra
   return guard(c, [&] {
     require(c->has_mesh && eps_r && R_out, MW_EINVAL, "bad tikhonov arguments");
     const int64_t T = c->topo.n_tet;
-    double* de = upload(c, eps_r, 2 * T);
-    double* dg = dalloc<double>(c, 2 * T);
+    Temps tmp(c);
+    double* de = tmp.get<double>(2 * T);
+    double* dg = tmp.get<double>(2 * T);
+    CK(cudaMemcpyAsync(de, eps_r, sizeof(double) * 2 * T, cudaMemcpyHostToDevice, c->stream));
     tikhonov_dev(c, de, R_out, dg);
     if (grad) {
       CK(cudaMemcpyAsync(grad, dg, sizeof(double) * 2 * T, cudaMemcpyDeviceToHost, c->stream));
       CK(cudaStreamSynchronize(c->stream));
     }
-    dfree(c, de);
-    dfree(c, dg);
   });
 }
 
@@ -3451,9 +3458,10 @@ mw_status mw_krylov_dots(mw_ctx* c, int32_t nvec, const void* V_dev, int64_t vst
     require(nvec >= 1 && nvec <= 64 && V_dev && w_dev && h_out && n_rows >= 1 && n_cols >= 1 && n_cols <= 128 &&
                 vstride >= n_rows * (int64_t)n_cols,
             MW_EINVAL, "bad arguments");
-    double2* part = dalloc<double2>(c, (size_t)mwk::kCgsDotsMaxParts * nvec * n_cols);
-    double2* h = dalloc<double2>(c, (size_t)nvec * n_cols);
-    int32_t* err = dalloc<int32_t>(c, 1);
+    Temps tmp(c);
+    double2* part = tmp.get<double2>((size_t)mwk::kCgsDotsMaxParts * nvec * n_cols);
+    double2* h = tmp.get<double2>((size_t)nvec * n_cols);
+    int32_t* err = tmp.get<int32_t>(1);
     CK(cudaMemsetAsync(err, 0, sizeof(int32_t), c->stream));
     const int np = mwk::cgs_dots_f32((const float2*)V_dev, vstride, nvec, (const float2*)w_dev, n_rows, n_cols, part,
                                      err, c->stream);
@@ -3462,9 +3470,6 @@ mw_status mw_krylov_dots(mw_ctx* c, int32_t nvec, const void* V_dev, int64_t vst
     CK(cudaMemcpyAsync(h_out, h, sizeof(double2) * nvec * n_cols, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaMemcpyAsync(&e, err, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
-    dfree(c, part);
-    dfree(c, h);
-    dfree(c, err);
     check_launch("krylov dots");
     require(e == 0, MW_ETIMEOUT, "streaming Gram-Schmidt dots: bounded wait ran out");
   });
@@ -3883,15 +3888,16 @@ mw_status mw_nn_grid_to_tets(mw_ctx* c, const float* grid, int32_t G, const doub
   return guard(c, [&] {
     require(c->has_mesh && grid && box && deps && G >= 2 && G <= 1024, MW_EINVAL, "bad grid arguments");
     const int64_t T = c->topo.n_tet;
-    float* dg = upload(c, grid, (size_t)2 * G * G * G);
-    double* out = dalloc<double>(c, 2 * T);
+    const size_t ng = (size_t)2 * G * G * G;
+    Temps tmp(c);
+    float* dg = tmp.get<float>(ng);
+    double* out = tmp.get<double>(2 * T);
+    CK(cudaMemcpyAsync(dg, grid, sizeof(float) * ng, cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemsetAsync(out, 0, sizeof(double) * 2 * T, c->stream));
     mwk::nn_grid_to_tets(dg, G, box, c->d_xyz, c->d_tets, T, out, c->stream);
     check_launch("grid to tets");
     CK(cudaMemcpyAsync(deps, out, sizeof(double) * 2 * T, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
-    dfree(c, dg);
-    dfree(c, out);
   });
 }
 
@@ -3899,13 +3905,13 @@ mw_status mw_nn_grid_to_tets(mw_ctx* c, const float* grid, int32_t G, const doub
 mw_status mw_selftest_bounded_wait(mw_ctx* c, int64_t spins, int32_t* code_out) {
   return guard(c, [&] {
     require(code_out && spins >= 1 && spins <= (int64_t)1 << 26, MW_EINVAL, "spins in [1, 2^26]");
-    int32_t* d = dalloc<int32_t>(c, 1);
+    Temps tmp(c);
+    int32_t* d = tmp.get<int32_t>(1);
     CK(cudaMemsetAsync(d, 0xff, sizeof(int32_t), c->stream));
     mwk::bounded_wait_probe((long long)spins, d, c->stream);
     check_launch("bounded wait probe");
     CK(cudaMemcpyAsync(code_out, d, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
-    dfree(c, d);
   });
 }
 

@@ -1,0 +1,68 @@
+"""Allocations refused one after the other: a memory cap that rises in small steps makes every allocation of a call
+fail once.  A refused call reports MW_ENOMEM and keeps nothing."""
+import numpy as np
+import pytest
+
+from phantom import EPS_MATCHING, box_partition, kuhn_mesh
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+LIMIT = 3000   # steps of a climb: a call that kept buffers when it is refused would never get past its cap
+
+
+def _climb(c, call, between=lambda: None, step=1 << 16):
+    """call() under a rising cap until it succeeds; between() after every refusal.  Returns the refusals; the cap
+    that sufficed is 1 + refusals * step."""
+    from paper_2311_05322_gb300 import mw
+    for refused in range(LIMIT):
+        c.set_memory_cap(1 + refused * step)
+        for f in (call, between):
+            try:
+                f()
+                if f is call:
+                    c.set_memory_cap(0)
+                    return refused
+            except mw.MWError as e:
+                assert e.status == mw.MW_ENOMEM, e
+    pytest.fail("the cap never sufficed")
+
+
+def _context(prec, eps=None):
+    from paper_2311_05322_gb300 import mw
+    m = kuhn_mesh(5, 4, 3, lo=(-0.02, -0.015, -0.01), hi=(0.02, 0.015, 0.01))
+    c = mw.Context(0)
+    E = c.set_mesh(m.xyz, m.tets).n_edge
+    c.assemble([1e9], np.tile([EPS_MATCHING.real, EPS_MATCHING.imag], (m.n_tet, 1)), EPS_MATCHING)
+    if prec is not None:
+        c.setup_preconditioner(4, box_partition(m, (2, 2, 1)), 1, prec)
+    return mw, m, c, E
+
+
+@pytest.mark.parametrize("what", ["matrix", "preconditioner", "dots", "grid", "tikhonov"])
+def test_refused_calls_keep_nothing(what):
+    """A cap that a climb of refused calls found sufficient is no larger than a fresh context needs."""
+    def ready():
+        from paper_2311_05322_gb300 import mw as lib
+        mw, m, c, E = _context(lib.MW_PREC_FP32)
+        x = torch.ones((E, 6), dtype=torch.complex128, device="cuda")
+        y = torch.empty_like(x)
+        v = torch.ones(4 * 6 * E, dtype=torch.complex64, device="cuda")
+        call = {"matrix": lambda: c.apply_matrix(0, 3, x, y, 6),
+                "preconditioner": lambda: c.apply_preconditioner(0, x, y, 6),
+                "dots": lambda: c.krylov_dots(v, v, 3, 6 * E, E, 6),
+                "grid": lambda: c.nn_grid_to_tets(np.ones((2, 32, 32, 32), np.float32), [-0.02] * 3 + [0.02] * 3),
+                "tikhonov": lambda: c.tikhonov(np.ones((m.n_tet, 2)))}[what]
+        return mw, c, call
+    step = 1 << 13
+    mw, c, call = ready()
+    refused = _climb(c, call, step=step)
+    assert refused > 0
+    c.close()
+    mw, c, call = ready()
+    c.set_memory_cap(1 + (refused - 1) * step)
+    with pytest.raises(mw.MWError) as e:
+        call()
+    assert e.value.status == mw.MW_ENOMEM
+    c.set_memory_cap(1 + refused * step)
+    call()
+    c.close()
