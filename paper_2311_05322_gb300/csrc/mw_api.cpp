@@ -450,79 +450,75 @@ void ensure_work(Ctx* c, int R, int m, int prec) {
   free_work(c);
   const size_t es = prec == 0 ? sizeof(double2) : sizeof(float2);
   const size_t n = (size_t)E * R;
+  try {
+    const size_t nv = (size_t)krylov_stride(E, R);
+    w.V = dalloc<unsigned char>(c, es * nv * (m + 1));
+    w.Z = dalloc<unsigned char>(c, es * nv * m);
+    w.vscale = dalloc<double>(c, (size_t)(m + 1) * R);
+    w.r = dalloc<double2>(c, n);
+    w.x = dalloc<double2>(c, n);
+    if (prec == 1) {
+      w.xdf = dalloc<float4>(c, n);
+      w.bdf = dalloc<float4>(c, n);
+      w.r32 = dalloc<float2>(c, n);
+    }
+    w.bblk = dalloc<double2>(c, n);
+    w.part = dalloc<double2>(c, (size_t)std::max(mwk::kCgsDotsMaxParts, kRedBlocks) * (kMaxRestart + 1) * R);
+    w.h = dalloc<double2>(c, (size_t)(kMaxRestart + 1) * R);
+    w.H = dalloc<double2>(c, (size_t)R * m * (m + 1));
+    w.cs = dalloc<double2>(c, (size_t)R * 2 * m);
+    w.g = dalloc<double2>(c, (size_t)R * (m + 1));
+    w.y = dalloc<double2>(c, (size_t)R * m);
+    w.npart = dalloc<double>(c, (size_t)kRedBlocks * R);
+    w.target = dalloc<double>(c, R);
+    w.rnorm = dalloc<double>(c, R);
+    w.bnorm = dalloc<double>(c, R);
+    w.scale = dalloc<double>(c, R);
+    w.done = dalloc<int32_t>(c, R);
+    w.kcol = dalloc<int32_t>(c, R);
+    w.active = dalloc<int32_t>(c, 2);
+    CK(cudaMemsetAsync(w.active, 0, 2 * sizeof(int32_t), c->stream));
+    CK(cudaMallocHost(&w.h_vec, sizeof(double) * R));
+    CK(cudaMallocHost(&w.h_ivec, sizeof(int32_t) * R));
+  } catch (...) {
+    free_work(c);   // nothing half allocated that a later, smaller solve would take for complete
+    throw;
+  }
   w.E = E;
   w.R = R;
   w.m = m;
   w.prec = prec;
-  const size_t nv = (size_t)krylov_stride(E, R);
-  w.V = dalloc<unsigned char>(c, es * nv * (m + 1));
-  w.Z = dalloc<unsigned char>(c, es * nv * m);
-  w.vscale = dalloc<double>(c, (size_t)(m + 1) * R);
-  w.r = dalloc<double2>(c, n);
-  w.x = dalloc<double2>(c, n);
-  if (prec == 1) {
-    w.xdf = dalloc<float4>(c, n);
-    w.bdf = dalloc<float4>(c, n);
-    w.r32 = dalloc<float2>(c, n);
-  }
-  w.bblk = dalloc<double2>(c, n);
-  w.part = dalloc<double2>(c, (size_t)std::max(mwk::kCgsDotsMaxParts, kRedBlocks) * (kMaxRestart + 1) * R);
-  w.h = dalloc<double2>(c, (size_t)(kMaxRestart + 1) * R);
-  w.H = dalloc<double2>(c, (size_t)R * m * (m + 1));
-  w.cs = dalloc<double2>(c, (size_t)R * 2 * m);
-  w.g = dalloc<double2>(c, (size_t)R * (m + 1));
-  w.y = dalloc<double2>(c, (size_t)R * m);
-  w.npart = dalloc<double>(c, (size_t)kRedBlocks * R);
-  w.target = dalloc<double>(c, R);
-  w.rnorm = dalloc<double>(c, R);
-  w.bnorm = dalloc<double>(c, R);
-  w.scale = dalloc<double>(c, R);
-  w.done = dalloc<int32_t>(c, R);
-  w.kcol = dalloc<int32_t>(c, R);
-  w.active = dalloc<int32_t>(c, 2);
-  CK(cudaMemsetAsync(w.active, 0, 2 * sizeof(int32_t), c->stream));
-  CK(cudaMallocHost(&w.h_vec, sizeof(double) * R));
-  CK(cudaMallocHost(&w.h_ivec, sizeof(int32_t) * R));
 }
 
 // ---------------------------------------------------------------------------------------
 // preconditioner apply on basis vectors of the working precision
 // ---------------------------------------------------------------------------------------
+// Grows a scratch buffer of `have` bytes to at least `need`; after a refused allocation it has none.
+void grow(Ctx* c, void*& p, size_t& have, size_t need) {
+  if (have >= need) return;
+  dfree(c, p);
+  p = nullptr;
+  have = 0;
+  p = dalloc<unsigned char>(c, need);
+  have = need;
+}
+
 // Size the tensor-core apply's gathered-operand scratch before a capture (no allocation may
 // happen while the stream is captured).
 void ensure_prec_scratch(Ctx* c, int R) {
   Prec& p = c->prec;
   Work& w = c->work;
   if (p.ready && (p.apply_prec == 4 || p.apply_prec == 5)) {
-    const size_t need = (size_t)p.mf.arena_rows * R * sizeof(float2);
-    if (w.mf_bytes < need) {
-      dfree(c, w.mf_arena);
-      w.mf_arena = nullptr;
-      w.mf_arena = dalloc<unsigned char>(c, need);
-      w.mf_bytes = need;
-    }
-    const size_t pneed = (size_t)std::max<int64_t>(p.mf.max_slots, 1) * mwk::kMfTileRows * R * sizeof(float2);
-    if (p.apply_prec == 4 && w.mf_pbytes < pneed) {
-      dfree(c, w.mf_partial);
-      w.mf_partial = nullptr;
-      w.mf_partial = dalloc<unsigned char>(c, pneed);
-      w.mf_pbytes = pneed;
-    }
-    if (p.apply_prec == 5 && w.tc_bytes < p.mf.tc_scratch) {
-      dfree(c, w.tc_scratch);
-      w.tc_scratch = nullptr;
-      w.tc_scratch = dalloc<unsigned char>(c, p.mf.tc_scratch);
-      w.tc_bytes = p.mf.tc_scratch;
-    }
+    grow(c, w.mf_arena, w.mf_bytes, (size_t)p.mf.arena_rows * R * sizeof(float2));
+    if (p.apply_prec == 4)
+      grow(c, w.mf_partial, w.mf_pbytes,
+           (size_t)std::max<int64_t>(p.mf.max_slots, 1) * mwk::kMfTileRows * R * sizeof(float2));
+    else
+      grow(c, w.tc_scratch, w.tc_bytes, p.mf.tc_scratch);
     return;
   }
   if (!p.ready || p.apply_prec != 2) return;
-  const size_t need = mwk::tc_scratch_bytes(p.tc, R);
-  if (w.tc_bytes < need) {
-    dfree(c, w.tc_scratch);
-    w.tc_scratch = dalloc<unsigned char>(c, need);
-    w.tc_bytes = need;
-  }
+  grow(c, w.tc_scratch, w.tc_bytes, mwk::tc_scratch_bytes(p.tc, R));
 }
 
 // ---------------------------------------------------------------------------------------

@@ -1,5 +1,6 @@
 """Allocations refused one after the other: a memory cap that rises in small steps makes every allocation of a call
-fail once.  A refused call reports MW_ENOMEM and keeps nothing."""
+fail once.  A refused call reports MW_ENOMEM and keeps nothing; a smaller call between two refusals either does too or
+gives the right result, and without the cap everything gives the results of a context that saw no refusal."""
 import numpy as np
 import pytest
 
@@ -65,4 +66,40 @@ def test_refused_calls_keep_nothing(what):
     assert e.value.status == mw.MW_ENOMEM
     c.set_memory_cap(1 + refused * step)
     call()
+    c.close()
+
+
+@pytest.mark.parametrize("prec", ["BF16", "SPARSE_BF16", "SPARSE", "FP32"])
+def test_solver_workspace(prec):
+    """Workspace and preconditioner scratch are recorded as present only when they are complete: a solve of fewer
+    columns after a refused one used to take the record of the larger workspace for memory it did not have."""
+    from paper_2311_05322_gb300 import mw as lib
+    mw, m, c, E = _context(getattr(lib, "MW_PREC_" + prec))
+    g = torch.Generator().manual_seed(3)
+    b = torch.complex(*(torch.randn(6, E, generator=g, dtype=torch.float64) for _ in range(2))).cuda()
+    o = mw.solve_opts(mode=1, restart=10, tol=1e-9, inner_tol=1e-2)
+    c.set_autotune(False)
+    want = torch.empty_like(b)
+    c.solve_rhs(6, b, want, o)
+    small_want = torch.empty_like(b[:2])
+    c.solve_rhs(2, b[:2], small_want, o)
+    z_want = torch.empty((E, 6), dtype=torch.complex128, device="cuda")
+    r = b.T.contiguous()
+    c.apply_preconditioner(0, r, z_want, 6)
+    c.close()
+    _, _, c, _ = _context(getattr(lib, "MW_PREC_" + prec))
+    c.set_autotune(False)
+    x, small, z = torch.empty_like(b), torch.empty_like(b[:2]), torch.empty_like(z_want)
+
+    def between():
+        small.zero_()
+        c.solve_rhs(2, b[:2], small, o)
+        assert torch.equal(torch.view_as_real(small), torch.view_as_real(small_want))
+
+    assert _climb(c, lambda: c.solve_rhs(6, b, x, o), between) > 5
+    assert torch.equal(torch.view_as_real(x), torch.view_as_real(want))
+    _climb(c, lambda: c.apply_preconditioner(0, r, z, 6), step=1 << 14)
+    assert torch.equal(torch.view_as_real(z), torch.view_as_real(z_want))
+    c.solve_rhs(6, b, x, o)
+    assert torch.equal(torch.view_as_real(x), torch.view_as_real(want))
     c.close()
