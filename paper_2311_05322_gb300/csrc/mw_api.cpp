@@ -1857,12 +1857,20 @@ void reassemble_all(Ctx* c) {
   check_launch("reassemble");
 }
 
+// One vector of all sources' columns per frequency; v is filled or, after a refused allocation, empty.
 void alloc_fields(Ctx* c, std::vector<double2*>& v) {
   const int64_t n = c->topo.n_edge * (int64_t)c->n_src;
   if ((int)v.size() == c->n_freq && !v.empty()) return;
   for (auto p : v) dfree(c, p);
-  v.assign(c->n_freq, nullptr);
-  for (int f = 0; f < c->n_freq; ++f) v[f] = dalloc<double2>(c, n);
+  v.clear();
+  v.reserve(c->n_freq);
+  try {
+    for (int f = 0; f < c->n_freq; ++f) v.push_back(dalloc<double2>(c, n));
+  } catch (...) {
+    for (auto p : v) dfree(c, p);
+    v.clear();
+    throw;
+  }
 }
 
 void forward(Ctx* c, const mw_solve_opts& o, mw_solve_stats* stats) {
@@ -2986,11 +2994,7 @@ static void gradient_dev_impl(Ctx* c, const mw_solve_opts& o, const double2* dSo
   if (!c->d_S) c->d_S = dalloc<double2>(c, 64 * 128 * 128);
   if (!c->d_C) c->d_C = dalloc<double2>(c, 64 * 128 * 128);
   if (!c->d_J) c->d_J = dalloc<double>(c, 4);
-  if (c->d_Badj.size() != (size_t)nf) {
-    for (auto p : c->d_Badj) dfree(c, p);
-    c->d_Badj.assign(nf, nullptr);
-    for (int f = 0; f < nf; ++f) c->d_Badj[f] = dalloc<double2>(c, E * ns);
-  }
+  alloc_fields(c, c->d_Badj);
   for (int f = 0; f < nf; ++f)
     mwk::s_project(c->Xf[f], c->d_q_ptr, c->d_q_edge, c->d_q_w, c->d_q_norm, ns, c->d_S + (size_t)f * ns * ns,
                    c->stream);

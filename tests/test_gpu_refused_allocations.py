@@ -103,3 +103,46 @@ def test_solver_workspace(prec):
     c.solve_rhs(6, b, x, o)
     assert torch.equal(torch.view_as_real(x), torch.view_as_real(want))
     c.close()
+
+
+def _data(n, nf=1):
+    rng = np.random.default_rng(n)
+    s = lambda: torch.from_numpy(rng.normal(size=(nf, n, n)) + 1j * rng.normal(size=(nf, n, n))).cuda()
+    return s(), s()
+
+
+@pytest.mark.parametrize("reciprocal", [False, True])
+def test_fields_of_an_evaluation(reciprocal):
+    """Forward and adjoint fields of several frequencies: an evaluation that was refused some of them leaves none."""
+    from paper_2311_05322_gb300 import mw as lib
+    pos = np.array([[0.012, 0.0, 0.002], [-0.012, 0.0, 0.002], [0.0, 0.01, 0.002]])
+    freqs = [0.9e9, 1.0e9, 1.1e9]
+    obs, emp = _data(3, 3)
+
+    def ready():
+        mw, m, c, E = _context(None)
+        eps = np.tile([EPS_MATCHING.real, EPS_MATCHING.imag], (m.n_tet, 1))
+        c.assemble(freqs, eps, EPS_MATCHING)
+        c.set_sources(pos, np.tile([0.0, 0.0, 1.0], (3, 1)))
+        c.setup_preconditioner(4, box_partition(m, (2, 2, 1)), 1, lib.MW_PREC_BF16)
+        c.set_autotune(False)
+        c.set_adjoint_mode(reciprocal)
+        g = torch.zeros((m.n_tet, 2), dtype=torch.float64, device="cuda")
+        o = mw.solve_opts(mode=1, restart=10, tol=1e-9, inner_tol=1e-2)
+        return c, g, o, lambda: c.gradient_dev(obs, emp, g, 0.0, o)
+
+    c, want, o, call = ready()
+    J = call()
+    S, _ = c.solve(o)
+    c.close()
+    c, g, o, call = ready()
+    got = []
+
+    def between():
+        s, _ = c.solve(o)
+        assert np.array_equal(s, S)
+
+    _climb(c, lambda: got.append(call()), between, step=1 << 15)
+    assert got[-1] == J and torch.equal(g, want)
+    assert np.array_equal(c.solve(o)[0], S)
+    c.close()
