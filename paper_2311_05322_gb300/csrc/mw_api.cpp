@@ -2302,7 +2302,9 @@ mw_status mw_assemble(mw_ctx* c, int32_t n_freq, const double* freq_hz, const do
     for (int f = 0; f < n_freq; ++f) require(freq_hz[f] > 0 && std::isfinite(freq_hz[f]), MW_EINVAL, "bad frequency");
     for (int64_t i = 0; i < 2 * T; ++i) require(std::isfinite(eps_r[i]), MW_EINVAL, "non-finite permittivity");
     require(std::isfinite(eps_bg[0]) && std::isfinite(eps_bg[1]), MW_EINVAL, "non-finite background permittivity");
+    if (!c->d_eps) c->d_eps = dalloc<double>(c, 2 * T);
     if (n_freq != c->n_freq) {
+      c->n_freq = 0;   // nothing is assembled until every buffer is there
       for (auto p : c->A64) dfree(c, p);
       for (auto p : c->A32) dfree(c, p);
       for (auto p : c->A32b) dfree(c, p);
@@ -2329,9 +2331,13 @@ mw_status mw_assemble(mw_ctx* c, int32_t n_freq, const double* freq_hz, const do
     c->freqs.assign(freq_hz, freq_hz + n_freq);
     c->eps_bg[0] = eps_bg[0];
     c->eps_bg[1] = eps_bg[1];
-    if (!c->d_eps) c->d_eps = dalloc<double>(c, 2 * T);
     CK(cudaMemcpyAsync(c->d_eps, eps_r, sizeof(double) * 2 * T, cudaMemcpyHostToDevice, c->stream));
-    reassemble_all(c);
+    try {
+      reassemble_all(c);
+    } catch (...) {
+      c->n_freq = 0;
+      throw;
+    }
   });
 }
 

@@ -11,12 +11,29 @@ torch = pytest.importorskip("torch")
 LIMIT = 3000   # steps of a climb: a call that kept buffers when it is refused would never get past its cap
 
 
-def _climb(c, call, between=lambda: None, step=1 << 16):
+def _used(c):
+    """Bytes the context holds: the largest cap at which the self-test's 16 bytes are refused, less 15."""
+    from paper_2311_05322_gb300 import mw
+    lo, hi = 1, 1 << 34
+    while lo < hi:
+        mid = (lo + hi) // 2
+        c.set_memory_cap(mid)
+        try:
+            c.selftest_bounded_wait(16)
+            hi = mid
+        except mw.MWError as e:
+            assert e.status == mw.MW_ENOMEM
+            lo = mid + 1
+    c.set_memory_cap(0)
+    return lo - 16
+
+
+def _climb(c, call, between=lambda: None, step=1 << 16, start=1):
     """call() under a rising cap until it succeeds; between() after every refusal.  Returns the refusals; the cap
-    that sufficed is 1 + refusals * step."""
+    that sufficed is start + refusals * step."""
     from paper_2311_05322_gb300 import mw
     for refused in range(LIMIT):
-        c.set_memory_cap(1 + refused * step)
+        c.set_memory_cap(start + refused * step)
         for f in (call, between):
             try:
                 f()
@@ -145,4 +162,27 @@ def test_fields_of_an_evaluation(reciprocal):
     _climb(c, lambda: got.append(call()), between, step=1 << 15)
     assert got[-1] == J and torch.equal(g, want)
     assert np.array_equal(c.solve(o)[0], S)
+    c.close()
+
+
+def test_matrices_of_several_frequencies():
+    """An assembly that was refused a buffer leaves nothing assembled."""
+    freqs = [0.9e9, 1.0e9, 1.1e9]
+    mw, m, c, E = _context(None)
+    eps = np.tile([EPS_MATCHING.real, EPS_MATCHING.imag], (m.n_tet, 1))
+    c.assemble(freqs, eps, EPS_MATCHING)
+    want = [c.get_matrix(f) for f in range(3)]
+    c.close()
+    mw, m, c, E = _context(None)
+    x = torch.ones((E, 3), dtype=torch.complex64, device="cuda")
+    y = torch.empty_like(x)
+
+    def between():
+        for call in (lambda: c.apply_matrix(0, mw.MW_PREC_FP32, x, y, 3), c.solve):
+            with pytest.raises(mw.MWError) as e:
+                call()
+            assert e.value.status in (mw.MW_EINVAL, mw.MW_ESTATE)
+
+    assert _climb(c, lambda: c.assemble(freqs, eps, EPS_MATCHING), between, step=1 << 14) > 10
+    assert all(np.array_equal(c.get_matrix(f), want[f]) for f in range(3))
     c.close()
