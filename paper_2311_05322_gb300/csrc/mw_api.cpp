@@ -1779,17 +1779,11 @@ void free_sources(Ctx* c) {
 }
 
 // Installs n sources given as CSR (host ptr / edges) with entry values and norms already on
-// the device (ownership passes to the context); builds the edge-major transpose.
+// the device (ownership passes to the context); builds the edge-major transpose.  After an exception the context has
+// no sources, and d_w and d_norm are still the caller's.
 void install_sources(Ctx* c, int n, bool ports, const std::vector<int64_t>& ptr, const std::vector<int32_t>& edge,
                      double* d_w, double* d_norm) {
   free_sources(c);
-  c->n_src = n;
-  c->src_ports = ports;
-  c->q_ptr_h = ptr;
-  c->d_q_ptr = upload(c, ptr.data(), ptr.size());
-  c->d_q_edge = upload_vec(c, edge);
-  c->d_q_w = d_w;
-  c->d_q_norm = d_norm;
   // transpose: pairs (edge, source, entry) sorted by edge, then source
   std::vector<std::array<int32_t, 3>> pr;
   pr.reserve(edge.size());
@@ -1807,11 +1801,23 @@ void install_sources(Ctx* c, int n, bool ports, const std::vector<int64_t>& ptr,
     tk.push_back(pr[i][2]);
   }
   if (!pr.empty()) tptr.push_back((int64_t)pr.size());
+  try {
+    c->d_q_ptr = upload(c, ptr.data(), ptr.size());
+    c->d_q_edge = upload_vec(c, edge);
+    c->d_qt_ptr = upload(c, tptr.data(), tptr.size());
+    c->d_qt_edge = upload_vec(c, tedge);
+    c->d_qt_src = upload_vec(c, tsrc);
+    c->d_qt_k = upload_vec(c, tk);
+    c->q_ptr_h = ptr;
+  } catch (...) {
+    free_sources(c);
+    throw;
+  }
   c->n_qt = (int64_t)tedge.size();
-  c->d_qt_ptr = upload(c, tptr.data(), tptr.size());
-  c->d_qt_edge = upload_vec(c, tedge);
-  c->d_qt_src = upload_vec(c, tsrc);
-  c->d_qt_k = upload_vec(c, tk);
+  c->d_q_w = d_w;
+  c->d_q_norm = d_norm;
+  c->src_ports = ports;
+  c->n_src = n;
 }
 
 // Face-class coefficient table [n_freq][2 + n_port]: i k0 sqrt(eps_bg) (open), 0 (metal),
@@ -2431,8 +2437,8 @@ mw_status mw_set_sources(mw_ctx* c, int32_t n_src, const double* pos, const doub
       d_n = upload(c, nrm.data(), nrm.size());
       install_sources(c, n_src, false, ptr, c->src_edge, d_w, d_n);
     } catch (...) {
-      if (c->d_q_w != d_w) dfree(c, d_w);
-      if (c->d_q_norm != d_n) dfree(c, d_n);
+      dfree(c, d_w);
+      dfree(c, d_n);
       throw;
     }
     if (edge_out) std::memcpy(edge_out, c->src_edge.data(), sizeof(int32_t) * n_src);
@@ -2627,8 +2633,8 @@ mw_status mw_set_ports(mw_ctx* c, int32_t n_port, const mw_port* ports, int64_t 
       install_sources(c, n_port, true, qptr, qedge, d_w, d_n);
     } catch (...) {
       for (void* q : tmp) dfree(c, q);
-      if (c->d_q_w != d_w) dfree(c, d_w);
-      if (c->d_q_norm != d_n) dfree(c, d_n);
+      dfree(c, d_w);
+      dfree(c, d_n);
       throw;
     }
     c->src_edge.clear();

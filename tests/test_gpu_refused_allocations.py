@@ -186,3 +186,31 @@ def test_matrices_of_several_frequencies():
     assert _climb(c, lambda: c.assemble(freqs, eps, EPS_MATCHING), between, step=1 << 14) > 10
     assert all(np.array_equal(c.get_matrix(f), want[f]) for f in range(3))
     c.close()
+
+
+def test_sources():
+    """Sources that were refused a table are no sources, and their vectors are freed once."""
+    from paper_2311_05322_gb300 import mw as lib
+    mw, m, c, E = _context(lib.MW_PREC_BF16)
+    c.set_autotune(False)
+    rng = np.random.default_rng(1)
+    pos = rng.uniform(-0.009, 0.009, (40, 3))
+    z = np.tile([0.0, 0.0, 1.0], (40, 1))
+    o = mw.solve_opts(mode=1, restart=10, tol=1e-9, inner_tol=1e-2)
+    c.set_sources(pos, z)
+    want, _ = c.solve(o)
+    c.set_sources(pos[:7], z[:7])           # drops the fields, which the tables would otherwise find room in
+    seen = set()
+
+    def between():
+        with pytest.raises(mw.MWError) as e:
+            c.solve(o)                      # no sources, or no memory for the fields of the old ones
+        seen.add(e.value.status)
+        if e.value.status == mw.MW_ESTATE:
+            c.set_memory_cap(0)
+            c.set_sources(pos[:7], z[:7])
+
+    _climb(c, lambda: c.set_sources(pos, z), between, step=16, start=_used(c))
+    assert seen == {mw.MW_ENOMEM, mw.MW_ESTATE}
+    assert np.array_equal(c.solve(o)[0], want)
+    c.close()
