@@ -3655,11 +3655,14 @@ static void nn_free(Ctx* c) {
 static void nn_batch_buffers(Ctx* c, int B) {
   NnState& n = c->nn;
   if (B <= n.bcap) return;
-  for (void* p : {(void*)n.x, (void*)n.h1, (void*)n.h2, (void*)n.g1,
-                  (void*)n.g2, (void*)n.y, (void*)n.t, (void*)n.dy, (void*)n.da2,
-                  (void*)n.da1, (void*)n.dz2, (void*)n.dz1, (void*)n.gws,
-                  (void*)n.cpart, (void*)n.wpart, (void*)n.part})
-    dfree(c, p);
+  n.bcap = 0;   // no batch fits until every buffer is there
+  for (float** p : {&n.x, &n.h1, &n.h2, &n.g1, &n.g2, &n.y, &n.t, &n.dy, &n.da2, &n.da1, &n.dz2, &n.dz1, &n.gws, &n.cpart,
+                    &n.wpart}) {
+    dfree(c, *p);
+    *p = nullptr;
+  }
+  dfree(c, n.part);
+  n.part = nullptr;
   n.wpart = dalloc<float>(c, (size_t)mwk::kConvChunks * 400 * 64);
   n.gws = dalloc<float>(c, (size_t)32 * B * kHid);
   n.cpart = dalloc<float>(c, (size_t)26 * B);
@@ -3758,18 +3761,23 @@ mw_status mw_nn_init(mw_ctx* c, int32_t n_in, const float* theta) {
     n.oC3 = o; o += 8 * 2 * 64;
     n.oc3 = o; o += 2;
     for (int64_t i = 0; i < n.np; ++i) require(std::isfinite(theta[i]), MW_EINVAL, "non-finite parameter");
-    n.theta = upload(c, theta, n.np);
-    n.grad = dalloc<float>(c, n.np);
-    n.m = dalloc<float>(c, n.np);
-    n.v = dalloc<float>(c, n.np);
-    CK(cudaMemsetAsync(n.m, 0, sizeof(float) * n.np, c->stream));
-    CK(cudaMemsetAsync(n.v, 0, sizeof(float) * n.np, c->stream));
-    n.W1b = dalloc<uint16_t>(c, (size_t)kHid * n_in);
-    n.W2b = dalloc<uint16_t>(c, (size_t)kHid * kHid);
-    n.loss = dalloc<double>(c, 1);
-    nn_refresh_bf16(c);
-    check_launch("nn init");
-    CK(cudaStreamSynchronize(c->stream));
+    try {
+      n.theta = upload(c, theta, n.np);
+      n.grad = dalloc<float>(c, n.np);
+      n.m = dalloc<float>(c, n.np);
+      n.v = dalloc<float>(c, n.np);
+      CK(cudaMemsetAsync(n.m, 0, sizeof(float) * n.np, c->stream));
+      CK(cudaMemsetAsync(n.v, 0, sizeof(float) * n.np, c->stream));
+      n.W1b = dalloc<uint16_t>(c, (size_t)kHid * n_in);
+      n.W2b = dalloc<uint16_t>(c, (size_t)kHid * kHid);
+      n.loss = dalloc<double>(c, 1);
+      nn_refresh_bf16(c);
+      check_launch("nn init");
+      CK(cudaStreamSynchronize(c->stream));
+    } catch (...) {
+      nn_free(c);   // theta alone would pass for a network
+      throw;
+    }
   });
 }
 

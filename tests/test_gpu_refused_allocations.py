@@ -214,3 +214,35 @@ def test_sources():
     assert seen == {mw.MW_ENOMEM, mw.MW_ESTATE}
     assert np.array_equal(c.solve(o)[0], want)
     c.close()
+
+
+def test_network():
+    """A network that was refused a buffer is none, and a batch that was refused one leaves no room for smaller ones."""
+    from paper_2311_05322_gb300 import inversion, mw
+    n_in, rng = 9, np.random.default_rng(2)
+    th = inversion.he_init(n_in, 2)
+    x = rng.normal(size=(24, n_in)).astype(np.float32)
+    t = (0.1 * rng.normal(size=(24, 2, 32, 32, 32))).astype(np.float32)
+    c = mw.Context(0)
+    c.nn_init(n_in, th)
+    want, small = c.nn_infer(x), c.nn_infer(x[:2])
+    losses, _ = c.nn_train(x, t, batch=10, epochs=2, lr=1e-3, seed=1)
+    params = c.nn_get_params()
+    c.close()
+    c = mw.Context(0)
+
+    def none():
+        with pytest.raises(mw.MWError) as e:
+            c.nn_infer(x[:2])
+        assert e.value.status == mw.MW_ESTATE
+
+    assert _climb(c, lambda: c.nn_init(n_in, th), none, step=1 << 18) > 10
+    assert np.array_equal(c.nn_infer(x[:2]), small)
+    got = []
+    between = lambda: np.testing.assert_array_equal(c.nn_infer(x[:2]), small)
+    assert _climb(c, lambda: got.append(c.nn_infer(x)), between, step=1 << 18, start=_used(c)) > 5
+    assert np.array_equal(got[-1], want)
+    assert _climb(c, lambda: got.append(c.nn_train(x, t, batch=10, epochs=2, lr=1e-3, seed=1)), between, step=1 << 18,
+                  start=_used(c)) > 5
+    assert np.array_equal(got[-1][0], losses) and np.array_equal(c.nn_get_params(), params)
+    c.close()
