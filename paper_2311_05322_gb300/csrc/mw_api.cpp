@@ -2009,6 +2009,20 @@ void drop_assembly(Ctx* c) {
   c->n_freq = 0;
 }
 
+// Drops the boundary classes and the ports, with the ports' sources (dipoles stay).
+void drop_classes(Ctx* c) {
+  for (void* q : {(void*)c->d_bface_cls, (void*)c->d_metal, (void*)c->d_nzmask, (void*)c->d_zc}) dfree(c, q);
+  c->d_bface_cls = nullptr;
+  c->d_metal = c->d_nzmask = nullptr;
+  c->d_zc = nullptr;
+  if (c->src_ports) free_sources(c);
+  c->src_ports = false;
+  c->n_port = 0;
+  c->ports.clear();
+  c->bface_cls.clear();
+  c->metal.clear();
+}
+
 // Boundary face with sorted vertices (a, b, c): index into bface_vert (sorted triples), or -1.
 int64_t find_bface(const mw::Topology& t, int32_t a, int32_t b, int32_t cc) {
   int64_t lo = 0, hi = t.n_bface;
@@ -2567,10 +2581,13 @@ mw_status mw_set_ports(mw_ctx* c, int32_t n_port, const mw_port* ports, int64_t 
     }
     // commit: the boundary changed, so everything assembled from it goes
     drop_assembly(c);
-    for (void* q : {(void*)c->d_bface_cls, (void*)c->d_metal, (void*)c->d_nzmask, (void*)c->d_zc}) dfree(c, q);
-    c->d_bface_cls = nullptr;
-    c->d_metal = c->d_nzmask = nullptr;
-    c->d_zc = nullptr;
+    drop_classes(c);
+    struct Undo {   // an exception on the way leaves a boundary without classes and no ports
+      Ctx* c;
+      ~Undo() {
+        if (c) drop_classes(c);
+      }
+    } undo{c};
     c->n_port = n_port;
     c->ports.assign(ports, ports + n_port);
     const bool any_class = n_face > 0;
@@ -2581,8 +2598,10 @@ mw_status mw_set_ports(mw_ctx* c, int32_t n_port, const mw_port* ports, int64_t 
       c->d_metal = upload(c, metal.data(), metal.size());
       c->d_nzmask = upload(c, nzm.data(), nzm.size());
     }
-    if (c->src_ports) free_sources(c);  // the previous ports' sources are stale
-    if (n_port == 0) return;
+    if (n_port == 0) {
+      undo.c = nullptr;
+      return;
+    }
     // port load vectors and norms on the device
     std::vector<double> pdesc(10 * n_port), gx, gw;
     for (int p = 0; p < n_port; ++p) {
@@ -2637,6 +2656,7 @@ mw_status mw_set_ports(mw_ctx* c, int32_t n_port, const mw_port* ports, int64_t 
       dfree(c, d_n);
       throw;
     }
+    undo.c = nullptr;
     c->src_edge.clear();
     c->src_sign.clear();
   });

@@ -246,3 +246,41 @@ def test_network():
                   start=_used(c)) > 5
     assert np.array_equal(got[-1][0], losses) and np.array_equal(c.nn_get_params(), params)
     c.close()
+
+
+def test_ports():
+    """Ports that were refused a buffer leave a boundary without classes: the matrix of an open boundary, no sources."""
+    from paper_2311_05322_gb300 import mw
+    from phantom import waveguide_section
+    m, fv, lab, ps = waveguide_section((4, 2, 6), 0.02, 0.01, 0.03, 59.0 - 1.0j)
+    eps = np.tile([59.0, -1.0], (m.n_tet, 1))
+    c = mw.Context(0)
+    c.set_mesh(m.xyz, m.tets)
+    c.assemble([8e8], eps, EPS_MATCHING)
+    open_ = c.get_matrix(0)
+    ports = lambda: c.set_ports(ps.origin, ps.u, ps.v, ps.a, ps.eps_fill, fv, lab)
+    ports()
+    W, n = c.get_port_vectors()
+    c.assemble([8e8], eps, EPS_MATCHING)
+    closed = c.get_matrix(0)
+    assert not np.array_equal(open_, closed)
+    c.close()
+    c = mw.Context(0)
+    c.set_mesh(m.xyz, m.tets)
+    ports()                                  # the ports that the refused ones replace
+
+    def between():
+        with pytest.raises(mw.MWError) as e:
+            c.get_port_vectors()
+        assert e.value.status == mw.MW_ESTATE
+        c.set_memory_cap(0)
+        c.assemble([8e8], eps, EPS_MATCHING)
+        assert np.array_equal(c.get_matrix(0), open_)
+
+    ports()
+    start = _used(c) - 4096                  # the classes go first: refusals begin below what is held
+    _climb(c, ports, between, step=256, start=start)
+    W2, n2 = c.get_port_vectors()
+    c.assemble([8e8], eps, EPS_MATCHING)
+    assert np.array_equal(W, W2) and np.array_equal(n, n2) and np.array_equal(c.get_matrix(0), closed)
+    c.close()
