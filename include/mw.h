@@ -441,7 +441,8 @@ mw_status mw_forward_cols(mw_ctx* ctx, const mw_solve_opts* opts, int32_t j0, in
 /* For the window of the last mw_forward_cols (same eps): J_out = the data cost of the whole
  * S_full (host complex128 [n_freq][n_src][n_src], the gathered S), the adjoint solves of the
  * window's columns with c_ij = w_ij conj(S_full_ij - S_obs_ij), and grad_part (host [n_tet][2])
- * = that window's share of dJ/d(Re eps, Im eps).  MW_ESTATE without a prior window.
+ * = that window's share of dJ/d(Re eps, Im eps).  n_freq n_src^2 <= 2^20 (MW_EINVAL).  MW_ESTATE
+ * without a prior window.
  * Synchronises. */
 mw_status mw_gradient_cols(mw_ctx* ctx, const mw_solve_opts* opts, const double* S_full, const double* S_obs,
                            const double* S_empty, double* J_out, double* grad_part);

@@ -42,6 +42,7 @@ void normalize_start_f32(const double2* r, const double* rnorm, const int32_t* d
 namespace mwimpl {
 
 constexpr int kMaxRestart = 63;
+constexpr size_t kMaxS = 64 * 128 * 128;   // values of S, of its data and weights: 64 frequencies of 128 sources
 
 // Launch-shape value (mw_launch_shapes.spmm_threads) that selects the halo-tiled SpMM.
 constexpr int kSpmmHaloShape = 1;
@@ -3023,8 +3024,8 @@ static void gradient_dev_impl(Ctx* c, const mw_solve_opts& o, const double2* dSo
   const size_t nS = (size_t)nf * ns * ns;
   forward(c, o, nullptr);
   alloc_fields(c, c->Lf);
-  if (!c->d_S) c->d_S = dalloc<double2>(c, 64 * 128 * 128);
-  if (!c->d_C) c->d_C = dalloc<double2>(c, 64 * 128 * 128);
+  if (!c->d_S) c->d_S = dalloc<double2>(c, kMaxS);
+  if (!c->d_C) c->d_C = dalloc<double2>(c, kMaxS);
   if (!c->d_J) c->d_J = dalloc<double>(c, 4);
   alloc_fields(c, c->d_Badj);
   for (int f = 0; f < nf; ++f)
@@ -3118,10 +3119,11 @@ static void gradient_cols_impl(Ctx* c, const mw_solve_opts& o, const double* S_f
   const int64_t E = c->topo.n_edge, T = c->topo.n_tet;
   const int ns = c->n_src, nf = c->n_freq, j0 = c->win_j0, nl = c->win_nl;
   const size_t nS = (size_t)nf * ns * ns;
-  if (!c->d_S) c->d_S = dalloc<double2>(c, 64 * 128 * 128);
-  if (!c->d_C) c->d_C = dalloc<double2>(c, 64 * 128 * 128);
-  if (!c->d_So) c->d_So = dalloc<double2>(c, 64 * 128 * 128);
-  if (!c->d_Se) c->d_Se = dalloc<double2>(c, 64 * 128 * 128);
+  require(nS <= kMaxS, MW_EINVAL, "the sharded gradient holds n_freq n_src^2 <= 2^20 values of S");
+  if (!c->d_S) c->d_S = dalloc<double2>(c, kMaxS);
+  if (!c->d_C) c->d_C = dalloc<double2>(c, kMaxS);
+  if (!c->d_So) c->d_So = dalloc<double2>(c, kMaxS);
+  if (!c->d_Se) c->d_Se = dalloc<double2>(c, kMaxS);
   if (!c->d_J) c->d_J = dalloc<double>(c, 4);
   if (!c->d_grad) c->d_grad = dalloc<double>(c, 2 * T);
   CK(cudaMemcpyAsync(c->d_S, S_full, sizeof(double2) * nS, cudaMemcpyHostToDevice, c->stream));
@@ -3189,11 +3191,12 @@ mw_status mw_gradient_cols(mw_ctx* c, const mw_solve_opts* opts, const double* S
 static void gradient_impl(Ctx* c, const mw_solve_opts& o, const double* S_obs, const double* S_empty, double alpha,
                           double* J_out, double* grad, double* S_out) {
   require(c->has_mesh && c->n_freq > 0 && c->n_src > 0, MW_ESTATE, "assemble and set sources first");
+  require(c->n_src <= 128, MW_EINVAL, "gradient supports at most 128 sources");   // before S is copied
   require(S_obs && S_empty && J_out, MW_EINVAL, "null S_obs / S_empty / J_out");
   const int64_t T = c->topo.n_tet;
   const size_t nS = (size_t)c->n_freq * c->n_src * c->n_src;
-  if (!c->d_So) c->d_So = dalloc<double2>(c, 64 * 128 * 128);
-  if (!c->d_Se) c->d_Se = dalloc<double2>(c, 64 * 128 * 128);
+  if (!c->d_So) c->d_So = dalloc<double2>(c, kMaxS);
+  if (!c->d_Se) c->d_Se = dalloc<double2>(c, kMaxS);
   if (!c->d_grad) c->d_grad = dalloc<double>(c, 2 * T);
   CK(cudaMemcpyAsync(c->d_So, S_obs, sizeof(double2) * nS, cudaMemcpyHostToDevice, c->stream));
   CK(cudaMemcpyAsync(c->d_Se, S_empty, sizeof(double2) * nS, cudaMemcpyHostToDevice, c->stream));

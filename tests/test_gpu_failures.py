@@ -64,3 +64,22 @@ def test_bounded_wait_runs_out_and_context_stays_usable():
     c.setup_preconditioner(4, box_partition(m, (2, 2, 1)), 1, mw.MW_PREC_FP64)
     S, st = c.solve(mw.solve_opts(tol=1e-10))
     assert st["n_converged"] == 1
+
+
+def test_s_matrices_beyond_their_buffers_are_refused():
+    """The buffers of S hold 2^20 values: more sources are an error before anything is copied."""
+    mw, m, c = _small()
+    c.assemble([1e9], np.tile([44.0, -20.0], (m.n_tet, 1)), EPS_MATCHING)
+    n = 1100
+    pos = np.random.default_rng(3).uniform(-0.015, 0.015, (n, 3))
+    c.set_sources(pos, np.tile([0.0, 0.0, 1.0], (n, 1)))
+    c.setup_preconditioner(4, box_partition(m, (2, 2, 1)), 1, mw.MW_PREC_FP64)
+    S = np.ones((1, n, n), complex)
+    o = mw.solve_opts(tol=1e-8)
+    for call in (lambda: c.gradient(S, S, 0.0, o), lambda: (c.forward_cols(5, 2, o), c.gradient_cols(S, S, S, o))):
+        with pytest.raises(mw.MWError) as e:
+            call()
+        assert e.value.status == mw.MW_EINVAL
+    c.set_sources(pos[:3], np.tile([0.0, 0.0, 1.0], (3, 1)))
+    S3, _ = c.solve(o)
+    assert np.isfinite(c.gradient(S3 * 1.1, np.ones_like(S3), 0.0, o)[0])
