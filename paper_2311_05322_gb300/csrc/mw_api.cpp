@@ -2231,6 +2231,12 @@ mw_status mw_set_mesh(mw_ctx* c, int64_t n_vert, const double* xyz, int64_t n_te
   return guard(c, [&] {
     require(xyz && tv, MW_EINVAL, "null mesh arrays");
     release_mesh(c);
+    struct Undo {   // an exception on the way leaves no mesh and none of its buffers
+      Ctx* c;
+      ~Undo() {
+        if (!c->has_mesh) release_mesh(c);
+      }
+    } undo{c};
     Error err{MW_OK, ""};
     if (!mw::build_topology(n_vert, n_tet, tv, c->topo, err)) throw Fail{err.code, err.msg};
     for (int64_t i = 0; i < 3 * n_vert; ++i) require(std::isfinite(xyz[i]), MW_EINVAL, "non-finite vertex coordinate");
@@ -2691,6 +2697,12 @@ mw_status mw_setup_preconditioner(mw_ctx* c, int32_t n_sub, const int32_t* part,
                                                        "BF16 tensor-core sweeps)");
     release_prec(c);
     Prec& p = c->prec;
+    struct Undo {   // an exception on the way leaves no preconditioner and none of its buffers
+      Ctx* c;
+      ~Undo() {
+        if (!c->prec.ready) release_prec(c);
+      }
+    } undo{c};
     Error err{MW_OK, ""};
     if (!mw::build_subdomains(c->topo, n_sub, part, overlap, p.sd, err)) throw Fail{err.code, err.msg};
     const mw::Subdomains& sd = p.sd;
@@ -2730,12 +2742,7 @@ mw_status mw_setup_preconditioner(mw_ctx* c, int32_t n_sub, const int32_t* part,
     mwk::face_geom(c->d_xyz, p.surf_vert, n_surf, p.Bsurf, c->stream);
     if (inv_prec == 4 || inv_prec == 5) {
       for (int s = 0; s < n_sub; ++s) p.sum_n += (double)(sd.dof_ptr[s + 1] - sd.dof_ptr[s]);
-      try {
-        setup_sparse(c);
-      } catch (...) {
-        release_prec(c);
-        throw;
-      }
+      setup_sparse(c);
       p.ready = true;
       return;
     }
@@ -2882,7 +2889,6 @@ mw_status mw_setup_preconditioner(mw_ctx* c, int32_t n_sub, const int32_t* part,
       require(st == 0, MW_ESINGULAR, "a subdomain matrix had a near-zero pivot");
     } catch (...) {
       for (void* q : tmp) dfree(c, q);
-      release_prec(c);
       throw;
     }
     for (void* q : tmp) dfree(c, q);

@@ -284,3 +284,40 @@ def test_ports():
     c.assemble([8e8], eps, EPS_MATCHING)
     assert np.array_equal(W, W2) and np.array_equal(n, n2) and np.array_equal(c.get_matrix(0), closed)
     c.close()
+
+
+@pytest.mark.parametrize("prec", ["FP64", "FP32", "BF16", "SPARSE", "SPARSE_BF16"])
+def test_mesh_and_preconditioner(prec):
+    """A mesh or a preconditioner that was refused a buffer is none, and holds nothing."""
+    from paper_2311_05322_gb300 import mw as lib
+    mw, m, c, E = _context(None)
+    part = box_partition(m, (2, 2, 1))
+    code = getattr(lib, "MW_PREC_" + prec)
+    held = _used(c)
+    r = torch.ones((E, 3), dtype=torch.complex128, device="cuda")
+    want, z = torch.empty_like(r), torch.empty_like(r)
+    c.setup_preconditioner(4, part, 1, code)
+    c.apply_preconditioner(0, r, want, 3)
+    c.close()
+    mw, m, c, E = _context(None)
+
+    def between():
+        with pytest.raises(mw.MWError) as e:
+            c.apply_preconditioner(0, r, z, 3)
+        assert e.value.status == mw.MW_ESTATE
+        assert _used(c) == held
+
+    assert _climb(c, lambda: c.setup_preconditioner(4, part, 1, code), between, step=1 << 14, start=held) > 5
+    c.apply_preconditioner(0, r, z, 3)
+    assert torch.equal(torch.view_as_real(z), torch.view_as_real(want))
+    c.close()
+    c = mw.Context(0)
+
+    def none():
+        with pytest.raises(mw.MWError) as e:
+            c.assemble([1e9], np.tile([EPS_MATCHING.real, EPS_MATCHING.imag], (m.n_tet, 1)), EPS_MATCHING)
+        assert e.value.status == mw.MW_ESTATE
+        assert _used(c) == 0
+
+    assert _climb(c, lambda: c.set_mesh(m.xyz, m.tets), none, step=1 << 13) > 5
+    c.close()
